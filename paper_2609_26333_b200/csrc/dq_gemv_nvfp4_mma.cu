@@ -118,17 +118,17 @@ gemv_nvfp4_mma_kernel(const uint8_t *__restrict__ codes, const uint8_t *__restri
     const int c_begin = w * kChunksPerSlice;
     const int c_end = min(c_begin + kChunksPerSlice, nchunks);
 
-    // Register ring of NPF chunks in flight per lane.  Every tile takes eight ring positions (a short last
-    // slice leaves some unused), so position p of the warp's stream is chunk c_begin + p % 8 of tile
-    // first + (p / 8) * stride and lives in ring[p % NPF].
+    // Register ring of NPF chunks in flight per lane.  Every tile takes kPos ring positions: its eight chunks (a short
+    // last slice leaves some unused) rounded up to a multiple of NPF, so that a tile's chunk k8 lives in ring[k8 % NPF]
+    // whatever tile it is.  Position p of the warp's stream is chunk c_begin + p % kPos of tile first + (p / kPos) * stride.
     // The weights are constant data: start streaming before waiting for the kernel ahead of this one.
+    constexpr int kPos = (kChunksPerSlice + NPF - 1) / NPF * NPF;
     ChunkRegs ring[NPF];
 #pragma unroll
     for (int p = 0; p < NPF; ++p) {
         ring[p].c[0] = ring[p].c[1] = make_uint4(0, 0, 0, 0);
         ring[p].sc[0] = ring[p].sc[1] = 0;
-        const int tile2 = first + (p >> 3) * stride, c2 = c_begin + (p & 7);
-        if (tile2 < ntiles && c2 < c_end) load_chunk(ring[p], tile2, c2);
+        if (first < ntiles && c_begin + p < c_end) load_chunk(ring[p], first, c_begin + p);
     }
 
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -188,12 +188,12 @@ gemv_nvfp4_mma_kernel(const uint8_t *__restrict__ codes, const uint8_t *__restri
     for (int tile = first; tile < ntiles; tile += stride, ++it) {
         float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int k8 = 0; k8 < 8; ++k8) {
+        for (int k8 = 0; k8 < kPos; ++k8) {                      // positions past the eight chunks: loads ahead only
             const int c = c_begin + k8;
             const ChunkRegs cur = ring[k8 % NPF];
             {   // issue the loads of the chunk NPF positions ahead into this slot before working on the current one
                 const int k2 = k8 + NPF;
-                const int tile2 = tile + (k2 >> 3) * stride, c2 = c_begin + (k2 & 7);
+                const int tile2 = tile + (k2 / kPos) * stride, c2 = c_begin + (k2 % kPos);
                 if (tile2 < ntiles && c2 < c_end) load_chunk(ring[k8 % NPF], tile2, c2);
             }
             if (c < c_end) {

@@ -304,6 +304,19 @@ def test_decode_nvfp4_parity(dq, oracle, N, K, seed, B):
             dq.decode_linear_nvfp4(w3, X.to(DEV))
 
 
+@pytest.mark.parametrize("N,K,seed,B", [(19200, 1152, 35, 1), (9600, 5120, 36, 9), (3200, 17408, 37, 2)])
+def test_decode_nvfp4_several_row_tiles_per_cta(dq, oracle, N, K, seed, B):
+    """More row tiles than the grid takes in one round, at the row lengths whose warps keep three chunks in flight (the
+    eight chunks of a tile are not a multiple of three)."""
+    W, ref = _layer(oracle, N, K, seed)
+    w = dq.pack_weights(W.to(DEV), formats=dq.FMT_NVFP4)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, seed + 200 + B)
+    Y = dq.decode_linear_nvfp4(w, X.to(DEV))
+    _status_ok(dq)
+    Yr, S = oracle.decode_linear_nvfp4(dq_inputs.bf16_to_f32_numpy(X), ref["nvfp4_codes"], ref["nvfp4_scales"], ref["s"])
+    check_outputs(_f64(Y), Yr, S, f"nvfp4 decode {B}x{N}x{K}")
+
+
 def test_decode_nvfp4_kernels_agree_and_handle_wide_range_activations(dq, oracle):
     """The tensor-core kernel (default) and the CUDA-core kernel both meet the oracle; activations spanning
     many binades (the tensor-core kernel rescales them to fp16) and strided, guarded outputs."""
