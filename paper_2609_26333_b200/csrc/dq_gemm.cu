@@ -7,8 +7,8 @@
 //   warp 0      : TMA producer (packed FP4 tiles, 128B swizzle) + bulk copies of the scale atoms
 //   warp 1      : tcgen05.cp of the scales into TMEM and tcgen05.mma (kind::mxf4nvf4, block 16)
 //   warps 2..5  : epilogue, TMEM -> registers -> bf16 -> global
-// The fp32 accumulator lives in TMEM (256 columns); the per-stage scale factors
-// occupy 2 x 48 further columns.  Every mbarrier wait is bounded: when it runs
+// The fp32 accumulator lives in TMEM (256 columns); the scale factors of the four stages
+// occupy 4 x 48 further columns.  Every mbarrier wait is bounded: when it runs
 // out the CTA records DQ_ERR_TIMEOUT in the status word and leaves normally.
 #include <cuda.h>
 
@@ -33,7 +33,7 @@ constexpr uint32_t SMEM_BYTES = kStages * STAGE_BYTES + 1024 /*align*/ + 256 /*b
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemSfBase = 256;         // accumulator uses columns [0, 256)
-constexpr uint32_t kTmemSfBufCols = 48;       // 16 (A) + 32 (B) per stage, double buffered
+constexpr uint32_t kTmemSfBufCols = 48;       // 16 (A) + 32 (B), one buffer per smem stage: free again when the stage is
 
 static_assert(STAGE_BYTES % 1024 == 0, "stage must keep 1024-byte alignment for the 128B swizzle");
 
@@ -105,70 +105,78 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0) {
+        {
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
                 int mb, nb;
                 tile_coords(t, tiles_m, tiles_n, mb, nb);
                 for (int ks = 0; ks < num_ks; ++ks) {
-                    if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
                     const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
                     const uint32_t sA = smem_base + stage * STAGE_BYTES;
                     const uint32_t sB = sA + A_STAGE_BYTES;
                     const uint32_t sSFA = sB + B_STAGE_BYTES;
                     const uint32_t sSFB = sSFA + SFA_STAGE_BYTES;
                     const uint32_t sf_bytes = (uint32_t)nkb * 512u;
-                    mbar_expect_tx(full_bar(stage), A_STAGE_BYTES + B_STAGE_BYTES + 3u * sf_bytes);
-                    tma_load_2d(sA, &tmap_a, ks * 128, mb * BM, full_bar(stage));
-                    tma_load_2d(sB, &tmap_w, ks * 128, nb * BN, full_bar(stage));
                     const size_t koff = (size_t)ks * kKbPerStage * 512;
-                    bulk_load(sSFA, a_sf + ((size_t)mb * katoms) * 512 + koff, sf_bytes, full_bar(stage));
-                    bulk_load(sSFB, w_sf + ((size_t)(2 * nb) * katoms) * 512 + koff, sf_bytes, full_bar(stage));
-                    bulk_load(sSFB + kKbPerStage * 512, w_sf + ((size_t)(2 * nb + 1) * katoms) * 512 + koff, sf_bytes,
-                              full_bar(stage));
+                    if (elect_one()) {
+                        mbar_expect_tx(full_bar(stage), A_STAGE_BYTES + B_STAGE_BYTES + 3u * sf_bytes);
+                        tma_load_2d(sA, &tmap_a, ks * 128, mb * BM, full_bar(stage));
+                        tma_load_2d(sB, &tmap_w, ks * 128, nb * BN, full_bar(stage));
+                        bulk_load(sSFA, a_sf + ((size_t)mb * katoms) * 512 + koff, sf_bytes, full_bar(stage));
+                        bulk_load(sSFB, w_sf + ((size_t)(2 * nb) * katoms) * 512 + koff, sf_bytes, full_bar(stage));
+                        bulk_load(sSFB + kKbPerStage * 512, w_sf + ((size_t)(2 * nb + 1) * katoms) * 512 + koff, sf_bytes,
+                                  full_bar(stage));
+                    }
+                    __syncwarp();
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
-        if (lane == 0) {
+        {
             int stage = 0; uint32_t phase = 0;
             uint32_t acc_phase = 0;
-            uint32_t sfbuf = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-                if (!mbar_wait(tmem_empty_bar, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(tmem_empty_bar, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 for (int ks = 0; ks < num_ks; ++ks) {
-                    if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
                     const uint32_t sA = smem_base + stage * STAGE_BYTES;
                     const uint32_t sB = sA + A_STAGE_BYTES;
                     const uint32_t sSFA = sB + B_STAGE_BYTES;
                     const uint32_t sSFB = sSFA + SFA_STAGE_BYTES;
-                    const uint32_t t_sfa = tmem_base + kTmemSfBase + sfbuf * kTmemSfBufCols;
+                    const uint32_t t_sfa = tmem_base + kTmemSfBase + (uint32_t)stage * kTmemSfBufCols;
                     const uint32_t t_sfb = t_sfa + 16u;
-                    for (int kb = 0; kb < nkb; ++kb) {
-                        tmem_cp_sf(t_sfa + 4u * kb, make_desc_sf(sSFA + 512u * kb));
-                        tmem_cp_sf(t_sfb + 8u * kb, make_desc_sf(sSFB + 512u * kb));
-                        tmem_cp_sf(t_sfb + 8u * kb + 4u, make_desc_sf(sSFB + kKbPerStage * 512u + 512u * kb));
+                    const uint64_t adesc = make_desc_sw128(sA), bdesc = make_desc_sw128(sB);
+                    const uint64_t fadesc = make_desc_sf(sSFA), fbdesc = make_desc_sf(sSFB);
+                    if (elect_one()) {
+#pragma unroll
+                        for (int kb = 0; kb < kKbPerStage; ++kb) {
+                            if (kb < nkb) {
+                                tmem_cp_sf(t_sfa + 4u * kb, fadesc + 32ull * kb);
+                                tmem_cp_sf(t_sfb + 8u * kb, fbdesc + 32ull * kb);
+                                tmem_cp_sf(t_sfb + 8u * kb + 4u, fbdesc + (kKbPerStage * 512u >> 4) + 32ull * kb);
+                            }
+                        }
+#pragma unroll
+                        for (int kb = 0; kb < kKbPerStage; ++kb) {
+                            // one k-step is 64 elements = 32 bytes inside the 128-byte swizzle row
+                            if (kb < nkb)
+                                mma_nvf4(tmem_base, adesc + 2ull * kb, bdesc + 2ull * kb, kInstrDesc, t_sfa + 4u * kb,
+                                         t_sfb + 8u * kb, (ks > 0 || kb > 0) ? 1u : 0u);
+                        }
+                        mma_commit(empty_bar(stage));          // frees the stage once these MMAs have read it
+                        if (ks + 1 == num_ks) mma_commit(tmem_full_bar);       // accumulator complete
                     }
-                    const uint64_t adesc = make_desc_sw128(sA);
-                    const uint64_t bdesc = make_desc_sw128(sB);
-                    for (int kb = 0; kb < nkb; ++kb) {
-                        // one k-step is 64 elements = 32 bytes inside the 128-byte swizzle row
-                        mma_nvf4(tmem_base, adesc + 2ull * kb, bdesc + 2ull * kb, kInstrDesc, t_sfa + 4u * kb,
-                                 t_sfb + 8u * kb, (ks > 0 || kb > 0) ? 1u : 0u);
-                    }
-                    mma_commit(empty_bar(stage));          // frees the stage once these MMAs have read it
-                    sfbuf ^= 1u;
+                    __syncwarp();
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
-                if (!ok) break;
-                mma_commit(tmem_full_bar);                 // accumulator complete
                 acc_phase ^= 1u;
             }
         }

@@ -11,11 +11,9 @@
 //                 signal barriers of the leader (scales and operands separately)
 //   warp 1      : (leader) tcgen05.mma; commits release the smem stage in both CTAs and
 //                 publish the accumulator to both
-//   warps 2, 3  : (leader) tcgen05.cp of the stage's scale atoms into TMEM, one TMEM
-//                 scale buffer per smem stage; the two warps take alternate k-steps.  Copies issued from their own thread
-//                 run concurrently with the MMAs; issued from the MMA thread they
-//                 serialise with them (measured: 490 us vs 240 us on 8192x17408x5120)
-//   warps 4..11 : epilogue; TMEM -> registers, TMEM released at once, then scale, bf16
+//   warp 2      : (leader) tcgen05.cp of the stage's scale atoms into TMEM, one TMEM
+//                 scale buffer per smem stage, ahead of the MMAs that read it
+//   warps 3..10 : epilogue; TMEM -> registers, TMEM released at once, then scale, bf16
 //                 convert, swizzled smem staging and TMA stores overlap the next tile's MMAs
 // Every wait is bounded; a wait that runs out sets DQ_ERR_TIMEOUT and all roles
 // of both CTAs leave through the common exit.
@@ -62,8 +60,7 @@ struct Cfg {
     static constexpr uint32_t STG_OFF = kStages * STAGE_BYTES;                    // epilogue staging, 1024-byte aligned
     static constexpr uint32_t BAR_OFF = STG_OFF + kEpiWarps * STG_WARP_BYTES;
     static constexpr uint32_t SMEM_BYTES = BAR_OFF + 1024 + 256;
-    static constexpr int kScaleWarps = 2;                          // warps 2 .. 1 + kScaleWarps
-    static constexpr int kFirstEpiWarp = 2 + kScaleWarps;
+    static constexpr int kFirstEpiWarp = 3;                        // producer, MMA issue, scale copies
     static constexpr int kThreads = 32 * (kFirstEpiWarp + kEpiWarps);
     static constexpr uint32_t kTmemSfBase = BN;                                   // accumulator: BN fp32 columns
     static constexpr uint32_t kTmemSfACols = 4 * kKbPerStage;
@@ -117,15 +114,14 @@ __device__ __forceinline__ void tmem2_cp_sf(uint32_t taddr, uint32_t lo, uint32_
     asm volatile("{\n\t.reg .b64 d;\n\tmov.b64 d, {%1, %2};\n\t"
                  "tcgen05.cp.cta_group::2.32x128b.warpx4 [%0], d;\n\t}" ::"r"(taddr), "r"(lo), "r"(hi) : "memory");
 }
-template <bool ACC>
 __device__ __forceinline__ void mma2_nvf4(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t sfa,
-                                          uint32_t sfb, uint32_t idesc)
+                                          uint32_t sfb, uint32_t idesc, bool accumulate)
 {
     asm volatile("{\n\t.reg .b64 da, db;\n\t.reg .pred p;\n\tmov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
                  "setp.ne.b32 p, %7, 0;\n\t"
                  "tcgen05.mma.cta_group::2.kind::mxf4nvf4.block_scale.block16 [%0], da, db, %4, [%5], [%6], p;\n\t}"
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(sfa), "r"(sfb),
-                   "r"(ACC ? 1u : 0u) : "memory");
+                   "r"(accumulate ? 1u : 0u) : "memory");
 }
 // TMA store of one staged box (shared -> global); out-of-range rows / columns are clipped by the hardware
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *tmap, uint32_t src, int c0, int c1)
@@ -163,6 +159,26 @@ __device__ __forceinline__ bool mbar_wait2(uint32_t bar, uint32_t parity, volati
         if ((++it & 63u) == 0u) {
             if (*abort_flag) return false;
             if (clock64() - t0 > kWaitBudgetCycles) {
+                *abort_flag = 1;
+                st_remote_u32(peer_abort_addr, 1u);
+                return false;
+            }
+        }
+    }
+}
+
+// the same for a whole converged warp: every lane returns the same answer
+__device__ __forceinline__ bool mbar_wait2_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag,
+                                                uint32_t peer_abort_addr)
+{
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    const long long t0 = clock64();
+    uint32_t it = 0;
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if ((++it & 63u) == 0u) {
+            const bool over = clock64() - t0 > kWaitBudgetCycles;
+            if (__any_sync(0xffffffffu, over || *abort_flag != 0)) {
                 *abort_flag = 1;
                 st_remote_u32(peer_abort_addr, 1u);
                 return false;
@@ -269,41 +285,44 @@ gemm_nvfp4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0) {
+        {
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
+            const uint32_t leader_full0 = mapa(full_bar(0), 0u), leader_sf_full0 = mapa(sf_full_bar(0), 0u);
             for (int t = pair; t < num_tiles && ok; t += npairs) {
                 int mb, nb;
                 tile_coords2(t, tiles_m, tiles_n, mb, nb, gm);
                 const int rowblk = mb * 2 + (int)rank;            // 128-row block of A this CTA owns
                 for (int ks = 0; ks < num_ks; ++ks) {
-                    if (!mbar_wait2(empty_bar(stage), phase ^ 1u, abort_flag, peer_abort)) { ok = false; break; }
+                    if (!mbar_wait2_warp(empty_bar(stage), phase ^ 1u, abort_flag, peer_abort)) { ok = false; break; }
                     const uint32_t sA = smem_base + stage * STAGE_BYTES;
                     const uint32_t sB = sA + A_BYTES;
                     const uint32_t sSFA = sB + B_BYTES;
                     const uint32_t sSFB = sSFA + SFA_BYTES;
                     // the small scale atoms go first and have their own barrier, so that their copy
                     // into TMEM overlaps the arrival of the operand tiles
-                    const uint32_t leader_full = mapa(full_bar(stage), 0u);
-                    const uint32_t leader_sf_full = mapa(sf_full_bar(stage), 0u);
-                    if (rank == 0) {
-                        mbar_expect_tx(sf_full_bar(stage), 2u * (SFA_BYTES + SFB_BYTES));
-                        mbar_expect_tx(full_bar(stage), 2u * (A_BYTES + B_BYTES));
-                    }
-                    if (!MMA_ONLY) {
-                        tma2_load_2d(sSFA, &tmap_sfa, 0, rowblk * katoms + ks * kKbPerStage, leader_sf_full);
+                    const uint32_t leader_full = leader_full0 + 8u * stage, leader_sf_full = leader_sf_full0 + 8u * stage;
+                    if (elect_one()) {
+                        if (rank == 0) {
+                            mbar_expect_tx(sf_full_bar(stage), 2u * (SFA_BYTES + SFB_BYTES));
+                            mbar_expect_tx(full_bar(stage), 2u * (A_BYTES + B_BYTES));
+                        }
+                        if (!MMA_ONLY) {
+                            tma2_load_2d(sSFA, &tmap_sfa, 0, rowblk * katoms + ks * kKbPerStage, leader_sf_full);
 #pragma unroll
-                        for (int at = 0; at < kSfbAtoms; ++at)
-                            tma2_load_2d(sSFB + (uint32_t)at * kKbPerStage * 512, &tmap_sfw, 0,
-                                         (kSfbAtoms * nb + at) * katoms + ks * kKbPerStage, leader_sf_full);
-                        tma2_load_2d(sA, &tmap_a, ks * 128, rowblk * BM, leader_full);
-                        tma2_load_2d(sB, &tmap_w, ks * 128, nb * BN + (int)rank * (BN / 2), leader_full);
-                    } else if (rank == 0) {
-                        asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(sf_full_bar(stage)),
-                                     "r"(2u * (SFA_BYTES + SFB_BYTES)) : "memory");
-                        asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(full_bar(stage)),
-                                     "r"(2u * (A_BYTES + B_BYTES)) : "memory");
+                            for (int at = 0; at < kSfbAtoms; ++at)
+                                tma2_load_2d(sSFB + (uint32_t)at * kKbPerStage * 512, &tmap_sfw, 0,
+                                             (kSfbAtoms * nb + at) * katoms + ks * kKbPerStage, leader_sf_full);
+                            tma2_load_2d(sA, &tmap_a, ks * 128, rowblk * BM, leader_full);
+                            tma2_load_2d(sB, &tmap_w, ks * 128, nb * BN + (int)rank * (BN / 2), leader_full);
+                        } else if (rank == 0) {
+                            asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(sf_full_bar(stage)),
+                                         "r"(2u * (SFA_BYTES + SFB_BYTES)) : "memory");
+                            asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(full_bar(stage)),
+                                         "r"(2u * (A_BYTES + B_BYTES)) : "memory");
+                        }
                     }
+                    __syncwarp();
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }
@@ -314,20 +333,20 @@ gemm_nvfp4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         // for everything it does, and a barrier probe alone is a round trip to shared memory.  The barriers of the
         // NEXT stage are therefore probed (without blocking) before the MMAs of this stage are issued and the answer
         // is read after them; the bounded blocking wait is only the fallback when the ring is not ahead.
-        if (rank == 0 && lane == 0) {
+        if (rank == 0) {
             int stage = 0; uint32_t phase = 0;
             uint32_t acc_phase = 0;
             bool ok = true;
             bool seen = false;          // barriers of `stage` already seen complete by the look-ahead probe
             const uint32_t a_lo0 = ((smem_base & 0x3FFFFu) >> 4) | (1u << 16);
             for (int t = pair; t < num_tiles && ok; t += npairs) {
-                if (!mbar_wait2(tmem_empty_bar, acc_phase ^ 1u, abort_flag, peer_abort)) { ok = false; break; }
+                if (!mbar_wait2_warp(tmem_empty_bar, acc_phase ^ 1u, abort_flag, peer_abort)) { ok = false; break; }
                 tc_fence_after();
                 for (int ks = 0; ks < num_ks; ++ks) {
                     // operand tiles of this stage are in smem and its scales are in TMEM
                     if (!seen) {
-                        if (!mbar_wait2(full_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
-                        if (!mbar_wait2(sf_ready_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
+                        if (!mbar_wait2_warp(full_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
+                        if (!mbar_wait2_warp(sf_ready_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
                     }
                     tc_fence_after();
                     const int nstage = (stage + 1 == kStages) ? 0 : stage + 1;
@@ -339,46 +358,43 @@ gemm_nvfp4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                     const uint32_t b_lo = a_lo + (A_BYTES >> 4);
                     const uint32_t t_sfa = tmem_base + kTmemSfBase + (uint32_t)stage * kTmemSfBufCols;
                     const uint32_t t_sfb = t_sfa + kTmemSfACols;
-                    {
-                        if (ks == 0) mma2_nvf4<false>(tmem_base, a_lo, b_lo, kDescHiSw128, t_sfa, t_sfb, kInstrDesc);
-                        else mma2_nvf4<true>(tmem_base, a_lo, b_lo, kDescHiSw128, t_sfa, t_sfb, kInstrDesc);
+                    if (elect_one()) {
+                        mma2_nvf4(tmem_base, a_lo, b_lo, kDescHiSw128, t_sfa, t_sfb, kInstrDesc, ks != 0);
 #pragma unroll
                         for (int kb = 1; kb < kKbPerStage; ++kb) {
                             if (kb < nkb)
-                                mma2_nvf4<true>(tmem_base, a_lo + 2u * kb, b_lo + 2u * kb, kDescHiSw128, t_sfa + 4u * kb,
-                                                t_sfb + 4u * kSfbAtoms * kb, kInstrDesc);
+                                mma2_nvf4(tmem_base, a_lo + 2u * kb, b_lo + 2u * kb, kDescHiSw128, t_sfa + 4u * kb,
+                                          t_sfb + 4u * kSfbAtoms * kb, kInstrDesc, true);
                         }
+                        mma2_commit_pair(empty_bar(stage));     // stage (smem and TMEM scales) reusable in both CTAs
+                        if (ks + 1 == num_ks) mma2_commit_pair(tmem_full_bar);
                     }
-                    mma2_commit_pair(empty_bar(stage));     // stage (smem and TMEM scales) reusable in both CTAs
-                    seen = next_full && next_sf;
+                    __syncwarp();
+                    seen = __all_sync(0xffffffffu, next_full && next_sf);
                     stage = nstage;
                     phase = nphase;
                 }
-                if (!ok) break;
-                mma2_commit_pair(tmem_full_bar);
                 acc_phase ^= 1u;
             }
         }
     } else if (warp < C::kFirstEpiWarp) {
         // ------------------------------- scale copies smem -> TMEM (leader CTA only)
-        // One thread can issue only about one copy per 30 ns, and a stage needs 12 of them plus the
-        // barrier round trips, which is more than the 0.4 us its MMAs take; so two threads take
-        // alternate stages (warp 2 the even k-steps, warp 3 the odd ones).
-        if (rank == 0 && lane == 0) {
+        // One warp takes all k-steps, in order.  (Two warps on alternate steps are wrong: the warp that is ahead would wait
+        // for the second phase of a stage whose first phase has not completed yet, and a parity wait lets it pass.)
+        if (rank == 0) {
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
             const uint32_t sf_lo0 = ((smem_base + A_BYTES + B_BYTES) & 0x3FFFFu) >> 4;
-            uint32_t step = 0;
             for (int t = pair; t < num_tiles && ok; t += npairs) {
-                for (int ks = 0; ks < num_ks; ++ks, ++step) {
-                    if (step % (uint32_t)C::kScaleWarps == (uint32_t)(warp - 2)) {
-                        if (!mbar_wait2(sf_full_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
-                        tc_fence_after();
-                        const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
-                        const uint32_t sfa_lo = sf_lo0 + (uint32_t)stage * (STAGE_BYTES >> 4);
-                        const uint32_t sfb_lo = sfa_lo + (SFA_BYTES >> 4);
-                        const uint32_t t_sfa = tmem_base + kTmemSfBase + (uint32_t)stage * kTmemSfBufCols;
-                        const uint32_t t_sfb = t_sfa + kTmemSfACols;
+                for (int ks = 0; ks < num_ks; ++ks) {
+                    if (!mbar_wait2_warp(sf_full_bar(stage), phase, abort_flag, peer_abort)) { ok = false; break; }
+                    tc_fence_after();
+                    const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
+                    const uint32_t sfa_lo = sf_lo0 + (uint32_t)stage * (STAGE_BYTES >> 4);
+                    const uint32_t sfb_lo = sfa_lo + (SFA_BYTES >> 4);
+                    const uint32_t t_sfa = tmem_base + kTmemSfBase + (uint32_t)stage * kTmemSfBufCols;
+                    const uint32_t t_sfb = t_sfa + kTmemSfACols;
+                    if (elect_one()) {
                         if (!MMA_ONLY) {
 #pragma unroll
                             for (int kb = 0; kb < kKbPerStage; ++kb) {
@@ -393,6 +409,7 @@ gemm_nvfp4_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
                         }
                         mma2_commit_local(sf_ready_bar(stage));    // arrives once the copies have landed in both CTAs
                     }
+                    __syncwarp();
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }

@@ -14,6 +14,19 @@ constexpr long long kWaitBudgetCycles = 4000000000ll;   // about two seconds
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of a converged warp, always the same one.  The warps that issue tcgen05 and TMA instructions walk their
+// loops and waits together and only wrap the instructions themselves in this: inside the branch the compiler knows that
+// one thread is left and keeps descriptors and addresses in uniform registers.  Under `lane == 0` it cannot, and a
+// tcgen05.mma takes 45 cycles to issue whatever its size; under elect.sync it takes what the tensor pipe needs
+// (128 x 16 x 16 with A in tensor memory: 9 cycles, 128 x 64 x 16: 32).  The branch holds straight-line code only: no lane
+// of the warp runs anything else meanwhile.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -58,6 +71,21 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
         if ((++it & 63u) == 0u) {
             if (*abort_flag) return false;
             if (clock64() - t0 > kWaitBudgetCycles) { *abort_flag = 1; return false; }
+        }
+    }
+}
+
+// The same for a whole converged warp: every lane returns the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag)
+{
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    const long long t0 = clock64();
+    uint32_t it = 0;
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+        if ((++it & 63u) == 0u) {
+            const bool over = clock64() - t0 > kWaitBudgetCycles;
+            if (__any_sync(0xffffffffu, over || *abort_flag != 0)) { *abort_flag = 1; return false; }
         }
     }
 }
