@@ -120,6 +120,15 @@ bool valid_codebook(const uint16_t cb[8])
     return has_zero && prev == 6.0f;
 }
 
+// Scale rows that pad the matrix to the GEMM's 256-row tiles read as zero; the band that holds them is cleared before the
+// real rows are written.
+int clear_sf_padding(const dq::PackedLayout &L, uint8_t *base, int64_t N, int64_t K, cudaStream_t s)
+{
+    if (L.nv_sf_bytes == 0 || N % dq::kSfRowPad == 0) return DQ_OK;
+    const size_t full = (size_t)(N / dq::kSfRowPad) * dq::kSfRowPad * (size_t)(K / dq::kBlock);
+    return cudaMemsetAsync(base + L.nv_sf_off + full, 0, L.nv_sf_bytes - full, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+}
+
 }  // namespace
 
 extern "C" {
@@ -178,38 +187,26 @@ int dq_pack_weights(const void *W_dev, int w_dtype, int64_t N, int64_t K, int64_
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint8_t *base = reinterpret_cast<uint8_t *>(packed_dev);
     dq::PackedHeader *hdr = reinterpret_cast<dq::PackedHeader *>(base);
-    if (cudaMemsetAsync(base, 0, dq::kHeaderBytes, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_pack_header(hdr, cb, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_absmax(W_dev, w_dtype, N, K, ldw, hdr, s) != cudaSuccess) return DQ_ERR_CUDA;
-    if (L.nv_sf_bytes) {
-        if (cudaMemsetAsync(base + L.nv_sf_off, 0, L.nv_sf_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
-    }
-    if (formats & DQ_FMT_NVFP4) {
-        if (dq::launch_pack_nvfp4(W_dev, w_dtype, N, K, ldw, hdr, base + L.nv_codes_off, base + L.nv_sf_off, s) !=
-            cudaSuccess)
-            return DQ_ERR_CUDA;
-    }
+    if (clear_sf_padding(L, base, N, K, s) != DQ_OK) return DQ_ERR_CUDA;
+    // NVFP4 shares the pass over W with a LUT format; a second LUT format takes its own
+    uint8_t *codes = (formats & DQ_FMT_NVFP4) ? base + L.nv_codes_off : nullptr;
+    uint8_t *sf = codes ? base + L.nv_sf_off : nullptr;
     if (formats & DQ_FMT_LUT3) {
-        if (K % dq::kLutSlice != 0) {       // partial last slice: padding must read as zero
-            if (cudaMemsetAsync(base + L.lut_off, 0, L.lut_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
-        }
-        if (dq::launch_pack_lut(3, W_dev, w_dtype, N, K, ldw, hdr, base + L.lut_off, s) != cudaSuccess)
-            return DQ_ERR_CUDA;
+        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, base + L.lut_off, 3, s) != cudaSuccess) return DQ_ERR_CUDA;
+        codes = sf = nullptr;
     }
     if (formats & DQ_FMT_LUT2) {
-        if (K % dq::kLutSlice != 0) {
-            if (cudaMemsetAsync(base + L.lut2_off, 0, L.lut2_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
-        }
-        if (dq::launch_pack_lut(2, W_dev, w_dtype, N, K, ldw, hdr, base + L.lut2_off, s) != cudaSuccess)
-            return DQ_ERR_CUDA;
+        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, base + L.lut2_off, 2, s) != cudaSuccess) return DQ_ERR_CUDA;
+        codes = sf = nullptr;
     }
+    if (codes && dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, nullptr, 0, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (formats & DQ_FMT_NVFP4_FROM_LUT3) {
         if (dq::launch_autocast(hdr, base + L.lut_off, N, K, base + L.nv_codes_off, base + L.nv_sf_off, s) !=
             cudaSuccess)
             return DQ_ERR_CUDA;
     }
-    if ((formats & (DQ_FMT_NVFP4 | DQ_FMT_NVFP4_FROM_LUT3)) && dq::launch_fill_e2m1_table(s) != cudaSuccess)
-        return DQ_ERR_CUDA;
     if (dq::launch_pack_done(s) != cudaSuccess) return DQ_ERR_CUDA;
     dq_weights *w = new (std::nothrow) dq_weights;
     if (!w) return DQ_ERR_INTERNAL;
@@ -254,7 +251,6 @@ int dq_import_canonical(int64_t N, int64_t K, unsigned formats, const void *nvfp
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint8_t *base = reinterpret_cast<uint8_t *>(packed_dev);
     dq::PackedHeader *hdr = reinterpret_cast<dq::PackedHeader *>(base);
-    if (cudaMemsetAsync(base, 0, dq::kHeaderBytes, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_pack_header(hdr, cb, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_set_scale(hdr, global_scale, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (L.nv_sf_bytes && cudaMemsetAsync(base + L.nv_sf_off, 0, L.nv_sf_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
@@ -277,8 +273,6 @@ int dq_import_canonical(int64_t N, int64_t K, unsigned formats, const void *nvfp
             cudaSuccess)
             return DQ_ERR_CUDA;
     }
-    if ((formats & (DQ_FMT_NVFP4 | DQ_FMT_NVFP4_FROM_LUT3)) && dq::launch_fill_e2m1_table(s) != cudaSuccess)
-        return DQ_ERR_CUDA;
     if (dq::launch_pack_done(s) != cudaSuccess) return DQ_ERR_CUDA;
     dq_weights *w = new (std::nothrow) dq_weights;
     if (!w) return DQ_ERR_INTERNAL;
@@ -312,7 +306,6 @@ int dq_import_canonical_lut2(int64_t N, int64_t K, const void *lut2_planes_dev, 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     uint8_t *base = reinterpret_cast<uint8_t *>(packed_dev);
     dq::PackedHeader *hdr = reinterpret_cast<dq::PackedHeader *>(base);
-    if (cudaMemsetAsync(base, 0, dq::kHeaderBytes, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_pack_header(hdr, cb, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (dq::launch_set_scale(hdr, global_scale, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (K % dq::kLutSlice != 0 && cudaMemsetAsync(base + L.lut2_off, 0, L.lut2_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
@@ -573,8 +566,16 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
     g.ldy = ldy;
     g.N = w->N;
     g.K = w->K;
-    const cudaError_t ce = tensor_cores ? dq::launch_gemv_nvfp4_mma(g, reinterpret_cast<cudaStream_t>(stream))
-                                        : dq::launch_gemv_nvfp4(g, reinterpret_cast<cudaStream_t>(stream));
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    cudaError_t ce;
+    if (tensor_cores) {
+        ce = dq::launch_gemv_nvfp4_mma(g, s);
+    } else {
+        // the comparison kernel's table of value pairs; with a launch in between it is never written by the kernel ahead
+        ce = dq::launch_fill_e2m1_table(s);
+        if (ce == cudaSuccess) ce = dq::launch_pack_done(s);
+        if (ce == cudaSuccess) ce = dq::launch_gemv_nvfp4(g, s);
+    }
     if (ce != cudaSuccess) return DQ_ERR_CUDA;
     return DQ_OK;
 }

@@ -13,13 +13,14 @@ namespace dq {
 // ------------------------------------------------------------------ header
 
 struct Codebook8 { unsigned short h[8]; };
+static_assert(kHeaderBytes == 256 * 4, "one word per thread of pack_header_kernel");
 
-__global__ void pack_header_kernel(PackedHeader *hdr, Codebook8 cb)
+__global__ void __launch_bounds__(256) pack_header_kernel(PackedHeader *hdr, Codebook8 cb)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    hdr->amax_bits = 0u;
+    reinterpret_cast<uint32_t *>(hdr)[threadIdx.x] = 0u;                     // the whole kilobyte
+    __syncthreads();
+    if (threadIdx.x != 0) return;
     hdr->s = 1.0f;
-    hdr->rc6 = 0.0f;
     int zero_idx = 0;
     unsigned int amap = 0;
     for (int j = 0; j < 8; ++j) {
@@ -60,178 +61,297 @@ cudaError_t launch_pack_header(PackedHeader *hdr, const uint16_t *codebook_f16_h
 {
     Codebook8 cb;
     for (int j = 0; j < 8; ++j) cb.h[j] = codebook_f16_host[j];
-    pack_header_kernel<<<1, 32, 0, stream>>>(hdr, cb);
+    pack_header_kernel<<<1, 256, 0, stream>>>(hdr, cb);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ absmax
 
-template <bool FP32IN>
-__global__ void absmax_kernel(const void *W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr)
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
 {
-    const int64_t nb = K / 16;
-    const int64_t total = N * nb;
-    float a = 0.0f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        float x[16];
-        load16<FP32IN>(W, i / nb, (i % nb) * 16, ldw, x);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) a = fmaxf(a, fabsf(x[j]));
+    uint32_t r;
+    asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+// Largest magnitude of W: one streaming read, four 16-byte loads in flight per thread.  grid.y walks rows, grid.x the
+// 16-byte pieces of a row; a matrix without gaps between its rows is one long row.  HBM-bound: 17408 x 5120 bf16
+// (178 MB) in 29 us, 6.1 TB/s.
+template <bool FP32IN>
+__global__ void __launch_bounds__(256) absmax_kernel(const uint4 *__restrict__ W, int64_t rows, int64_t len, int64_t ld, PackedHeader *hdr)
+{
+    uint32_t m[4] = {0u, 0u, 0u, 0u};                       // fp32 bits, or two bf16 magnitudes; a NaN is passed over
+    auto take = [&](uint32_t &acc, const uint4 &v) {
+        if (FP32IN) {
+            const float a = fmaxf(fabsf(__uint_as_float(v.x)), fabsf(__uint_as_float(v.y)));
+            const float b = fmaxf(fabsf(__uint_as_float(v.z)), fabsf(__uint_as_float(v.w)));
+            acc = __float_as_uint(fmaxf(__uint_as_float(acc), fmaxf(a, b)));
+        } else {
+            acc = max_bf16x2(max_bf16x2(acc, max_bf16x2(v.x & 0x7FFF7FFFu, v.y & 0x7FFF7FFFu)),
+                             max_bf16x2(v.z & 0x7FFF7FFFu, v.w & 0x7FFF7FFFu));
+        }
+    };
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t r = blockIdx.y; r < rows; r += gridDim.y) {
+        const uint4 *p = W + r * ld;
+        int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        for (; i + 3 * stride < len; i += 4 * stride) {
+            const uint4 v0 = __ldg(p + i), v1 = __ldg(p + i + stride), v2 = __ldg(p + i + 2 * stride), v3 = __ldg(p + i + 3 * stride);
+            take(m[0], v0);
+            take(m[1], v1);
+            take(m[2], v2);
+            take(m[3], v3);
+        }
+        for (; i < len; i += stride) take(m[0], __ldg(p + i));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-    __shared__ float red[32];
+    uint32_t a;                                             // magnitudes order like unsigned integers
+    if (FP32IN) {
+        a = max(max(m[0], m[1]), max(m[2], m[3]));
+    } else {
+        const uint32_t q = max_bf16x2(max_bf16x2(m[0], m[1]), max_bf16x2(m[2], m[3]));
+        a = max(q >> 16, q & 0xFFFFu) << 16;
+    }
+    a = __reduce_max_sync(0xffffffffu, a);
+    __shared__ uint32_t red[8];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        a = (threadIdx.x < (blockDim.x >> 5)) ? red[threadIdx.x] : 0.0f;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-        if (threadIdx.x == 0) atomicMax(&hdr->amax_bits, __float_as_uint(a));
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < 8; ++i) a = max(a, red[i]);
+        atomicMax(&hdr->amax_bits, a);
     }
-}
-
-__global__ void finalize_scale_kernel(PackedHeader *hdr)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const float amax = __uint_as_float(hdr->amax_bits);
-    const float s = (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);      // 6 * 448
-    hdr->s = s;
-    hdr->rc6 = __frcp_rn(__fmul_rn(6.0f, s));
 }
 
 cudaError_t launch_absmax(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
                           cudaStream_t stream)
 {
-    const int64_t total = N * (K / 16);
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 148 * 8) blocks = 148 * 8;
-    if (w_dtype == DQ_DT_FP32) absmax_kernel<true><<<blocks, 256, 0, stream>>>(W, N, K, ldw, hdr);
-    else absmax_kernel<false><<<blocks, 256, 0, stream>>>(W, N, K, ldw, hdr);
-    finalize_scale_kernel<<<1, 32, 0, stream>>>(hdr);
+    const int64_t per16 = (w_dtype == DQ_DT_FP32) ? 4 : 8;
+    int64_t rows = N, len = K / per16;
+    if (ldw == K) { len *= rows; rows = 1; }
+    const int64_t want = (len + 1023) / 1024, slots = 148 * 8;
+    const unsigned gx = (unsigned)(want < slots ? want : slots);
+    int64_t gy = slots / gx;
+    if (gy > rows) gy = rows;
+    const dim3 grid(gx, (unsigned)(gy < 1 ? 1 : gy));
+    const uint4 *p = reinterpret_cast<const uint4 *>(W);
+    if (w_dtype == DQ_DT_FP32) absmax_kernel<true><<<grid, 256, 0, stream>>>(p, rows, len, ldw / per16, hdr);
+    else absmax_kernel<false><<<grid, 256, 0, stream>>>(p, rows, len, ldw / per16, hdr);
     return cudaGetLastError();
 }
 
-// -------------------------------------------------------------- NVFP4 pack
+// -------------------------------------------------------------------- pack
 
-template <bool FP32IN>
-__global__ void pack_nvfp4_kernel(const void *W, int64_t N, int64_t K, int64_t ldw, const PackedHeader *hdr,
-                                  uint8_t *codes, uint8_t *sf)
+// tensor scale from the largest magnitude (App. A.3): s = max|W| / (6 * 448), 1 for an all-zero tensor
+__device__ __forceinline__ float tensor_scale(const PackedHeader *hdr)
 {
-    const int64_t nb = K / 16;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N * nb) return;
-    const int64_t r = i / nb, b = i % nb;
-    float x[16];
-    load16<FP32IN>(W, r, b * 16, ldw, x);
-    uint2 c;
-    const uint32_t d8 = quant_block_nvfp4(x, hdr->s, hdr->rc6, c);
-    *reinterpret_cast<uint2 *>(codes + r * (K / 2) + b * 8) = c;
-    sf[sf_swizzled_offset(r, b, K)] = (uint8_t)d8;
+    const float amax = __uint_as_float(hdr->amax_bits);
+    return (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
 }
 
-cudaError_t launch_pack_nvfp4(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw,
-                              const PackedHeader *hdr, uint8_t *codes, uint8_t *sf_swizzled, cudaStream_t stream)
+// four floats -> two bytes of E2M1 codes (element 0 in the low nibble of byte 0)
+__device__ __forceinline__ uint32_t f32x4_to_e2m1x4(float f0, float f1, float f2, float f3)
 {
-    const int64_t total = N * (K / 16);
-    const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (w_dtype == DQ_DT_FP32) pack_nvfp4_kernel<true><<<blocks, 256, 0, stream>>>(W, N, K, ldw, hdr, codes, sf_swizzled);
-    else pack_nvfp4_kernel<false><<<blocks, 256, 0, stream>>>(W, N, K, ldw, hdr, codes, sf_swizzled);
-    return cudaGetLastError();
+    uint32_t r;
+    asm("{\n\t.reg .b8 b0, b1;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
+        "mov.b32 %0, {b0, b1, b0, b1};\n\t}"
+        : "=r"(r) : "f"(f0), "f"(f1), "f"(f2), "f"(f3));
+    return r & 0xFFFFu;
+}
+// Transpose of 16-bit pieces between the four threads of a quad.  Thread t comes with v[j] = its pieces of blocks 2j (low
+// half) and 2j + 1 (high half) and leaves with the sixteen bytes of blocks 2t and 2t + 1, pieces in thread order.
+__device__ __forceinline__ uint4 quad_transpose(const uint32_t (&v)[4], int t)
+{
+    const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
+    const uint32_t a0 = hi2 ? v[2] : v[0], a1 = hi2 ? v[3] : v[1];
+    const uint32_t b0 = __shfl_xor_sync(0xffffffffu, hi2 ? v[0] : v[2], 2), b1 = __shfl_xor_sync(0xffffffffu, hi2 ? v[1] : v[3], 2);
+    const uint32_t k0 = hi1 ? a1 : a0, k1 = hi1 ? b1 : b0;              // from thread t and from thread t ^ 2
+    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, hi1 ? a0 : a1, 1), g1 = __shfl_xor_sync(0xffffffffu, hi1 ? b0 : b1, 1);
+    const uint32_t p0 = hi1 ? g0 : k0, p1 = hi1 ? k0 : g0;              // from threads (t & 2), (t & 2) + 1
+    const uint32_t q0 = hi1 ? g1 : k1, q1 = hi1 ? k1 : g1;              // from the other two
+    const uint32_t u0 = hi2 ? q0 : p0, u1 = hi2 ? q1 : p1, u2 = hi2 ? p0 : q0, u3 = hi2 ? p1 : q1;
+    return make_uint4(__byte_perm(u0, u1, 0x5410), __byte_perm(u2, u3, 0x5410), __byte_perm(u0, u1, 0x7632),
+                      __byte_perm(u2, u3, 0x7632));
 }
 
-// ---------------------------------------------------------------- LUT pack
-
-template <bool FP32IN>
-__device__ __forceinline__ void load4(const void *base, int64_t row, int64_t k0, int64_t ld, float (&x)[4])
+// Number of thresholds below y (the index of the nearest level, a value on a threshold taking the lower level), as index
+// bits in the sign bits of the results: T - y is negative exactly where y > T, and with increasing thresholds the bits of the count
+// are parities of those signs.
+template <int BITS>
+__device__ __forceinline__ void level_bits(float y, const float (&T)[(1 << BITS) - 1], uint32_t (&bit)[BITS])
 {
-    if (FP32IN) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(base) + row * ld + k0));
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    uint32_t d[(1 << BITS) - 1];
+#pragma unroll
+    for (int l = 0; l < (1 << BITS) - 1; ++l) d[l] = __float_as_uint(__fsub_rn(T[l], y));
+    if (BITS == 3) {
+        bit[BITS - 1] = d[3];
+        bit[1] = d[1] ^ d[3] ^ d[BITS == 3 ? 5 : 0];
+        bit[0] = (d[0] ^ d[1] ^ d[2]) ^ (d[3] ^ d[BITS == 3 ? 4 : 0] ^ d[BITS == 3 ? 5 : 0]) ^ d[BITS == 3 ? 6 : 0];
     } else {
-        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(base) + row * ld + k0));
-        x[0] = __uint_as_float(v.x << 16); x[1] = __uint_as_float(v.x & 0xFFFF0000u);
-        x[2] = __uint_as_float(v.y << 16); x[3] = __uint_as_float(v.y & 0xFFFF0000u);
+        bit[1] = d[1];
+        bit[0] = d[0] ^ d[1] ^ d[2];
     }
 }
-
-// the larger magnitude of two signed values; equal magnitudes: the positive one
-__device__ __forceinline__ float signed_extreme(float m, float v)
+// appends a nibble [index bits, BITS of them][garbage bit] at the low end of acc (LUT2: [0][bits][garbage])
+template <int BITS>
+__device__ __forceinline__ uint32_t push_level(uint32_t acc, const uint32_t (&bit)[BITS])
 {
-    return (fabsf(v) > fabsf(m) || (fabsf(v) == fabsf(m) && v > m)) ? v : m;
+    if (BITS == 2) acc <<= 1;
+#pragma unroll
+    for (int b = BITS - 1; b > 0; --b) acc = __funnelshift_l(bit[b], acc, 1);
+    return __funnelshift_l(bit[0], acc, 2);
 }
 
-// LUT3 / LUT2 round-to-nearest (App. A.3 "LUT formats").  Four neighbouring threads (t = 0..3) quantise the 128
-// weights 128 q .. 128 q + 127 of one row: thread t holds weights 4t .. 4t+3 of each of the eight 16-blocks, which is
-// exactly what its word group of the device layout stores; the block extreme is found across the four threads.
-template <bool FP32IN, int BITS>
-__global__ void __launch_bounds__(128) pack_lut_kernel(const void *W, int64_t N, int64_t K, int64_t ldw,
-                                                       const PackedHeader *hdr, uint8_t *lut)
+// Round-to-nearest packing of the master weights (App. A.3): NVFP4 (NV) and / or one LUT format (BITS = 3 or 2) in one
+// read of W.  A warp takes an atom of 8 rows x 512 weights; lane (g, t) = (row, quarter of a 16-block) takes weights
+// 4t .. 4t+3 of every block of its row, which is what its index words of the LUT layout store, 128 weights at a time.
+// Both encodings share the block's largest magnitude, its E4M3 scale and the reciprocal (a table of the 127 scales per CTA);
+// index words and scales leave as whole 512- and 256-byte rows of the atom, E2M1 codes after a transpose inside
+// the quad as 16 bytes per lane.
+// Bound by instruction issue (the thresholds: 7 subtractions, 4 logic ops and 3 shifts per weight).  17408 x 5120 bf16 to
+// NVFP4 and LUT3: 120 us, 2.2 TB/s; a pass per format with compares and one bit placed at a time took about 250.
+template <bool FP32IN, bool NV, int BITS>
+__global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
+                                                   uint8_t *__restrict__ codes, uint8_t *__restrict__ sf, uint8_t *__restrict__ lut)
 {
-    const int64_t nq = K / 128;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t quad = i >> 2;
-    const int t = (int)(i & 3);
-    const bool live = quad < N * nq;                      // whole quads are live or not; shuffles stay inside a quad
-    const int64_t r = live ? quad / nq : 0, q = live ? quad % nq : 0;
-    const float s = hdr->s, rc6 = hdr->rc6;
-    constexpr int NT = (1 << BITS) - 1;
-    float T[NT];
+    constexpr bool LUT = BITS > 0;
+    constexpr int B = LUT ? BITS : 2;                      // dummy where there is no LUT format
+    __shared__ float rtab[128];                            // 1 / (s * d) by the byte of d; 0 for a scale that rounded to zero
+    const float s = tensor_scale(hdr);
+    const float rc6 = __frcp_rn(__fmul_rn(6.0f, s));
+    if (blockIdx.x == 0 && threadIdx.x == 0) { hdr->s = s; hdr->rc6 = rc6; }
+    rtab[threadIdx.x] = (threadIdx.x == 0) ? 0.0f : __frcp_rn(__fmul_rn(s, e4m3_to_f32(threadIdx.x)));
+    __syncthreads();
+    const uint32_t atoms_k = (uint32_t)(2 * lut_slices(K));               // atoms along a row, a short last slice padded
+    const uint32_t katoms = NV && !LUT ? (uint32_t)((K + 511) / 512) : atoms_k;
+    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int64_t rowgrp = task / katoms;
+    if (rowgrp >= N / 8) return;
+    const uint32_t atom = (uint32_t)(task - rowgrp * katoms);
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int64_t r = rowgrp * 8 + g;
+    const int nwi = max(0, min(4, (int)(K / 128) - 4 * (int)atom));
+    float T[(1 << B) - 1];
+    if (LUT) {
 #pragma unroll
-    for (int l = 0; l < NT; ++l) T[l] = (BITS == 3) ? hdr->lut_thresholds[l] : hdr->lut2_thresholds[l];
-    const int zero_idx = (BITS == 3) ? hdr->lut_zero_idx : hdr->lut2_zero_idx;
-    uint32_t wd[BITS];
+        for (int l = 0; l < (1 << B) - 1; ++l) T[l] = (BITS == 3) ? hdr->lut_thresholds[l] : hdr->lut2_thresholds[l & 3];
+    }
+    uint32_t words[4][B];
+    uint2 my_scales = make_uint2(0u, 0u);                  // LUT scale bytes of word group t
 #pragma unroll
-    for (int p = 0; p < BITS; ++p) wd[p] = 0u;
-    uint32_t sc_lo = 0u, sc_hi = 0u;
+    for (int wi = 0; wi < 4; ++wi) {
 #pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        float x[4];
-        load4<FP32IN>(W, r, q * 128 + bb * 16 + t * 4, ldw, x);
-        // the block's maximum-magnitude weight with its sign; equal magnitudes: the positive one
-        float m = signed_extreme(signed_extreme(x[0], x[1]), signed_extreme(x[2], x[3]));
-        m = signed_extreme(m, __shfl_xor_sync(0xffffffffu, m, 1));
-        m = signed_extreme(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        uint32_t d8 = f32_to_e4m3(__fmul_rn(m, rc6));
-        if ((d8 & 0x7Fu) == 0u) d8 = 0u;
-        if (bb < 4) sc_lo |= d8 << (8 * bb); else sc_hi |= d8 << (8 * (bb - 4));
-        const float rr = (d8 != 0u) ? __frcp_rn(__fmul_rn(s, e4m3_to_f32(d8))) : 0.0f;
+        for (int p = 0; p < B; ++p) words[wi][p] = 0u;
+        if (wi >= nwi) continue;                           // whole warps
+        const int64_t k0 = (int64_t)atom * 512 + wi * 128;
+        uint4 raw[8];                                      // bf16: two words of it are used
 #pragma unroll
-        for (int n4 = 0; n4 < 4; ++n4) {
-            int idx = zero_idx;
-            if (d8 != 0u) {
-                const float y = __fmul_rn(x[n4], rr);
-                idx = 0;
-#pragma unroll
-                for (int l = 0; l < NT; ++l) idx += (y > T[l]) ? 1 : 0;
-            }
-#pragma unroll
-            for (int b = 0; b < BITS; ++b) {
-                int word, pos;
-                lut_locate<BITS>(bb, n4, b, word, pos);            // compile-time constants after unrolling
-                wd[word] |= (uint32_t)((idx >> b) & 1) << pos;
+        for (int bb = 0; bb < 8; ++bb) {
+            if (FP32IN) {
+                raw[bb] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(W) + r * ldw + k0 + bb * 16 + t * 4));
+            } else {
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(W) + r * ldw + k0 + bb * 16 + t * 4));
+                raw[bb] = make_uint4(v.x, v.y, 0u, 0u);
             }
         }
-    }
-    if (!live) return;
+        uint32_t nv_pieces[4] = {0u, 0u, 0u, 0u};
+        uint32_t nv_sc[2] = {0u, 0u}, lut_sc[2] = {0u, 0u};
+        uint32_t sel[4];
 #pragma unroll
-    for (int p = 0; p < BITS; ++p) *reinterpret_cast<uint32_t *>(lut + lut_word_offset(r, q, t, p, K, BITS)) = wd[p];
-    if (t == 0) *reinterpret_cast<uint2 *>(lut + lut_scale_offset(r, q * 8, K, BITS)) = make_uint2(sc_lo, sc_hi);
+        for (int a = 3; a >= 0; --a) {
+            uint32_t acc = 0u;
+#pragma unroll
+            for (int h = 1; h >= 0; --h) {                 // selector nibbles from the top: second block first
+                const int bb = 2 * a + h;
+                // largest and most negative value of the block across the quad
+                float mx, mn;
+                float x[4];
+                if (FP32IN) {
+                    x[0] = __uint_as_float(raw[bb].x); x[1] = __uint_as_float(raw[bb].y);
+                    x[2] = __uint_as_float(raw[bb].z); x[3] = __uint_as_float(raw[bb].w);
+                    mx = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+                    mn = fmaxf(fmaxf(-x[0], -x[1]), fmaxf(-x[2], -x[3]));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+                    mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+                    mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
+                } else {
+                    x[0] = __uint_as_float(raw[bb].x << 16); x[1] = __uint_as_float(raw[bb].x & 0xFFFF0000u);
+                    x[2] = __uint_as_float(raw[bb].y << 16); x[3] = __uint_as_float(raw[bb].y & 0xFFFF0000u);
+                    const uint32_t pm = max_bf16x2(raw[bb].x, raw[bb].y);
+                    const uint32_t nm = max_bf16x2(raw[bb].x ^ 0x80008000u, raw[bb].y ^ 0x80008000u);
+                    uint32_t e = max_bf16x2(__byte_perm(pm, nm, 0x5410), __byte_perm(pm, nm, 0x7632));    // (max, -min)
+                    e = max_bf16x2(e, __shfl_xor_sync(0xffffffffu, e, 1));
+                    e = max_bf16x2(e, __shfl_xor_sync(0xffffffffu, e, 2));
+                    mx = __uint_as_float(e << 16);
+                    mn = __uint_as_float(e & 0xFFFF0000u);
+                }
+                const uint32_t d8 = f32_to_e4m3(__fmul_rn(fmaxf(mx, mn), rc6)) & 0x7Fu;
+                const float rr = rtab[d8];
+                if (NV) {
+                    const uint32_t c = f32x4_to_e2m1x4(__fmul_rn(x[0], rr), __fmul_rn(x[1], rr), __fmul_rn(x[2], rr), __fmul_rn(x[3], rr));
+                    nv_pieces[a] |= (d8 ? c : 0u) << (16 * h);
+                    nv_sc[bb >> 2] |= d8 << (8 * (bb & 3));
+                }
+                if (LUT) {
+                    // the scale takes the sign of the block's extreme; where both signs reach the magnitude, plus
+                    const bool neg = mn > mx;
+                    lut_sc[bb >> 2] |= (d8 ? (d8 | (neg ? 0x80u : 0u)) : 0u) << (8 * (bb & 3));
+                    const float rs = neg ? -rr : rr;
+#pragma unroll
+                    for (int n4 = 3; n4 >= 0; --n4) {
+                        uint32_t bit[B];
+                        level_bits<B>(__fmul_rn(x[n4], rs), T, bit);
+                        acc = push_level<B>(acc, bit);
+                    }
+                }
+            }
+            sel[a] = acc >> 1;
+        }
+        if (LUT) {
+            if (BITS == 3) {
+#pragma unroll
+                for (int p = 0; p < B; ++p)
+                    words[wi][p] = (sel[p] & 0x77777777u) | (((sel[3] >> p) & 0x11111111u) << 3);
+            } else {
+#pragma unroll
+                for (int p = 0; p < 2; ++p)
+                    words[wi][p] = (sel[2 * p] & 0x33333333u) | ((sel[2 * p + 1] & 0x33333333u) << 2);
+            }
+            if (t == wi) my_scales = make_uint2(lut_sc[0], lut_sc[1]);
+        }
+        if (NV) {
+            *reinterpret_cast<uint4 *>(codes + r * (K / 2) + k0 / 2 + t * 16) = quad_transpose(nv_pieces, t);
+            if (t < 2) *reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, k0 / 16 + 4 * t, K)) = t ? nv_sc[1] : nv_sc[0];
+        }
+    }
+    if (LUT) {
+        uint8_t *out = lut + lut_atom_offset(rowgrp * 8, atom, K, B);
+#pragma unroll
+        for (int p = 0; p < B; ++p)
+            *reinterpret_cast<uint4 *>(out + p * 512 + lane * 16) = make_uint4(words[0][p], words[1][p], words[2][p], words[3][p]);
+        *reinterpret_cast<uint2 *>(out + lut_plane_bytes(B) + lane * 8) = my_scales;
+    }
 }
 
-cudaError_t launch_pack_lut(int bits, const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw,
-                            const PackedHeader *hdr, uint8_t *lut_dev, cudaStream_t stream)
+template <bool FP32IN>
+static void launch_pack_typed(const void *W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes, uint8_t *sf,
+                              uint8_t *lut, int bits, cudaStream_t stream)
 {
-    const int64_t total = N * (K / 128) * 4;
-    const unsigned blocks = (unsigned)((total + 127) / 128);
-    const bool f32 = (w_dtype == DQ_DT_FP32);
-    if (bits == 3) {
-        if (f32) pack_lut_kernel<true, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, lut_dev);
-        else pack_lut_kernel<false, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, lut_dev);
-    } else {
-        if (f32) pack_lut_kernel<true, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, lut_dev);
-        else pack_lut_kernel<false, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, lut_dev);
-    }
+    const int64_t atoms_k = bits ? 2 * lut_slices(K) : (K + 511) / 512;
+    const unsigned blocks = (unsigned)((N / 8 * atoms_k + 3) / 4);
+    if (codes && bits == 3) pack_kernel<FP32IN, true, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    else if (codes && bits == 2) pack_kernel<FP32IN, true, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    else if (codes) pack_kernel<FP32IN, true, 0><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    else if (bits == 3) pack_kernel<FP32IN, false, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    else pack_kernel<FP32IN, false, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+}
+
+// codes / sf: NVFP4 output or nullptr; lut with bits = 3 or 2: LUT output, bits = 0: none
+cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes,
+                        uint8_t *sf_swizzled, uint8_t *lut_dev, int bits, cudaStream_t stream)
+{
+    if (w_dtype == DQ_DT_FP32) launch_pack_typed<true>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, stream);
+    else launch_pack_typed<false>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, stream);
     return cudaGetLastError();
 }
 
@@ -239,58 +359,118 @@ cudaError_t launch_pack_lut(int bits, const void *W, int w_dtype, int64_t N, int
 
 // NVFP4 view of the LUT3 codes (Sec. 2.3): level -> nearest E2M1 value, element signs
 // flipped under a negative block scale, block scale |d|, same tensor scale.
-// One thread per word group (32 weights: four of each of eight blocks).  A selector byte holds the indices of a
-// weight pair as nibbles; a small shared-memory table maps such a byte to the byte of two E2M1 codes, in three
-// variants: positive scale, negative scale (sign bits of non-zero codes flipped), zero scale (all codes zero).
-// Selector word a holds blocks 2a (low half) and 2a+1 (high half); the thread's four codes of a block are two
-// consecutive bytes of the row's code bytes.
-__global__ void __launch_bounds__(256) autocast_kernel(const PackedHeader *hdr, const uint8_t *lut, int64_t N,
-                                                       int64_t K, uint8_t *codes, uint8_t *sf)
+// A warp takes an atom (8 rows x 512 weights): 16-byte loads of index words, a byte permute looks up the E2M1 codes of four
+// weights (one table per sign of the block scale), and a transpose inside the quad leaves every lane 16 bytes of codes to
+// store.  5120 x 17408 (39 MB in, 50 MB out): 26 us; with two table bytes looked up in shared memory and 2-byte stores per
+// block it took 78.
+__global__ void __launch_bounds__(128) autocast_kernel(const PackedHeader *__restrict__ hdr, const uint8_t *__restrict__ lut, int64_t N,
+                                                       int64_t K, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf)
 {
-    __shared__ uint8_t table[3][128];               // [variant][idx_b << 4 | idx_a] -> two E2M1 codes
+    const uint32_t natoms = (uint32_t)((K + 511) / 512);
+    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int64_t rowgrp = task / natoms;
+    if (rowgrp >= N / 8) return;
+    const uint32_t atom = (uint32_t)(task - rowgrp * natoms);
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int64_t r = rowgrp * 8 + g;
+    const uint8_t *src = lut + lut_atom_offset(rowgrp * 8, atom, K, 3);
+    uint4 w[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) w[p] = __ldg(reinterpret_cast<const uint4 *>(src + p * 512 + lane * 16));
+    const uint2 s8 = __ldg(reinterpret_cast<const uint2 *>(src + lut_plane_bytes(3) + lane * 8));
+    // E2M1 codes of the levels as bytes; negative block scale: sign bits of non-zero codes flipped
     const uint32_t amap = hdr->autocast_map;
-    for (int i = threadIdx.x; i < 3 * 128; i += blockDim.x) {
-        const int v = i >> 7, e = i & 127;
-        uint32_t ca = (amap >> (4 * (e & 7))) & 0xFu, cb = (amap >> (4 * ((e >> 4) & 7))) & 0xFu;
-        if (v == 1) { if (ca & 7u) ca ^= 8u; if (cb & 7u) cb ^= 8u; }
-        if (v == 2) { ca = 0u; cb = 0u; }
-        table[v][e] = (uint8_t)(ca | (cb << 4));
+    uint32_t pos[2], neg[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t m = amap >> (16 * i);
+        pos[i] = (m & 0xFu) | ((m & 0xF0u) << 4) | ((m & 0xF00u) << 8) | ((m & 0xF000u) << 12);
+        const uint32_t nz = (pos[i] | (pos[i] >> 1) | (pos[i] >> 2)) & 0x01010101u;
+        neg[i] = pos[i] ^ (nz << 3);
     }
-    __syncthreads();
-    const int64_t nq = K / 128;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t quad = i >> 2;
-    const int t = (int)(i & 3);
-    if (quad >= N * nq) return;
-    const int64_t r = quad / nq, q = quad % nq;
-    uint32_t w[3], sel[4];
+    const int nwi = min(4, (int)(K / 128) - 4 * (int)atom);
 #pragma unroll
-    for (int p = 0; p < 3; ++p) w[p] = *reinterpret_cast<const uint32_t *>(lut + lut_word_offset(r, q, t, p, K, 3));
-    lut_selectors<3>(w, sel);
-    const uint2 d8x8 = *reinterpret_cast<const uint2 *>(lut + lut_scale_offset(r, q * 8, K, 3));
+    for (int wi = 0; wi < 4; ++wi) {
+        if (wi >= nwi) break;                              // whole warps
+        uint32_t wd[3], sel[4];
 #pragma unroll
-    for (int bb = 0; bb < 8; ++bb) {
-        const uint32_t d8 = ((bb < 4 ? d8x8.x : d8x8.y) >> (8 * (bb & 3))) & 0xFFu;
-        const uint8_t *tab = table[d8 == 0u ? 2 : ((d8 & 0x80u) ? 1 : 0)];
-        const uint32_t u = (sel[bb >> 1] >> (16 * (bb & 1))) & 0xFFFFu;
-        const unsigned short two = (unsigned short)((uint32_t)tab[u & 0xFFu] | ((uint32_t)tab[u >> 8] << 8));
-        *reinterpret_cast<unsigned short *>(codes + r * (K / 2) + q * 64 + bb * 8 + t * 2) = two;
-        if (t == (bb & 3)) sf[sf_swizzled_offset(r, q * 8 + bb, K)] = (uint8_t)(d8 & 0x7Fu);
+        for (int p = 0; p < 3; ++p) wd[p] = wi == 0 ? w[p].x : wi == 1 ? w[p].y : wi == 2 ? w[p].z : w[p].w;
+        lut_selectors<3>(wd, sel);
+        // the row's scales of this word group sit in lane wi of the quad
+        const uint32_t sc[2] = {__shfl_sync(0xffffffffu, s8.x, (lane & ~3) | wi), __shfl_sync(0xffffffffu, s8.y, (lane & ~3) | wi)};
+        uint32_t v[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            uint32_t c[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int bb = 2 * a + h;
+                const uint32_t d8 = (sc[bb >> 2] >> (8 * (bb & 3))) & 0xFFu;
+                const bool minus = (d8 & 0x80u) != 0u;
+                const uint32_t x = __byte_perm(minus ? neg[0] : pos[0], minus ? neg[1] : pos[1], h ? sel[a] >> 16 : sel[a] & 0xFFFFu);
+                c[h] = d8 ? (x | (x >> 4)) : 0u;           // bytes 0 and 2: two codes each
+            }
+            v[a] = __byte_perm(c[0], c[1], 0x6420);
+        }
+        const int64_t k0 = (int64_t)atom * 512 + wi * 128;
+        *reinterpret_cast<uint4 *>(codes + r * (K / 2) + k0 / 2 + t * 16) = quad_transpose(v, t);
+        if (t < 2) *reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, k0 / 16 + 4 * t, K)) = (t ? sc[1] : sc[0]) & 0x7F7F7F7Fu;
     }
 }
 
 cudaError_t launch_autocast(const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N,
                             int64_t K, uint8_t *codes, uint8_t *sf_swizzled, cudaStream_t stream)
 {
-    const int64_t total = N * (K / 128) * 4;
-    autocast_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(hdr, lut_dev, N, K, codes, sf_swizzled);
+    const int64_t warps = N / 8 * ((K + 511) / 512);
+    autocast_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, stream>>>(hdr, lut_dev, N, K, codes, sf_swizzled);
     return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ export
 
-__global__ void export_nvfp4_kernel(const PackedHeader *hdr, const uint8_t *codes, const uint8_t *sf, int64_t N,
-                                    int64_t K, uint8_t *codes_out, uint8_t *scales_out, float *s_out)
+// Codes are row-major on both sides: 16-byte copies, four in flight per thread.  Scales: a warp takes 32 rows of each quarter
+// of a 128-row band and four 64-wide k atoms, reads the atoms' 16-byte groups (scales of rows r, r+32, r+64, r+96)
+// and writes 16 scales of each of its rows at once.
+__global__ void __launch_bounds__(256) export_nvfp4_kernel(const PackedHeader *__restrict__ hdr, const uint4 *__restrict__ codes,
+                                                           const uint8_t *__restrict__ sf, int64_t N, int64_t K, uint4 *__restrict__ codes_out,
+                                                           uint8_t *__restrict__ scales_out, float *s_out, int code_blocks)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0 && s_out) *s_out = hdr->s;
+    if ((int)blockIdx.x < code_blocks) {
+        const int64_t n16 = N * (K / 2) / 16, base = (int64_t)blockIdx.x * 1024 + threadIdx.x;
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (base + u * 256 < n16) v[u] = __ldg(codes + base + u * 256);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) if (base + u * 256 < n16) codes_out[base + u * 256] = v[u];
+        return;
+    }
+    const int64_t katoms = K / 64, groups = (katoms + 3) / 4;
+    const int64_t task = ((int64_t)blockIdx.x - code_blocks) * 8 + (threadIdx.x >> 5);
+    const int64_t band = task / groups, kg = task - band * groups;
+    if (band * 128 >= N) return;
+    const int lane = threadIdx.x & 31;
+    const int nk = (int)min((int64_t)4, katoms - kg * 4);           // K % 128 == 0: two or four
+    uint4 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+        v[c] = (c < nk) ? __ldg(reinterpret_cast<const uint4 *>(sf + (band * katoms + kg * 4 + c) * 512 + lane * 16)) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int64_t r = band * 128 + q * 32 + lane;
+        if (r >= N) continue;
+        uint32_t o[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[c] = q == 0 ? v[c].x : q == 1 ? v[c].y : q == 2 ? v[c].z : v[c].w;
+        uint8_t *dst = scales_out + r * (K / 16) + kg * 16;          // 8-byte aligned (K / 16 is a multiple of 8)
+        *reinterpret_cast<uint2 *>(dst) = make_uint2(o[0], o[1]);
+        if (nk == 4) *reinterpret_cast<uint2 *>(dst + 8) = make_uint2(o[2], o[3]);
+    }
+}
+
+// codes_out and scales_out need 8-byte alignment only: the general form for pointers that are not 16-byte aligned
+__global__ void export_nvfp4_narrow_kernel(const PackedHeader *hdr, const uint8_t *codes, const uint8_t *sf, int64_t N,
+                                           int64_t K, uint8_t *codes_out, uint8_t *scales_out, float *s_out)
 {
     const int64_t nb = K / 16;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -306,60 +486,96 @@ cudaError_t launch_export_nvfp4(const PackedHeader *hdr, const uint8_t *codes, c
                                 int64_t K, uint8_t *codes_out, uint8_t *scales_out, float *s_out,
                                 cudaStream_t stream)
 {
-    const int64_t total = N * (K / 16);
-    export_nvfp4_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(hdr, codes, sf_swizzled, N, K,
-                                                                             codes_out, scales_out, s_out);
+    if (reinterpret_cast<uintptr_t>(codes_out) % 16 || reinterpret_cast<uintptr_t>(scales_out) % 8) {
+        const int64_t total = N * (K / 16);
+        export_nvfp4_narrow_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(hdr, codes, sf_swizzled, N, K, codes_out,
+                                                                                        scales_out, s_out);
+        return cudaGetLastError();
+    }
+    const int64_t code_blocks = (N * (K / 2) / 16 + 1023) / 1024;
+    const int64_t warps = (N + 127) / 128 * ((K / 64 + 3) / 4);
+    export_nvfp4_kernel<<<(unsigned)(code_blocks + (warps + 7) / 8), 256, 0, stream>>>(
+        hdr, reinterpret_cast<const uint4 *>(codes), sf_swizzled, N, K, reinterpret_cast<uint4 *>(codes_out), scales_out, s_out,
+        (int)code_blocks);
     return cudaGetLastError();
 }
 
-// index of weight k of row r, read from the device layout
+// LSB-first bit-planes (App. C.2) from the device layout.  A warp takes an atom; lane (g, t) holds weights 4t .. 4t+3 of every
+// block of row g, i.e. bits 4t .. 4t+3 of each half of a canonical word.  It gathers its bits of the sixteen words of the atom
+// per plane; two exchanges inside the quad OR them together so that lane t ends up with the four words of word group t.
 template <int BITS>
-__device__ __forceinline__ int lut_read_index(const uint8_t *lut, int64_t r, int64_t k, int64_t K)
+__global__ void __launch_bounds__(128) export_lut_kernel(const PackedHeader *__restrict__ hdr, const uint8_t *__restrict__ lut, int64_t N,
+                                                         int64_t K, uint32_t *__restrict__ planes_out, uint8_t *__restrict__ scales_out, float *s_out)
 {
-    const int64_t q = k >> 7;
-    const int bb = (int)((k >> 4) & 7), t = (int)((k >> 2) & 3), n4 = (int)(k & 3);
-    int idx = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && s_out) *s_out = hdr->s;
+    const uint32_t natoms = (uint32_t)((K + 511) / 512);
+    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int64_t rowgrp = task / natoms;
+    if (rowgrp >= N / 8) return;
+    const uint32_t atom = (uint32_t)(task - rowgrp * natoms);
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int64_t r = rowgrp * 8 + g;
+    const uint8_t *src = lut + lut_atom_offset(rowgrp * 8, atom, K, BITS);
+    uint4 w[BITS];
 #pragma unroll
-    for (int b = 0; b < BITS; ++b) {
-        int word, pos;
-        lut_locate<BITS>(bb, n4, b, word, pos);
-        const uint32_t w = *reinterpret_cast<const uint32_t *>(lut + lut_word_offset(r, q, t, word, K, BITS));
-        idx |= (int)((w >> pos) & 1u) << b;
+    for (int p = 0; p < BITS; ++p) w[p] = __ldg(reinterpret_cast<const uint4 *>(src + p * 512 + lane * 16));
+    const uint2 s8 = __ldg(reinterpret_cast<const uint2 *>(src + lut_plane_bytes(BITS) + lane * 8));
+    const bool mine = (int)(K / 128) - 4 * (int)atom > t;   // word group t of the atom lies inside the row
+    uint32_t sel[4][4];                                     // [word group][selector]
+#pragma unroll
+    for (int wi = 0; wi < 4; ++wi) {
+        uint32_t wd[BITS];
+#pragma unroll
+        for (int p = 0; p < BITS; ++p) wd[p] = wi == 0 ? w[p].x : wi == 1 ? w[p].y : wi == 2 ? w[p].z : w[p].w;
+        lut_selectors<BITS>(wd, sel[wi]);
     }
-    return idx;
-}
-
-template <int BITS>
-__global__ void export_lut_kernel(const PackedHeader *hdr, const uint8_t *lut, int64_t N,
-                                  int64_t K, uint32_t *planes_out, uint8_t *scales_out, float *s_out)
-{
-    const int64_t nw = K / 32;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && s_out) *s_out = hdr->s;
-    if (i >= N * nw) return;
-    const int64_t r = i / nw, j = i % nw;
-    uint32_t c[BITS];
+    const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
 #pragma unroll
-    for (int p = 0; p < BITS; ++p) c[p] = 0u;
-    for (int e = 0; e < 32; ++e) {
-        const int idx = lut_read_index<BITS>(lut, r, j * 32 + e, K);
+    for (int p = 0; p < BITS; ++p) {
+        uint32_t o[4];
 #pragma unroll
-        for (int p = 0; p < BITS; ++p) c[p] |= (uint32_t)((idx >> p) & 1) << e;      // canonical: LSB-first bit-planes
+        for (int a = 0; a < 4; ++a) {
+            uint32_t z[4];
+#pragma unroll
+            for (int wi = 0; wi < 4; ++wi) {                // bit p of the eight nibbles -> bits 0-3 of both halves, then to 4t
+                uint32_t x = (sel[wi][a] >> p) & 0x11111111u;
+                x = (x | (x >> 3)) & 0x03030303u;
+                x = (x | (x >> 6)) & 0x000F000Fu;
+                z[wi] = x << (4 * t);
+            }
+            const uint32_t a0 = (hi2 ? z[2] : z[0]) | __shfl_xor_sync(0xffffffffu, hi2 ? z[0] : z[2], 2);
+            const uint32_t a1 = (hi2 ? z[3] : z[1]) | __shfl_xor_sync(0xffffffffu, hi2 ? z[1] : z[3], 2);
+            o[a] = (hi1 ? a1 : a0) | __shfl_xor_sync(0xffffffffu, hi1 ? a0 : a1, 1);
+        }
+        if (mine) {
+            uint32_t *dst = planes_out + (r * BITS + p) * (K / 32) + (int64_t)atom * 16 + t * 4;
+            if ((reinterpret_cast<uintptr_t>(planes_out) & 15) == 0) {
+                *reinterpret_cast<uint4 *>(dst) = make_uint4(o[0], o[1], o[2], o[3]);
+            } else {
+#pragma unroll
+                for (int a = 0; a < 4; ++a) dst[a] = o[a];
+            }
+        }
     }
+    if (mine) {
+        uint8_t *dst = scales_out + r * (K / 16) + (int64_t)atom * 32 + t * 8;
+        if ((reinterpret_cast<uintptr_t>(scales_out) & 7) == 0) {
+            *reinterpret_cast<uint2 *>(dst) = s8;
+        } else {
 #pragma unroll
-    for (int p = 0; p < BITS; ++p) planes_out[(r * BITS + p) * nw + j] = c[p];
-    scales_out[r * (K / 16) + 2 * j] = lut[lut_scale_offset(r, 2 * j, K, BITS)];
-    scales_out[r * (K / 16) + 2 * j + 1] = lut[lut_scale_offset(r, 2 * j + 1, K, BITS)];
+            for (int i = 0; i < 8; ++i) dst[i] = (uint8_t)((i < 4 ? s8.x : s8.y) >> (8 * (i & 3)));
+        }
+    }
 }
 
 cudaError_t launch_export_lut(int bits, const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N,
                               int64_t K, uint32_t *planes_out, uint8_t *scales_out, float *s_out,
                               cudaStream_t stream)
 {
-    const int64_t total = N * (K / 32);
-    const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (bits == 3) export_lut_kernel<3><<<blocks, 256, 0, stream>>>(hdr, lut_dev, N, K, planes_out, scales_out, s_out);
-    else export_lut_kernel<2><<<blocks, 256, 0, stream>>>(hdr, lut_dev, N, K, planes_out, scales_out, s_out);
+    const int64_t warps = N / 8 * ((K + 511) / 512);
+    const unsigned blocks = (unsigned)((warps + 3) / 4);
+    if (bits == 3) export_lut_kernel<3><<<blocks, 128, 0, stream>>>(hdr, lut_dev, N, K, planes_out, scales_out, s_out);
+    else export_lut_kernel<2><<<blocks, 128, 0, stream>>>(hdr, lut_dev, N, K, planes_out, scales_out, s_out);
     return cudaGetLastError();
 }
 

@@ -760,3 +760,39 @@ def test_measurement_hooks_leave_results_alone(dq, oracle):
     assert torch.equal(dq.prefill_linear(w, A, sa, workspace=ws), Y0)
     with pytest.raises(dq.DQError):
         dq.bench_gemm_mma_only(w, 64, scratch, ws)             # the measurement mode exists for M > 128 only
+
+
+@pytest.mark.parametrize("N,K", [(16, 128), (272, 640), (48, 1664)])
+@pytest.mark.parametrize("fmt", ["nvfp4+lut3", "nvfp4+lut2", "lut3+lut2+nvfp4", "lut2", "nvfp4"])
+def test_pack_every_combination_of_formats(dq, oracle, N, K, fmt):
+    """One pass over W serves several encodings; row lengths that end inside an atom of 512 weights and inside a slice of 1024,
+    row counts that end inside the 128-row bands of the scale layout.  Bit exact, exports into unaligned buffers included."""
+    W, ref = _layer(oracle, N, K, 41 + N)
+    names = fmt.split("+")
+    w = dq.pack_weights(W.to(DEV), formats=sum({"nvfp4": dq.FMT_NVFP4, "lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2}[f] for f in names))
+    Wf = dq_inputs.bf16_to_f32_numpy(W)
+    if "nvfp4" in names:
+        codes, scales, s = dq.export_canonical(w, dq.FMT_NVFP4)
+        assert _np(s)[0] == np.float32(ref["s"])
+        assert np.array_equal(_np(codes), ref["nvfp4_codes"]) and np.array_equal(_np(scales), ref["nvfp4_scales"])
+    if "lut3" in names:
+        planes, lsc, _ = dq.export_canonical(w, dq.FMT_LUT3)
+        assert np.array_equal(_np(planes).view(np.uint32), ref["lut3_planes"]) and np.array_equal(_np(lsc), ref["lut3_scales"])
+    if "lut2" in names:
+        p2, s2 = oracle.quant_lut2(Wf, ref["s"])
+        planes, lsc, _ = dq.export_canonical(w, dq.FMT_LUT2)
+        assert np.array_equal(_np(planes).view(np.uint32), p2) and np.array_equal(_np(lsc), s2)
+    _status_ok(dq)
+    # destinations that are only as aligned as the entry point asks for
+    first = {"nvfp4": dq.FMT_NVFP4, "lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2}[names[0]]
+    want, wsc, _ = dq.export_canonical(w, first)
+    nb = want.numel() * want.element_size()
+    buf = torch.zeros(nb + 16, dtype=torch.uint8, device=DEV)
+    scb = torch.zeros(wsc.numel() + 16, dtype=torch.uint8, device=DEV)
+    off = 8 if names[0] == "nvfp4" else 4
+    st = dq.lib().dq_export_canonical(w.handle, first, buf.data_ptr() + off, scb.data_ptr() + 8 + (off == 4), None,
+                                      int(torch.cuda.current_stream().cuda_stream))
+    _status_ok(dq)
+    assert st == 0
+    assert torch.equal(buf[off:off + nb], want.view(torch.uint8).flatten())
+    assert torch.equal(scb[8 + (off == 4):][:wsc.numel()], wsc.flatten())
