@@ -381,9 +381,13 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           variant 4 runs the kernel that dq_decode_linear takes for batches above 8 on matrices
  *           of 8192 rows and more (up to 32 columns in one pass over the weights, 16-row
  *           tiles, K walked in slices of 1024 with a power-of-two activation scale per slice) on
- *           any shape and batch; groups_per_cta (1..9) then sets its warps per CTA.
- *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = the tensor-core
- *           kernel dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison.
+ *           any shape and batch; groups_per_cta (1..9) then sets its warps per CTA.  variant 5 runs the
+ *           batch kernel that dequantises every weight once into tensor memory (all columns in one pass,
+ *           256-row tiles; DQ_ERR_INVALID_ARG for a codebook with levels that are not multiples of
+ *           2^-15); warps_per_group (1..8) then sets the CTAs that share a tile.
+ *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what
+ *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 5 = the batch
+ *           kernel as above, 6 = the mma.sync kernel.
  * Other arguments as dq_decode_linear.
  */
 int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int warps_per_group,

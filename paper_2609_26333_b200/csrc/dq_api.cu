@@ -17,6 +17,7 @@ struct dq_weights {
     unsigned formats;
     uint8_t *base;
     dq::PackedLayout layout;
+    bool lut3_split_exact;               // every LUT3 level is a multiple of 2^-15
 };
 
 namespace {
@@ -129,6 +130,16 @@ int clear_sf_padding(const dq::PackedLayout &L, uint8_t *base, int64_t N, int64_
     return cudaMemsetAsync(base + L.nv_sf_off + full, 0, L.nv_sf_bytes - full, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
+// levels times E4M3 scales then fit a pair of fp16 numbers exactly (the batch decode kernel asks for it)
+bool split_exact(const uint16_t cb[8])
+{
+    for (int j = 0; j < 8; ++j) {
+        const float v = __half2float(__ushort_as_half(cb[j])) * 32768.0f;
+        if (v != std::rint(v)) return false;
+    }
+    return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -217,6 +228,7 @@ int dq_pack_weights(const void *W_dev, int w_dtype, int64_t N, int64_t K, int64_
     w->formats = formats;
     w->base = base;
     w->layout = L;
+    w->lut3_split_exact = split_exact(cb);
     *out_host = w;
     return DQ_OK;
 }
@@ -283,6 +295,7 @@ int dq_import_canonical(int64_t N, int64_t K, unsigned formats, const void *nvfp
     w->formats = formats;
     w->base = base;
     w->layout = L;
+    w->lut3_split_exact = split_exact(cb);
     *out_host = w;
     return DQ_OK;
 }
@@ -322,6 +335,7 @@ int dq_import_canonical_lut2(int64_t N, int64_t K, const void *lut2_planes_dev, 
     w->formats = formats;
     w->base = base;
     w->layout = L;
+    w->lut3_split_exact = split_exact(cb);
     *out_host = w;
     return DQ_OK;
 }
@@ -544,7 +558,7 @@ int dq_prefill_linear(const dq_weights *w, const void *A_dev, int64_t M, int64_t
 }
 
 static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
-                        void *stream, bool tensor_cores)
+                        void *stream, int variant, int csize = 0)
 {
     if (!valid_handle(w) || !X_dev || !Y_dev) return DQ_ERR_INVALID_ARG;
     if (!has_nvfp4_view(w) || !on_handle_device(w)) return DQ_ERR_INVALID_ARG;
@@ -568,7 +582,16 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
     g.K = w->K;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t ce;
-    if (tensor_cores) {
+    // From five columns on, and where shared memory would cut a smaller batch into passes of the mma.sync kernel, the weights
+    // are dequantised once for all columns; below that the two are level but for long rows (measured, us, mma.sync kernel /
+    // that kernel: 34816x5120 batch 1 27.7 / 31, batch 8 33.3 / 31.6, batch 16 64 / 32; 4096x14336 batch 4 16.1 / 17.6,
+    // batch 5 28 / 17.8; 5120x17408 batch 4 42 / 21; few rows, 1024x4096 batch 1 7.6 / 6.5).  Rows above 32768 are refused by
+    // the mma.sync kernel, as for every batch.
+    const bool tc = variant == 5 || (variant == 0 && w->K <= 32768 &&
+                                     (B > 4 || w->N <= 1024 || (int64_t)(2 * w->K + 32) * B > 128 * 1024));
+    if (tc) {
+        ce = dq::launch_decode_tc_nvfp4(g, csize, s);
+    } else if (variant == 0 || variant == 6) {
         ce = dq::launch_gemv_nvfp4_mma(g, s);
     } else {
         // the comparison kernel's table of value pairs; with a launch in between it is never written by the kernel ahead
@@ -583,7 +606,7 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
 int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
                            void *stream)
 {
-    return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, true);
+    return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, 0);
 }
 
 static int decode_lut(const dq_weights *w, unsigned format, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev,
@@ -617,6 +640,7 @@ static int decode_lut(const dq_weights *w, unsigned format, const void *X_dev, i
     g.wait_cycles = wait_cycles;
     g.drop_first_copy = drop_first_copy;
     g.kernel = kernel;
+    g.split_exact = format != DQ_FMT_LUT3 || w->lut3_split_exact;
     const cudaError_t ce = dq::launch_gemv_lut(g, reinterpret_cast<cudaStream_t>(stream));
     if (ce == cudaErrorInvalidValue) return DQ_ERR_INVALID_ARG;
     if (ce != cudaSuccess) return DQ_ERR_CUDA;
@@ -640,12 +664,12 @@ int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int
                           int64_t ldy, void *stream)
 {
     if (format == DQ_FMT_NVFP4 || format == DQ_FMT_NVFP4_FROM_LUT3)
-        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant == 0);
+        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 ? warps_per_group : 0);
     if (warps_per_group < 0 || groups_per_cta < 0 || ring_stages < 0 || ring_stages > 8 || wait_cycles < 0)
         return DQ_ERR_INVALID_ARG;
-    if (variant < 0 || variant > 4) return DQ_ERR_INVALID_ARG;
+    if (variant < 0 || variant > 5) return DQ_ERR_INVALID_ARG;
     return decode_lut(w, format, X_dev, B, ldx, Y_dev, ldy, stream, warps_per_group, groups_per_cta, ring_stages,
-                      wait_cycles, variant == 1 ? 1 : 0, variant == 2 ? 1 : variant == 3 ? 2 : variant == 4 ? 3 : 0);
+                      wait_cycles, variant == 1 ? 1 : 0, variant == 2 ? 1 : variant == 3 ? 2 : variant >= 4 ? variant - 1 : 0);
 }
 
 int dq_export_canonical(const dq_weights *w, unsigned format, void *codes_dev, void *scales_dev,

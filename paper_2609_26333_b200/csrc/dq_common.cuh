@@ -214,6 +214,7 @@ struct GemmArgs {
 cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream);
 cudaError_t launch_gemm_nvfp4_pair(const GemmArgs &args, void *encode_fn, cudaStream_t stream);
 int gemm_init_driver_api();   // resolves the tensor-map encoder; 0 on success
+void *gemm_encode_fn();       // the encoder, after gemm_init_driver_api
 
 struct GemvArgs {
     int bits = 3;                                         // 3 = LUT3, 2 = LUT2
@@ -227,12 +228,18 @@ struct GemvArgs {
     int force_P = 0, force_G = 0, force_S = 0;
     long long wait_cycles = 0;
     int drop_first_copy = 0;                              // one warp's first copy is never requested (its wait must run out)
-    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8)
+    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8), 4 = dequantised through tcgen05 (any batch)
+    bool split_exact = true;                              // codebook levels are multiples of 2^-15 (launch_decode_tc)
 };
 cudaError_t launch_gemv_lut(const GemvArgs &args, cudaStream_t stream);     // picks one of the two kernels below
 // tcgen05 kernel (batch 1): number of warpgroups it would run this shape with, 0 where it does not take it
 int gemv_lut_tc_warpgroups(int bits, int64_t N, int64_t K, int64_t B, int sms, bool any_size);
 cudaError_t launch_gemv_lut_tc(const GemvArgs &args, int warpgroups, cudaStream_t stream);
+
+// dq_decode_tc.cu: up to 64 columns in one pass, dequantised weights through tcgen05.  LUT3 asks for a codebook whose levels
+// are multiples of 2^-15 (split_exact); force_P = CTAs per tile (test hook)
+cudaError_t launch_decode_tc(const GemvArgs &args, cudaStream_t stream);
+double decode_tc_slices(int64_t N, int64_t K, int sms);
 
 struct GemvNvArgs {
     const uint8_t *codes; const uint8_t *sf;              // NVFP4 view: [N][K/2] codes, MMA-layout scales
@@ -244,6 +251,7 @@ struct GemvNvArgs {
 };
 cudaError_t launch_gemv_nvfp4(const GemvNvArgs &args, cudaStream_t stream);          // CUDA cores, pair-table lookups
 cudaError_t launch_gemv_nvfp4_mma(const GemvNvArgs &args, cudaStream_t stream);      // tensor cores (mma.sync), no lookups
+cudaError_t launch_decode_tc_nvfp4(const GemvNvArgs &args, int force_csize, cudaStream_t stream);     // dq_decode_tc.cu
 cudaError_t launch_fill_e2m1_table(cudaStream_t stream);
 // read-only streaming sum with 128-bit loads (measurement): 8 bytes of result at out_dev
 cudaError_t launch_stream_read(const void *src_dev, size_t bytes, void *out_dev, cudaStream_t stream);   // value-pair table of the NVFP4 decode kernel

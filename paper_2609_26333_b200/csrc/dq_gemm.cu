@@ -269,6 +269,8 @@ int gemm_init_driver_api()
     return 0;
 }
 
+void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
+
 cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
 {
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;

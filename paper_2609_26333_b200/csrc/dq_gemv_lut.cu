@@ -1005,6 +1005,32 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
     return launch_one<BITS, 1024, 1, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
 }
 
+static bool wide_rows(int64_t N, int B) { return N >= 8192 || (B >= 16 && N >= 4096); }
+
+// Which calls the batch kernel of dq_decode_tc.cu takes from the two kernels of this file.  It dequantises a weight once for
+// all columns, at about 1.5 times what a pass of the kernels here costs for few columns (it multiplies the block scale in),
+// in tiles of 256 rows x 512 weights.  Measured (us; LUT3, this file's / that file's kernel):
+//   up to 8 columns: faster only where shared memory cuts the batch into passes (5120x17408 batch 8: 51 / 34; 4096x14336
+//     batch 6: 33 / 29) or there are few rows (512x256 batch 8: 7.0 / 4.8; 1024x4096: 10.3 / 8.5); 17408x5120 batch 8: 23.5 / 29;
+//   9 to 32 columns: against the slice-by-slice kernel, whose rounds over the rows a CTA of eight warps covers and slices of
+//     1024 cost 5.2 us up to 16 columns, 7.9 up to 24 and 8.7 up to 32 where a slice here costs 5.3 and the launch
+//     1.7 more (17408x5120 batch 16: 26.7 / 30.2; 16384x1024: 6.5 / 10.4; 10240x5120: 25.1 / 24.9; batch 24: 38.7 / 26.1); against
+//     passes of eight, always but for short rows (2048x1024 batch 16: 6.2 / 8.6; 4096x4096: 19.8 / 13.8);
+//   above 32: always (17408x5120 batch 40: 66 / 37).
+static bool tc_is_faster(int bits, int64_t N, int64_t K, int B, int sms)
+{
+    if (B <= 8) {
+        if (N <= 1024) return B >= 5;
+        return B >= 4 && choose_split(bits, N, K, sms, B).cols < B;
+    }
+    if (B > 32) return true;
+    if (!wide_rows(N, B)) return K > 1024 || B > 16;
+    const int64_t per_round = 8 * (int64_t)sms;
+    const double rounds = (double)((N / 16 + per_round - 1) / per_round) * (double)lut_slices(K);
+    const double wide = rounds * (B <= 16 ? 5.2 : B <= 24 ? 7.9 : 8.7) + 1.0;
+    return decode_tc_slices(N, K, sms) * 5.3 + 2.7 < wide;
+}
+
 // up to eight columns per pass
 cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
 {
@@ -1021,11 +1047,12 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
         if (wgs == 0) return cudaErrorInvalidValue;
         return launch_gemv_lut_tc(a, wgs, stream);
     }
-    // batches above 8 on enough rows to give every SM several 16-row tiles: the kernel that walks K slice by slice
-    // Batches above 8: one slice-by-slice pass over the weights per 32 columns instead of one pass per 8 columns, where
-    // that is faster (measured: from 8192 rows on, and from 4096 rows on for 16 columns and more)
-    if ((a.kernel == 3 || (a.kernel == 0 && a.force_P == 0 && B > 8 && (N >= 8192 || (B >= 16 && N >= 4096)))))
-        return launch_wide(a, sms, stream);
+    if (a.kernel == 4) return a.split_exact ? launch_decode_tc(a, stream) : cudaErrorInvalidValue;
+    const bool choose = a.kernel == 0 && a.force_P == 0;
+    if (choose && a.split_exact && tc_is_faster(a.bits, N, K, B, sms)) return launch_decode_tc(a, stream);
+    // Batches above 8 that stay here: one slice-by-slice pass over the weights per 32 columns instead of one pass per 8 columns,
+    // where that is faster (measured: from 8192 rows on, and from 4096 rows on for 16 columns and more)
+    if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, B))) return launch_wide(a, sms, stream);
     const int want_cols = B;                    // the split decides how many of them one pass takes
     Split sp = choose_split(a.bits, N, K, sms, want_cols);
     LutPlan L;

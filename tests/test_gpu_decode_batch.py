@@ -1,0 +1,161 @@
+"""GPU parity of the batch decode kernel (dequantised weights through tensor memory) against the CPU oracle, with the
+tolerances of parity_utils: every encoding, every column padding, ragged rows and row lengths, one and several CTAs a tile."""
+import numpy as np
+import pytest
+import torch
+
+import dq_inputs
+from parity_utils import check_outputs
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+TC = 5                                   # test-hook variant: this kernel whatever the batch
+
+
+@pytest.fixture(scope="module")
+def dq():
+    import __graft_entry__ as g
+    g.build()
+    import paper_2609_26333_b200 as dq
+    return dq
+
+
+def _status_ok(dq):
+    torch.cuda.synchronize()
+    st, det = dq.get_status()
+    assert st == 0, f"device status {dq.status_string(st)} detail {det}"
+
+
+_cache = {}
+
+
+def _layer(oracle, N, K):
+    if (N, K) not in _cache:
+        W = dq_inputs.gaussian_bf16(N, K, 0.02, 500 + N + K)
+        Wf = dq_inputs.bf16_to_f32_numpy(W)
+        ref = oracle.pack_weights(Wf)
+        ref["lut2_planes"], ref["lut2_scales"] = oracle.quant_lut2(Wf, ref["s"])
+        _cache[(N, K)] = (W, ref)
+    return _cache[(N, K)]
+
+
+def _reference(oracle, ref, fmt, X):
+    Xf = dq_inputs.bf16_to_f32_numpy(X)
+    if fmt == "lut3":
+        return oracle.decode_linear(Xf, ref["lut3_planes"], ref["lut3_scales"], ref["s"])
+    if fmt == "lut2":
+        return oracle.decode_linear_lut2(Xf, ref["lut2_planes"], ref["lut2_scales"], ref["s"])
+    return oracle.decode_linear_nvfp4(Xf, ref["nvfp4_codes"], ref["nvfp4_scales"], ref["s"])
+
+
+def _f64(t):
+    return t.detach().float().cpu().numpy().astype(np.float64)
+
+
+# one row tile and less, the last half tile missing or ragged, K inside a slice of 512 and inside a 128-weight pair
+SHAPES = [(16, 128), (144, 384), (272, 640), (400, 1152), (1040, 2048)]
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
+@pytest.mark.parametrize("N,K", SHAPES)
+@pytest.mark.parametrize("B", [1, 9, 16, 17, 33, 48, 64])
+def test_decode_batch_parity(dq, oracle, fmt, N, K, B):
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 900 + B)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    big = torch.zeros(B, K + 24, dtype=torch.bfloat16, device=DEV)        # strided activations, guarded strided outputs
+    big[:, :K] = X.to(DEV)
+    out = torch.full((B + 1, N + 8), 7.0, dtype=torch.bfloat16, device=DEV)
+    dq.test_decode_linear(w, code, big[:, :K], out=out[:B, :N], variant=TC)
+    _status_ok(dq)
+    check_outputs(_f64(out[:B, :N]), Yr, S, f"{fmt} {B}x{N}x{K}")
+    assert torch.all(out[B] == 7.0) and torch.all(out[:, N:] == 7.0)
+    if B > 8:                                                             # what the public entry point runs
+        y = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2, "nvfp4": dq.decode_linear_nvfp4}[fmt](w, X.to(DEV))
+        _status_ok(dq)
+        check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K} public")
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "nvfp4"])
+@pytest.mark.parametrize("csize", [1, 2, 3, 5, 8])
+@pytest.mark.parametrize("B", [10, 40, 61])
+def test_decode_batch_ctas_per_tile(dq, oracle, fmt, csize, B):
+    N, K = 784, 4224                                                      # nine slices, the last one short
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 700 + B)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    outs = []
+    for _ in range(2):
+        y = torch.full((B, N), float("nan"), dtype=torch.bfloat16, device=DEV)
+        dq.test_decode_linear(w, code, X.to(DEV), out=y, variant=TC, warps_per_group=csize)
+        outs.append(y)
+    _status_ok(dq)
+    check_outputs(_f64(outs[0]), Yr, S, f"{fmt} {csize} CTAs a tile, batch {B}")
+    assert torch.equal(outs[0], outs[1])                                  # sums in a fixed order
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
+def test_decode_batch_wide_range_and_sparse_activations(dq, oracle, fmt):
+    """Columns that differ by 2^60, elements down to 2^-28 of a slice's largest, zero columns, single non-zeros."""
+    N, K, B = 272, 1152, 20
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 77).float()
+    g = torch.Generator().manual_seed(5)
+    X *= torch.pow(2.0, torch.randint(-20, 1, (B, K), generator=g).float())
+    X *= torch.pow(2.0, torch.linspace(-30, 30, B).round())[:, None]
+    X[3] = 0
+    X[4, 1:] = 0
+    X[5, :1000] = 0
+    X = X.to(torch.bfloat16)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    y = dq.test_decode_linear(w, code, X.to(DEV), variant=TC)
+    _status_ok(dq)
+    Y = _f64(y)
+    for b in range(B):                                                    # per column: the Frobenius check must not hide small ones
+        check_outputs(Y[b:b + 1], Yr[b:b + 1], S[b:b + 1], f"{fmt} column {b}")
+    # one-hot columns: the weight itself, rounded to bf16 once
+    E = torch.zeros(16, K, dtype=torch.bfloat16)
+    ks = [0, 3, 4, 15, 16, 37, 127, 128, 511, 512, 639, 640, 1000, 1023, 1024, 1151]
+    E[torch.arange(16), torch.tensor(ks)] = 1.0
+    Yr, _ = _reference(oracle, ref, fmt, E)
+    y = dq.test_decode_linear(w, code, E.to(DEV), variant=TC)
+    _status_ok(dq)
+    assert torch.equal(y.float().cpu(), torch.from_numpy(Yr).to(torch.float32).to(torch.bfloat16).float())
+
+
+def test_decode_batch_fine_codebook_takes_the_general_path(dq, oracle):
+    """Levels that are not multiples of 2^-15 do not fit the kernel's pair of fp16 numbers under every block scale."""
+    N, K, B = 272, 640, 12
+    W, _ = _layer(oracle, N, K)
+    cb = torch.tensor([-4.0, -2.0, -0.001, 0.0, 0.0011, 2.5, 4.0, 6.0], dtype=torch.float16)
+    bits = [int(v) & 0xFFFF for v in cb.view(torch.int16)]
+    w = dq.pack_weights(W.to(DEV), formats=dq.FMT_LUT3, codebook_f16=bits)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 12).to(DEV)
+    with pytest.raises(dq.DQError):
+        dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=TC)
+    planes, scales, s = dq.export_canonical(w, dq.FMT_LUT3)
+    bit = (planes.long()[:, :, :, None] >> torch.arange(32, device=DEV)) & 1
+    idx = (bit[:, 0] + 2 * bit[:, 1] + 4 * bit[:, 2]).flatten(1)
+    Wd = cb.double().to(DEV)[idx] * scales.view(torch.float8_e4m3fn).double().repeat_interleave(16, dim=1) * s.double()
+    Y = dq.decode_linear(w, X)
+    _status_ok(dq)
+    check_outputs(_f64(Y), (X.double() @ Wd.T).cpu().numpy(), (X.double().abs() @ Wd.abs().T).cpu().numpy(), "fine codebook")
+
+
+def test_decode_batch_wait_runs_out(dq):
+    """A ring stage that is never requested: the waits run out, the launch returns and reports."""
+    w = dq.pack_weights(dq_inputs.gaussian_bf16(256, 512, 0.02, 1).to(DEV), formats=dq.FMT_LUT3)
+    X = dq_inputs.gaussian_bf16(12, 512, 1.0, 2).to(DEV)
+    good = dq.decode_linear(w, X)
+    dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=1, wait_cycles=2_000_000)
+    torch.cuda.synchronize()
+    st, _ = dq.get_status()
+    assert dq.status_string(st) == "device-side wait ran out"
+    assert torch.equal(dq.decode_linear(w, X), good)
+    _status_ok(dq)
