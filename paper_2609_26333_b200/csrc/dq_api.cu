@@ -465,6 +465,7 @@ static int prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, 
     g.a_sf = ws + L.a_sf;
     g.w_codes = has_nvfp4_view(w) ? w->base + w->layout.nv_codes_off : ws + L.w_codes;
     g.w_sf = has_nvfp4_view(w) ? w->base + w->layout.nv_sf_off : ws + L.w_sf;
+    g.w_const = has_nvfp4_view(w);
     g.hdr = reinterpret_cast<const dq::PackedHeader *>(w->base);
     g.act_scale = act_global_scale;
     g.Y = Y_dev;

@@ -206,6 +206,7 @@ struct GemmArgs {
     void *Y; int64_t ldy;
     int64_t M, N, K;
     StatusWord *status;
+    bool w_const = false;    // w_codes / w_sf belong to the handle (not cast into the workspace for this call)
     bool mma_only = false;   // measurement: MMA issue sequence only (pair kernel; no loads, scale copies or stores)
     // gated epilogue (pair kernel only): W is a fused gate/up matrix with interleaved rows, and instead of Y the kernel
     // writes NVFP4(bf16(SiLU(gate) * up)) with input scale gated_scale: codes [M][N/4], block scales in the MMA's layout

@@ -3,13 +3,21 @@
 // tensor scales):
 //   Y[m][n] = bf16( s_a * s_w * sum_blk dA[m][blk] dW[n][blk] sum_{k in blk} eA[m][k] eW[n][k] )
 //
-// One persistent CTA per SM, 128 x 256 output tiles, 256-element k-steps.
-//   warp 0      : TMA producer (packed FP4 tiles, 128B swizzle) + bulk copies of the scale atoms
+// One CTA per SM and 128-row tile: the kernel of short prompts, where the weights stream from HBM and what counts is that every
+// SM streams its share of them.  Tiles are 128 x 256 or 128 x 128; where there are too few of them for the chip a cluster of up to
+// 8 CTAs shares one, each taking a range of k-steps, and they exchange partial sums through distributed shared memory at
+// the end (added in rank order; no workspace).  256-element k-steps.
+//   warp 0      : TMA producer (packed FP4 tiles, 128B swizzle) + bulk copies of the scale atoms; weights that are part of the
+//                 handle are requested before the kernel ahead (the activation quantiser) has finished
 //   warp 1      : tcgen05.cp of the scales into TMEM and tcgen05.mma (kind::mxf4nvf4, block 16)
 //   warps 2..5  : epilogue, TMEM -> registers -> bf16 -> global
-// The fp32 accumulator lives in TMEM (256 columns); the scale factors of the four stages
-// occupy 4 x 48 further columns.  Every mbarrier wait is bounded: when it runs
+// The fp32 accumulator lives in TMEM (two of 128 columns or one of 256) beside the scale factors of every stage.  Producer and MMA
+// roles are one elected thread each, waits included: see elect_one.  Every mbarrier wait is bounded: when it runs
 // out the CTA records DQ_ERR_TIMEOUT in the status word and leaves normally.
+// Bound by the weights' way from HBM and the launches: one layer of the 27B-class stack (203 MB) at 77 tokens, quantisers and GEMMs,
+// takes 71 us; with lone CTAs on 128 x 256 tiles, 20 to 136 of them, it took 104.
+#include <atomic>
+
 #include <cuda.h>
 
 #include "dq_common.cuh"
@@ -19,29 +27,32 @@ namespace dq {
 
 namespace {
 
+using namespace tc;
+
 constexpr int BM = 128;
-constexpr int BN = 256;
-constexpr int BK = 256;                       // elements; 128 bytes of packed FP4 = one swizzle row
-constexpr int kStages = 4;
-constexpr int kKbPerStage = BK / 64;          // MMA k-steps (64 elements) per stage
-constexpr uint32_t A_STAGE_BYTES = BM * 128;  // 16 KiB
-constexpr uint32_t B_STAGE_BYTES = BN * 128;  // 32 KiB
-constexpr uint32_t SFA_STAGE_BYTES = kKbPerStage * 512;
-constexpr uint32_t SFB_STAGE_BYTES = 2 * kKbPerStage * 512;
-constexpr uint32_t STAGE_BYTES = A_STAGE_BYTES + B_STAGE_BYTES + SFA_STAGE_BYTES + SFB_STAGE_BYTES;
-constexpr uint32_t SMEM_BYTES = kStages * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
+constexpr int kKbPerStage = 4;                // 64-element MMA k-steps per 256-element stage (128 bytes of FP4: one swizzle row)
 constexpr int kThreads = 192;
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kTmemSfBase = 256;         // accumulator uses columns [0, 256)
-constexpr uint32_t kTmemSfBufCols = 48;       // 16 (A) + 32 (B), one buffer per smem stage: free again when the stage is
 
-static_assert(STAGE_BYTES % 1024 == 0, "stage must keep 1024-byte alignment for the 128B swizzle");
-
-// instruction descriptor: dense, A/B = E2M1 (kind::mxf4nvf4), both K-major, scale type UE4M3,
-// N >> 3 at bit 17, M >> 4 at bit 24, scale-factor ids 0, K = 64
-constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-
-using namespace tc;
+template <int BN>
+struct Cfg {
+    static constexpr int kStages = BN == 128 ? 6 : 4;
+    static constexpr int kAccs = BN == 128 ? 2 : 1;                    // accumulators
+    static constexpr int kSfbAtoms = BN / 128;
+    static constexpr uint32_t A_BYTES = BM * 128, B_BYTES = BN * 128;
+    static constexpr uint32_t SFA_BYTES = kKbPerStage * 512, SFB_BYTES = kSfbAtoms * kKbPerStage * 512;
+    static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES + SFA_BYTES + SFB_BYTES;
+    static constexpr uint32_t SMEM_BYTES = kStages * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
+    static constexpr uint32_t kSfBase = kAccs * BN;                    // TMEM columns: accumulators, then scales per stage
+    static constexpr uint32_t kSfbCol = 4 * kKbPerStage, kSfCols = kSfbCol + 4 * kKbPerStage * kSfbAtoms;
+    static_assert(kSfBase + kStages * kSfCols <= kTmemCols, "scale buffers must fit in TMEM");
+    static_assert(STAGE_BYTES % 1024 == 0, "stages must keep 1024-byte alignment for the 128B swizzle");
+    static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+    static_assert((BN / 8 + 8) * BM * 32 <= kStages * (int)STAGE_BYTES, "partial sums of a cluster must fit the ring");
+    // instruction descriptor: dense, A/B = E2M1 (kind::mxf4nvf4), both K-major, scale type UE4M3,
+    // N >> 3 at bit 17, M >> 4 at bit 24, scale-factor ids 0, K = 64
+    static constexpr uint32_t kInstrDesc = (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+};
 
 // tile index -> (m block, n block): m fastest inside groups of 16 m-blocks so that
 // the CTAs running at the same time share A row-blocks and W column-blocks in L2
@@ -56,24 +67,47 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
     mb = first_m + r % gsz;
     nb = r / gsz;
 }
+__device__ __forceinline__ uint32_t cluster_ctarank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t rank, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("{\n\t.reg .b32 p;\n\tmapa.shared::cluster.u32 p, %0, %1;\n\tst.shared::cluster.v4.b32 [p], {%2, %3, %4, %5};\n\t}"
+                 ::"r"(addr), "r"(rank), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ float4 lds_v4f(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
 
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const uint8_t *__restrict__ a_sf, const uint8_t *__restrict__ w_sf,
                   const PackedHeader *__restrict__ hdr, float act_scale, __nv_bfloat16 *__restrict__ Y, int64_t ldy,
-                  int M, int N, int K, StatusWord *status)
+                  int M, int N, int K, int csize, int early_weights, StatusWord *status)
 {
+    using C = Cfg<BN>;
+    constexpr int kStages = C::kStages, kAccs = C::kAccs;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-    // per stage: [A 16K][B 32K][SFA 2K][SFB 4K]
-    const uint32_t bar_base = smem_base + kStages * STAGE_BYTES;
-    // barriers: full[kStages], empty[kStages], tmem_full, tmem_empty ; then tmem ptr, abort flag
+    // per stage: [A][B][SFA][SFB]; barriers: full[kStages], empty[kStages], tmem_full[2], tmem_empty[2]; then tmem ptr, abort flag
+    const uint32_t bar_base = smem_base + kStages * C::STAGE_BYTES;
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
-    const uint32_t tmem_full_bar = bar_base + 8u * (2 * kStages);
-    const uint32_t tmem_empty_bar = bar_base + 8u * (2 * kStages + 1);
-    uint32_t *tmem_ptr_smem = reinterpret_cast<uint32_t *>(smem_gen + kStages * STAGE_BYTES + 8 * (2 * kStages + 2));
+    auto tmem_full_bar = [&](int i) { return bar_base + 8u * (2 * kStages + i); };
+    auto tmem_empty_bar = [&](int i) { return bar_base + 8u * (2 * kStages + 2 + i); };
+    uint32_t *tmem_ptr_smem = reinterpret_cast<uint32_t *>(smem_gen + kStages * C::STAGE_BYTES + 8 * (2 * kStages + 4));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_ptr_smem + 1);
 
     const int warp = threadIdx.x >> 5;
@@ -81,8 +115,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-        mbar_init(tmem_full_bar, 1);
-        mbar_init(tmem_empty_bar, 4);
+        for (int i = 0; i < 2; ++i) { mbar_init(tmem_full_bar(i), 1); mbar_init(tmem_empty_bar(i), 4); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -96,131 +129,201 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_ptr_smem;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     const int tiles_m = (M + BM - 1) / BM;
     const int tiles_n = (N + BN - 1) / BN;
     const int num_tiles = tiles_m * tiles_n;
     const int katoms = K / 64;                                // 64-element k atoms in K
     const int num_ks = (katoms + kKbPerStage - 1) / kKbPerStage;
+    const uint32_t rank = csize > 1 ? cluster_ctarank() : 0u;
+    const int first_tile = (int)blockIdx.x / csize, tile_stride = (int)gridDim.x / csize;
+    const int k0 = (int)((long long)num_ks * rank / csize), k1 = (int)((long long)num_ks * (rank + 1) / csize);
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        {
+        if (elect_one()) {
+            auto load_w = [&](int stage, int nb, int ks) {
+                const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
+                const uint32_t sB = smem_base + stage * C::STAGE_BYTES + C::A_BYTES, sSFB = sB + C::B_BYTES + C::SFA_BYTES;
+                const uint32_t sf_bytes = (uint32_t)nkb * 512u;
+                mbar_expect_tx(full_bar(stage), C::A_BYTES + C::B_BYTES + (1u + C::kSfbAtoms) * sf_bytes);
+                tma_load_2d(sB, &tmap_w, ks * 128, nb * BN, full_bar(stage));
+#pragma unroll
+                for (int at = 0; at < C::kSfbAtoms; ++at)
+                    bulk_load(sSFB + (uint32_t)at * kKbPerStage * 512u,
+                              w_sf + ((size_t)(C::kSfbAtoms * nb + at) * katoms + (size_t)ks * kKbPerStage) * 512, sf_bytes, full_bar(stage));
+            };
+            auto load_a = [&](int stage, int mb, int ks) {
+                const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
+                const uint32_t sA = smem_base + stage * C::STAGE_BYTES, sSFA = sA + C::A_BYTES + C::B_BYTES;
+                tma_load_2d(sA, &tmap_a, ks * 128, mb * BM, full_bar(stage));
+                bulk_load(sSFA, a_sf + ((size_t)mb * katoms + (size_t)ks * kKbPerStage) * 512, (uint32_t)nkb * 512u, full_bar(stage));
+            };
+            // The weights of a handle are constant data: the first stages of them are requested before waiting for the kernel ahead,
+            // which makes the activations (weights cast into the workspace for this call are made by it too)
+            int early = 0;
+            if (early_weights && first_tile < num_tiles) {
+                int mb, nb;
+                tile_coords(first_tile, tiles_m, tiles_n, mb, nb);
+                early = min(kStages, k1 - k0);
+                for (int i = 0; i < early; ++i) load_w(i, nb, k0 + i);
+            }
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+            for (int t = first_tile; t < num_tiles && ok; t += tile_stride) {
                 int mb, nb;
                 tile_coords(t, tiles_m, tiles_n, mb, nb);
-                for (int ks = 0; ks < num_ks; ++ks) {
-                    if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
-                    const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
-                    const uint32_t sA = smem_base + stage * STAGE_BYTES;
-                    const uint32_t sB = sA + A_STAGE_BYTES;
-                    const uint32_t sSFA = sB + B_STAGE_BYTES;
-                    const uint32_t sSFB = sSFA + SFA_STAGE_BYTES;
-                    const uint32_t sf_bytes = (uint32_t)nkb * 512u;
-                    const size_t koff = (size_t)ks * kKbPerStage * 512;
-                    if (elect_one()) {
-                        mbar_expect_tx(full_bar(stage), A_STAGE_BYTES + B_STAGE_BYTES + 3u * sf_bytes);
-                        tma_load_2d(sA, &tmap_a, ks * 128, mb * BM, full_bar(stage));
-                        tma_load_2d(sB, &tmap_w, ks * 128, nb * BN, full_bar(stage));
-                        bulk_load(sSFA, a_sf + ((size_t)mb * katoms) * 512 + koff, sf_bytes, full_bar(stage));
-                        bulk_load(sSFB, w_sf + ((size_t)(2 * nb) * katoms) * 512 + koff, sf_bytes, full_bar(stage));
-                        bulk_load(sSFB + kKbPerStage * 512, w_sf + ((size_t)(2 * nb + 1) * katoms) * 512 + koff, sf_bytes,
-                                  full_bar(stage));
+                for (int ks = k0; ks < k1; ++ks) {
+                    if (early > 0) {
+                        --early;
+                    } else {
+                        if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
+                        load_w(stage, nb, ks);
                     }
-                    __syncwarp();
+                    load_a(stage, mb, ks);
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA issuer
-        {
+        if (elect_one()) {
             int stage = 0; uint32_t phase = 0;
-            uint32_t acc_phase = 0;
+            uint32_t it = 0;                                   // tiles: accumulator it % kAccs
             bool ok = true;
-            for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-                if (!mbar_wait_warp(tmem_empty_bar, acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+            for (int t = first_tile; t < num_tiles && ok; t += tile_stride, ++it) {
+                const uint32_t acc = it % kAccs;
+                ok = mbar_wait(tmem_empty_bar(acc), ((it / kAccs) & 1u) ^ 1u, abort_flag);
+                if (!ok) break;
                 tc_fence_after();
-                for (int ks = 0; ks < num_ks; ++ks) {
-                    if (!mbar_wait_warp(full_bar(stage), phase, abort_flag)) { ok = false; break; }
+                const uint32_t d_tmem = tmem_base + acc * BN;
+                for (int ks = k0; ks < k1; ++ks) {
+                    if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const int nkb = min(kKbPerStage, katoms - ks * kKbPerStage);
-                    const uint32_t sA = smem_base + stage * STAGE_BYTES;
-                    const uint32_t sB = sA + A_STAGE_BYTES;
-                    const uint32_t sSFA = sB + B_STAGE_BYTES;
-                    const uint32_t sSFB = sSFA + SFA_STAGE_BYTES;
-                    const uint32_t t_sfa = tmem_base + kTmemSfBase + (uint32_t)stage * kTmemSfBufCols;
-                    const uint32_t t_sfb = t_sfa + 16u;
+                    const uint32_t sA = smem_base + stage * C::STAGE_BYTES;
+                    const uint32_t sB = sA + C::A_BYTES, sSFA = sB + C::B_BYTES, sSFB = sSFA + C::SFA_BYTES;
+                    const uint32_t t_sfa = tmem_base + C::kSfBase + (uint32_t)stage * C::kSfCols;
+                    const uint32_t t_sfb = t_sfa + C::kSfbCol;
                     const uint64_t adesc = make_desc_sw128(sA), bdesc = make_desc_sw128(sB);
                     const uint64_t fadesc = make_desc_sf(sSFA), fbdesc = make_desc_sf(sSFB);
-                    if (elect_one()) {
 #pragma unroll
-                        for (int kb = 0; kb < kKbPerStage; ++kb) {
-                            if (kb < nkb) {
-                                tmem_cp_sf(t_sfa + 4u * kb, fadesc + 32ull * kb);
-                                tmem_cp_sf(t_sfb + 8u * kb, fbdesc + 32ull * kb);
-                                tmem_cp_sf(t_sfb + 8u * kb + 4u, fbdesc + (kKbPerStage * 512u >> 4) + 32ull * kb);
-                            }
-                        }
+                    for (int kb = 0; kb < kKbPerStage; ++kb) {
+                        if (kb < nkb) {
+                            tmem_cp_sf(t_sfa + 4u * kb, fadesc + 32ull * kb);
 #pragma unroll
-                        for (int kb = 0; kb < kKbPerStage; ++kb) {
-                            // one k-step is 64 elements = 32 bytes inside the 128-byte swizzle row
-                            if (kb < nkb)
-                                mma_nvf4(tmem_base, adesc + 2ull * kb, bdesc + 2ull * kb, kInstrDesc, t_sfa + 4u * kb,
-                                         t_sfb + 8u * kb, (ks > 0 || kb > 0) ? 1u : 0u);
+                            for (int at = 0; at < C::kSfbAtoms; ++at)
+                                tmem_cp_sf(t_sfb + 4u * C::kSfbAtoms * kb + 4u * at, fbdesc + (uint64_t)(at * (kKbPerStage * 512 >> 4)) + 32ull * kb);
                         }
-                        mma_commit(empty_bar(stage));          // frees the stage once these MMAs have read it
-                        if (ks + 1 == num_ks) mma_commit(tmem_full_bar);       // accumulator complete
                     }
-                    __syncwarp();
+#pragma unroll
+                    for (int kb = 0; kb < kKbPerStage; ++kb) {
+                        // one k-step is 64 elements = 32 bytes inside the 128-byte swizzle row
+                        if (kb < nkb)
+                            mma_nvf4(d_tmem, adesc + 2ull * kb, bdesc + 2ull * kb, C::kInstrDesc, t_sfa + 4u * kb,
+                                     t_sfb + 4u * C::kSfbAtoms * kb, (ks > k0 || kb > 0) ? 1u : 0u);
+                    }
+                    mma_commit(empty_bar(stage));          // frees the stage once these MMAs have read it
                     if (++stage == kStages) { stage = 0; phase ^= 1u; }
                 }
-                acc_phase ^= 1u;
+                if (ok) mma_commit(tmem_full_bar(acc));    // accumulator complete
             }
         }
     } else {
         // ------------------------------------------------------------ epilogue
         const int wq = warp & 3;                           // TMEM lane quarter this warp may read
+        const uint32_t lanes = (uint32_t)(wq * 32) << 16;
         const float alpha = __fmul_rn(act_scale, hdr->s);
-        uint32_t acc_phase = 0;
         bool ok = true;
-        for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
-            int mb, nb;
-            tile_coords(t, tiles_m, tiles_n, mb, nb);
-            if (!mbar_wait(tmem_full_bar, acc_phase, abort_flag)) { ok = false; break; }
-            tc_fence_after();
-            const int row = mb * BM + wq * 32 + lane;
-            __nv_bfloat16 *yrow = Y + (int64_t)row * ldy + (int64_t)nb * BN;
+        if (csize == 1) {
+            uint32_t it = 0;
+            for (int t = first_tile; t < num_tiles && ok; t += tile_stride, ++it) {
+                const uint32_t acc = it % kAccs;
+                int mb, nb;
+                tile_coords(t, tiles_m, tiles_n, mb, nb);
+                ok = mbar_wait_warp(tmem_full_bar(acc), (it / kAccs) & 1u, abort_flag);
+                if (!ok) break;
+                tc_fence_after();
+                const int row = mb * BM + wq * 32 + lane;
+                __nv_bfloat16 *yrow = Y + (int64_t)row * ldy + (int64_t)nb * BN;
+                if (mb * BM + wq * 32 < M) {               // whole warps of padding rows read nothing
 #pragma unroll 1
-            for (int c = 0; c < BN / 32; ++c) {
-                uint32_t v[32];
-                tmem_ld32(tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(c * 32), v);
-                tmem_ld_wait();
-                if (row < M) {
+                    for (int c = 0; c < BN / 32; ++c) {
+                        uint32_t v[32];
+                        tmem_ld32(tmem_base + acc * BN + lanes + (uint32_t)(c * 32), v);
+                        tmem_ld_wait();
+                        if (row < M) {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int col = nb * BN + c * 32 + q * 8;
-                        if (col < N) {
-                            uint4 o;
-                            o.x = pack_bf16x2(__uint_as_float(v[8 * q + 0]) * alpha, __uint_as_float(v[8 * q + 1]) * alpha);
-                            o.y = pack_bf16x2(__uint_as_float(v[8 * q + 2]) * alpha, __uint_as_float(v[8 * q + 3]) * alpha);
-                            o.z = pack_bf16x2(__uint_as_float(v[8 * q + 4]) * alpha, __uint_as_float(v[8 * q + 5]) * alpha);
-                            o.w = pack_bf16x2(__uint_as_float(v[8 * q + 6]) * alpha, __uint_as_float(v[8 * q + 7]) * alpha);
-                            *reinterpret_cast<uint4 *>(yrow + c * 32 + q * 8) = o;
+                            for (int q = 0; q < 4; ++q) {
+                                if (nb * BN + c * 32 + q * 8 < N) {
+                                    uint4 o;
+                                    o.x = pack_bf16x2(__uint_as_float(v[8 * q + 0]) * alpha, __uint_as_float(v[8 * q + 1]) * alpha);
+                                    o.y = pack_bf16x2(__uint_as_float(v[8 * q + 2]) * alpha, __uint_as_float(v[8 * q + 3]) * alpha);
+                                    o.z = pack_bf16x2(__uint_as_float(v[8 * q + 4]) * alpha, __uint_as_float(v[8 * q + 5]) * alpha);
+                                    o.w = pack_bf16x2(__uint_as_float(v[8 * q + 6]) * alpha, __uint_as_float(v[8 * q + 7]) * alpha);
+                                    *reinterpret_cast<uint4 *>(yrow + c * 32 + q * 8) = o;
+                                }
+                            }
+                        }
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tmem_empty_bar(acc));
+            }
+        } else {
+            // One tile per cluster.  Eight columns i of the tile go to CTA i % csize; after the first barrier everybody's copies and MMAs
+            // are over and the ring takes the partial sums: [source][group of this CTA][128 rows][8 columns].
+            int mb, nb;
+            tile_coords(first_tile, tiles_m, tiles_n, mb, nb);
+            ok = mbar_wait_warp(tmem_full_bar(0), 0u, abort_flag);
+            tc_fence_after();
+            cluster_sync();
+            const int per = (BN / 8 + csize - 1) / csize;
+            const int row = mb * BM + wq * 32 + lane;
+            const uint32_t mine = smem_base + (uint32_t)(wq * 32 + lane) * 16u;       // + 2048 for the second half of a group
+            if (ok && mb * BM + wq * 32 < M) {
+#pragma unroll 1
+                for (int c = 0; c < BN / 32; ++c) {
+                    uint32_t v[32];
+                    tmem_ld32(tmem_base + lanes + (uint32_t)(c * 32), v);
+                    tmem_ld_wait();
+                    if (row < M) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int i = c * 4 + q;
+                            const uint32_t dst = mine + (uint32_t)((int)rank * per + i / csize) * 4096u;
+                            st_cluster_v4(dst, (uint32_t)(i % csize), v[8 * q], v[8 * q + 1], v[8 * q + 2], v[8 * q + 3]);
+                            st_cluster_v4(dst + 2048u, (uint32_t)(i % csize), v[8 * q + 4], v[8 * q + 5], v[8 * q + 6], v[8 * q + 7]);
                         }
                     }
                 }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tmem_empty_bar);
-            acc_phase ^= 1u;
+            cluster_sync();
+            if (ok && row < M) {
+                for (int i = (int)rank, l = 0; i < BN / 8 && nb * BN + 8 * i < N; i += csize, ++l) {
+                    float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+                    for (int src = 0; src < csize; ++src) {
+                        const uint32_t at = mine + (uint32_t)(src * per + l) * 4096u;
+                        const float4 x = lds_v4f(at), y = lds_v4f(at + 2048u);
+                        a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+                        b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
+                    }
+                    uint4 o;
+                    o.x = pack_bf16x2(a.x * alpha, a.y * alpha);
+                    o.y = pack_bf16x2(a.z * alpha, a.w * alpha);
+                    o.z = pack_bf16x2(b.x * alpha, b.y * alpha);
+                    o.w = pack_bf16x2(b.z * alpha, b.w * alpha);
+                    *reinterpret_cast<uint4 *>(Y + (int64_t)row * ldy + (int64_t)nb * BN + 8 * i) = o;
+                }
+            }
         }
     }
-
     __syncwarp();
+    if (csize > 1 && warp < 2) { cluster_sync(); cluster_sync(); }
+
     tc_fence_before();
     __syncthreads();
     if (*abort_flag) {
@@ -256,6 +359,87 @@ bool make_codes_tmap(CUtensorMap *tm, const void *ptr, int64_t rows, int64_t K, 
     return r == CUDA_SUCCESS;
 }
 
+constexpr int kMaxCluster = 8;
+struct Split { int csize; double cost; };
+
+template <int BN>
+cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int csize, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = Cfg<BN>::SMEM_BYTES;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)csize;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = csize > 1 ? 2 : 1;
+    return cfg;
+}
+
+template <int BN>
+cudaError_t set_attributes(int dev)
+{
+    static std::atomic<bool> done[kMaxDevices];
+    if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
+    if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
+    return e;
+}
+
+// CTAs per tile of 128 x BN: bytes of weights (rows x k-steps) that the busiest CTA streams, the activation tile of a step counted
+// as 48 rows (it comes from L2) and a cluster's exchange as 600.  A cluster takes one tile, and all must be resident;
+// how many of a size fit is asked once per device.
+template <int BN>
+Split choose_split(const GemmArgs &a, int dev, int sms)
+{
+    static std::atomic<int> max_clusters[kMaxDevices][kMaxCluster + 1];          // + 1; 0 = not asked yet
+    const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
+    const int num_ks = (int)((a.K / 64 + kKbPerStage - 1) / kKbPerStage);
+    const double step = BN + 48.0;
+    Split best = {1, (double)((tiles + sms - 1) / sms) * num_ks * step};
+    for (int c = 2; c <= kMaxCluster && c <= num_ks && tiles * c <= sms; ++c) {
+        int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
+        if (fit == 0) {
+            cudaLaunchAttribute attr[2];
+            const cudaLaunchConfig_t cfg = launch_config<BN>(attr, c * (sms / c), c, nullptr);
+            int n = 0;
+            if (set_attributes<BN>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN>, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            fit = n + 1;
+            max_clusters[dev][c].store(fit, std::memory_order_relaxed);
+        }
+        if (tiles > fit - 1) continue;
+        const double cost = (double)((num_ks + c - 1) / c) * step + 600.0;
+        if (cost < best.cost) best = {c, cost};
+    }
+    return best;
+}
+
+template <int BN>
+cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaError_t e = set_attributes<BN>(dev);
+    if (e != cudaSuccess) return e;
+    CUtensorMap tmap_a, tmap_w;
+    if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
+    if (!make_codes_tmap(&tmap_w, a.w_codes, a.N, a.K, BN)) return cudaErrorInvalidValue;
+    const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
+    const int grid = (int)(sp.csize > 1 ? tiles * sp.csize : (tiles < sms ? tiles : sms));
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = launch_config<BN>(attr, grid, sp.csize, stream);
+    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
+                              reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M, (int)a.N, (int)a.K, sp.csize,
+                              a.w_const ? 1 : 0, a.status);
+}
+
 }  // namespace
 
 int gemm_init_driver_api()
@@ -276,26 +460,12 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
     // more than one 128-row block: CTA pairs share the W tile; otherwise a lone CTA per tile
     // (the gated epilogue exists in the pair kernel only)
-    if (a.M > BM || a.gated_codes) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
-    static bool attr_set[kMaxDevices] = {};
-    int dev = 0;
+    int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        attr_set[dev] = true;
-    }
-    CUtensorMap tmap_a, tmap_w;
-    if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
-    if (!make_codes_tmap(&tmap_w, a.w_codes, a.N, a.K, BN)) return cudaErrorInvalidValue;
-    int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tiles = (int)(((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN));
-    const int grid = tiles < sms ? tiles : sms;
-    gemm_nvfp4_kernel<<<grid, kThreads, SMEM_BYTES, stream>>>(tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
-                                                             reinterpret_cast<__nv_bfloat16 *>(a.Y), a.ldy, (int)a.M,
-                                                             (int)a.N, (int)a.K, a.status);
-    return cudaGetLastError();
+    if (a.M > BM || a.gated_codes) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
+    const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
+    return s128.cost < s256.cost ? launch_tile<128>(a, s128, sms, stream) : launch_tile<256>(a, s256, sms, stream);
 }
 
 }  // namespace dq

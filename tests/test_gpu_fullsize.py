@@ -149,13 +149,16 @@ def test_c3_gated_ffn_sampled(dq, oracle):
     assert np.linalg.norm(Yg - Yd) <= 2.5e-3 * np.linalg.norm(Yd)
 
 
-@pytest.mark.parametrize("M", [129, 256])
-def test_gemm_on_weights_that_stream_from_hbm(dq, M):
-    """Few row tiles against a matrix larger than what the GEMM keeps in flight: tile loads arrive late and out of order,
-    and every stage of the ring is waited for.  Repeated launches on fresh inputs agree with the fp64 product of the
-    exported codes; status stays clear."""
-    N, K = 34816, 5120
-    gen = torch.Generator(device=DEV).manual_seed(91 + M)
+@pytest.mark.parametrize("N,K,Ms", [
+    (34816, 5120, (129, 256)),             # few row tiles of the pair kernel: tile loads arrive late and out of order
+    (34816, 5120, (1, 77, 128)),           # one 128-row tile: one round of 256-column tiles, or two of 128
+    (10240, 5120, (77,)), (5120, 17408, (100,)), (5120, 8192, (3,)), (1040, 2176, (33, 128)), (528, 640, (1, 65)), (16, 128, (9,)),
+])
+def test_gemm_on_weights_that_stream_from_hbm(dq, N, K, Ms):
+    """Short prompts: the weights stream from HBM, every ring stage is waited for, and one to eight CTAs share a tile.  Repeated
+    launches on fresh inputs agree with the fp64 product of the exported codes; rows around the output stay as they were; the
+    same call twice gives the same bits; status stays clear."""
+    gen = torch.Generator(device=DEV).manual_seed(91 + N + Ms[0])
     w = dq.pack_weights((torch.randn(N, K, generator=gen, device=DEV) * 0.02).to(torch.bfloat16), formats=dq.FMT_NVFP4)
     e2m1 = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, -0., -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device=DEV)
 
@@ -164,14 +167,18 @@ def test_gemm_on_weights_that_stream_from_hbm(dq, M):
         return v * scales.view(torch.float8_e4m3fn).double().repeat_interleave(16, dim=1)
 
     codes, scales, s = dq.export_canonical(w, dq.FMT_NVFP4)
-    rows = torch.randperm(N, generator=gen, device=DEV)[:2048].sort().values
-    Wd = dequantise(codes[rows], scales[rows]) * s.double()
-    for _ in range(6):
-        A = torch.randn(M, K, generator=gen, device=DEV).to(torch.bfloat16)
-        sa = float(A.float().abs().max()) / 2688.0
-        Y = dq.prefill_linear(w, A, sa)
-        ref = (dequantise(*dq.quantize_activations(A, sa)) * sa) @ Wd.T
-        rel = ((Y[:, rows].double() - ref).norm() / ref.norm()).item()
-        assert rel <= 2e-3, rel
+    cols = torch.randperm(N, generator=gen, device=DEV)[:2048].sort().values
+    Wd = dequantise(codes[cols], scales[cols]) * s.double()
+    for M in Ms:
+        for _ in range(4):
+            A = torch.randn(M, K, generator=gen, device=DEV).to(torch.bfloat16)
+            sa = float(A.float().abs().max()) / 2688.0
+            out = torch.full((M + 1, N + 8), 7.0, dtype=torch.bfloat16, device=DEV)
+            Y = dq.prefill_linear(w, A, sa, out=out[:M, :N])
+            ref = (dequantise(*dq.quantize_activations(A, sa)) * sa) @ Wd.T
+            rel = ((Y[:, cols].double() - ref).norm() / ref.norm()).item()
+            assert rel <= 2e-3, (M, rel)
+            assert torch.all(out[M] == 7.0) and torch.all(out[:, N:] == 7.0)
+            assert torch.equal(dq.prefill_linear(w, A, sa), Y)
     torch.cuda.synchronize()
     assert dq.get_status() == (0, 0)
