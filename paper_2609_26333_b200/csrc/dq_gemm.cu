@@ -458,13 +458,23 @@ void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
 cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
 {
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
-    // more than one 128-row block: CTA pairs share the W tile; otherwise a lone CTA per tile
-    // (the gated epilogue exists in the pair kernel only)
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (a.M > BM || a.gated_codes) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
+    // the gated epilogue and the measurement mode exist in the pair kernel only
+    if (a.gated_codes || a.mma_only) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
     const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
+    if (a.M > BM) {
+        // CTA pairs on 256 x 256 tiles move half as many bytes per flop but have few tiles to share out: 0.36 us per k-step and round
+        // and 1 us per tile against 1.75 ns per unit of the other cost.  Measured (us, quantiser included, pair / here): 5120x17408
+        // 200 tokens 29.7 / 21.7, 300 tokens 31.3 / 26.0, 512 tokens 32.7 / 37.3; 6144x4096 256 tokens 12.6 / 11.5, 512 tokens
+        // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
+        const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
+        const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
+        const double pair_cost = (double)rounds * ((double)num_ks * 206.0 + 571.0);
+        if (pair_cost <= s128.cost && pair_cost <= s256.cost)
+            return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
+    }
     return s128.cost < s256.cost ? launch_tile<128>(a, s128, sms, stream) : launch_tile<256>(a, s256, sms, stream);
 }
 
