@@ -471,8 +471,29 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
         // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
         const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
         const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
-        const double pair_cost = (double)rounds * ((double)num_ks * 206.0 + 571.0);
-        if (pair_cost <= s128.cost && pair_cost <= s256.cost)
+        const auto pair_cost = [&](int64_t r) { return (double)r * ((double)num_ks * 206.0 + 571.0); };
+        // Where the last round would be nearly empty its columns go to the cluster kernel in a launch of their own, about 7 us of
+        // ramp before its k-steps count (5120x17408, 1000 tokens, 80 tiles on 74 pairs: 59.6 -> 50.0 us; 10240x5120,
+        // where a round is 9 us, would lose: 31.7 -> 37.3)
+        const int64_t tiles_m = (a.M + 255) / 256, head = (rounds - 1) * (sms / 2) / tiles_m;      // 256-column blocks of the full rounds
+        if (rounds > 1 && head > 0 && head * 256 < a.N) {
+            GemmArgs tail = a;
+            tail.N = a.N - head * 256;
+            tail.w_codes = a.w_codes + head * 256 * (a.K / 2);
+            tail.w_sf = a.w_sf + head * 256 * (a.K / kBlock);
+            tail.Y = reinterpret_cast<__nv_bfloat16 *>(a.Y) + head * 256;
+            const Split t128 = choose_split<128>(tail, dev, sms), t256 = choose_split<256>(tail, dev, sms);
+            const double tail_cost = (t128.cost < t256.cost ? t128.cost : t256.cost) + 4000.0;
+            const double split_cost = pair_cost(rounds - 1) + tail_cost;
+            if (split_cost < pair_cost(rounds) && split_cost < s128.cost && split_cost < s256.cost) {
+                GemmArgs front = a;
+                front.N = head * 256;
+                const cudaError_t e = launch_gemm_nvfp4_pair(front, reinterpret_cast<void *>(g_encode), stream);
+                if (e != cudaSuccess) return e;
+                return t128.cost < t256.cost ? launch_tile<128>(tail, t128, sms, stream) : launch_tile<256>(tail, t256, sms, stream);
+            }
+        }
+        if (pair_cost(rounds) <= s128.cost && pair_cost(rounds) <= s256.cost)
             return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
     }
     return s128.cost < s256.cost ? launch_tile<128>(a, s128, sms, stream) : launch_tile<256>(a, s256, sms, stream);
