@@ -379,13 +379,21 @@ static int prefill_checks(const dq_weights *w, int64_t M, float act_global_scale
     return DQ_OK;
 }
 
+// rows that pad the scale layout of a cast view to the GEMM's 256-row tiles read as zero
+static int clear_view_padding(const dq_weights *w, uint8_t *ws, const WsLayout &L, cudaStream_t s)
+{
+    if (w->N % dq::kSfRowPad == 0) return DQ_OK;
+    const size_t full = (size_t)(w->N / dq::kSfRowPad) * dq::kSfRowPad * (size_t)(w->K / dq::kBlock);
+    return cudaMemsetAsync(ws + L.w_sf + full, 0, L.w_sf_bytes - full, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+}
+
 // the part of the activation stage that does not depend on how the activations were produced: for a handle that stores
 // only LUT3, cast the weights to NVFP4 for this call (Sec. 2.3, same code map as the pack-time view); rows that pad the
 // scale layout to the GEMM tile must read as zero
 static int prefill_weight_view(const dq_weights *w, uint8_t *ws, const WsLayout &L, cudaStream_t s)
 {
     if (has_nvfp4_view(w)) return DQ_OK;
-    if (w->N % dq::kSfRowPad != 0 && cudaMemsetAsync(ws + L.w_sf, 0, L.w_sf_bytes, s) != cudaSuccess) return DQ_ERR_CUDA;
+    if (clear_view_padding(w, ws, L, s) != DQ_OK) return DQ_ERR_CUDA;
     if (dq::launch_autocast(reinterpret_cast<const dq::PackedHeader *>(w->base), w->base + w->layout.lut_off, w->N, w->K,
                             ws + L.w_codes, ws + L.w_sf, s) != cudaSuccess)
         return DQ_ERR_CUDA;
@@ -404,9 +412,12 @@ int dq_prefill_quantize(const dq_weights *w, const void *A_dev, int64_t M, int64
     uint8_t *ws = reinterpret_cast<uint8_t *>(workspace_dev);
     const WsLayout L = ws_layout(w, M);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (dq::launch_quant_act(A_dev, M, w->K, lda, act_global_scale, ws, ws + L.a_sf, 1, s) != cudaSuccess)
-        return DQ_ERR_CUDA;
-    return prefill_weight_view(w, ws, L, s);
+    if (has_nvfp4_view(w))
+        return dq::launch_quant_act(A_dev, M, w->K, lda, act_global_scale, ws, ws + L.a_sf, 1, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+    if (clear_view_padding(w, ws, L, s) != DQ_OK) return DQ_ERR_CUDA;
+    return dq::launch_quant_act_cast(A_dev, M, w->K, lda, act_global_scale, ws, ws + L.a_sf,
+                                     reinterpret_cast<const dq::PackedHeader *>(w->base), w->base + w->layout.lut_off, w->N,
+                                     ws + L.w_codes, ws + L.w_sf, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
 int dq_prefill_rmsnorm_quantize(const dq_weights *w, const void *X_dev, int64_t M, int64_t ldx, const void *gamma_dev,

@@ -190,6 +190,10 @@ cudaError_t launch_import_lut(int bits, const uint32_t *planes_in, const uint8_t
 // (swizzled != 0) or canonical [M][K/16].
 cudaError_t launch_quant_act(const void *A_bf16, int64_t M, int64_t K, int64_t lda, float act_scale, uint8_t *codes,
                              uint8_t *sf, int swizzled, cudaStream_t stream);
+// the quantiser (MMA layout) and the cast of a LUT3 matrix to NVFP4 in one launch
+cudaError_t launch_quant_act_cast(const void *A_bf16, int64_t M, int64_t K, int64_t lda, float act_scale, uint8_t *codes, uint8_t *sf,
+                                  const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N, uint8_t *w_codes, uint8_t *w_sf,
+                                  cudaStream_t stream);
 
 // fused activation processing + quantiser (dq_fused_quant.cu); outputs as launch_quant_act
 cudaError_t launch_rmsnorm_quant(const void *X_bf16, int64_t M, int64_t K, int64_t ldx, const void *gamma_bf16, float eps,

@@ -208,7 +208,7 @@ __device__ __forceinline__ uint32_t push_level(uint32_t acc, const uint32_t (&bi
 // index words and scales leave as whole 512- and 256-byte rows of the atom, E2M1 codes after a transpose inside
 // the quad as 16 bytes per lane.
 // Bound by instruction issue (the thresholds: 7 subtractions, 4 logic ops and 3 shifts per weight).  17408 x 5120 bf16 to
-// NVFP4 and LUT3: 120 us, 2.2 TB/s; a pass per format with compares and one bit placed at a time took about 250.
+// NVFP4 and LUT3: 116 us, 2.3 TB/s; a pass per format with compares and one bit placed at a time took about 250.
 template <bool FP32IN, bool NV, int BITS>
 __global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
                                                    uint8_t *__restrict__ codes, uint8_t *__restrict__ sf, uint8_t *__restrict__ lut)
@@ -235,6 +235,13 @@ __global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, i
 #pragma unroll
         for (int l = 0; l < (1 << B) - 1; ++l) T[l] = (BITS == 3) ? hdr->lut_thresholds[l] : hdr->lut2_thresholds[l & 3];
     }
+    uint4 *out_codes = nullptr;
+    uint32_t *out_sf = nullptr;
+    if (NV) {
+        out_codes = reinterpret_cast<uint4 *>(codes + r * (K / 2) + (int64_t)atom * 256 + t * 16);
+        out_sf = reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, (int64_t)atom * 32 + 4 * (t & 1), K));
+    }
+    const int64_t src = r * ldw + (int64_t)atom * 512 + t * 4;
     uint32_t words[4][B];
     uint2 my_scales = make_uint2(0u, 0u);                  // LUT scale bytes of word group t
 #pragma unroll
@@ -242,14 +249,13 @@ __global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, i
 #pragma unroll
         for (int p = 0; p < B; ++p) words[wi][p] = 0u;
         if (wi >= nwi) continue;                           // whole warps
-        const int64_t k0 = (int64_t)atom * 512 + wi * 128;
         uint4 raw[8];                                      // bf16: two words of it are used
 #pragma unroll
         for (int bb = 0; bb < 8; ++bb) {
             if (FP32IN) {
-                raw[bb] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(W) + r * ldw + k0 + bb * 16 + t * 4));
+                raw[bb] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(W) + src + wi * 128 + bb * 16));
             } else {
-                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(W) + r * ldw + k0 + bb * 16 + t * 4));
+                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(W) + src + wi * 128 + bb * 16));
                 raw[bb] = make_uint4(v.x, v.y, 0u, 0u);
             }
         }
@@ -320,8 +326,8 @@ __global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, i
             if (t == wi) my_scales = make_uint2(lut_sc[0], lut_sc[1]);
         }
         if (NV) {
-            *reinterpret_cast<uint4 *>(codes + r * (K / 2) + k0 / 2 + t * 16) = quad_transpose(nv_pieces, t);
-            if (t < 2) *reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, k0 / 16 + 4 * t, K)) = t ? nv_sc[1] : nv_sc[0];
+            out_codes[wi * 4] = quad_transpose(nv_pieces, t);
+            if (t < 2) out_sf[wi * 256] = t ? nv_sc[1] : nv_sc[0];              // two k atoms of 512 bytes per word group
         }
     }
     if (LUT) {
@@ -360,17 +366,20 @@ cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_
 // NVFP4 view of the LUT3 codes (Sec. 2.3): level -> nearest E2M1 value, element signs
 // flipped under a negative block scale, block scale |d|, same tensor scale.
 // A warp takes an atom (8 rows x 512 weights): 16-byte loads of index words, a byte permute looks up the E2M1 codes of four
-// weights (one table per sign of the block scale), and a transpose inside the quad leaves every lane 16 bytes of codes to
-// store.  5120 x 17408 (39 MB in, 50 MB out): 26 us; with two table bytes looked up in shared memory and 2-byte stores per
-// block it took 78.
-__global__ void __launch_bounds__(128) autocast_kernel(const PackedHeader *__restrict__ hdr, const uint8_t *__restrict__ lut, int64_t N,
-                                                       int64_t K, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf)
+// weights, and a transpose inside the quad leaves every lane 16 bytes of codes to store.  Signs and zero scales are masks made
+// by the permute's sign replication: under a negative scale the looked-up table is exchanged for the one with the signs of
+// non-zero codes flipped, under a zero scale the codes are cleared.
+// byte permute with the selector as it is: the intrinsic clears the top bits of its nibbles first
+__device__ __forceinline__ uint32_t prmt_raw(uint32_t a, uint32_t b, uint32_t sel)
 {
-    const uint32_t natoms = (uint32_t)((K + 511) / 512);
-    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int64_t rowgrp = task / natoms;
-    if (rowgrp >= N / 8) return;
-    const uint32_t atom = (uint32_t)(task - rowgrp * natoms);
+    uint32_t r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+__device__ __forceinline__ uint32_t prmt_sign(uint32_t a, uint32_t sel) { return prmt_raw(a, a, sel); }      // nibbles 8-11: sign of byte 0-3
+__device__ __forceinline__ void autocast_atom(const PackedHeader *hdr, const uint8_t *lut, int64_t rowgrp, uint32_t atom, int64_t K,
+                                              uint8_t *codes, uint8_t *sf)
+{
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int64_t r = rowgrp * 8 + g;
     const uint8_t *src = lut + lut_atom_offset(rowgrp * 8, atom, K, 3);
@@ -378,17 +387,18 @@ __global__ void __launch_bounds__(128) autocast_kernel(const PackedHeader *__res
 #pragma unroll
     for (int p = 0; p < 3; ++p) w[p] = __ldg(reinterpret_cast<const uint4 *>(src + p * 512 + lane * 16));
     const uint2 s8 = __ldg(reinterpret_cast<const uint2 *>(src + lut_plane_bytes(3) + lane * 8));
-    // E2M1 codes of the levels as bytes; negative block scale: sign bits of non-zero codes flipped
+    // E2M1 codes of the levels as bytes, and what a negative block scale flips: the sign bits of non-zero codes
     const uint32_t amap = hdr->autocast_map;
-    uint32_t pos[2], neg[2];
+    uint32_t pos[2], flip[2];
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
         const uint32_t m = amap >> (16 * i);
         pos[i] = (m & 0xFu) | ((m & 0xF0u) << 4) | ((m & 0xF00u) << 8) | ((m & 0xF000u) << 12);
-        const uint32_t nz = (pos[i] | (pos[i] >> 1) | (pos[i] >> 2)) & 0x01010101u;
-        neg[i] = pos[i] ^ (nz << 3);
+        flip[i] = ((pos[i] | (pos[i] >> 1) | (pos[i] >> 2)) & 0x01010101u) << 3;
     }
     const int nwi = min(4, (int)(K / 128) - 4 * (int)atom);
+    uint4 *out = reinterpret_cast<uint4 *>(codes + r * (K / 2) + (int64_t)atom * 256 + t * 16);
+    uint32_t *out_sf = reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, (int64_t)atom * 32 + 4 * (t & 1), K));
 #pragma unroll
     for (int wi = 0; wi < 4; ++wi) {
         if (wi >= nwi) break;                              // whole warps
@@ -400,22 +410,32 @@ __global__ void __launch_bounds__(128) autocast_kernel(const PackedHeader *__res
         const uint32_t sc[2] = {__shfl_sync(0xffffffffu, s8.x, (lane & ~3) | wi), __shfl_sync(0xffffffffu, s8.y, (lane & ~3) | wi)};
         uint32_t v[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            uint32_t c[2];
+        for (int i = 0; i < 2; ++i) {
+            // top bit of every byte: the block's scale byte is not zero
+            const uint32_t live = (((sc[i] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | sc[i]) & 0x80808080u;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int bb = 2 * a + h;
-                const uint32_t d8 = (sc[bb >> 2] >> (8 * (bb & 3))) & 0xFFu;
-                const bool minus = (d8 & 0x80u) != 0u;
-                const uint32_t x = __byte_perm(minus ? neg[0] : pos[0], minus ? neg[1] : pos[1], h ? sel[a] >> 16 : sel[a] & 0xFFFFu);
-                c[h] = d8 ? (x | (x >> 4)) : 0u;           // bytes 0 and 2: two codes each
+            for (int k = 0; k < 2; ++k) {                  // blocks 4 i + 2 k and the next
+                const int a = 2 * i + k;
+                const uint32_t m0 = prmt_sign(sc[i], 0x8888u + 0x1111u * (2 * k)), m1 = prmt_sign(sc[i], 0x8888u + 0x1111u * (2 * k + 1));
+                const uint32_t x0 = prmt_raw(pos[0] ^ (m0 & flip[0]), pos[1] ^ (m0 & flip[1]), sel[a]);
+                const uint32_t x1 = prmt_raw(pos[0] ^ (m1 & flip[0]), pos[1] ^ (m1 & flip[1]), sel[a] >> 16);
+                // codes 0, 2 of both blocks and codes 1, 3 of both blocks
+                const uint32_t e = __byte_perm(x0, x1, 0x6420), o = __byte_perm(x0, x1, 0x7531);
+                v[a] = (e | (o << 4)) & prmt_sign(live, k ? 0xBBAAu : 0x9988u);
             }
-            v[a] = __byte_perm(c[0], c[1], 0x6420);
         }
-        const int64_t k0 = (int64_t)atom * 512 + wi * 128;
-        *reinterpret_cast<uint4 *>(codes + r * (K / 2) + k0 / 2 + t * 16) = quad_transpose(v, t);
-        if (t < 2) *reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, k0 / 16 + 4 * t, K)) = (t ? sc[1] : sc[0]) & 0x7F7F7F7Fu;
+        out[wi * 4] = quad_transpose(v, t);
+        if (t < 2) out_sf[wi * 256] = (t ? sc[1] : sc[0]) & 0x7F7F7F7Fu;      // two k atoms of 512 bytes per word group
     }
+}
+
+__global__ void __launch_bounds__(128) autocast_kernel(const PackedHeader *__restrict__ hdr, const uint8_t *__restrict__ lut, int64_t N,
+                                                       int64_t K, uint8_t *__restrict__ codes, uint8_t *__restrict__ sf)
+{
+    const uint32_t natoms = (uint32_t)((K + 511) / 512);
+    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int64_t rowgrp = task / natoms;
+    if (rowgrp < N / 8) autocast_atom(hdr, lut, rowgrp, (uint32_t)(task - rowgrp * natoms), K, codes, sf);
 }
 
 cudaError_t launch_autocast(const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N,
@@ -711,17 +731,13 @@ cudaError_t launch_stream_read(const void *src_dev, size_t bytes, void *out_dev,
 // bf16 -> NVFP4 with a static tensor scale (App. A.3 "NVFP4").  One thread per
 // 16-block: 32 B in, 8 B of codes out; four neighbouring lanes (one 64-wide k
 // atom) merge their scale bytes into one 32-bit store of the MMA scale layout.
+// Block (bx, by): 64 blocks of one row per 64 threads, four rows; no division, 32-bit index arithmetic.
 template <bool SWIZZLED>
-__global__ void __launch_bounds__(256) quant_act_kernel(const __nv_bfloat16 *A, int M, int nb, int64_t lda,
-                                                        float s, uint8_t *codes, uint8_t *sf)
+__device__ __forceinline__ void quant_act_block(const __nv_bfloat16 *A, int M, int nb, int64_t lda, float s, uint8_t *codes, uint8_t *sf,
+                                                int bx, int by, int tx, int ty)
 {
-    // launched with programmatic stream serialization (hides the launch latency behind the previous
-    // kernel); that kernel may produce A or still read the workspace, so wait for it before anything else
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // 64 blocks of one row per 64 threads, four rows per CTA: no division, 32-bit index arithmetic
-    const int b = blockIdx.y * 64 + threadIdx.x;
-    const int r = blockIdx.x * 4 + threadIdx.y;
+    const int b = by * 64 + tx;
+    const int r = bx * 4 + ty;
     const bool live = (b < nb) && (r < M);
     const float rc6 = __frcp_rn(__fmul_rn(6.0f, s));
     uint32_t d8 = 0;
@@ -734,10 +750,10 @@ __global__ void __launch_bounds__(256) quant_act_kernel(const __nv_bfloat16 *A, 
         *reinterpret_cast<uint2 *>(codes + ((int64_t)r * nb + b) * 8) = c;
     }
     // K % 64 == 0, so lanes 4q..4q+3 always hold the four blocks of one k atom of one row
-    uint32_t w = d8 << (8 * (threadIdx.x & 3));
+    uint32_t w = d8 << (8 * (tx & 3));
     w |= __shfl_xor_sync(0xffffffffu, w, 1);
     w |= __shfl_xor_sync(0xffffffffu, w, 2);
-    if (live && (threadIdx.x & 3) == 0) {
+    if (live && (tx & 3) == 0) {
         if (SWIZZLED) {
             // atom (r / 128, b / 4) of 512 bytes; row rr of the atom at (rr % 32) * 16 + (rr / 32) * 4
             const int rr = r & 127;
@@ -749,23 +765,78 @@ __global__ void __launch_bounds__(256) quant_act_kernel(const __nv_bfloat16 *A, 
     }
 }
 
+template <bool SWIZZLED>
+__global__ void __launch_bounds__(256) quant_act_kernel(const __nv_bfloat16 *A, int M, int nb, int64_t lda,
+                                                        float s, uint8_t *codes, uint8_t *sf)
+{
+    // launched with programmatic stream serialization (hides the launch latency behind the previous
+    // kernel); that kernel may produce A or still read the workspace, so wait for it before anything else
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    quant_act_block<SWIZZLED>(A, M, nb, lda, s, codes, sf, (int)blockIdx.x, (int)blockIdx.y, (int)threadIdx.x, (int)threadIdx.y);
+}
+
+// The activation quantiser and the cast of a LUT3 matrix to NVFP4 in one launch: the first `cast_blocks` blocks take eight atoms
+// each, the others a block of the quantiser.  Both are bound by instruction issue, and nothing orders them.  5120 x 17408 and 1000
+// rows of activations: 31.6 us, one after the other 36.
+__global__ void __launch_bounds__(256) quant_act_cast_kernel(const __nv_bfloat16 *A, int M, int nb, int64_t lda, float s, uint8_t *codes,
+                                                             uint8_t *sf, const PackedHeader *hdr, const uint8_t *lut, int64_t N, int64_t K,
+                                                             uint8_t *w_codes, uint8_t *w_sf, int64_t cast_blocks, int quant_x)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if ((int64_t)blockIdx.x < cast_blocks) {
+        const uint32_t natoms = (uint32_t)((K + 511) / 512);
+        const int64_t task = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+        const int64_t rowgrp = task / natoms;
+        if (rowgrp < N / 8) autocast_atom(hdr, lut, rowgrp, (uint32_t)(task - rowgrp * natoms), K, w_codes, w_sf);
+        return;
+    }
+    const uint32_t q = (uint32_t)((int64_t)blockIdx.x - cast_blocks), by = q / (uint32_t)quant_x;
+    quant_act_block<true>(A, M, nb, lda, s, codes, sf, (int)(q - by * (uint32_t)quant_x), (int)by, (int)(threadIdx.x & 63), (int)(threadIdx.x >> 6));
+}
+
+static cudaLaunchConfig_t overlapped(cudaLaunchAttribute (&attr)[1], dim3 grid, dim3 block, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = stream;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 cudaError_t launch_quant_act(const void *A_bf16, int64_t M, int64_t K, int64_t lda, float act_scale, uint8_t *codes,
                              uint8_t *sf, int swizzled, cudaStream_t stream)
 {
     const int nb = (int)(K / 16);
     const int m = (int)M;
     const __nv_bfloat16 *A = reinterpret_cast<const __nv_bfloat16 *>(A_bf16);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((m + 3) / 4), (unsigned)((nb + 63) / 64));
-    cfg.blockDim = dim3(64, 4);
-    cfg.stream = stream;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = overlapped(attr, dim3((unsigned)((m + 3) / 4), (unsigned)((nb + 63) / 64)), dim3(64, 4), stream);
     if (swizzled) return cudaLaunchKernelEx(&cfg, quant_act_kernel<true>, A, m, nb, lda, act_scale, codes, sf);
     return cudaLaunchKernelEx(&cfg, quant_act_kernel<false>, A, m, nb, lda, act_scale, codes, sf);
+}
+
+cudaError_t launch_quant_act_cast(const void *A_bf16, int64_t M, int64_t K, int64_t lda, float act_scale, uint8_t *codes, uint8_t *sf,
+                                  const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N, uint8_t *w_codes, uint8_t *w_sf,
+                                  cudaStream_t stream)
+{
+    const int nb = (int)(K / 16), m = (int)M;
+    const int64_t cast_blocks = (N / 8 * ((K + 511) / 512) + 7) / 8;
+    const int quant_x = (m + 3) / 4;
+    const int64_t blocks = cast_blocks + (int64_t)quant_x * ((nb + 63) / 64);
+    if (blocks > 0x7FFFFFFFll) {                             // beyond one grid: one after the other
+        const cudaError_t e = launch_quant_act(A_bf16, M, K, lda, act_scale, codes, sf, 1, stream);
+        return e != cudaSuccess ? e : launch_autocast(hdr, lut_dev, N, K, w_codes, w_sf, stream);
+    }
+    cudaLaunchAttribute attr[1];
+    const cudaLaunchConfig_t cfg = overlapped(attr, dim3((unsigned)blocks), dim3(256), stream);
+    return cudaLaunchKernelEx(&cfg, quant_act_cast_kernel, reinterpret_cast<const __nv_bfloat16 *>(A_bf16), m, nb, lda, act_scale, codes,
+                              sf, hdr, lut_dev, N, K, w_codes, w_sf, cast_blocks, quant_x);
 }
 
 }  // namespace dq
