@@ -133,9 +133,23 @@ def _check(code: int, where: str):
         raise DQError(code, where)
 
 
+def _current_stream_ptr() -> int:
+    return int(torch.cuda.current_stream().cuda_stream)
+
+
+try:                                     # the same without building a Stream object: 0.2 us for 2
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream, _cuda_getDevice as _raw_device
+
+    def _current_stream_ptr() -> int:    # noqa: F811
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return _raw_stream(_raw_device())
+except ImportError:                      # a build of torch without CUDA
+    pass
+
+
 def _stream_ptr(stream=None) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return int(s.cuda_stream)
+    return _current_stream_ptr() if stream is None else int(stream.cuda_stream)
 
 
 def packed_bytes(N: int, K: int, formats: int) -> int:

@@ -1,5 +1,6 @@
 // C ABI (include/dq.h): argument checks, handle bookkeeping and kernel launches.
 // No device allocation, no synchronisation except in dq_get_status.
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -8,6 +9,34 @@
 
 namespace dq {
 __device__ StatusWord g_status_word;
+
+const DeviceInfo *device_info()
+{
+    static DeviceInfo info[kMaxDevices];
+    static std::atomic<int> known[kMaxDevices];              // 0 = not asked, 1 = being filled in, 2 = there
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    if (known[dev].load(std::memory_order_acquire) == 2) return &info[dev];
+    DeviceInfo d = {dev, DQ_OK, 0, nullptr};
+    int major = 0, minor = 0;
+    void *p = nullptr;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return nullptr;
+    if (major != 10 || minor != 0) d.arch = DQ_ERR_ARCH;
+    else if (cudaGetSymbolAddress(&p, g_status_word) != cudaSuccess) return nullptr;
+    d.status = reinterpret_cast<StatusWord *>(p);
+    int expected = 0;
+    if (known[dev].compare_exchange_strong(expected, 1, std::memory_order_acq_rel)) {
+        info[dev] = d;
+        known[dev].store(2, std::memory_order_release);
+        return &info[dev];
+    }
+    static thread_local DeviceInfo mine;                     // another thread is filling it in: the same answers
+    mine = d;
+    return &mine;
+}
 }
 
 struct dq_weights {
@@ -28,13 +57,8 @@ inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_
 
 int check_arch()
 {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return DQ_ERR_CUDA;
-    int major = 0, minor = 0;
-    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) return DQ_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev) != cudaSuccess) return DQ_ERR_CUDA;
-    if (major != 10 || minor != 0) return DQ_ERR_ARCH;
-    return DQ_OK;
+    const dq::DeviceInfo *d = dq::device_info();
+    return d ? d->arch : DQ_ERR_CUDA;
 }
 
 int check_shape(int64_t N, int64_t K, unsigned formats)
@@ -95,9 +119,8 @@ WsLayout ws_layout(const dq_weights *w, int64_t M)
 
 dq::StatusWord *status_word_ptr()
 {
-    void *p = nullptr;
-    if (cudaGetSymbolAddress(&p, dq::g_status_word) != cudaSuccess) return nullptr;
-    return reinterpret_cast<dq::StatusWord *>(p);
+    const dq::DeviceInfo *d = dq::device_info();
+    return d ? d->status : nullptr;
 }
 
 // default codebook: the paper's LUT3A16 grid (App. A.3 "LUT formats") rounded to fp16

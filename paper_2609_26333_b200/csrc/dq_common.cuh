@@ -162,6 +162,11 @@ __host__ __device__ inline size_t sf_swizzled_offset(int64_t r, int64_t b, int64
 // SM of its first CTA: SM clock cycles and nanoseconds of the global timer from the CTA's start to its end.
 struct StatusWord { int status; int detail; unsigned long long gemm_cycles; unsigned long long gemm_ns; };
 
+// What the entry points ask about the current device, looked up once per device: arch is DQ_OK on compute capability 10.0.
+// nullptr where the runtime does not answer.
+struct DeviceInfo { int device; int arch; int sms; StatusWord *status; };
+const DeviceInfo *device_info();
+
 bool handle_on_current_device(const dq_weights *w);      // defined beside the handle (dq_api.cu)
 
 // ---- launchers (each enqueues on `stream`, returns a cudaError_t) ----

@@ -765,9 +765,9 @@ cudaError_t launch_one(const CUtensorMap &tmap, TcDecodeArgs P, int force_csize,
     auto kernel = decode_tc_kernel<FMT, NC>;
     static std::atomic<bool> attr_set[kMaxDevices];
     static std::atomic<int> max_clusters[kMaxDevices][kMaxCluster + 1];          // + 1; 0 = not asked yet
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device, sms = di->sms;
     if (!attr_set[dev].load(std::memory_order_acquire)) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);

@@ -424,9 +424,9 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
 template <int BN>
 cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaError_t e = set_attributes<BN>(dev);
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    cudaError_t e = set_attributes<BN>(di->device);
     if (e != cudaSuccess) return e;
     CUtensorMap tmap_a, tmap_w;
     if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
@@ -458,9 +458,9 @@ void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
 cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
 {
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device, sms = di->sms;
     // the gated epilogue and the measurement mode exist in the pair kernel only
     if (a.gated_codes || a.mma_only) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
     const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);

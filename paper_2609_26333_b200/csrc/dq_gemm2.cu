@@ -578,8 +578,9 @@ template <class C>
 static cudaError_t launch_pair_cfg(const GemmArgs &a, EncodeTiledFn enc, cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device, sms = di->sms;
     if (!attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_pair_kernel<false, 0, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              C::SMEM_BYTES);
@@ -602,7 +603,6 @@ static cudaError_t launch_pair_cfg(const GemmArgs &a, EncodeTiledFn enc, cudaStr
     if (gated) tmap_y = tmap_a;
     else if (!make_y_tmap(enc, &tmap_y, a.Y, a.M, a.N, a.ldy)) return cudaErrorInvalidValue;
     GatedOut go = {a.gated_codes, a.gated_sf, a.gated_scale, (int)(a.N / 2)};
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int tiles = (int)(((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN));
     int pairs = sms / 2 * C::kMinCtas;
     if (tiles < pairs) pairs = tiles;

@@ -499,8 +499,9 @@ cudaError_t launch_one(const GemvArgs &a, int b0, int cols, int grid, int thread
                        cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device;
     if (!attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemv_lut_kernel<BITS, MAXT, MINB, CG, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemLimit);
@@ -834,8 +835,9 @@ cudaError_t launch_wide_one(const GemvArgs &a, int b0, int cols, int grid, int t
                             cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device;
     if (!attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemv_lut_wide_kernel<BITS, CG8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
         if (e != cudaSuccess) return e;
@@ -1017,12 +1019,9 @@ static bool wide_rows(int64_t N, int B) { return N >= 8192 || (B >= 16 && N >= 4
 //     1.7 more (17408x5120 batch 16: 26.7 / 30.2; 16384x1024: 6.5 / 10.4; 10240x5120: 25.1 / 24.9; batch 24: 38.7 / 26.1); against
 //     passes of eight, always but for short rows (2048x1024 batch 16: 6.2 / 8.6; 4096x4096: 19.8 / 13.8);
 //   above 32: always (17408x5120 batch 40: 66 / 37).
-static bool tc_is_faster(int bits, int64_t N, int64_t K, int B, int sms)
+static bool tc_is_faster(int64_t N, int64_t K, int B, int sms, const Split &narrow)
 {
-    if (B <= 8) {
-        if (N <= 1024) return B >= 5;
-        return B >= 4 && choose_split(bits, N, K, sms, B).cols < B;
-    }
+    if (B <= 8) return N <= 1024 ? B >= 5 : (B >= 4 && narrow.cols < B);
     if (B > 32) return true;
     if (!wide_rows(N, B)) return K > 1024 || B > 16;
     const int64_t per_round = 8 * (int64_t)sms;
@@ -1037,9 +1036,9 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     const int K = (int)a.K, N = (int)a.N, B = (int)a.B;
     if (a.bits != 2 && a.bits != 3) return cudaErrorInvalidValue;
     if (K > kLutMaxK) return cudaErrorInvalidValue;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int sms = di->sms;
     // The tcgen05 kernel runs only where the caller asks for it (test hook): measured, it is the slower of the two
     // (23.7 against 16.3 us on 17408x5120; its header says why).
     if (a.kernel == 2) {
@@ -1049,12 +1048,12 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     }
     if (a.kernel == 4) return a.split_exact ? launch_decode_tc(a, stream) : cudaErrorInvalidValue;
     const bool choose = a.kernel == 0 && a.force_P == 0;
-    if (choose && a.split_exact && tc_is_faster(a.bits, N, K, B, sms)) return launch_decode_tc(a, stream);
+    const int want_cols = B;                    // the split decides how many of them one pass takes
+    Split sp = choose_split(a.bits, N, K, sms, want_cols);
+    if (choose && a.split_exact && tc_is_faster(N, K, B, sms, sp)) return launch_decode_tc(a, stream);
     // Batches above 8 that stay here: one slice-by-slice pass over the weights per 32 columns instead of one pass per 8 columns,
     // where that is faster (measured: from 8192 rows on, and from 4096 rows on for 16 columns and more)
     if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, B))) return launch_wide(a, sms, stream);
-    const int want_cols = B;                    // the split decides how many of them one pass takes
-    Split sp = choose_split(a.bits, N, K, sms, want_cols);
     LutPlan L;
     if (a.force_P > 0 && a.force_G > 0) {
         if (a.force_P * a.force_G > 32 || a.force_G > kMaxGroups) return cudaErrorInvalidValue;

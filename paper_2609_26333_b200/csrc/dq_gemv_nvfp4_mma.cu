@@ -276,8 +276,9 @@ cudaError_t launch_one(const GemvNvArgs &a, int b0, int cols, int grid, int thre
                        uint32_t smem, cudaStream_t stream)
 {
     static bool attr_set[kMaxDevices] = {};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int dev = di->device;
     if (!attr_set[dev]) {
         cudaError_t e = cudaFuncSetAttribute(gemv_nvfp4_mma_kernel<MAXT, NPF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)(kCtrlBytes + kRedBytes + kMaxXBytes));
@@ -319,9 +320,9 @@ cudaError_t launch_gemv_nvfp4_mma(const GemvNvArgs &a, cudaStream_t stream)
     int cols_max = (int)(kMaxXBytes / col_stride);
     if (cols_max > 8) cols_max = 8;
     if (cols_max < 1) return cudaErrorInvalidValue;
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const int sms = di->sms;
     const int ntiles = ((N + 127) / 128) * 8;
     int grid = (ntiles + G - 1) / G;
     if (grid > sms) grid = sms;
