@@ -238,7 +238,7 @@ struct GemvArgs {
     int force_P = 0, force_G = 0, force_S = 0;
     long long wait_cycles = 0;
     int drop_first_copy = 0;                              // one warp's first copy is never requested (its wait must run out)
-    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8), 4 = dequantised through tcgen05 (any batch)
+    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8), 4 = dequantised through tcgen05 (any batch), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns)
     bool split_exact = true;                              // codebook levels are multiples of 2^-15 (launch_decode_tc)
 };
 cudaError_t launch_gemv_lut(const GemvArgs &args, cudaStream_t stream);     // picks one of the two kernels below

@@ -906,6 +906,317 @@ cudaError_t launch_wide(const GemvArgs &a, int sms, cudaStream_t stream)
     return cudaSuccess;
 }
 
+// ---------------------------------------------------------------------------------------------------------------
+// Five to eight columns: tiles of 16 rows (the two row halves of the device layout side by side), so that the 16 rows of the
+// mma's A operand are 16 rows of one block and its 8 columns the batch: one mma and four FFMA per 16 x 16 weights where the
+// 8-row tiles above take two and eight.  Activations of the whole row stay in shared memory as there, in the wide kernel's layout;
+// a ring stage is a tile's 512 weights (two atoms), a warp takes halves w, w + P, .. of the slices.  Bound by instruction
+// issue like the kernel above.  Measured (us, 8-row tiles / these): 6144x4096 batch 8 12.5 / 11.5, 34816x5120 39.8 / 34.1,
+// 28672x8192 batch 5 55.1 / 49.2; 17408x5120 batch 4 17.9 / 19.1.
+template <int BITS>
+__global__ void __launch_bounds__(512, 1)
+gemv_lut_rows16_kernel(const uint8_t *__restrict__ lut, const PackedHeader *__restrict__ hdr,
+                       const __nv_bfloat16 *__restrict__ X, int64_t ldx, int b0, int cols,
+                       __nv_bfloat16 *__restrict__ Y, int64_t ldy, int N, int K, LutPlan L, StatusWord *status)
+{
+    constexpr uint32_t kAtom = (uint32_t)lut_atom_bytes(BITS);
+    constexpr uint32_t kChunk = 2u * kAtom;                 // one ring stage: 16 rows x 512 weights
+    constexpr uint32_t kPlanes = (uint32_t)lut_plane_bytes(BITS);
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t win0 = (uint32_t)__cvta_generic_to_shared(smem_raw);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_raw);
+    int *sync_words = reinterpret_cast<int *>(smem_raw + 64);                           // [G][kSlots] x (generation, count)
+    float *xmax_s = reinterpret_cast<float *>(smem_raw + 640);                          // per-warp maxima
+    float *red = reinterpret_cast<float *>(smem_raw + L.red_off);
+
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    const int P = L.P, G = L.G, S = L.S;
+    const int grp = warp / P;
+    const int w = warp - grp * P;
+    const int g = lane >> 2, t = lane & 3;
+    const int nslices = (int)lut_slices(K);
+    const int kpad = nslices * kLutSlice;
+    const int nunits = (K + kLutAtomK - 1) / kLutAtomK;
+
+    const uint32_t ring0 = win0 + L.ring_off + (uint32_t)warp * (uint32_t)S * kChunk;
+    const uint32_t bars0 = win0 + L.bar_off + (uint32_t)warp * (uint32_t)S * 8u;
+    const uint32_t ring_end = ring0 + (uint32_t)S * kChunk;
+    if (lane == 0) {
+        for (int i = 0; i < S; ++i) tc::mbar_init(bars0 + 8u * i, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    if (threadIdx.x < kMaxGroups * kSlots * 2) sync_words[threadIdx.x] = 0;
+    if (threadIdx.x == 0) *abort_flag = 0;
+    __syncwarp();
+
+    const int ns = (w < nunits) ? (nunits - w + P - 1) / P : 0;          // units of every tile this warp takes
+    const int ntiles = N / 16;
+    const int stride = gridDim.x * G;
+    const int first = blockIdx.x * G + grp;
+    // producer state, as in the kernel above; the two atoms of a unit (row halves) lie 2 atoms apart
+    int pu = w, ptile = (ns > 0) ? first : ntiles;
+    uint32_t pdst = ring0, pbar = bars0;
+    auto issue_next = [&]() {
+        const uint32_t doit = (lane == 0 && ptile < ntiles) ? 1u : 0u;
+        const uint8_t *src = lut + ((size_t)ptile * nslices * 4u + (size_t)(pu >> 1) * 4u + (size_t)(pu & 1)) * kAtom;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %0, 0;\n\t"
+            "@p fence.proxy.async.shared::cta;\n\t"
+            "@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], %2;\n\t"
+            "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%3], [%4], %5, [%1];\n\t"
+            "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%6], [%7], %5, [%1];\n\t}"
+            ::"r"(doit), "r"(pbar), "r"(kChunk), "r"(pdst), "l"(src), "r"(kAtom), "r"(pdst + kAtom), "l"(src + 2u * kAtom) : "memory");
+        pu += P;
+        if (pu >= nunits) { pu = w; ptile += stride; }
+        pdst += kChunk;
+        pbar += 8u;
+        if (pdst == ring_end) { pdst = ring0; pbar = bars0; }
+    };
+    // The weights are constant data: start streaming before waiting for the kernel ahead of this one.
+    for (int i = 0; i < S && ptile < ntiles; ++i) issue_next();
+    const uint4 cbv = *reinterpret_cast<const uint4 *>(BITS == 3 ? hdr->lut_prmt : hdr->lut2_prmt);
+    const Codebook cb = {cbv.x, cbv.y, cbv.z, cbv.w};
+    const float s_w = hdr->s;
+
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    // ---- activations: raw bf16 parked in shared memory, largest magnitude on the way, then power-of-two scale -> fp16 in place
+    uint8_t *xh = smem_raw + L.x_off;
+    auto x_at = [&](int c, int i) {                              // eight weights 8 i .. 8 i + 7 of column c; the other quarter 16 bytes on
+        return xh + (size_t)c * L.col_stride + (size_t)(i >> 7) * 2048u + x16_offset(((uint32_t)i >> 1) & 63u, ((uint32_t)i & 1u) * 2u);
+    };
+    float m = 0.0f;
+    for (int c = 0; c < cols; ++c) {
+        const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)(b0 + c) * ldx);
+        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);                 // the padding of a short last slice reads as zero
+            if (i < K / 8) v = __ldg(xp + i);
+            const uint32_t a0 = v.x & 0x7FFF7FFFu, a1 = v.y & 0x7FFF7FFFu, a2 = v.z & 0x7FFF7FFFu, a3 = v.w & 0x7FFF7FFFu;
+            const uint32_t hi = max(max(a0 >> 16, a1 >> 16), max(a2 >> 16, a3 >> 16));
+            const uint32_t lo = max(max(a0 & 0xFFFFu, a1 & 0xFFFFu), max(a2 & 0xFFFFu, a3 & 0xFFFFu));
+            m = fmaxf(m, __uint_as_float(max(hi, lo) << 16));
+            uint8_t *dst = x_at(c, i);
+            *reinterpret_cast<uint2 *>(dst) = make_uint2(v.x, v.y);
+            *reinterpret_cast<uint2 *>(dst + 16) = make_uint2(v.z, v.w);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) xmax_s[warp] = m;
+    __syncthreads();
+    m = (lane < nwarps) ? xmax_s[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int ex = (int)((__float_as_uint(m) >> 23) & 0xFFu) - 127;           // floor(log2(max)); -127 for zero / subnormal
+    ex = max(-100, min(100, ex));
+    const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
+    const float out_scale = s_w * __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
+    for (int c = 0; c < cols; ++c) {
+        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {        // every thread converts what it parked itself
+            uint8_t *px = x_at(c, i);
+            const uint2 va = *reinterpret_cast<const uint2 *>(px), vb = *reinterpret_cast<const uint2 *>(px + 16);
+            const uint32_t ww[4] = {va.x, va.y, vb.x, vb.y};
+            uint32_t r[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z) {
+                const __half2 h = __floats2half2_rn(__uint_as_float(ww[z] << 16) * xscale,
+                                                    __uint_as_float(ww[z] & 0xFFFF0000u) * xscale);
+                r[z] = *reinterpret_cast<const uint32_t *>(&h);
+            }
+            *reinterpret_cast<uint2 *>(px) = make_uint2(r[0], r[1]);
+            *reinterpret_cast<uint2 *>(px + 16) = make_uint2(r[2], r[3]);
+        }
+    }
+    __syncthreads();
+    // B operand of this lane: column g (column 0 where the pass has fewer), weights 4t .. 4t+3 of a pair of blocks per 16-byte load
+    const uint32_t xlane = win0 + L.x_off + (uint32_t)(g < cols ? g : 0) * L.col_stride + (uint32_t)t * 16u;
+    const uint32_t lane_plane = (uint32_t)lane * 16u;
+    const uint32_t sbuf = win0 + L.sbuf_off + (uint32_t)warp * (2u * kScaleBufBytes);
+    const uint32_t srow = sbuf + (uint32_t)g * 144u;
+    const uint32_t swr = sbuf + (uint32_t)(lane >> 2) * 144u + (uint32_t)(lane & 3) * 32u;
+    const uint32_t sync0 = win0 + 64u + (uint32_t)grp * kSlots * 8u;
+
+    uint32_t cbase = ring0, cbar = bars0, phase = 0;
+    int tile = first;
+    for (int it = 0; tile < ntiles; ++it, tile += stride) {
+        float acc[1][4] = {{0.0f, 0.0f, 0.0f, 0.0f}};
+        for (int i = 0, u = w; i < ns; ++i, u += P) {
+            if (!__any_sync(0xffffffffu, tc::mbar_try(cbar, phase))) {
+                const long long t0 = clock64();
+                bool got = false;
+                while (true) {
+                    __nanosleep(32);
+                    got = __any_sync(0xffffffffu, tc::mbar_try(cbar, phase));
+                    if (got) break;
+                    if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > L.wait_cycles)) break;
+                }
+                if (!got) { *abort_flag = 1; goto give_up; }
+            }
+            uint4 pw0[BITS], pw1[BITS];
+            pw0[0] = lds_v4_at<0>(cbase + lane_plane);
+            pw0[1] = lds_v4_at<512>(cbase + lane_plane);
+            if (BITS == 3) pw0[BITS - 1] = lds_v4_at<1024>(cbase + lane_plane);
+            pw1[0] = lds_v4_at<(int)kAtom>(cbase + lane_plane);
+            pw1[1] = lds_v4_at<(int)kAtom + 512>(cbase + lane_plane);
+            if (BITS == 3) pw1[BITS - 1] = lds_v4_at<(int)kAtom + 1024>(cbase + lane_plane);
+            const uint2 sa = lds_v2_at<(int)kPlanes>(cbase + (uint32_t)lane * 8u);
+            const uint2 sb = lds_v2_at<(int)(kAtom + kPlanes)>(cbase + (uint32_t)lane * 8u);
+            __syncwarp();                                          // the stage is in registers, the scale buffers are free
+            issue_next();
+            sts_v4f(swr, e4m3x4_to_f32(sa.x));
+            sts_v4f(swr + 16u, e4m3x4_to_f32(sa.y));
+            sts_v4f(swr + kScaleBufBytes, e4m3x4_to_f32(sb.x));
+            sts_v4f(swr + kScaleBufBytes + 16u, e4m3x4_to_f32(sb.y));
+            __syncwarp();
+            atom_dot16<BITS, 1>(pw0, pw1, xlane + (uint32_t)u * 1024u, 0u, srow, srow + kScaleBufBytes, cb, acc);
+            cbase += kChunk;
+            cbar += 8u;
+            if (cbase == ring_end) { cbase = ring0; cbar = bars0; phase ^= 1u; }
+        }
+        if (P == 1) {
+            // lane (g, t): rows g and g + 8, columns 2t and 2t + 1
+            const int row = tile * 16 + g, col = 2 * t;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (col + (j & 1) < cols) Y[(int64_t)(b0 + col + (j & 1)) * ldy + row + 8 * (j >> 1)] = __float2bfloat16_rn(acc[0][j] * out_scale);
+            continue;
+        }
+        // ---- cross-warp sum: last-arriving warp of the group adds the P partial tiles in order and stores
+        const int slot = it & (kSlots - 1);
+        const uint32_t gen_addr = sync0 + (uint32_t)slot * 8u;
+        int *cnt = sync_words + (grp * kSlots + slot) * 2 + 1;
+        {
+            uint32_t good = 1;
+            if (lane == 0) {
+                const uint32_t want = (uint32_t)(it / kSlots);
+                long long t0 = 0;
+                uint32_t spins = 0;
+                while (lds_u32_volatile(gen_addr) != want) {
+                    if ((++spins & 255u) == 0u) {
+                        if (t0 == 0) t0 = clock64();
+                        if (*abort_flag || clock64() - t0 > L.wait_cycles) { *abort_flag = 1; good = 0; break; }
+                    }
+                }
+            }
+            if (__shfl_sync(0xffffffffu, good, 0) == 0) goto give_up;
+        }
+        float *rbuf = red + (size_t)((grp * kSlots + slot) * P) * 128;              // [warp][row 16][column 8]
+        *reinterpret_cast<float2 *>(rbuf + w * 128 + g * 8 + 2 * t) = make_float2(acc[0][0], acc[0][1]);
+        *reinterpret_cast<float2 *>(rbuf + w * 128 + (g + 8) * 8 + 2 * t) = make_float2(acc[0][2], acc[0][3]);
+        __syncwarp();
+        int prev = 0;
+        if (lane == 0) { fence_cta(); prev = atomicAdd(cnt, 1); }
+        prev = __shfl_sync(0xffffffffu, prev, 0);
+        if (prev == P - 1) {
+            fence_cta();
+            const int row = lane & 15;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int col = (lane >> 4) + 2 * j;
+                float tot = 0.0f;
+                for (int ww = 0; ww < P; ++ww) tot += *reinterpret_cast<const volatile float *>(rbuf + ww * 128 + row * 8 + col);
+                if (col < cols) Y[(int64_t)(b0 + col) * ldy + tile * 16 + row] = __float2bfloat16_rn(tot * out_scale);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                *cnt = 0;
+                fence_cta();
+                asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(gen_addr), "r"((uint32_t)(it / kSlots + 1)) : "memory");
+            }
+        }
+    }
+give_up:
+    if (*abort_flag) {
+        for (int i = 0; i < 200; ++i) __nanosleep(1000);
+        if (lane == 0) {
+            atomicExch(&status->status, (int)DQ_ERR_TIMEOUT);
+            atomicExch(&status->detail, 0x3C000 | (int)blockIdx.x);
+        }
+    }
+}
+
+constexpr int kRows16Warps = 16;
+
+// shared memory of P x G warps, rings two stages deep, `cols` activation columns
+uint32_t plan_rows16(int bits, int K, int P, int G, int cols, LutPlan &L)
+{
+    const uint32_t nwarps = (uint32_t)(P * G);
+    L.P = P; L.G = G; L.S = 2;
+    L.bar_off = 1024;
+    L.red_off = 2048;
+    L.sbuf_off = (L.red_off + (P > 1 ? nwarps * kSlots * 512u : 0u) + 127u) & ~127u;
+    L.ring_off = L.sbuf_off + nwarps * 2u * kScaleBufBytes;
+    L.x_off = (L.ring_off + nwarps * 2u * 2u * (uint32_t)lut_atom_bytes(bits) + 127u) & ~127u;
+    L.col_stride = (uint32_t)lut_slices(K) * kLutSlice * 2u + 64u;     // 64 mod 128: the 16-byte loads of two columns hit different banks
+    return L.x_off + (uint32_t)cols * L.col_stride;
+}
+
+// Split of a launch: P warps share a 16-row tile, G tiles at a time per CTA, one CTA per SM; the cost model of choose_split in units of
+// 512 weights.  0 where fewer than eight warps fit beside the activations.
+int choose_rows16(int bits, int64_t N, int64_t K, int sms, int cols, LutPlan &best)
+{
+    const int nunits = (int)((K + kLutAtomK - 1) / kLutAtomK);
+    const int64_t ntiles = N / 16;
+    double best_cost = 1e300;
+    int grid_best = 0;
+    for (int p = 1; p <= nunits && p <= kRows16Warps; ++p) {
+        for (int gg = 1; gg * p <= kRows16Warps; ++gg) {
+            LutPlan L = {};
+            if (plan_rows16(bits, (int)K, p, gg, cols, L) > kSmemLimit) break;
+            if (gg * p < 8 && (gg + 1) * p <= kRows16Warps) continue;
+            const int64_t need = (ntiles + gg - 1) / gg;
+            const int64_t grid = need < sms ? need : sms;
+            const int64_t rounds = (ntiles + grid * gg - 1) / (grid * gg);
+            const double warps = (double)(gg * p);
+            const double cost = (double)(gg * rounds) * ((double)((nunits + p - 1) / p) + 0.5) * p * (warps < 12.0 ? 12.0 / warps : 1.0);
+            if (cost < best_cost) { best_cost = cost; best = L; grid_best = (int)grid; }
+        }
+    }
+    return grid_best;
+}
+
+template <int BITS>
+cudaError_t launch_rows16_bits(const GemvArgs &a, const LutPlan &L, int grid, cudaStream_t stream)
+{
+    static bool attr_set[kMaxDevices] = {};
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    if (!attr_set[di->device]) {
+        cudaError_t e = cudaFuncSetAttribute(gemv_lut_rows16_kernel<BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(gemv_lut_rows16_kernel<BITS>, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        attr_set[di->device] = true;
+    }
+    const uint32_t smem = L.x_off + (uint32_t)a.B * L.col_stride;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)(L.P * L.G * 32));
+    cfg.dynamicSmemBytes = smem < 114u * 1024u ? 114u * 1024u : smem;       // one CTA per SM
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, gemv_lut_rows16_kernel<BITS>, a.lut, a.hdr, reinterpret_cast<const __nv_bfloat16 *>(a.X), (int64_t)a.ldx, 0,
+                              (int)a.B, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.N, (int)a.K, L, a.status);
+}
+
+// B <= 8 columns in one pass; cudaErrorInvalidValue where the row is too long for it
+cudaError_t launch_rows16(const GemvArgs &a, int sms, cudaStream_t stream)
+{
+    LutPlan L = {};
+    const int grid = a.B <= 8 ? choose_rows16(a.bits, a.N, a.K, sms, (int)a.B, L) : 0;
+    if (grid == 0) return cudaErrorInvalidValue;
+    L.wait_cycles = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitBudgetCycles;
+    return a.bits == 3 ? launch_rows16_bits<3>(a, L, grid, stream) : launch_rows16_bits<2>(a, L, grid, stream);
+}
+
 }  // namespace
 
 // column groups (of four batch columns, one mma each) the kernel is instantiated for
@@ -1047,10 +1358,17 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
         return launch_gemv_lut_tc(a, wgs, stream);
     }
     if (a.kernel == 4) return a.split_exact ? launch_decode_tc(a, stream) : cudaErrorInvalidValue;
+    if (a.kernel == 5) return launch_rows16(a, sms, stream);
     const bool choose = a.kernel == 0 && a.force_P == 0;
     const int want_cols = B;                    // the split decides how many of them one pass takes
     Split sp = choose_split(a.bits, N, K, sms, want_cols);
     if (choose && a.split_exact && tc_is_faster(N, K, B, sms, sp)) return launch_decode_tc(a, stream);
+    // five to eight columns on rows whose activations leave room for the warps (above 8192 weights they do not: 4096x11008 batch 5
+    // 17.3 / 18.3 us)
+    if (choose && B > 4 && B <= 8 && K <= 8192) {
+        const cudaError_t e = launch_rows16(a, sms, stream);
+        if (e != cudaErrorInvalidValue) return e;
+    }
     // Batches above 8 that stay here: one slice-by-slice pass over the weights per 32 columns instead of one pass per 8 columns,
     // where that is faster (measured: from 8192 rows on, and from 4096 rows on for 16 columns and more)
     if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, B))) return launch_wide(a, sms, stream);

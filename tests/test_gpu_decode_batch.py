@@ -159,3 +159,25 @@ def test_decode_batch_wait_runs_out(dq):
     assert dq.status_string(st) == "device-side wait ran out"
     assert torch.equal(dq.decode_linear(w, X), good)
     _status_ok(dq)
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2"])
+@pytest.mark.parametrize("N,K", SHAPES + [(4112, 1536)])
+@pytest.mark.parametrize("B", [1, 5, 8])
+def test_decode_rows16_parity(dq, oracle, fmt, N, K, B):
+    """The kernel with 16-row tiles (what batches of five to eight take): ragged slices, one and several warps per tile, more tiles
+    than one round takes."""
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 300 + B)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    out = torch.full((B + 1, N + 8), 7.0, dtype=torch.bfloat16, device=DEV)
+    dq.test_decode_linear(w, code, X.to(DEV), out=out[:B, :N], variant=6)
+    _status_ok(dq)
+    check_outputs(_f64(out[:B, :N]), Yr, S, f"{fmt} {B}x{N}x{K}")
+    assert torch.all(out[B] == 7.0) and torch.all(out[:, N:] == 7.0)
+    if B > 4:
+        y = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2}[fmt](w, X.to(DEV))
+        _status_ok(dq)
+        check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K} public")
