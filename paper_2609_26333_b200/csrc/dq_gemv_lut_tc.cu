@@ -33,14 +33,13 @@
 // buffers and two accumulators per warpgroup (160 of the 512 tensor-memory columns).  Every wait is bounded.
 //
 // Status: exact (outputs equal the mma.sync kernel's up to the order of the fp32 sums) but slower, and therefore only
-// reachable through the test hook.  Measured on 17408 x 5120 (LUT3, launches back to back): 23.7 us against 16.3 us.
-// One MMA of 128 x 16 x 16 from tensor memory takes 45 cycles whatever N is (the A operand is what it reads), so the
-// 24 MMAs of a round of three warpgroups keep the tensor pipe busy for 1080 cycles, as long as the three dequantising
-// warps of a scheduler need to issue their permutes; with two buffers per warpgroup a step cannot start before the
-// MMAs two steps back have finished, the two costs add up instead of overlapping (1850 cycles per step measured, 840
-// with the dequantisation left out), more buffers do not fit tensor memory beside three warpgroups, and set-up
+// reachable through the test hook.  Measured on 17408 x 5120 (LUT3, launches back to back): 20.9 us against 15.3 us.
+// The MMAs are not what costs (issued under elect.sync one of 128 x 16 x 16 from tensor memory takes 9 cycles; under `lane == 0` it
+// took 45 and the launch 23.7 us): with two buffers per warpgroup a step cannot start before the
+// MMAs two steps back have finished, more buffers do not fit tensor memory beside three warpgroups, and set-up
 // (tensor-memory allocation, 8 bytes of shared memory per activation to fill) costs about 3 us more than the
-// mma.sync kernel's.  Kept as the measured answer to whether tcgen05 helps this contraction on this GPU.
+// mma.sync kernel's.  Kept as the measured answer to whether tcgen05 helps this contraction at one column; for batches it does
+// (dq_decode_tc.cu).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -425,7 +424,7 @@ gemv_lut_tc_kernel(const uint8_t *__restrict__ lut, const PackedHeader *__restri
                 if (ok && !*abort_flag && row < N) Y[row] = __float2bfloat16_rn(tot * out_scale);
             }
         }
-    } else if (lane == 0) {
+    } else if (tc::elect_one()) {
         // ================= MMA issue: one warp per warpgroup =================
         const int g_ = warp - ndq;
         const uint32_t xaddr = win0 + L.x_off + kZeroPad, zlo = win0 + L.x_off, zhi = xaddr + L.x_bytes;
