@@ -10,7 +10,7 @@
 //   warp 0      : TMA producer (packed FP4 tiles, 128B swizzle) + bulk copies of the scale atoms; weights that are part of the
 //                 handle are requested before the kernel ahead (the activation quantiser) has finished
 //   warp 1      : tcgen05.cp of the scales into TMEM and tcgen05.mma (kind::mxf4nvf4, block 16)
-//   warps 2..5  : epilogue, TMEM -> registers -> bf16 -> global
+//   warps 2..   : epilogue, TMEM -> registers -> bf16 -> global; four warps, or eight beside an exchange (launch_tile)
 // The fp32 accumulator lives in TMEM (two of 128 columns or one of 256) beside the scale factors of every stage.  Producer and MMA
 // roles are one elected thread each, waits included: see elect_one.  Every mbarrier wait is bounded: when it runs
 // out the CTA records DQ_ERR_TIMEOUT in the status word and leaves normally.
@@ -31,7 +31,7 @@ using namespace tc;
 
 constexpr int BM = 128;
 constexpr int kKbPerStage = 4;                // 64-element MMA k-steps per 256-element stage (128 bytes of FP4: one swizzle row)
-constexpr int kThreads = 192;
+constexpr int threads_of(int halves) { return 64 + 128 * halves; }     // `halves` epilogue warps per TMEM lane quarter
 constexpr uint32_t kTmemCols = 512;
 
 template <int BN>
@@ -89,8 +89,8 @@ __device__ __forceinline__ float4 lds_v4f(uint32_t addr)
     return v;
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int BN, int HALVES>
+__global__ void __launch_bounds__(threads_of(HALVES), 1)
 gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const uint8_t *__restrict__ a_sf, const uint8_t *__restrict__ w_sf,
                   const PackedHeader *__restrict__ hdr, float act_scale, __nv_bfloat16 *__restrict__ Y, int64_t ldy,
@@ -237,7 +237,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const uint32_t lanes = (uint32_t)(wq * 32) << 16;
         const float alpha = __fmul_rn(act_scale, hdr->s);
         bool ok = true;
-        if (csize == 1) {
+        if (HALVES == 1 && csize == 1) {
             uint32_t it = 0;
             for (int t = first_tile; t < num_tiles && ok; t += tile_stride, ++it) {
                 const uint32_t acc = it % kAccs;
@@ -281,12 +281,13 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             ok = mbar_wait_warp(tmem_full_bar(0), 0u, abort_flag);
             tc_fence_after();
             cluster_sync();
+            const int half = HALVES > 1 ? (warp - 2) >> 2 : 0;                        // each takes its part of the columns
             const int per = (BN / 8 + csize - 1) / csize;
             const int row = mb * BM + wq * 32 + lane;
             const uint32_t mine = smem_base + (uint32_t)(wq * 32 + lane) * 16u;       // + 2048 for the second half of a group
             if (ok && mb * BM + wq * 32 < M) {
 #pragma unroll 1
-                for (int c = 0; c < BN / 32; ++c) {
+                for (int c = half * (BN / 32 / HALVES); c < (half + 1) * (BN / 32 / HALVES); ++c) {
                     uint32_t v[32];
                     tmem_ld32(tmem_base + lanes + (uint32_t)(c * 32), v);
                     tmem_ld_wait();
@@ -303,7 +304,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             }
             cluster_sync();
             if (ok && row < M) {
-                for (int i = (int)rank, l = 0; i < BN / 8 && nb * BN + 8 * i < N; i += csize, ++l) {
+                for (int l = half, i = (int)rank + half * csize; i < BN / 8 && nb * BN + 8 * i < N; i += HALVES * csize, l += HALVES) {
                     float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
                     for (int src = 0; src < csize; ++src) {
                         const uint32_t at = mine + (uint32_t)(src * per + l) * 4096u;
@@ -362,12 +363,12 @@ bool make_codes_tmap(CUtensorMap *tm, const void *ptr, int64_t rows, int64_t K, 
 constexpr int kMaxCluster = 8;
 struct Split { int csize; double cost; };
 
-template <int BN>
+template <int BN, int HALVES>
 cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int csize, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3((unsigned)threads_of(HALVES));
     cfg.dynamicSmemBytes = Cfg<BN>::SMEM_BYTES;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -380,12 +381,12 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int c
     return cfg;
 }
 
-template <int BN>
+template <int BN, int HALVES>
 cudaError_t set_attributes(int dev)
 {
     static std::atomic<bool> done[kMaxDevices];
     if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN, HALVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
     return e;
 }
@@ -405,9 +406,9 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
         int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
         if (fit == 0) {
             cudaLaunchAttribute attr[2];
-            const cudaLaunchConfig_t cfg = launch_config<BN>(attr, c * (sms / c), c, nullptr);
+            const cudaLaunchConfig_t cfg = launch_config<BN, 1>(attr, c * (sms / c), c, nullptr);
             int n = 0;
-            if (set_attributes<BN>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN>, &cfg) != cudaSuccess) {
+            if (set_attributes<BN, 1>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1>, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
             }
@@ -421,12 +422,12 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
     return best;
 }
 
-template <int BN>
-cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
+template <int BN, int HALVES>
+cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
-    cudaError_t e = set_attributes<BN>(di->device);
+    cudaError_t e = set_attributes<BN, HALVES>(di->device);
     if (e != cudaSuccess) return e;
     CUtensorMap tmap_a, tmap_w;
     if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
@@ -434,10 +435,20 @@ cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_
     const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
     const int grid = (int)(sp.csize > 1 ? tiles * sp.csize : (tiles < sms ? tiles : sms));
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = launch_config<BN>(attr, grid, sp.csize, stream);
-    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
+    const cudaLaunchConfig_t cfg = launch_config<BN, HALVES>(attr, grid, sp.csize, stream);
+    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN, HALVES>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
                               reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M, (int)a.N, (int)a.K, sp.csize,
                               a.w_const ? 1 : 0, a.status);
+}
+
+// An exchange whose row tile leaves a lane quarter empty hangs on the one to three warps that have rows: two warps a quarter then save
+// 0.2 to 1 us (5120x17408, 1 row: 16.7 -> 15.9; 10240x5120, 1 / 16 / 77 / 96 rows: 13.7 / 14.0 / 14.2 / 14.5 -> 12.7 / 13.1 / 13.7 /
+// 14.2).  With all four quarters busy, or no exchange, the extra warps gain 0.2 us at best and cost up to 0.5 (2048x1024, 128 rows:
+// 6.5 -> 7.0; 34816x5120, 128 rows: 26.3 -> 26.9).  The count is a template parameter: as a variable it cost the four-warp form 1 %.
+template <int BN>
+cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
+{
+    return sp.csize > 1 && a.M <= 3 * 32 ? launch_with<BN, 2>(a, sp, sms, stream) : launch_with<BN, 1>(a, sp, sms, stream);
 }
 
 }  // namespace

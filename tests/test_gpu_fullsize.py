@@ -152,11 +152,13 @@ def test_c3_gated_ffn_sampled(dq, oracle):
 @pytest.mark.parametrize("N,K,Ms", [
     (34816, 5120, (129, 256)),             # few row tiles of the pair kernel: tile loads arrive late and out of order
     (34816, 5120, (1, 77, 128)),           # one 128-row tile: one round of 256-column tiles, or two of 128
-    (10240, 5120, (77,)), (5120, 17408, (100,)), (5120, 8192, (3,)), (1040, 2176, (33, 128)), (528, 640, (1, 65)), (16, 128, (9,)),
+    (10240, 5120, (77, 300)), (5136, 17408, (100, 300, 1000)), (5120, 8192, (3, 97)),
+    (2048, 1024, (96, 129, 700)), (1040, 2176, (33, 128)), (528, 640, (1, 65)), (16, 128, (9,)),
 ])
 def test_gemm_on_weights_that_stream_from_hbm(dq, N, K, Ms):
-    """Short prompts: the weights stream from HBM, every ring stage is waited for, and one to eight CTAs share a tile.  Repeated
-    launches on fresh inputs agree with the fp64 product of the exported codes; rows around the output stay as they were; the
+    """Short prompts: the weights stream from HBM, every ring stage is waited for, and one to eight CTAs share a tile (with
+    eight epilogue warps up to 96 rows, four above); longer ones that take the same kernel, or hand it the columns of a nearly empty
+    last round.  Repeated launches on fresh inputs agree with the fp64 product of the exported codes; rows around the output stay as they were; the
     same call twice gives the same bits; status stays clear."""
     gen = torch.Generator(device=DEV).manual_seed(91 + N + Ms[0])
     w = dq.pack_weights((torch.randn(N, K, generator=gen, device=DEV) * 0.02).to(torch.bfloat16), formats=dq.FMT_NVFP4)
