@@ -378,14 +378,14 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           levels stored to tensor memory, one tcgen05.mma per 16-weight block, the same exact
  *           arithmetic; measured slower than the default kernel, it is kept for comparison and is
  *           not what dq_decode_linear launches.  The three split arguments do not apply to it.
- *           variant 4 runs the kernel that dq_decode_linear takes for batches above 8 on matrices
- *           of 8192 rows and more (up to 32 columns in one pass over the weights, 16-row
+ *           variant 4 runs the kernel that dq_decode_linear takes for batches above 8 where the
+ *           batch kernel of variant 5 is not the faster one (up to 32 columns in one pass over the weights, 16-row
  *           tiles, K walked in slices of 1024 with a power-of-two activation scale per slice) on
  *           any shape and batch; groups_per_cta (1..9) then sets its warps per CTA.  variant 5 runs the
  *           batch kernel that dequantises every weight once into tensor memory (all columns in one pass,
  *           256-row tiles; DQ_ERR_INVALID_ARG for a codebook with levels that are not multiples of
  *           2^-15); warps_per_group (1..8) then sets the CTAs that share a tile.  variant 6 runs the kernel
- *           with 16-row tiles that dq_decode_linear takes for batches of 5 to 8 (DQ_ERR_INVALID_ARG where
+ *           with 16-row tiles that dq_decode_linear takes for most batches of 5 to 8 (DQ_ERR_INVALID_ARG where
  *           the row is too long for it).
  *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what
  *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 5 = the batch

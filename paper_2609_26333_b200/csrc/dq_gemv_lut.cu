@@ -32,6 +32,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <cmath>
+
 #include "dq_common.cuh"
 #include "dq_tcgen05.cuh"
 
@@ -1157,11 +1159,11 @@ uint32_t plan_rows16(int bits, int K, int P, int G, int cols, LutPlan &L)
 
 // Split of a launch: P warps share a 16-row tile, G tiles at a time per CTA, one CTA per SM; the cost model of choose_split in units of
 // 512 weights.  0 where fewer than eight warps fit beside the activations.
-int choose_rows16(int bits, int64_t N, int64_t K, int sms, int cols, LutPlan &best)
+int choose_rows16(int bits, int64_t N, int64_t K, int sms, int cols, LutPlan &best, double &best_cost)
 {
     const int nunits = (int)((K + kLutAtomK - 1) / kLutAtomK);
     const int64_t ntiles = N / 16;
-    double best_cost = 1e300;
+    best_cost = 1e300;
     int grid_best = 0;
     for (int p = 1; p <= nunits && p <= kRows16Warps; ++p) {
         for (int gg = 1; gg * p <= kRows16Warps; ++gg) {
@@ -1211,7 +1213,8 @@ cudaError_t launch_rows16_bits(const GemvArgs &a, const LutPlan &L, int grid, cu
 cudaError_t launch_rows16(const GemvArgs &a, int sms, cudaStream_t stream)
 {
     LutPlan L = {};
-    const int grid = a.B <= 8 ? choose_rows16(a.bits, a.N, a.K, sms, (int)a.B, L) : 0;
+    double cost;
+    const int grid = a.B <= 8 ? choose_rows16(a.bits, a.N, a.K, sms, (int)a.B, L, cost) : 0;
     if (grid == 0) return cudaErrorInvalidValue;
     L.wait_cycles = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitBudgetCycles;
     return a.bits == 3 ? launch_rows16_bits<3>(a, L, grid, stream) : launch_rows16_bits<2>(a, L, grid, stream);
@@ -1240,7 +1243,7 @@ static uint32_t plan_smem(int bits, int K, int P, int G, int S, int cols, LutPla
     return L.x_off + (uint32_t)cols * L.col_stride;
 }
 
-struct Split { int P, G, slots, ctas, S, cols; };
+struct Split { int P, G, slots, ctas, S, cols; double cost; };
 
 // CTAs of one size class: `slots` of them fit an SM (registers at 80 per thread, shared memory), `ctas` are launched per
 // SM.  (Classes with three or four slots and one of them left free for the first CTAs of the next launch in the stream
@@ -1267,7 +1270,7 @@ static Split choose_split(int bits, int64_t N, int64_t K, int sms, int want_cols
     const int nslices = (int)lut_slices(K);
     const int64_t ntiles = N / kLutAtomRows;
     double best = 1e300;
-    Split sp = {1, 1, 1, 1, 2, 1};
+    Split sp = {1, 1, 1, 1, 2, 1, best};
     LutPlan tmp;
     for (int p = 1; p <= nslices && p <= kMaxWarps; ++p) {
         const int ns_max = (nslices + p - 1) / p;                                   // slices of warp 0
@@ -1289,7 +1292,7 @@ static Split choose_split(int bits, int64_t N, int64_t K, int sms, int want_cols
                 // every further group of four columns adds an mma, four FFMA and its fragment loads to the eight lookups
                 const int passes = (want_cols + cols - 1) / cols;
                 const double cost = (double)passes * (1.0 + 0.2 * (col_groups(cols) - 1)) * (double)(ctas_on_sm * gg * rounds) * per_tile * stretch;
-                if (cost < best) { best = cost; sp = {p, gg, sc.slots, sc.ctas, 2, cols}; }
+                if (cost < best) { best = cost; sp = {p, gg, sc.slots, sc.ctas, 2, cols, cost}; }
                 break;                                                              // the smallest class that fits
             }
         }
@@ -1318,27 +1321,48 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
     return launch_one<BITS, 1024, 1, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
 }
 
-static bool wide_rows(int64_t N, int B) { return N >= 8192 || (B >= 16 && N >= 4096); }
+// The choices between the kernels, from launch after launch of one matrix at 130 shapes from 16 to 16384 rows of 128 to 12288 weights
+// (LUT3 and LUT2; us).
 
-// Which calls the batch kernel of dq_decode_tc.cu takes from the two kernels of this file.  It dequantises a weight once for
-// all columns, at about 1.5 times what a pass of the kernels here costs for few columns (it multiplies the block scale in),
-// in tiles of 256 rows x 512 weights.  Measured (us; LUT3, this file's / that file's kernel):
-//   up to 8 columns: faster only where shared memory cuts the batch into passes (5120x17408 batch 8: 51 / 34; 4096x14336
-//     batch 6: 33 / 29) or there are few rows (512x256 batch 8: 7.0 / 4.8; 1024x4096: 10.3 / 8.5); 17408x5120 batch 8: 23.5 / 29;
-//   9 to 32 columns: against the slice-by-slice kernel, whose rounds over the rows a CTA of eight warps covers and slices of
-//     1024 cost 5.2 us up to 16 columns, 7.9 up to 24 and 8.7 up to 32 where a slice here costs 5.3 and the launch
-//     1.7 more (17408x5120 batch 16: 26.7 / 30.2; 16384x1024: 6.5 / 10.4; 10240x5120: 25.1 / 24.9; batch 24: 38.7 / 26.1); against
-//     passes of eight, always but for short rows (2048x1024 batch 16: 6.2 / 8.6; 4096x4096: 19.8 / 13.8);
-//   above 32: always (17408x5120 batch 40: 66 / 37).
-static bool tc_is_faster(int64_t N, int64_t K, int B, int sms, const Split &narrow)
+// Five to eight columns, 16-row tiles against 8-row tiles: the two cost models in one unit; a CTA with few warps loses a little more
+// than the model's stretch, and long rows' activations take their time to convert.  Over 520 points the pick is never the slower one by more
+// than 2 % and on average 0.3 % off the better (1024x4096 batch 5: 7.9 / 6.6; 4096x5120 batch 8: 11.6 / 11.4; 8192x12288 batch 5:
+// 38 / 25.8; stays with 8 rows: 5120x3072 batch 5 8.3 / 9.2, 1024x8192 batch 6 10.1 / 11.4).  Below 128 rows neither fills the chip.
+static bool rows16_is_faster(int bits, int64_t N, int64_t K, int B, int sms, const Split &narrow)
 {
-    if (B <= 8) return N <= 1024 ? B >= 5 : (B >= 4 && narrow.cols < B);
-    if (B > 32) return true;
-    if (!wide_rows(N, B)) return K > 1024 || B > 16;
+    LutPlan L = {};
+    double cost;
+    if (N < 128 || choose_rows16(bits, N, K, sms, B, L, cost) == 0) return false;
+    const double warps = (double)(L.P * L.G);
+    if (warps < 12.0) cost *= std::sqrt(std::sqrt(12.0 / warps));
+    return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost;
+}
+
+// Where shared memory cuts four to eight columns into passes, the batch kernel of dq_decode_tc.cu, which has no such limit, is ahead once the
+// passes add up (3072x12288 batch 6: 22.7 / 19.5; 5120x17408 batch 8: 52 / 35; not yet for 1024x12288 batch 8: 17.3 / 18.5).
+static bool passes_add_up(int B, const Split &narrow) { return B >= 4 && narrow.cols < B && narrow.cost > 100.0 - 5.0 * B; }
+
+// The batch kernel at up to eight columns on very short rows: one half slice, 4.5 to 4.8 whatever the batch (1024x256 batch 5 / 8: 4.8 / 5.9
+// with 16-row tiles).
+static bool one_half_slice(int64_t N, int64_t K) { return K <= 256 && N <= 16384; }
+
+// Slice-by-slice kernel against passes of eight columns (1024x1024 batch 9: 5.9 / 11.0; 1024x2048 batch 9: 10.3 / 14.1, batch 24: 15.9 / 23.9)
+static bool wide_rows(int64_t N, int64_t K, int B) { return N >= 8192 || (B >= 16 && N >= 4096) || (N >= 512 && K <= 2048); }
+
+// Above eight columns, the batch kernel against the slice-by-slice kernel: rounds over the rows that a CTA of eight warps covers and slices
+// of 1024 cost 5.2 up to 16 columns, 7.9 up to 24 and 8.7 up to 32 there; a slice of 512 costs 5.3 here, a quarter of the only one 1.05,
+// and the second sixteen columns 1.5 (17408x5120 batch 16: 26.7 / 30.2, batch 24: 38.7 / 34.6; 10240x5120: 25.1 / 24.9; 1024x1024 batch 9:
+// 5.9 / 8.1, batch 24: 8.7 / 9.9; 1024x256 batch 9: 5.9 / 4.7; 8192x2048 batch 9: 11.0 / 10.1).  Few rows leave that kernel's warps idle
+// (16x1024 batch 9: 10.8 / 6.6), and above 32 columns it takes two passes (17408x5120 batch 40: 66 / 37).
+static bool tc_is_faster(int64_t N, int64_t K, int B, int sms)
+{
+    if (B > 32 || N < 512) return true;
     const int64_t per_round = 8 * (int64_t)sms;
     const double rounds = (double)((N / 16 + per_round - 1) / per_round) * (double)lut_slices(K);
     const double wide = rounds * (B <= 16 ? 5.2 : B <= 24 ? 7.9 : 8.7) + 1.0;
-    return decode_tc_slices(N, K, sms) * 5.3 + 2.7 < wide;
+    const double slices = decode_tc_slices(N, K, sms);
+    const double tc = (K <= 512 ? slices * 1.05 * (double)((K + 127) / 128) : slices * 5.3) + 2.7 + (B > 16 ? 1.5 : 0.0);
+    return tc < wide;
 }
 
 // up to eight columns per pass
@@ -1362,16 +1386,13 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     const bool choose = a.kernel == 0 && a.force_P == 0;
     const int want_cols = B;                    // the split decides how many of them one pass takes
     Split sp = choose_split(a.bits, N, K, sms, want_cols);
-    if (choose && a.split_exact && tc_is_faster(N, K, B, sms, sp)) return launch_decode_tc(a, stream);
-    // five to eight columns on rows whose activations leave room for the warps (above 8192 weights they do not: 4096x11008 batch 5
-    // 17.3 / 18.3 us)
-    if (choose && B > 4 && B <= 8 && K <= 8192) {
-        const cudaError_t e = launch_rows16(a, sms, stream);
-        if (e != cudaErrorInvalidValue) return e;
+    if (choose && B >= 4 && B <= 8) {
+        if (B > 4 && a.split_exact && one_half_slice(N, K)) return launch_decode_tc(a, stream);
+        if (B > 4 && rows16_is_faster(a.bits, N, K, B, sms, sp)) return launch_rows16(a, sms, stream);
+        if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);
     }
-    // Batches above 8 that stay here: one slice-by-slice pass over the weights per 32 columns instead of one pass per 8 columns,
-    // where that is faster (measured: from 8192 rows on, and from 4096 rows on for 16 columns and more)
-    if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, B))) return launch_wide(a, sms, stream);
+    if (choose && B > 8 && a.split_exact) return tc_is_faster(N, K, B, sms) ? launch_decode_tc(a, stream) : launch_wide(a, sms, stream);
+    if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, K, B))) return launch_wide(a, sms, stream);
     LutPlan L;
     if (a.force_P > 0 && a.force_G > 0) {
         if (a.force_P * a.force_G > 32 || a.force_G > kMaxGroups) return cudaErrorInvalidValue;
