@@ -617,13 +617,10 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
     g.K = w->K;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     cudaError_t ce;
-    // From five columns on, and where shared memory would cut a smaller batch into passes of the mma.sync kernel, the weights
-    // are dequantised once for all columns; below that the two are level but for long rows (measured, us, mma.sync kernel /
-    // that kernel: 34816x5120 batch 1 27.7 / 31, batch 8 33.3 / 31.6, batch 16 64 / 32; 4096x14336 batch 4 16.1 / 17.6,
-    // batch 5 28 / 17.8; 5120x17408 batch 4 42 / 21; few rows, 1024x4096 batch 1 7.6 / 6.5).  Rows above 32768 are refused by
-    // the mma.sync kernel, as for every batch.
-    const bool tc = variant == 5 || (variant == 0 && w->K <= 32768 &&
-                                     (B > 4 || w->N <= 1024 || (int64_t)(2 * w->K + 32) * B > 128 * 1024));
+    const dq::DeviceInfo *di = dq::device_info();
+    if (!di) return DQ_ERR_CUDA;
+    // Rows above 32768 are refused by the mma.sync kernel, as for every batch.
+    const bool tc = variant == 5 || (variant == 0 && w->K <= 32768 && dq::nvfp4_batch_kernel_is_faster(w->N, w->K, B, di->sms));
     if (tc) {
         ce = dq::launch_decode_tc_nvfp4(g, csize, s);
     } else if (variant == 0 || variant == 6) {

@@ -261,6 +261,7 @@ struct GemvNvArgs {
 };
 cudaError_t launch_gemv_nvfp4(const GemvNvArgs &args, cudaStream_t stream);          // CUDA cores, pair-table lookups
 cudaError_t launch_gemv_nvfp4_mma(const GemvNvArgs &args, cudaStream_t stream);      // tensor cores (mma.sync), no lookups
+bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms);
 cudaError_t launch_decode_tc_nvfp4(const GemvNvArgs &args, int force_csize, cudaStream_t stream);     // dq_decode_tc.cu
 cudaError_t launch_fill_e2m1_table(cudaStream_t stream);
 // read-only streaming sum with 128-bit loads (measurement): 8 bytes of result at out_dev

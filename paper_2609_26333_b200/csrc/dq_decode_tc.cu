@@ -825,12 +825,12 @@ cudaError_t launch_cols(const CUtensorMap &tmap, const TcDecodeArgs &P, int forc
 }  // namespace
 
 // 512-weight slices the busiest CTA of a launch works through, before the exchange of a cluster (the launcher's own choice,
-// with the cluster sizes that fit a B200 taken as those whose CTAs fit the chip)
+// by what fits a B200 at once: clusters do not straddle its groups of SMs, so the last few SMs stay out, more of them at eight CTAs)
 double decode_tc_slices(int64_t N, int64_t K, int sms)
 {
     const int tiles = (int)((N + 255) / 256), ns = (int)((K + kSlice - 1) / kSlice);
     double best = (double)((tiles + sms - 1) / sms) * ns;
-    for (int c = 2; c <= kMaxCluster && c <= ns && tiles * c <= sms; ++c) {
+    for (int c = 2; c <= kMaxCluster && c <= ns && tiles * c <= sms - (c == 8 ? 28 : 8); ++c) {
         const double cost = (double)((ns + c - 1) / c) + 0.5;
         if (cost < best) best = cost;
     }

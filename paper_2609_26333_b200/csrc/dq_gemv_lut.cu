@@ -1338,6 +1338,10 @@ static bool rows16_is_faster(int bits, int64_t N, int64_t K, int B, int sms, con
     return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost;
 }
 
+// Four columns: 16-row tiles only where every CTA gets one of them at most and the rows are short (512x1024: 5.7 / 5.0; 1024x2048: 6.1 / 5.4;
+// 2048x256: 5.2 / 4.6; longer, 1024x2560: 6.2 / 6.5; more rows, 3072x1024: 4.4 / 5.3)
+static bool few_rows(int64_t N, int64_t K, int sms) { return N >= 512 && N <= 16 * (int64_t)sms && K <= 2048; }
+
 // Where shared memory cuts four to eight columns into passes, the batch kernel of dq_decode_tc.cu, which has no such limit, is ahead once the
 // passes add up (3072x12288 batch 6: 22.7 / 19.5; 5120x17408 batch 8: 52 / 35; not yet for 1024x12288 batch 8: 17.3 / 18.5).
 static bool passes_add_up(int B, const Split &narrow) { return B >= 4 && narrow.cols < B && narrow.cost > 100.0 - 5.0 * B; }
@@ -1387,6 +1391,7 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     const int want_cols = B;                    // the split decides how many of them one pass takes
     Split sp = choose_split(a.bits, N, K, sms, want_cols);
     if (choose && B >= 4 && B <= 8) {
+        if (B == 4 && few_rows(N, K, sms)) return launch_rows16(a, sms, stream);
         if (B > 4 && a.split_exact && one_half_slice(N, K)) return launch_decode_tc(a, stream);
         if (B > 4 && rows16_is_faster(a.bits, N, K, B, sms, sp)) return launch_rows16(a, sms, stream);
         if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);

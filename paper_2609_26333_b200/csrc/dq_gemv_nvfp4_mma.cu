@@ -303,17 +303,39 @@ cudaError_t launch_one(const GemvNvArgs &a, int b0, int cols, int grid, int thre
 
 }  // namespace
 
+// warps per row group (one 1024-weight slice each) and row groups per CTA
+static int row_groups(int W)
+{
+    // measured: 20 warps with three chunks in flight per lane beat 16 warps with four (17408x5120: 15.0 vs 17.4 us);
+    // 24 warps with two and any configuration that spills are slower
+    const int G = (W > 20 ? 32 : 20) / W;
+    return G < 1 ? 1 : G > 15 ? 15 : G;
+}
+
+// Whether the batch kernel of dq_decode_tc.cu is ahead of this file's, from 396 points between 16x256 and 17408x8192, batch 1 to 8, launch
+// after launch of one matrix: here 2.4 us a pass, 4.6 for each round over the rows (less where a slice is short) and about half a
+// microsecond a column; there 2.2 and 2.7 for each slice of 512 weights that a CTA dequantises, whatever the batch.  The pick is never
+// the slower one by more than 2 % (us, here / there: 2048x4096 batch 1 / 4 7.6 / 6.6, 9.3 / 6.7; 8192x256 batch 4 5.6 / 3.8; 1024x8192
+// batch 1 / 8 7.1 / 8.8, 20.4 / 9.2; 8192x5120 batch 5 10.5 / 12.3; 17408x5120 batch 5 / 6 15.8 / 17.4, 16.4 / 17.4).  Above eight columns a second
+// pass is due here.
+bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms)
+{
+    const int64_t W = (K + 1023) / 1024, G = row_groups((int)W), ntiles = ((N + 127) / 128) * 8;
+    const int64_t cols_max = kMaxXBytes / (2 * K + 32);
+    if (B > 8 || cols_max < 1) return true;
+    const int64_t cols = cols_max < 8 ? cols_max : 8;
+    const double rounds = (double)((ntiles + G * sms - 1) / (G * sms)), passes = (double)((B + cols - 1) / cols);
+    const double here = passes * (2.4 + 4.6 * rounds * (K < 1280 ? (double)K / 1280.0 : 1.0)) + 0.58 * (double)B * (0.8 + 0.2 * rounds);
+    const double there = 2.2 + 2.7 * decode_tc_slices(N, K, sms) * (K < 512 ? (double)K / 512.0 : 1.0);
+    return there < here;
+}
+
 cudaError_t launch_gemv_nvfp4_mma(const GemvNvArgs &a, cudaStream_t stream)
 {
     const int K = (int)a.K, N = (int)a.N, B = (int)a.B;
-    const int W = (K + 1023) / 1024;                  // warps per row group (one 1024-weight slice each)
+    const int W = (K + 1023) / 1024;
     if (W > 32) return cudaErrorInvalidValue;
-    // measured: 20 warps with three chunks in flight per lane beat 16 warps with four (17408x5120: 15.0 vs 17.4 us);
-    // 24 warps with two and any configuration that spills are slower
-    const int max_warps = (W > 20) ? 32 : 20;
-    int G = max_warps / W;
-    if (G < 1) G = 1;
-    if (G > 15) G = 15;
+    const int G = row_groups(W);
     const int threads = G * W * 32;
     if ((size_t)G * kSlots * W * 32 * 16 > kRedBytes) return cudaErrorInvalidValue;
     const uint32_t col_stride = (uint32_t)K * 2u + 32u;          // 32 mod 128: see the layout note in the kernel

@@ -181,3 +181,21 @@ def test_decode_rows16_parity(dq, oracle, fmt, N, K, B):
         y = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2}[fmt](w, X.to(DEV))
         _status_ok(dq)
         check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K} public")
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
+@pytest.mark.parametrize("N,K", [(512, 256), (528, 1024), (1024, 2176), (2384, 640)])
+@pytest.mark.parametrize("B", [4, 6, 9, 16, 24])
+def test_decode_takes_any_kernel_on_few_rows(dq, oracle, fmt, N, K, B):
+    """Small matrices on both sides of the lines between the kernels, through the public calls."""
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    call = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2, "nvfp4": dq.decode_linear_nvfp4}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 700 + B)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    out = torch.full((B + 1, N + 8), 7.0, dtype=torch.bfloat16, device=DEV)
+    call(w, X.to(DEV), out=out[:B, :N])
+    _status_ok(dq)
+    check_outputs(_f64(out[:B, :N]), Yr, S, f"{fmt} {B}x{N}x{K}")
+    assert torch.all(out[B] == 7.0) and torch.all(out[:, N:] == 7.0)
