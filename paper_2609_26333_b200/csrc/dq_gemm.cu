@@ -394,6 +394,9 @@ cudaError_t set_attributes(int dev)
 // CTAs per tile of 128 x BN: bytes of weights (rows x k-steps) that the busiest CTA streams, the activation tile of a step counted
 // as 48 rows (it comes from L2) and a cluster's exchange as 600.  A cluster takes one tile, and all must be resident;
 // how many of a size fit is asked once per device.
+// Against the pair kernel, above one tile of rows, the output counts as well: a round takes no less than its epilogue and half its k-steps
+// (34816 columns, 16384 rows: 2.3 us a round at K = 128, 2.9 at 1024), the exchange of full row tiles up to 1500 more where few
+// k-steps hide it (512x1536, 793 rows: 9.6 us against 8.2 in the pair kernel; 5120x17408, 300 rows: 25.2 with it, 27.0 without), and the ramp is 600 shorter than the pair kernel's.
 template <int BN>
 Split choose_split(const GemmArgs &a, int dev, int sms)
 {
@@ -401,7 +404,9 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
     const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
     const int num_ks = (int)((a.K / 64 + kKbPerStage - 1) / kKbPerStage);
     const double step = BN + 48.0;
-    Split best = {1, (double)((tiles + sms - 1) / sms) * num_ks * step};
+    const double rounds = (double)((tiles + sms - 1) / sms), stream = num_ks * step, output = 0.54 * stream + 1290.0 * (BN / 128);
+    const bool many = a.M > BM;
+    Split best = {1, many ? rounds * (stream > output ? stream : output) - 600.0 : rounds * stream};
     for (int c = 2; c <= kMaxCluster && c <= num_ks && tiles * c <= sms; ++c) {
         int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
         if (fit == 0) {
@@ -416,7 +421,7 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
             max_clusters[dev][c].store(fit, std::memory_order_relaxed);
         }
         if (tiles > fit - 1) continue;
-        const double cost = (double)((num_ks + c - 1) / c) * step + 600.0;
+        const double cost = (double)((num_ks + c - 1) / c) * step + 600.0 + (many && num_ks < 50 ? 1500.0 - 30.0 * num_ks : 0.0);
         if (cost < best.cost) best = {c, cost};
     }
     return best;
@@ -477,12 +482,16 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
     const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
     if (a.M > BM) {
         // CTA pairs on 256 x 256 tiles move half as many bytes per flop but have few tiles to share out: 0.36 us per k-step and round
-        // and 1 us per tile against 1.75 ns per unit of the other cost.  Measured (us, quantiser included, pair / here): 5120x17408
+        // and 1 us per tile against 1.75 ns per unit of the other cost, and no less than the output of a round on short rows
+        // (34816x256, 16384 rows: 293 us here, 568 with the other kernel; 5120x1024, 2048 rows 13.3 / 16.7).  Measured (us, quantiser included, pair / here): 5120x17408
         // 200 tokens 29.7 / 21.7, 300 tokens 31.3 / 26.0, 512 tokens 32.7 / 37.3; 6144x4096 256 tokens 12.6 / 11.5, 512 tokens
         // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
         const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
         const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
-        const auto pair_cost = [&](int64_t r) { return (double)r * ((double)num_ks * 206.0 + 571.0); };
+        const auto pair_cost = [&](int64_t r) {
+            const double stream = (double)num_ks * 206.0 + 571.0, output = (double)num_ks * 150.0 + 900.0;
+            return (double)r * (stream > output ? stream : output);
+        };
         // Where the last round would be nearly empty its columns go to the cluster kernel in a launch of their own, about 7 us of
         // ramp before its k-steps count (5120x17408, 1000 tokens, 80 tiles on 74 pairs: 59.6 -> 50.0 us; 10240x5120,
         // where a round is 9 us, would lose: 31.7 -> 37.3)
