@@ -384,7 +384,7 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           any shape and batch; groups_per_cta (1..9) then sets its warps per CTA.  variant 5 runs the
  *           batch kernel that dequantises every weight once into tensor memory (all columns in one pass,
  *           256-row tiles; DQ_ERR_INVALID_ARG for a codebook with levels that are not multiples of
- *           2^-15); warps_per_group (1..8) then sets the CTAs that share a tile.  variant 6 runs the kernel
+ *           2^-15 or beyond +-146.2); warps_per_group (1..8) then sets the CTAs that share a tile.  variant 6 runs the kernel
  *           with 16-row tiles that dq_decode_linear takes for most batches of 5 to 8 (DQ_ERR_INVALID_ARG where
  *           the row is too long for it).
  *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what

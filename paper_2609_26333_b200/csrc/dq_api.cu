@@ -46,7 +46,7 @@ struct dq_weights {
     unsigned formats;
     uint8_t *base;
     dq::PackedLayout layout;
-    bool lut3_split_exact;               // every LUT3 level is a multiple of 2^-15
+    bool lut3_split_exact;               // every LUT3 level times a block scale is a pair of fp16 numbers
 };
 
 namespace {
@@ -153,12 +153,14 @@ int clear_sf_padding(const dq::PackedLayout &L, uint8_t *base, int64_t N, int64_
     return cudaMemsetAsync(base + L.nv_sf_off + full, 0, L.nv_sf_bytes - full, s) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
-// levels times E4M3 scales then fit a pair of fp16 numbers exactly (the batch decode kernel asks for it)
+// Levels times E4M3 scales then fit a pair of fp16 numbers exactly (the batch decode kernel asks for it): multiples of 2^-15 times
+// multiples of 2^-9, and no product beyond the largest fp16.  The negative side of a codebook has no limit of its own: -200 under
+// a scale of 448 would be an infinity, and its rest a NaN.
 bool split_exact(const uint16_t cb[8])
 {
     for (int j = 0; j < 8; ++j) {
-        const float v = __half2float(__ushort_as_half(cb[j])) * 32768.0f;
-        if (v != std::rint(v)) return false;
+        const float v = __half2float(__ushort_as_half(cb[j])), t = v * 32768.0f;
+        if (t != std::rint(t) || std::fabs(v) * 448.0f > 65504.0f) return false;
     }
     return true;
 }

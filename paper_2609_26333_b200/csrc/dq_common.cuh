@@ -239,7 +239,7 @@ struct GemvArgs {
     long long wait_cycles = 0;
     int drop_first_copy = 0;                              // one warp's first copy is never requested (its wait must run out)
     int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8), 4 = dequantised through tcgen05 (any batch), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns)
-    bool split_exact = true;                              // codebook levels are multiples of 2^-15 (launch_decode_tc)
+    bool split_exact = true;                              // codebook levels times block scales are exact as pairs of fp16 numbers (launch_decode_tc)
 };
 cudaError_t launch_gemv_lut(const GemvArgs &args, cudaStream_t stream);     // picks one of the two kernels below
 // tcgen05 kernel (batch 1): number of warpgroups it would run this shape with, 0 where it does not take it
@@ -247,7 +247,7 @@ int gemv_lut_tc_warpgroups(int bits, int64_t N, int64_t K, int64_t B, int sms, b
 cudaError_t launch_gemv_lut_tc(const GemvArgs &args, int warpgroups, cudaStream_t stream);
 
 // dq_decode_tc.cu: up to 64 columns in one pass, dequantised weights through tcgen05.  LUT3 asks for a codebook whose levels
-// are multiples of 2^-15 (split_exact); force_P = CTAs per tile (test hook)
+// are multiples of 2^-15 up to 146.2 in magnitude (split_exact); force_P = CTAs per tile (test hook)
 cudaError_t launch_decode_tc(const GemvArgs &args, cudaStream_t stream);
 double decode_tc_slices(int64_t N, int64_t K, int sms);
 

@@ -4,8 +4,8 @@
 //
 // Arithmetic.  A weight is dequantised with its block scale to fp16: E2M1 * E4M3 is exact (3 + 4 bits of significand); an
 // fp16 codebook level times E4M3 has up to 15 bits and is kept as a pair hi = rn(G d), lo = G d - hi, both fp16 and exact for
-// codebooks whose levels are multiples of 2^-15 (every d is a multiple of 2^-9, fp16 reaches down to 2^-24; the launcher
-// asks for it).  Activations: per batch column and slice of 512 weights one power of two brings the largest
+// codebooks whose levels are multiples of 2^-15 (every d is a multiple of 2^-9, fp16 reaches down to 2^-24) and at most 146.2 in
+// magnitude (d goes to 448, fp16 to 65504); the launcher asks for it.  Activations: per batch column and slice of 512 weights one power of two brings the largest
 // magnitude into [2^14, 2^15); fp16 then holds every element within 2^28 of it exactly.  So products are exact; a group (128
 // weights of a LUT format, a slice of NVFP4) is summed in fp32 by the tensor cores, groups are added in fp32 by FMA with the inverse
 // power of two.

@@ -148,6 +148,41 @@ def test_decode_batch_fine_codebook_takes_the_general_path(dq, oracle):
     check_outputs(_f64(Y), (X.double() @ Wd.T).cpu().numpy(), (X.double().abs() @ Wd.abs().T).cpu().numpy(), "fine codebook")
 
 
+def _imported_layer(dq, N, K, cb, seed):
+    """A LUT3 handle from random indices and every finite block scale, as an import may bring them, and its weights in fp64."""
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    planes = torch.randint(-2 ** 31, 2 ** 31, (N, 3, K // 32), generator=g, device=DEV, dtype=torch.int64).to(torch.int32)
+    scales = torch.randint(0, 256, (N, K // 16), generator=g, device=DEV, dtype=torch.int32)
+    scales = (scales - ((scales & 0x7F) == 0x7F).int()).to(torch.uint8)                # 0x7F and 0xFF are NaN
+    scales[:, :2] = 0x7E                                                               # the largest, 448
+    s = 2.0 ** -10
+    w = dq.import_canonical(N, K, dq.FMT_LUT3, s, lut3=(planes, scales), codebook_f16=[int(v) & 0xFFFF for v in cb.view(torch.int16)])
+    bit = (planes.long()[:, :, :, None] >> torch.arange(32, device=DEV)) & 1
+    idx = (bit[:, 0] + 2 * bit[:, 1] + 4 * bit[:, 2]).flatten(1)
+    return w, cb.double().to(DEV)[idx] * scales.view(torch.float8_e4m3fn).double().repeat_interleave(16, dim=1) * s
+
+
+@pytest.mark.parametrize("lowest,fits", [(-146.0, True), (-146.25, False), (-200.0, False), (-65504.0, False)])
+@pytest.mark.parametrize("N,K", [(512, 256), (512, 1024), (272, 640)])
+@pytest.mark.parametrize("B", [5, 9, 40])
+def test_decode_batch_codebooks_of_large_magnitude(dq, lowest, fits, N, K, B):
+    """The negative side of a codebook has no limit.  A level times the largest block scale, 448, fits fp16 up to 146.2; beyond, the
+    kernel refuses and the public call takes one that multiplies in fp32."""
+    w, Wd = _imported_layer(dq, N, K, torch.tensor([lowest, -2.0, -1.0, 0.0, 1.0, 2.5, 4.0, 6.0], dtype=torch.float16), 31 + N + K)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 40 + B).to(DEV)
+    Yr, S = (X.double() @ Wd.T).cpu().numpy(), (X.double().abs() @ Wd.abs().T).cpu().numpy()
+    Y = dq.decode_linear(w, X)
+    _status_ok(dq)
+    check_outputs(_f64(Y), Yr, S, f"lowest level {lowest}, batch {B}")
+    if fits:
+        Y = dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=TC)
+        _status_ok(dq)
+        check_outputs(_f64(Y), Yr, S, f"lowest level {lowest}, batch {B}, batch kernel")
+    else:
+        with pytest.raises(dq.DQError):
+            dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=TC)
+
+
 def test_decode_batch_wait_runs_out(dq):
     """A ring stage that is never requested: the waits run out, the launch returns and reports."""
     w = dq.pack_weights(dq_inputs.gaussian_bf16(256, 512, 0.02, 1).to(DEV), formats=dq.FMT_LUT3)
