@@ -640,6 +640,12 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 uint32_t cnt = 0, step = 0, grp = 0;
                 for (int tile = first_tile; tile < ntiles && ok; tile += tile_stride) {
                     const int nh = halves(tile);
+                    // A last tile without a second half: that half's warps may still be reading the tile before back, with inverse scales
+                    // whose place the activations of the fourth slice from then on take.  Steps of half 0 alone would not hold them off.
+                    if (nh == 1 && grp > 0) {
+                        const uint32_t n = grp - 1u;
+                        ok = wait_one(win0 + kDEmpty + ((n & 1u) * 2u + 1u) * 8u, (n >> 1) & 1u, abort_flag, budget);
+                    }
                     for (int sl = s0; sl < s1 && ok; ++sl, ++cnt) {
                         const uint32_t xb = cnt & 1u;
                         ok = wait_one(win0 + kXFull + xb * 8u, (cnt >> 1) & 1u, abort_flag, budget);

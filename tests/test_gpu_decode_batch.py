@@ -183,6 +183,44 @@ def test_decode_batch_codebooks_of_large_magnitude(dq, lowest, fits, N, K, B):
             dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=TC)
 
 
+def _dequantised(dq, w, fmt):
+    """The handle's weights in fp64 on the GPU, from its canonical export."""
+    codes, scales, s = dq.export_canonical(w, {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt])
+    if fmt == "nvfp4":
+        mags = torch.tensor([0, 0.5, 1, 1.5, 2, 3, 4, 6], dtype=torch.float64, device=DEV)
+        levels = torch.cat([mags, -mags])
+        idx = torch.stack([codes & 15, codes >> 4], dim=2).flatten(1).long()
+    else:
+        lo = {"lut3": [-4.703125, -2.869140625, -1.369140625, 0, 1.220703125, 2.529296875, 4.046875, 6],
+              "lut2": [-3.65234375, 0, 2.5234375, 6]}[fmt]
+        levels = torch.tensor(lo, dtype=torch.float64, device=DEV)
+        bit = (codes[:, :, :, None] >> torch.arange(32, device=DEV, dtype=torch.int32)) & 1
+        idx = sum(bit[:, p].int() << p for p in range(codes.shape[1])).flatten(1).long()
+    return levels[idx] * scales.view(torch.float8_e4m3fn).double().repeat_interleave(16, dim=1) * s.double()
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
+@pytest.mark.parametrize("B", [9, 40])
+@pytest.mark.parametrize("rest", [16, 128, 144])
+def test_decode_batch_last_tile_of_a_cta_has_one_half(dq, fmt, B, rest):
+    """More 256-row tiles than SMs and a last one with rows in its first half only (and, beside it, in both): a CTA then takes a
+    full tile and a half one, the second half's warps reading the full one back while the half one is under way.  Slices whose
+    magnitudes differ by many binades: an inverse scale of another slice would show."""
+    N, K = 256 * torch.cuda.get_device_properties(0).multi_processor_count + rest, 2688
+    g = torch.Generator(device=DEV).manual_seed(N + B)
+    W = (torch.randn(N, K, generator=g, device=DEV) * 0.02).to(torch.bfloat16)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights(W, formats=code)
+    X = torch.randn(B, K, generator=g, device=DEV) * torch.exp2(3.0 * torch.arange(K, device=DEV).div(512, rounding_mode="floor"))
+    X = X.to(torch.bfloat16)
+    Wd = _dequantised(dq, w, fmt)
+    Yr, S = (X.double() @ Wd.T).cpu().numpy(), (X.double().abs() @ Wd.abs().T).cpu().numpy()
+    for _ in range(3):
+        y = dq.test_decode_linear(w, code, X, variant=TC)
+        _status_ok(dq)
+        check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K}")
+
+
 def test_decode_batch_wait_runs_out(dq):
     """A ring stage that is never requested: the waits run out, the launch returns and reports."""
     w = dq.pack_weights(dq_inputs.gaussian_bf16(256, 512, 0.02, 1).to(DEV), formats=dq.FMT_LUT3)
