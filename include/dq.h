@@ -21,7 +21,8 @@
  *     and `workspace_dev` 1024-byte aligned (else DQ_ERR_ALIGN);
  *   - a handle belongs to the device that was current when it was packed; calls that
  *     use it with another device current return DQ_ERR_INVALID_ARG;
- *   - NaN/Inf in tensors give unspecified values, never a fault;
+ *   - NaN/Inf in tensors give unspecified values, never a fault (an infinite activation makes the outputs of its own row infinite
+ *     or NaN; the decode calls may lose the finite rows that share its power-of-two scale, see dq_decode_linear);
  *   - the device must be compute capability 10.0 (else DQ_ERR_ARCH).
  */
 #ifndef DQ_H_

@@ -41,8 +41,8 @@ using namespace tc;
 constexpr int kSlice = 512;                        // weights along K per accumulator
 constexpr int kThreads = 512;
 constexpr uint32_t kSmemMax = 227 * 1024;
-constexpr uint32_t kXinvOff = 512;                 // [4][64] floats: inverse activation scales of the last slices
-constexpr uint32_t kRingOff = 2048;
+constexpr uint32_t kXinvOff = 512;                 // [4][4][64] floats: inverse activation scales of the last slices' 128-weight groups
+constexpr uint32_t kRingOff = 5120;
 
 // FMT: 0 = NVFP4, 2 = LUT2, 3 = LUT3; NC: batch columns of the pass, padded
 template <int FMT, int NC>
@@ -126,6 +126,47 @@ __device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t a, uint32_t b)
     uint32_t r;
     asm("max.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
     return r;
+}
+// A bf16 pair as fp16: +-1 in the place of an infinity, NaN stays, anything else is zero
+__device__ __forceinline__ uint32_t inf_to_one(uint32_t w)
+{
+    uint32_t r = 0;
+#pragma unroll
+    for (int s = 0; s < 32; s += 16) {
+        const uint32_t h = (w >> s) & 0xFFFFu, mag = h & 0x7FFFu;
+        r |= (mag == 0x7F80u ? (h & 0x8000u) | 0x3C00u : mag > 0x7F80u ? 0x7FFFu : 0u) << s;
+    }
+    return r;
+}
+// Infinite activations of a LUT format.  Both parts of a weight meet the same activation, and a part that is zero would make a NaN of an
+// infinite one: a warp's columns of the slice (every fourth from c0) that hold an infinity are staged again with +-1 for it and
+// zeros beside it, and the inverse scale of their 128-weight groups is infinite.  A function of its own: inside the loop of the
+// activation warps its code costs every call of more than 32 columns 1 % (5120x17408 LUT3 batch 40: 44.5 us so, 45.0 inside).
+__device__ __noinline__ void stage_infinite(const __nv_bfloat16 *X, int64_t ldx, int c0, int cols, int live, uint32_t xb, uint32_t stride,
+                                            float *xinv)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int c = c0; c < cols && c < c0 + 16; c += 4) {
+        const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)c * ldx);
+        uint4 x[2];
+        uint32_t inf = 0;                                    // groups with an infinity
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint4 v = lane + 32 * i < live ? __ldg(xp + lane + 32 * i) : make_uint4(0u, 0u, 0u, 0u);
+            x[i] = make_uint4(inf_to_one(v.x), inf_to_one(v.y), inf_to_one(v.z), inf_to_one(v.w));
+            // 1 has bit 12 set and bit 14 clear, NaN has both
+            const uint32_t ones = (x[i].x & ~(x[i].x >> 2)) | (x[i].y & ~(x[i].y >> 2)) | (x[i].z & ~(x[i].z >> 2)) | (x[i].w & ~(x[i].w >> 2));
+            const uint32_t any = __ballot_sync(0xffffffffu, (ones & 0x10001000u) != 0u);
+            inf |= ((any & 0xFFFFu ? 1u : 0u) | (any >> 16 ? 2u : 0u)) << (2 * i);
+        }
+        if (inf == 0) continue;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                         ::"r"(xb + (uint32_t)c * 16u + (uint32_t)(lane + 32 * i) * stride), "r"(x[i].x), "r"(x[i].y), "r"(x[i].z), "r"(x[i].w) : "memory");
+        if (lane < 4) xinv[lane * 64 + c] = (inf >> lane) & 1u ? __uint_as_float(0x7F800000u) : 1.0f;
+    }
 }
 // four code bytes -> four fp16 pairs (low nibble first)
 __device__ __forceinline__ void e2m1x8_to_f16(uint32_t w, uint32_t (&p)[4])
@@ -338,7 +379,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
         uint32_t cnt = 0, step = 0, wst = 0, wph = 0;       // slices, A buffers filled, ring stage and its phase
         uint32_t grp = 0;                                   // groups handed over
         bool open = false;                                  // the last of them is not in the running sums yet
-        uint32_t open_xi = 0;                               // the inverse activation scales it takes
+        uint32_t next_xi = 0, open_xi = 0;                  // inverse activation scales of the next group and of that one
         // the last complete group from its accumulator into the running sums
         auto flush = [&]() {
             if (!open) return;
@@ -389,7 +430,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             if ((st + 1) % C::kGroupSteps == 0 || st + 1 == nsteps) {
                 ++grp;
                 open = true;
-                open_xi = win0 + kXinvOff + (cnt & 3u) * 256u;
+                open_xi = next_xi;
+                if (kLut) next_xi += 256u;
             }
         };
         for (int tile = first_tile; tile < ntiles && ok; tile += tile_stride) {
@@ -398,6 +440,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             for (int c = 0; c < NC; ++c) acc[c] = 0.0f;
             for (int sl = s0; sl < s1 && ok; ++sl, ++cnt) {
                 const int ng = groups(sl);
+                next_xi = win0 + kXinvOff + (cnt & 3u) * 1024u;
                 if constexpr (kLut) {
                     // Index words and scales of this warp's 32 rows: four atoms.  Scales of the slice and words of one half of it at a time
                     // are held in registers, and the halves are a loop: unrolled over the slice the code outgrows the instruction
@@ -576,6 +619,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 // four columns at a time: eight loads in flight per lane
                 for (int c0 = sw; c0 < P.cols; c0 += 16) {
                     uint4 v[4][2];
+                    uint32_t top = 0;                            // the four columns' largest magnitude
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int c = c0 + 4 * u;
@@ -592,10 +636,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                                                     max_abs_bf16x2(max_abs_bf16x2(v[u][1].x, v[u][1].y), max_abs_bf16x2(v[u][1].z, v[u][1].w)));
                         m &= 0x7FFF7FFFu;
                         m = __reduce_max_sync(0xffffffffu, max(m >> 16, m & 0xFFFFu));
-                        int ex = (int)(m >> 7) - 127;                               // floor(log2(max)); -127 for zero / subnormal
-                        ex = max(-100, min(100, ex));
+                        top = max(top, m);
+                        const int ex = max(-100, (int)(m >> 7) - 127);              // floor(log2(max)); -127 for zero / subnormal
                         const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
-                        if (lane == 0) xinv_s[(cnt & 3u) * 64u + c] = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
+                        if (lane < 4) xinv_s[((cnt & 3u) * 4u + (uint32_t)lane) * 64u + c] = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             const uint32_t ww[4] = {v[u][i].x, v[u][i].y, v[u][i].z, v[u][i].w};
@@ -620,6 +664,9 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                             }
                         }
                     }
+                    if (kLut && top >= 0x7F80u)
+                        stage_infinite(P.X + (int64_t)P.b0 * P.ldx + sl * kSlice, P.ldx, c0, P.cols, live, xb, C::kXStride,
+                                       xinv_s + (cnt & 3u) * 256u);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // the tensor cores read them
                 __syncwarp();

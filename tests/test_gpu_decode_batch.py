@@ -221,6 +221,44 @@ def test_decode_batch_last_tile_of_a_cta_has_one_half(dq, fmt, B, rest):
         check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K}")
 
 
+@pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
+@pytest.mark.parametrize("B", [9, 40])
+def test_decode_batch_infinite_and_huge_activations(dq, fmt, B):
+    """An infinite activation gives what its products give: an infinity where the weight is not zero, NaN where it is, as with one
+    column; infinities of several 128-weight groups add up; the columns beside it are not touched.  NaN stays in its column.
+    Huge finite magnitudes are scaled like any other."""
+    N, K = 272, 1152
+    g = torch.Generator(device=DEV).manual_seed(61 + B)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights((torch.randn(N, K, generator=g, device=DEV) * 0.02).to(torch.bfloat16), formats=code)
+    call = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2, "nvfp4": dq.decode_linear_nvfp4}[fmt]
+    Wd = _dequantised(dq, w, fmt)
+    X = torch.randn(B, K, generator=g, device=DEV).to(torch.bfloat16)
+    Y0 = dq.test_decode_linear(w, code, X, variant=TC)
+    X[0, 700] = float("inf")
+    X[1, 3] = float("-inf")
+    X[2, 129], X[2, 1151] = float("inf"), float("-inf")
+    X[3, 64] = float("nan")
+    X[4] *= 2.0 ** 104                                        # the sums, before the tensor scale of about 2^-15, stay below 2^128
+    X[5] = 0
+    X[5, 17] = 2.0 ** 115
+    Y = dq.test_decode_linear(w, code, X, variant=TC)
+    _status_ok(dq)
+    Yr = X.double() @ Wd.T                                    # 0 times infinity is NaN there too
+    for b in range(3):
+        assert not torch.isfinite(Yr[b]).any()
+        assert torch.equal(torch.isnan(Y[b]), torch.isnan(Yr[b])), f"column {b}"
+        assert torch.equal(Y[b].double().nan_to_num(0.0, 1.0, -1.0), Yr[b].nan_to_num(0.0, 1.0, -1.0)), f"column {b}"
+    assert torch.isnan(Y[3]).all()
+    S = X.double().abs() @ Wd.abs().T
+    for b in (4, 5):
+        check_outputs(_f64(Y[b:b + 1]), Yr[b:b + 1].cpu().numpy(), S[b:b + 1].cpu().numpy(), f"column {b}")
+    assert torch.equal(Y[6:], Y0[6:])
+    one = call(w, X[:1])
+    _status_ok(dq)
+    assert torch.equal(torch.isnan(one[0]), torch.isnan(Y[0])) and torch.equal(one[0].nan_to_num(0.0), Y[0].nan_to_num(0.0))
+
+
 def test_decode_batch_wait_runs_out(dq):
     """A ring stage that is never requested: the waits run out, the launch returns and reports."""
     w = dq.pack_weights(dq_inputs.gaussian_bf16(256, 512, 0.02, 1).to(DEV), formats=dq.FMT_LUT3)
