@@ -220,9 +220,9 @@ int dq_prefill_linear_static(const dq_weights *w, const void *A_dev, int64_t M, 
  * the total.  Nothing is rounded before the fp32 accumulation, so the error per output is a few
  * fp32 rounding errors of sum_k |x w| plus the bf16 rounding of the result, for any activation
  * pattern.  An activation more than 2^28 times smaller in magnitude than the largest activation
- * it shares a power-of-two scale with loses low bits or reads as zero: that is the largest of the
- * same pass (up to eight rows of X), or, for batches above 8 on matrices of 8192 rows and more (4096 and
- * more from batch 16 on), of the same 1024-element slice of K of the same pass (up to 32 rows of X).
+ * it shares a power-of-two scale with loses low bits or reads as zero: at most those of the rows of X that go
+ * through one pass together (eight consecutive rows), in most calls with batches above 8 only those of its own row
+ * in the same slice of K (512 or 1024 elements).
  * X_dev: B x K bf16, row stride ldx; Y_dev: B x N bf16, row stride ldy.
  */
 int dq_decode_linear(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx,
@@ -382,7 +382,7 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           variant 4 runs the kernel that dq_decode_linear takes for batches above 8 where the
  *           batch kernel of variant 5 is not the faster one (up to 32 columns in one pass over the weights, 16-row
  *           tiles, K walked in slices of 1024 with a power-of-two activation scale per slice) on
- *           any shape and batch; groups_per_cta (1..9) then sets its warps per CTA.  variant 5 runs the
+ *           any shape and batch; groups_per_cta (1..8) then sets its warps per CTA.  variant 5 runs the
  *           batch kernel that dequantises every weight once into tensor memory (all columns in one pass,
  *           256-row tiles; DQ_ERR_INVALID_ARG for a codebook with levels that are not multiples of
  *           2^-15 or beyond +-146.2); warps_per_group (1..8) then sets the CTAs that share a tile.  variant 6 runs the kernel

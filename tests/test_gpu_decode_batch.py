@@ -310,3 +310,24 @@ def test_decode_takes_any_kernel_on_few_rows(dq, oracle, fmt, N, K, B):
     _status_ok(dq)
     check_outputs(_f64(out[:B, :N]), Yr, S, f"{fmt} {B}x{N}x{K}")
     assert torch.all(out[B] == 7.0) and torch.all(out[:, N:] == 7.0)
+
+
+@pytest.mark.parametrize("fmt", ["lut3", "lut2"])
+@pytest.mark.parametrize("N,K", [(1040, 1024), (528, 2048), (2064, 640)])
+@pytest.mark.parametrize("B", [9, 16, 24, 29])
+def test_decode_columns_of_very_different_magnitude(dq, oracle, fmt, N, K, B):
+    """Columns that differ by 2^60 in the slice-by-slice kernel, whatever shares its pass, and through the public call, where these
+    shapes reach it."""
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 800 + B).float()
+    X = (X * torch.pow(2.0, torch.linspace(-30, 30, B).round())[:, None]).to(torch.bfloat16)
+    X[3] = 0
+    X[4, 300:] = 0
+    Yr, S = _reference(oracle, ref, fmt, X)
+    call = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2}[fmt]
+    for Y in (_f64(dq.test_decode_linear(w, code, X.to(DEV), variant=4)), _f64(call(w, X.to(DEV)))):
+        _status_ok(dq)
+        for b in range(B):
+            check_outputs(Y[b:b + 1], Yr[b:b + 1], S[b:b + 1], f"{fmt} {B}x{N}x{K} column {b}")
