@@ -1345,22 +1345,24 @@ static bool passes_add_up(int B, const Split &narrow) { return B >= 4 && narrow.
 // with 16-row tiles).
 static bool one_half_slice(int64_t N, int64_t K) { return K <= 256 && N <= 16384; }
 
-// Slice-by-slice kernel against passes of eight columns (1024x1024 batch 9: 5.9 / 11.0; 1024x2048 batch 9: 10.3 / 14.1, batch 24: 15.9 / 23.9)
+// Slice-by-slice kernel against passes of eight columns (1024x1024 batch 9: 4.9 / 11.0; 1024x2048 batch 9: 8.5 / 14.1, batch 24: 11.4 / 23.9)
 static bool wide_rows(int64_t N, int64_t K, int B) { return N >= 8192 || (B >= 16 && N >= 4096) || (N >= 512 && K <= 2048); }
 
-// Above eight columns, the batch kernel against the slice-by-slice kernel: rounds over the rows that a CTA of eight warps covers and slices
-// of 1024 cost 5.2 up to 16 columns, 7.9 up to 24 and 8.7 up to 32 there; a slice of 512 costs 5.3 here, a quarter of the only one 1.05,
-// and the second sixteen columns 1.5 (17408x5120 batch 16: 26.7 / 30.2, batch 24: 38.7 / 34.6; 10240x5120: 25.1 / 24.9; 1024x1024 batch 9:
-// 5.9 / 8.1, batch 24: 8.7 / 9.9; 1024x256 batch 9: 5.9 / 4.7; 8192x2048 batch 9: 11.0 / 10.1).  Few rows leave that kernel's warps idle
-// (16x1024 batch 9: 10.8 / 6.6), and above 32 columns it takes two passes (17408x5120 batch 40: 66 / 37).
+// Above eight columns, the batch kernel against the slice-by-slice kernel.  There: 1.15 and, for each round over the rows that a CTA of
+// eight warps covers and slice of 1024, 3.95 up to 16 columns, 5.2 up to 24, 6.25 up to 32.  Here: 1.1 and 5.05 for each slice of 512 up to
+// 16 columns, 1.8 and 5.72 above; with one slice at most, 1.05 for each quarter (17408x5120 batch 16: 21.4 / 29.7, batch 32: 33.6 / 34.0;
+// 10240x5120 batch 9: 20.5 / 24.2, batch 24: 28.3 / 27.9; 1024x1024 batch 9: 4.9 / 7.9, batch 24: 6.3 / 9.9; 1024x256 batch 9: 4.9 / 4.5;
+// 2048x1536 batch 9: 8.7 / 8.1).  Of 1218 points from 512 to 34816 rows and 128 to 17408 weights the pick is more than 2 % off the better
+// at 49.  Few rows leave that kernel's warps idle (16x1024 batch 9: 10.8 / 6.6), and above 32 columns it takes two passes.
 static bool tc_is_faster(int64_t N, int64_t K, int B, int sms)
 {
     if (B > 32 || N < 512) return true;
     const int64_t per_round = 8 * (int64_t)sms;
     const double rounds = (double)((N / 16 + per_round - 1) / per_round) * (double)lut_slices(K);
-    const double wide = rounds * (B <= 16 ? 5.2 : B <= 24 ? 7.9 : 8.7) + 1.0;
+    const double wide = rounds * (B <= 16 ? 3.95 : B <= 24 ? 5.2 : 6.25) + 1.15;
     const double slices = decode_tc_slices(N, K, sms);
-    const double tc = (K <= 512 ? slices * 1.05 * (double)((K + 127) / 128) : slices * 5.3) + 2.7 + (B > 16 ? 1.5 : 0.0);
+    const double tc = K <= 512 ? slices * 1.05 * (double)((K + 127) / 128) + (B > 16 ? 4.2 : 2.7)
+                               : B > 16 ? slices * 5.72 + 1.8 : slices * 5.05 + 1.1;
     return tc < wide;
 }
 
