@@ -147,7 +147,7 @@ __device__ __noinline__ void stage_infinite(const __nv_bfloat16 *X, int64_t ldx,
 {
     const int lane = threadIdx.x & 31;
 #pragma unroll 1
-    for (int c = c0; c < cols && c < c0 + 16; c += 4) {
+    for (int c = c0; c < cols; c += 4) {
         const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)c * ldx);
         uint4 x[2];
         uint32_t inf = 0;                                    // groups with an infinity
@@ -616,10 +616,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 if (!ok) break;
                 const uint32_t xb = win0 + C::kXOff + (cnt & 1u) * C::kXBytes;
                 const int live = groups(sl) * 16;            // 16-byte pieces (8 weights) of a column inside K
+                uint32_t top = 0;                                // largest magnitude of the warp's columns
                 // four columns at a time: eight loads in flight per lane
                 for (int c0 = sw; c0 < P.cols; c0 += 16) {
                     uint4 v[4][2];
-                    uint32_t top = 0;                            // the four columns' largest magnitude
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int c = c0 + 4 * u;
@@ -664,10 +664,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                             }
                         }
                     }
-                    if (kLut && top >= 0x7F80u)
-                        stage_infinite(P.X + (int64_t)P.b0 * P.ldx + sl * kSlice, P.ldx, c0, P.cols, live, xb, C::kXStride,
-                                       xinv_s + (cnt & 3u) * 256u);
                 }
+                if (kLut && top >= 0x7F80u)
+                    stage_infinite(P.X + (int64_t)P.b0 * P.ldx + sl * kSlice, P.ldx, sw, P.cols, live, xb, C::kXStride,
+                                   xinv_s + (cnt & 3u) * 256u);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // the tensor cores read them
                 __syncwarp();
                 if (lane == 0) mbar_arrive(win0 + kXFull + (cnt & 1u) * 8u);
