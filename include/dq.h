@@ -336,10 +336,10 @@ int dq_silu_mul_quantize_activations(const void *GU_dev, int64_t M, int64_t F, i
                                      void *stream);
 
 /*
- * Measurement hook: how long the last CTA-pair GEMM launch on the current device (dq_prefill_gemm with M > 128,
+ * Measurement hook: how long the last GEMM on the current device (dq_prefill_gemm with M > 128,
  * dq_prefill_gemm_silu_mul_quantize, dq_bench_gemm_mma_only) ran on the SM of its first CTA, in SM clock cycles
- * (clock64) and in nanoseconds of the global timer; their ratio is the SM clock under that load, which on a
- * power-capped part is lower than what a management query reports between launches.  Synchronises `stream`.
+ * (clock64) and in nanoseconds of the global timer, whichever kernel it took; where its columns are shared out over two launches,
+ * the sum of both.  Their ratio is the SM clock under that load, which on a power-capped part is lower than what a management query reports between launches.  Synchronises `stream`.
  * Both values are 0 before the first such launch.
  */
 int dq_bench_gemm_clocks(void *stream, unsigned long long *sm_cycles_host, unsigned long long *ns_host);

@@ -422,7 +422,7 @@ test_silu.__test__ = False
 
 
 def bench_gemm_clocks(stream=None):
-    """dq_bench_gemm_clocks: (SM clock cycles, nanoseconds) the last CTA-pair GEMM launch took on its first CTA's SM."""
+    """dq_bench_gemm_clocks: (SM clock cycles, nanoseconds) the last GEMM (M > 128, or gated) took on its first CTA's SM."""
     cyc, ns = C.c_ulonglong(0), C.c_ulonglong(0)
     _check(lib().dq_bench_gemm_clocks(_stream_ptr(stream), C.byref(cyc), C.byref(ns)), "dq_bench_gemm_clocks")
     return int(cyc.value), int(ns.value)

@@ -158,7 +158,7 @@ __host__ __device__ inline size_t sf_swizzled_offset(int64_t r, int64_t b, int64
     return (size_t)atom * 512 + (size_t)(rr % 32) * 16 + (size_t)(rr / 32) * 4 + (size_t)(b % 4);
 }
 
-// Device status word: [0] = dq_status, [1] = detail; then, for measurement, what the last pair-GEMM launch took on the
+// Device status word: [0] = dq_status, [1] = detail; then, for measurement, what the last GEMM above 128 tokens took on the
 // SM of its first CTA: SM clock cycles and nanoseconds of the global timer from the CTA's start to its end.
 struct StatusWord { int status; int detail; unsigned long long gemm_cycles; unsigned long long gemm_ns; };
 
@@ -216,6 +216,7 @@ struct GemmArgs {
     int64_t M, N, K;
     StatusWord *status;
     bool w_const = false;    // w_codes / w_sf belong to the handle (not cast into the workspace for this call)
+    int clocks = 0;          // 1: the launch leaves its cycles and nanoseconds in the status word, 2: adds them (the pair kernel always leaves its)
     bool mma_only = false;   // measurement: MMA issue sequence only (pair kernel; no loads, scale copies or stores)
     // gated epilogue (pair kernel only): W is a fused gate/up matrix with interleaved rows, and instead of Y the kernel
     // writes NVFP4(bf16(SiLU(gate) * up)) with input scale gated_scale: codes [M][N/4], block scales in the MMA's layout

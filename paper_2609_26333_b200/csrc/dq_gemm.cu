@@ -89,12 +89,12 @@ __device__ __forceinline__ float4 lds_v4f(uint32_t addr)
     return v;
 }
 
-template <int BN, int HALVES>
+template <int BN, int HALVES, bool CLOCKS>
 __global__ void __launch_bounds__(threads_of(HALVES), 1)
 gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const uint8_t *__restrict__ a_sf, const uint8_t *__restrict__ w_sf,
                   const PackedHeader *__restrict__ hdr, float act_scale, __nv_bfloat16 *__restrict__ Y, int64_t ldy,
-                  int M, int N, int K, int csize, int early_weights, StatusWord *status)
+                  int M, int N, int K, int csize, int early_weights, int clocks, StatusWord *status)
 {
     using C = Cfg<BN>;
     constexpr int kStages = C::kStages, kAccs = C::kAccs;
@@ -237,6 +237,15 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
         const uint32_t lanes = (uint32_t)(wq * 32) << 16;
         const float alpha = __fmul_rn(act_scale, hdr->s);
         bool ok = true;
+        // measurement, as in the pair kernel: SM cycles and global-timer nanoseconds of the first CTA, from the end of the kernel ahead until
+        // its first epilogue warp is done; clocks = 1: left in the status word, 2: added to what the launch before it left there
+        long long clk0 = 0, ns0 = 0;
+        const bool timed = CLOCKS && blockIdx.x == 0 && threadIdx.x == 64;
+        if (timed) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            clk0 = clock64();
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
+        }
         if (HALVES == 1 && csize == 1) {
             uint32_t it = 0;
             for (int t = first_tile; t < num_tiles && ok; t += tile_stride, ++it) {
@@ -321,6 +330,12 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
             }
         }
+        if (timed) {
+            long long ns1;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns1));
+            status->gemm_cycles = (unsigned long long)(clock64() - clk0) + (clocks == 2 ? status->gemm_cycles : 0ull);
+            status->gemm_ns = (unsigned long long)(ns1 - ns0) + (clocks == 2 ? status->gemm_ns : 0ull);
+        }
     }
     __syncwarp();
     if (csize > 1 && warp < 2) { cluster_sync(); cluster_sync(); }
@@ -381,12 +396,12 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int c
     return cfg;
 }
 
-template <int BN, int HALVES>
+template <int BN, int HALVES, bool CLOCKS>
 cudaError_t set_attributes(int dev)
 {
     static std::atomic<bool> done[kMaxDevices];
     if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN, HALVES>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN, HALVES, CLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
     if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
     return e;
 }
@@ -413,7 +428,7 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
             cudaLaunchAttribute attr[2];
             const cudaLaunchConfig_t cfg = launch_config<BN, 1>(attr, c * (sms / c), c, nullptr);
             int n = 0;
-            if (set_attributes<BN, 1>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1>, &cfg) != cudaSuccess) {
+            if (set_attributes<BN, 1, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false>, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
             }
@@ -427,12 +442,12 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
     return best;
 }
 
-template <int BN, int HALVES>
+template <int BN, int HALVES, bool CLOCKS>
 cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
-    cudaError_t e = set_attributes<BN, HALVES>(di->device);
+    cudaError_t e = set_attributes<BN, HALVES, CLOCKS>(di->device);
     if (e != cudaSuccess) return e;
     CUtensorMap tmap_a, tmap_w;
     if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
@@ -441,9 +456,9 @@ cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_
     const int grid = (int)(sp.csize > 1 ? tiles * sp.csize : (tiles < sms ? tiles : sms));
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = launch_config<BN, HALVES>(attr, grid, sp.csize, stream);
-    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN, HALVES>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
+    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN, HALVES, CLOCKS>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
                               reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M, (int)a.N, (int)a.K, sp.csize,
-                              a.w_const ? 1 : 0, a.status);
+                              a.w_const ? 1 : 0, a.clocks, a.status);
 }
 
 // An exchange whose row tile leaves a lane quarter empty hangs on the one to three warps that have rows: two warps a quarter then save
@@ -453,7 +468,8 @@ cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_
 template <int BN>
 cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
-    return sp.csize > 1 && a.M <= 3 * 32 ? launch_with<BN, 2>(a, sp, sms, stream) : launch_with<BN, 1>(a, sp, sms, stream);
+    if (a.clocks) return launch_with<BN, 1, true>(a, sp, sms, stream);       // above 128 tokens
+    return sp.csize > 1 && a.M <= 3 * 32 ? launch_with<BN, 2, false>(a, sp, sms, stream) : launch_with<BN, 1, false>(a, sp, sms, stream);
 }
 
 }  // namespace
@@ -471,8 +487,10 @@ int gemm_init_driver_api()
 
 void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
 
-cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
+cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
 {
+    GemmArgs a = args;
+    a.clocks = a.M > BM ? 1 : 0;
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
@@ -499,6 +517,7 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &a, cudaStream_t stream)
         if (rounds > 1 && head > 0 && head * 256 < a.N) {
             GemmArgs tail = a;
             tail.N = a.N - head * 256;
+            tail.clocks = 2;
             tail.w_codes = a.w_codes + head * 256 * (a.K / 2);
             tail.w_sf = a.w_sf + head * 256 * (a.K / kBlock);
             tail.Y = reinterpret_cast<__nv_bfloat16 *>(a.Y) + head * 256;

@@ -762,6 +762,36 @@ def test_measurement_hooks_leave_results_alone(dq, oracle):
         dq.bench_gemm_mma_only(w, 64, scratch, ws)             # the measurement mode exists for M > 128 only
 
 
+@pytest.mark.parametrize("M,N,K", [(2048, 4096, 1024), (512, 1024, 1024), (200, 5120, 4096), (1000, 5120, 17408)])
+def test_gemm_clocks_are_those_of_the_last_launch(dq, M, N, K):
+    """One launch of the pair kernel, lone CTAs, clusters, and a launch of each: the clocks are the last call's, not what an earlier one
+    left, and no longer than the events around it; a prompt of up to 128 tokens leaves them alone."""
+    g = torch.Generator(device=DEV).manual_seed(M)
+    w = dq.pack_weights((torch.randn(N, K, generator=g, device=DEV) * 0.02).to(torch.bfloat16), formats=dq.FMT_NVFP4)
+    A = torch.randn(M, K, generator=g, device=DEV).to(torch.bfloat16)
+    ws = dq.alloc_workspace(dq.prefill_workspace_bytes(w, M), DEV)
+    Y = torch.empty(M, N, dtype=torch.bfloat16, device=DEV)
+    dq.prefill_quantize(w, A, 4.0 / 2688.0, ws)
+    dq.prefill_gemm(w, M, 4.0 / 2688.0, Y, ws)
+    mine = dq.bench_gemm_clocks()
+    dq.bench_gemm_mma_only(w, M, Y, ws)                        # somebody else's launch in between
+    other = dq.bench_gemm_clocks()
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
+    dq.prefill_gemm(w, M, 4.0 / 2688.0, Y, ws)
+    end.record()
+    cycles, ns = dq.bench_gemm_clocks()
+    _status_ok(dq)
+    assert (cycles, ns) != other
+    assert 500.0 < cycles / ns * 1e3 < 2500.0
+    assert 0.4 * mine[1] < ns < 2.5 * mine[1]
+    assert ns <= start.elapsed_time(end) * 1e6 + 500.0
+    flops = 2.0 * M * N * K
+    assert flops / (cycles * 148) < 32768.0                    # not more than the tensor pipes can do in those cycles
+    dq.prefill_linear(w, A[:100], 4.0 / 2688.0)
+    assert dq.bench_gemm_clocks() == (cycles, ns)
+
+
 @pytest.mark.parametrize("N,K", [(16, 128), (272, 640), (48, 1664)])
 @pytest.mark.parametrize("fmt", ["nvfp4+lut3", "nvfp4+lut2", "lut3+lut2+nvfp4", "lut2", "nvfp4"])
 def test_pack_every_combination_of_formats(dq, oracle, N, K, fmt):
