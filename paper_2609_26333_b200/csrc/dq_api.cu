@@ -556,9 +556,7 @@ int dq_prefill_gemm_silu_mul_quantize(const dq_weights *w_gate_up, int64_t M, fl
     g.N = w_gate_up->N;
     g.K = w_gate_up->K;
     g.status = sw;
-    g.gated_codes = ows;
-    g.gated_sf = ows + LO.a_sf;
-    g.gated_scale = out_global_scale;
+    g.gated = {ows, ows + LO.a_sf, out_global_scale, (int)w_down->K};
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (dq::launch_gemm_nvfp4(g, s) != cudaSuccess) return DQ_ERR_CUDA;
     return prefill_weight_view(w_down, ows, LO, s);

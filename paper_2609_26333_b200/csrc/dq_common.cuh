@@ -207,6 +207,14 @@ cudaError_t launch_silu_mul_quant(const void *GU_bf16, int64_t M, int64_t F, int
                                   uint8_t *sf, int swizzled, cudaStream_t stream);
 cudaError_t launch_silu_probe(const void *g_bf16, int64_t n, float *out, cudaStream_t stream);
 
+// What a gated epilogue writes instead of Y
+struct GatedOut {
+    uint8_t *codes;          // [M][F/2] NVFP4 codes of bf16(SiLU(gate) * up)
+    uint8_t *sf;             // their block scales in the MMA's layout
+    float s;                 // static input scale of the layer that reads them
+    int F;                   // features a row of the output holds (N = 2F, or a range of columns of it)
+};
+
 struct GemmArgs {
     const uint8_t *a_codes;  const uint8_t *a_sf;      // activations: [M][K/2], MMA scale layout
     const uint8_t *w_codes;  const uint8_t *w_sf;      // weights:     [N][K/2], MMA scale layout
@@ -218,9 +226,9 @@ struct GemmArgs {
     bool w_const = false;    // w_codes / w_sf belong to the handle (not cast into the workspace for this call)
     int clocks = 0;          // 1: the launch leaves its cycles and nanoseconds in the status word, 2: adds them (the pair kernel always leaves its)
     bool mma_only = false;   // measurement: MMA issue sequence only (pair kernel; no loads, scale copies or stores)
-    // gated epilogue (pair kernel only): W is a fused gate/up matrix with interleaved rows, and instead of Y the kernel
-    // writes NVFP4(bf16(SiLU(gate) * up)) with input scale gated_scale: codes [M][N/4], block scales in the MMA's layout
-    uint8_t *gated_codes = nullptr; uint8_t *gated_sf = nullptr; float gated_scale = 0.0f;
+    // gated epilogue where gated.codes is not null: W is a fused gate/up matrix with interleaved rows, and instead of Y the kernel
+    // writes NVFP4(bf16(SiLU(gate) * up))
+    GatedOut gated = {nullptr, nullptr, 0.0f, 0};
 };
 cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream);
 cudaError_t launch_gemm_nvfp4_pair(const GemmArgs &args, void *encode_fn, cudaStream_t stream);

@@ -21,6 +21,7 @@
 #include <cuda.h>
 
 #include "dq_common.cuh"
+#include "dq_quant.cuh"
 #include "dq_tcgen05.cuh"
 
 namespace dq {
@@ -34,6 +35,19 @@ constexpr int kKbPerStage = 4;                // 64-element MMA k-steps per 256-
 constexpr int threads_of(int halves) { return 64 + 128 * halves; }     // `halves` epilogue warps per TMEM lane quarter
 constexpr uint32_t kTmemCols = 512;
 
+constexpr int kMaxCluster = 8;
+// largest area that the partial sums of a gated tile take: units of 16 gate and 16 up columns go round the CTAs of a cluster, four
+// groups of eight columns each
+constexpr uint32_t gated_bytes(int units)
+{
+    uint32_t most = 0;
+    for (int c = 2; c <= kMaxCluster; ++c) {
+        const uint32_t b = (uint32_t)(c * ((units + c - 1) / c) * 4) * 4096u;
+        if (b > most) most = b;
+    }
+    return most;
+}
+
 template <int BN>
 struct Cfg {
     static constexpr int kStages = BN == 128 ? 6 : 4;
@@ -42,12 +56,15 @@ struct Cfg {
     static constexpr uint32_t A_BYTES = BM * 128, B_BYTES = BN * 128;
     static constexpr uint32_t SFA_BYTES = kKbPerStage * 512, SFB_BYTES = kSfbAtoms * kKbPerStage * 512;
     static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES + SFA_BYTES + SFB_BYTES;
-    static constexpr uint32_t SMEM_BYTES = kStages * STAGE_BYTES + 1024 /*align*/ + 256 /*barriers*/;
+    // barriers behind the ring, which an exchange of partial sums uses again; that of a gated tile may reach beyond it
+    static constexpr uint32_t GATED_BYTES = gated_bytes(BN / 32);
+    static constexpr uint32_t BAR_OFF = kStages * STAGE_BYTES, BAR_OFF_GATED = GATED_BYTES > BAR_OFF ? GATED_BYTES : BAR_OFF;
+    static constexpr uint32_t SMEM_BYTES = BAR_OFF + 1024 /*align*/ + 256 /*barriers*/, SMEM_BYTES_GATED = BAR_OFF_GATED + 1024 + 256;
     static constexpr uint32_t kSfBase = kAccs * BN;                    // TMEM columns: accumulators, then scales per stage
     static constexpr uint32_t kSfbCol = 4 * kKbPerStage, kSfCols = kSfbCol + 4 * kKbPerStage * kSfbAtoms;
     static_assert(kSfBase + kStages * kSfCols <= kTmemCols, "scale buffers must fit in TMEM");
     static_assert(STAGE_BYTES % 1024 == 0, "stages must keep 1024-byte alignment for the 128B swizzle");
-    static_assert(SMEM_BYTES <= 227 * 1024, "shared memory");
+    static_assert(SMEM_BYTES_GATED <= 227 * 1024, "shared memory");
     static_assert((BN / 8 + 8) * BM * 32 <= kStages * (int)STAGE_BYTES, "partial sums of a cluster must fit the ring");
     // instruction descriptor: dense, A/B = E2M1 (kind::mxf4nvf4), both K-major, scale type UE4M3,
     // N >> 3 at bit 17, M >> 4 at bit 24, scale-factor ids 0, K = 64
@@ -89,25 +106,26 @@ __device__ __forceinline__ float4 lds_v4f(uint32_t addr)
     return v;
 }
 
-template <int BN, int HALVES, bool CLOCKS>
+template <int BN, int HALVES, bool CLOCKS, bool GATED>
 __global__ void __launch_bounds__(threads_of(HALVES), 1)
 gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_w,
                   const uint8_t *__restrict__ a_sf, const uint8_t *__restrict__ w_sf,
                   const PackedHeader *__restrict__ hdr, float act_scale, __nv_bfloat16 *__restrict__ Y, int64_t ldy,
-                  int M, int N, int K, int csize, int early_weights, int clocks, StatusWord *status)
+                  int M, int N, int K, int csize, int early_weights, int clocks, StatusWord *status, GatedOut gated)
 {
     using C = Cfg<BN>;
     constexpr int kStages = C::kStages, kAccs = C::kAccs;
+    constexpr uint32_t kBarOff = GATED ? C::BAR_OFF_GATED : C::BAR_OFF;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     // per stage: [A][B][SFA][SFB]; barriers: full[kStages], empty[kStages], tmem_full[2], tmem_empty[2]; then tmem ptr, abort flag
-    const uint32_t bar_base = smem_base + kStages * C::STAGE_BYTES;
+    const uint32_t bar_base = smem_base + kBarOff;
     auto full_bar = [&](int s) { return bar_base + 8u * s; };
     auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
     auto tmem_full_bar = [&](int i) { return bar_base + 8u * (2 * kStages + i); };
     auto tmem_empty_bar = [&](int i) { return bar_base + 8u * (2 * kStages + 2 + i); };
-    uint32_t *tmem_ptr_smem = reinterpret_cast<uint32_t *>(smem_gen + kStages * C::STAGE_BYTES + 8 * (2 * kStages + 4));
+    uint32_t *tmem_ptr_smem = reinterpret_cast<uint32_t *>(smem_gen + kBarOff + 8 * (2 * kStages + 4));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_ptr_smem + 1);
 
     const int warp = threadIdx.x >> 5;
@@ -246,7 +264,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             clk0 = clock64();
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(ns0));
         }
-        if (HALVES == 1 && csize == 1) {
+        if (HALVES == 1 && !GATED && csize == 1) {
             uint32_t it = 0;
             for (int t = first_tile; t < num_tiles && ok; t += tile_stride, ++it) {
                 const uint32_t acc = it % kAccs;
@@ -291,7 +309,9 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
             tc_fence_after();
             cluster_sync();
             const int half = HALVES > 1 ? (warp - 2) >> 2 : 0;                        // each takes its part of the columns
-            const int per = (BN / 8 + csize - 1) / csize;
+            // A gated tile goes out in units of 16 features instead, 16 columns of gate and the 16 of up that lie 64 further on: unit u to
+            // CTA u % csize, so that one thread has what a block of the output takes.
+            const int per = GATED ? (BN / 32 + csize - 1) / csize * 4 : (BN / 8 + csize - 1) / csize;
             const int row = mb * BM + wq * 32 + lane;
             const uint32_t mine = smem_base + (uint32_t)(wq * 32 + lane) * 16u;       // + 2048 for the second half of a group
             if (ok && mb * BM + wq * 32 < M) {
@@ -303,8 +323,10 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                     if (row < M) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const int i = c * 4 + q;
-                            const uint32_t dst = mine + (uint32_t)((int)rank * per + i / csize) * 4096u;
+                            // which of the columns' owners, and where in its share
+                            const int i = GATED ? (c >> 2) * 4 + (c & 1) * 2 + (q >> 1) : c * 4 + q;
+                            const int at = GATED ? i / csize * 4 + ((c >> 1) & 1) * 2 + (q & 1) : i / csize;
+                            const uint32_t dst = mine + (uint32_t)((int)rank * per + at) * 4096u;
                             st_cluster_v4(dst, (uint32_t)(i % csize), v[8 * q], v[8 * q + 1], v[8 * q + 2], v[8 * q + 3]);
                             st_cluster_v4(dst + 2048u, (uint32_t)(i % csize), v[8 * q + 4], v[8 * q + 5], v[8 * q + 6], v[8 * q + 7]);
                         }
@@ -312,7 +334,38 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_const
                 }
             }
             cluster_sync();
-            if (ok && row < M) {
+            if (GATED) {
+                const float rc6 = __frcp_rn(__fmul_rn(6.0f, gated.s));
+                if (ok && row < M) {
+                    for (int l = half, u = (int)rank + half * csize; u < BN / 32; u += HALVES * csize, l += HALVES) {
+                        uint32_t gu[2][8];                                            // gate and up, packed bf16 as the plain epilogue stores them
+#pragma unroll
+                        for (int sub = 0; sub < 4; ++sub) {
+                            float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
+                            for (int src = 0; src < csize; ++src) {
+                                const uint32_t at = mine + (uint32_t)(src * per + 4 * l + sub) * 4096u;
+                                const float4 x = lds_v4f(at), y = lds_v4f(at + 2048u);
+                                a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w;
+                                b.x += y.x; b.y += y.y; b.z += y.z; b.w += y.w;
+                            }
+                            uint32_t *o = &gu[sub >> 1][(sub & 1) * 4];
+                            o[0] = pack_bf16x2(a.x * alpha, a.y * alpha);
+                            o[1] = pack_bf16x2(a.z * alpha, a.w * alpha);
+                            o[2] = pack_bf16x2(b.x * alpha, b.y * alpha);
+                            o[3] = pack_bf16x2(b.z * alpha, b.w * alpha);
+                        }
+                        uint32_t h[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) h[i] = silu_mul_bf16x2(gu[0][i], gu[1][i]);
+                        uint2 codes;
+                        const uint32_t d8 = quant_block_nvfp4_bf16(h, gated.s, rc6, codes);
+                        const int blk = nb * (BN / 32) + u, rr = row & 127;           // 16-feature block of the output row
+                        *reinterpret_cast<uint2 *>(gated.codes + ((int64_t)row * (gated.F >> 4) + blk) * 8) = codes;
+                        gated.sf[((size_t)(row >> 7) * (size_t)(gated.F >> 6) + (size_t)(blk >> 2)) * 512 +
+                                 (size_t)((rr & 31) * 16 + (rr >> 5) * 4 + (blk & 3))] = (uint8_t)d8;
+                    }
+                }
+            } else if (ok && row < M) {
                 for (int l = half, i = (int)rank + half * csize; i < BN / 8 && nb * BN + 8 * i < N; i += HALVES * csize, l += HALVES) {
                     float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
                     for (int src = 0; src < csize; ++src) {
@@ -375,16 +428,15 @@ bool make_codes_tmap(CUtensorMap *tm, const void *ptr, int64_t rows, int64_t K, 
     return r == CUDA_SUCCESS;
 }
 
-constexpr int kMaxCluster = 8;
 struct Split { int csize; double cost; };
 
-template <int BN, int HALVES>
+template <int BN, int HALVES, bool GATED>
 cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int csize, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads_of(HALVES));
-    cfg.dynamicSmemBytes = Cfg<BN>::SMEM_BYTES;
+    cfg.dynamicSmemBytes = GATED ? Cfg<BN>::SMEM_BYTES_GATED : Cfg<BN>::SMEM_BYTES;
     cfg.stream = stream;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -396,12 +448,13 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int c
     return cfg;
 }
 
-template <int BN, int HALVES, bool CLOCKS>
+template <int BN, int HALVES, bool CLOCKS, bool GATED>
 cudaError_t set_attributes(int dev)
 {
     static std::atomic<bool> done[kMaxDevices];
     if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN, HALVES, CLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<BN>::SMEM_BYTES);
+    const cudaError_t e = cudaFuncSetAttribute(gemm_nvfp4_kernel<BN, HALVES, CLOCKS, GATED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(GATED ? Cfg<BN>::SMEM_BYTES_GATED : Cfg<BN>::SMEM_BYTES));
     if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
     return e;
 }
@@ -426,9 +479,9 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
         int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
         if (fit == 0) {
             cudaLaunchAttribute attr[2];
-            const cudaLaunchConfig_t cfg = launch_config<BN, 1>(attr, c * (sms / c), c, nullptr);
+            const cudaLaunchConfig_t cfg = launch_config<BN, 1, false>(attr, c * (sms / c), c, nullptr);
             int n = 0;
-            if (set_attributes<BN, 1, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false>, &cfg) != cudaSuccess) {
+            if (set_attributes<BN, 1, false, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false, false>, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
             }
@@ -442,12 +495,12 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
     return best;
 }
 
-template <int BN, int HALVES, bool CLOCKS>
+template <int BN, int HALVES, bool CLOCKS, bool GATED>
 cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
-    cudaError_t e = set_attributes<BN, HALVES, CLOCKS>(di->device);
+    cudaError_t e = set_attributes<BN, HALVES, CLOCKS, GATED>(di->device);
     if (e != cudaSuccess) return e;
     CUtensorMap tmap_a, tmap_w;
     if (!make_codes_tmap(&tmap_a, a.a_codes, a.M, a.K, BM)) return cudaErrorInvalidValue;
@@ -455,10 +508,10 @@ cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_
     const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
     const int grid = (int)(sp.csize > 1 ? tiles * sp.csize : (tiles < sms ? tiles : sms));
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = launch_config<BN, HALVES>(attr, grid, sp.csize, stream);
-    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN, HALVES, CLOCKS>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
+    const cudaLaunchConfig_t cfg = launch_config<BN, HALVES, GATED>(attr, grid, sp.csize, stream);
+    return cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<BN, HALVES, CLOCKS, GATED>, tmap_a, tmap_w, a.a_sf, a.w_sf, a.hdr, a.act_scale,
                               reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M, (int)a.N, (int)a.K, sp.csize,
-                              a.w_const ? 1 : 0, a.clocks, a.status);
+                              a.w_const ? 1 : 0, a.clocks, a.status, a.gated);
 }
 
 // An exchange whose row tile leaves a lane quarter empty hangs on the one to three warps that have rows: two warps a quarter then save
@@ -468,8 +521,11 @@ cudaError_t launch_with(const GemmArgs &a, const Split &sp, int sms, cudaStream_
 template <int BN>
 cudaError_t launch_tile(const GemmArgs &a, const Split &sp, int sms, cudaStream_t stream)
 {
-    if (a.clocks) return launch_with<BN, 1, true>(a, sp, sms, stream);       // above 128 tokens
-    return sp.csize > 1 && a.M <= 3 * 32 ? launch_with<BN, 2, false>(a, sp, sms, stream) : launch_with<BN, 1, false>(a, sp, sms, stream);
+    // SiLU and quantiser are worth a second warp a quarter where a CTA has more than one unit of the tile (gate/up 3328x8192, 129 tokens:
+    // 18.6 -> 13.7; with one unit, 1024x4096: 8.9 -> 9.5; in the pair kernel 29.7 and 25.0)
+    if (a.gated.codes) return BN / 32 > sp.csize ? launch_with<BN, 2, true, true>(a, sp, sms, stream) : launch_with<BN, 1, true, true>(a, sp, sms, stream);
+    if (a.clocks) return launch_with<BN, 1, true, false>(a, sp, sms, stream);       // above 128 tokens
+    return sp.csize > 1 && a.M <= 3 * 32 ? launch_with<BN, 2, false, false>(a, sp, sms, stream) : launch_with<BN, 1, false, false>(a, sp, sms, stream);
 }
 
 }  // namespace
@@ -487,55 +543,72 @@ int gemm_init_driver_api()
 
 void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
 
+// Kernel and tile of a GEMM: the pair kernel for the first `head` columns, tiles of 128 x bn with clusters of sp.csize for the rest
+struct Plan { int64_t head; int bn; Split sp; };
+
+static Plan choose_plan(const GemmArgs &a, int dev, int sms)
+{
+    const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
+    const Plan tiles_only = s128.cost < s256.cost ? Plan{0, 128, s128} : Plan{0, 256, s256};
+    if (a.M <= BM) return tiles_only;
+    // CTA pairs on 256 x 256 tiles move half as many bytes per flop but have few tiles to share out: 0.36 us per k-step and round
+    // and 1 us per tile against 1.75 ns per unit of the other cost, and no less than the output of a round on short rows
+    // (34816x256, 16384 rows: 293 us here, 568 with the other kernel; 5120x1024, 2048 rows 13.3 / 16.7).  Measured (us, quantiser included, pair / here): 5120x17408
+    // 200 tokens 29.7 / 21.7, 300 tokens 31.3 / 26.0, 512 tokens 32.7 / 37.3; 6144x4096 256 tokens 12.6 / 11.5, 512 tokens
+    // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
+    const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
+    const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
+    const auto pair_cost = [&](int64_t r) {
+        const double stream = (double)num_ks * 206.0 + 571.0, output = (double)num_ks * 150.0 + 900.0;
+        return (double)r * (stream > output ? stream : output);
+    };
+    // Where the last round would be nearly empty its columns go to the cluster kernel in a launch of their own, about 7 us of
+    // ramp before its k-steps count (5120x17408, 1000 tokens, 80 tiles on 74 pairs: 59.6 -> 50.0 us; 10240x5120,
+    // where a round is 9 us, would lose: 31.7 -> 37.3)
+    const int64_t tiles_m = (a.M + 255) / 256, head = (rounds - 1) * (sms / 2) / tiles_m;      // 256-column blocks of the full rounds
+    if (rounds > 1 && head > 0 && head * 256 < a.N) {
+        GemmArgs tail = a;
+        tail.N = a.N - head * 256;
+        const Split t128 = choose_split<128>(tail, dev, sms), t256 = choose_split<256>(tail, dev, sms);
+        const double tail_cost = (t128.cost < t256.cost ? t128.cost : t256.cost) + 4000.0;
+        const double split_cost = pair_cost(rounds - 1) + tail_cost;
+        if (split_cost < pair_cost(rounds) && split_cost < s128.cost && split_cost < s256.cost)
+            return t128.cost < t256.cost ? Plan{head * 256, 128, t128} : Plan{head * 256, 256, t256};
+    }
+    if (pair_cost(rounds) <= s128.cost && pair_cost(rounds) <= s256.cost) return {a.N, 256, {1, 0.0}};
+    return tiles_only;
+}
+
 cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
 {
-    GemmArgs a = args;
-    a.clocks = a.M > BM ? 1 : 0;
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
-    const int dev = di->device, sms = di->sms;
-    // the gated epilogue and the measurement mode exist in the pair kernel only
-    if (a.gated_codes || a.mma_only) return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
-    const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
-    if (a.M > BM) {
-        // CTA pairs on 256 x 256 tiles move half as many bytes per flop but have few tiles to share out: 0.36 us per k-step and round
-        // and 1 us per tile against 1.75 ns per unit of the other cost, and no less than the output of a round on short rows
-        // (34816x256, 16384 rows: 293 us here, 568 with the other kernel; 5120x1024, 2048 rows 13.3 / 16.7).  Measured (us, quantiser included, pair / here): 5120x17408
-        // 200 tokens 29.7 / 21.7, 300 tokens 31.3 / 26.0, 512 tokens 32.7 / 37.3; 6144x4096 256 tokens 12.6 / 11.5, 512 tokens
-        // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
-        const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
-        const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
-        const auto pair_cost = [&](int64_t r) {
-            const double stream = (double)num_ks * 206.0 + 571.0, output = (double)num_ks * 150.0 + 900.0;
-            return (double)r * (stream > output ? stream : output);
-        };
-        // Where the last round would be nearly empty its columns go to the cluster kernel in a launch of their own, about 7 us of
-        // ramp before its k-steps count (5120x17408, 1000 tokens, 80 tiles on 74 pairs: 59.6 -> 50.0 us; 10240x5120,
-        // where a round is 9 us, would lose: 31.7 -> 37.3)
-        const int64_t tiles_m = (a.M + 255) / 256, head = (rounds - 1) * (sms / 2) / tiles_m;      // 256-column blocks of the full rounds
-        if (rounds > 1 && head > 0 && head * 256 < a.N) {
-            GemmArgs tail = a;
-            tail.N = a.N - head * 256;
-            tail.clocks = 2;
-            tail.w_codes = a.w_codes + head * 256 * (a.K / 2);
-            tail.w_sf = a.w_sf + head * 256 * (a.K / kBlock);
-            tail.Y = reinterpret_cast<__nv_bfloat16 *>(a.Y) + head * 256;
-            const Split t128 = choose_split<128>(tail, dev, sms), t256 = choose_split<256>(tail, dev, sms);
-            const double tail_cost = (t128.cost < t256.cost ? t128.cost : t256.cost) + 4000.0;
-            const double split_cost = pair_cost(rounds - 1) + tail_cost;
-            if (split_cost < pair_cost(rounds) && split_cost < s128.cost && split_cost < s256.cost) {
-                GemmArgs front = a;
-                front.N = head * 256;
-                const cudaError_t e = launch_gemm_nvfp4_pair(front, reinterpret_cast<void *>(g_encode), stream);
-                if (e != cudaSuccess) return e;
-                return t128.cost < t256.cost ? launch_tile<128>(tail, t128, sms, stream) : launch_tile<256>(tail, t256, sms, stream);
-            }
+    GemmArgs a = args;
+    a.clocks = a.M > BM ? 1 : 0;
+    Plan p = {a.N, 256, {1, 0.0}};
+    // The measurement mode exists in the pair kernel only, and up to 128 tokens the gated epilogue too.  Above, a gated call adds its
+    // products up as the plain call does: clusters where that takes clusters.  A lone CTA's sums are those of the pair kernel bit
+    // for bit, k-step after k-step, so there the gated call keeps to the pair kernel, whose epilogue overlaps.
+    if (!a.mma_only && !(a.gated.codes && a.M <= BM)) p = choose_plan(a, di->device, di->sms);
+    if (a.gated.codes && p.sp.csize == 1) p.head = a.N;
+    if (p.head > 0) {
+        GemmArgs front = a;
+        front.N = p.head;
+        const cudaError_t e = launch_gemm_nvfp4_pair(front, reinterpret_cast<void *>(g_encode), stream);
+        if (e != cudaSuccess || p.head == a.N) return e;
+        a.N -= p.head;
+        a.w_codes += p.head * (a.K / 2);
+        a.w_sf += p.head * (a.K / kBlock);
+        a.clocks = 2;
+        if (a.gated.codes) {                                      // half as many features
+            a.gated.codes += p.head / 4;
+            a.gated.sf += p.head / 128 * 512;                     // 64 features to an atom
+        } else {
+            a.Y = reinterpret_cast<__nv_bfloat16 *>(a.Y) + p.head;
         }
-        if (pair_cost(rounds) <= s128.cost && pair_cost(rounds) <= s256.cost)
-            return launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
     }
-    return s128.cost < s256.cost ? launch_tile<128>(a, s128, sms, stream) : launch_tile<256>(a, s256, sms, stream);
+    return p.bn == 128 ? launch_tile<128>(a, p.sp, di->sms, stream) : launch_tile<256>(a, p.sp, di->sms, stream);
 }
 
 }  // namespace dq

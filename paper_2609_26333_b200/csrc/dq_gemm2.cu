@@ -200,14 +200,6 @@ __device__ __forceinline__ void tile_coords2(int t, int tiles_m, int tiles_n, in
     nb = r / gsz;
 }
 
-// what the gated epilogue (EPI = 1) writes instead of Y
-struct GatedOut {
-    uint8_t *codes;          // [M][F/2] NVFP4 codes of bf16(SiLU(gate) * up)
-    uint8_t *sf;             // their block scales in the MMA's layout
-    float s;                 // static input scale of the layer that reads them
-    int F;                   // features (N = 2F)
-};
-
 // MMA_ONLY (measurement): the same roles and barriers, but no operand or scale loads (the barriers are completed by
 // hand), no scale copies into TMEM and no stores: what is left is the MMA issue sequence on whatever shared memory
 // and TMEM hold, i.e. the tensor-core rate this kernel could reach if nothing else cost time.
@@ -599,10 +591,10 @@ static cudaError_t launch_pair_cfg(const GemmArgs &a, EncodeTiledFn enc, cudaStr
     if (!make_sf_tmap(enc, &tmap_sfa, a.a_sf, ((a.M + 127) / 128) * katoms)) return cudaErrorInvalidValue;
     if (!make_sf_tmap(enc, &tmap_sfw, a.w_sf, ((a.N + 255) / 256) * 2 * katoms)) return cudaErrorInvalidValue;
     // the gated epilogue stores with plain instructions: its output map is never used, any valid map will do
-    const bool gated = a.gated_codes != nullptr;
+    const bool gated = a.gated.codes != nullptr;
     if (gated) tmap_y = tmap_a;
     else if (!make_y_tmap(enc, &tmap_y, a.Y, a.M, a.N, a.ldy)) return cudaErrorInvalidValue;
-    GatedOut go = {a.gated_codes, a.gated_sf, a.gated_scale, (int)(a.N / 2)};
+    
     const int tiles = (int)(((a.M + 2 * BM - 1) / (2 * BM)) * ((a.N + BN - 1) / BN));
     int pairs = sms / 2 * C::kMinCtas;
     if (tiles < pairs) pairs = tiles;
@@ -623,14 +615,14 @@ static cudaError_t launch_pair_cfg(const GemmArgs &a, EncodeTiledFn enc, cudaStr
     if (gated)
         return cudaLaunchKernelEx(&cfg, gemm_nvfp4_pair_kernel<false, 1, C>, tmap_a, tmap_w, tmap_sfa, tmap_sfw, tmap_y, a.hdr,
                                   a.act_scale, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M,
-                                  (int)a.N, (int)a.K, a.status, group_m, go);
+                                  (int)a.N, (int)a.K, a.status, group_m, a.gated);
     if (a.mma_only)
         return cudaLaunchKernelEx(&cfg, gemm_nvfp4_pair_kernel<true, 0, C>, tmap_a, tmap_w, tmap_sfa, tmap_sfw, tmap_y, a.hdr,
                                   a.act_scale, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M,
-                                  (int)a.N, (int)a.K, a.status, group_m, go);
+                                  (int)a.N, (int)a.K, a.status, group_m, a.gated);
     return cudaLaunchKernelEx(&cfg, gemm_nvfp4_pair_kernel<false, 0, C>, tmap_a, tmap_w, tmap_sfa, tmap_sfw, tmap_y, a.hdr,
                               a.act_scale, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.M, (int)a.N,
-                              (int)a.K, a.status, group_m, go);
+                              (int)a.K, a.status, group_m, a.gated);
 }
 
 }  // namespace

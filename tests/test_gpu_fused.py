@@ -212,6 +212,40 @@ def test_gate_up_gemm_with_gated_epilogue(dq, oracle, M, H, F):
     assert np.linalg.norm(Yg - Yd) <= 2.5e-3 * np.linalg.norm(Yd)          # the bf16 rounding of Y alone is 1.7e-3
 
 
+def _wide_range(g, rows, K, std):
+    """Blocks of 16 whose magnitudes differ by up to 2^9: sums over K that fp32 does not hold exactly, so that their order shows."""
+    x = torch.randn(rows, K, generator=g, device=DEV) * std
+    e = torch.randint(-9, 1, (rows, K // 16), generator=g, device=DEV)
+    return (x * torch.exp2(e.float()).repeat_interleave(16, 1)).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("M,H,F", [(300, 17408, 2560), (512, 8192, 256), (1000, 17408, 2560), (300, 4096, 128), (129, 5120, 512),
+                                   (257, 2048, 128), (129, 4096, 512), (129, 8192, 896), (129, 8192, 1280), (129, 8192, 1408),
+                                   (129, 8192, 1664), (200, 8192, 1920), (257, 8192, 1664), (2048, 5120, 2560)])
+def test_gated_epilogue_adds_up_as_the_plain_gemm_does(dq, M, H, F):
+    """The same bits as the two calls also where the GEMM shares a tile's k-steps out over a cluster or splits its columns over two
+    launches, on operands whose sums depend on the order they are taken in."""
+    g = torch.Generator(device=DEV).manual_seed(M + H)
+    w_gu = dq.pack_weights(_wide_range(g, 2 * F, H, 0.02), formats=dq.FMT_NVFP4)
+    w_d = dq.pack_weights((torch.randn(128, F, generator=g, device=DEV) * 0.02).to(torch.bfloat16), formats=dq.FMT_NVFP4)
+    A = _wide_range(g, M, H, 1.0)
+    sa = float(A.abs().max()) / 2688.0
+    ws = dq.alloc_workspace(dq.prefill_workspace_bytes(w_gu, M), DEV)
+    out, want = (dq.alloc_workspace(dq.prefill_workspace_bytes(w_d, M), DEV) for _ in range(2))
+    dq.prefill_quantize(w_gu, A, sa, ws)
+    Y = torch.empty(M, 2 * F, dtype=torch.bfloat16, device=DEV)
+    dq.prefill_gemm(w_gu, M, sa, Y, ws)
+    GU = torch.empty_like(Y)
+    GU[:, dq.gate_up_row_order(F).to(DEV)] = Y
+    s_out = float((torch.nn.functional.silu(GU[:, :F].float()) * GU[:, F:].float()).abs().max()) / 2688.0
+    out.fill_(0xA5)
+    want.fill_(0xA5)
+    dq.prefill_silu_mul_quantize(w_d, GU, s_out, want)
+    dq.prefill_gemm_silu_mul_quantize(w_gu, M, sa, ws, w_d, s_out, out)
+    _status_ok(dq)
+    assert torch.equal(out, want)
+
+
 def test_gate_up_gemm_with_gated_epilogue_arguments(dq):
     F, H, M = 256, 256, 64
     w_gu = dq.pack_weights(dq_inputs.gaussian_bf16(2 * F, H, 0.05, 440).to(DEV), formats=dq.FMT_NVFP4)
