@@ -113,7 +113,8 @@ int dq_prefill_workspace_bytes(const dq_weights *w, int64_t M, size_t *bytes_hos
  * where A^ is the NVFP4 round-to-nearest of A with the static per-tensor input
  * scale `act_global_scale` (App. A.3 "NVFP4": s_a in  a^ = s_a * d_b * e2m1) and
  * W^ the handle's NVFP4 weights; block-scaled FP4 tensor-core GEMM, fp32
- * accumulation.
+ * accumulation.  Repeated calls give the same bits; the order of the sum over k depends on M, N and K, so a row
+ * need not have the same bits in calls of different M.
  * A handle packed with DQ_FMT_LUT3 alone stores one 3.5-bit matrix for both phases
  * (Sec. 2.3 "format-disaggregated LUT3"; the paper describes this on-the-fly cast but
  * does not build it): every prefill call first casts the LUT3 codes to NVFP4 into the
@@ -252,8 +253,8 @@ int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, in
 
 /*
  * dq_prefill_linear on host memory: A_host (M x K bf16, row stride lda) is copied to the device, the
- * prefill linear runs, Y_host (M x N bf16, row stride ldy) receives the result.  M is cut into row
- * chunks; the copy in of the next chunk and the copy out of the previous one overlap the kernels of the
+ * prefill linear runs, Y_host (M x N bf16, row stride ldy) receives the result, bit for bit that of
+ * dq_prefill_linear on the same M rows.  M is cut into row chunks; the copy in of the next chunk and the copy out of the previous one overlap the kernels of the
  * current one on two internal streams per device (created at the first call on that device, which
  * therefore must not happen during a stream capture; these calls are not capturable at all).
  * A_host and Y_host should be pinned (cudaHostAlloc / cudaHostRegister), else the copies serialise.

@@ -483,7 +483,7 @@ int dq_prefill_silu_mul_quantize(const dq_weights *w, const void *GU_dev, int64_
 }
 
 static int prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, void *Y_dev, int64_t ldy,
-                        const void *workspace_dev, size_t workspace_bytes, void *stream, bool mma_only)
+                        const void *workspace_dev, size_t workspace_bytes, void *stream, bool mma_only, int64_t plan_rows = 0)
 {
     if (!Y_dev) return DQ_ERR_INVALID_ARG;
     int st = prefill_checks(w, M, act_global_scale, workspace_dev, workspace_bytes);
@@ -507,6 +507,7 @@ static int prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, 
     g.Y = Y_dev;
     g.ldy = ldy;
     g.M = M;
+    g.plan_rows = plan_rows;
     g.N = w->N;
     g.K = w->K;
     g.status = sw;
@@ -582,6 +583,14 @@ int dq_bench_stream_read(const void *src_dev, size_t bytes, void *out_dev, void 
 int dq_prefill_linear(const dq_weights *w, const void *A_dev, int64_t M, int64_t lda, float act_global_scale,
                       void *Y_dev, int64_t ldy, void *workspace_dev, size_t workspace_bytes, void *stream)
 {
+    return dq::prefill_linear_rows(w, A_dev, M, lda, act_global_scale, Y_dev, ldy, workspace_dev, workspace_bytes, M, stream);
+}
+
+}  // extern "C"
+
+int dq::prefill_linear_rows(const dq_weights *w, const void *A_dev, int64_t M, int64_t lda, float act_global_scale, void *Y_dev,
+                            int64_t ldy, void *workspace_dev, size_t workspace_bytes, int64_t plan_rows, void *stream)
+{
     if (!A_dev || !Y_dev) return DQ_ERR_INVALID_ARG;
     int st = prefill_checks(w, M, act_global_scale, workspace_dev, workspace_bytes);
     if (st != DQ_OK) return st;
@@ -589,8 +598,10 @@ int dq_prefill_linear(const dq_weights *w, const void *A_dev, int64_t M, int64_t
     if (!aligned(A_dev, 16) || !aligned(Y_dev, 16)) return DQ_ERR_ALIGN;
     st = dq_prefill_quantize(w, A_dev, M, lda, act_global_scale, workspace_dev, workspace_bytes, stream);
     if (st != DQ_OK) return st;
-    return dq_prefill_gemm(w, M, act_global_scale, Y_dev, ldy, workspace_dev, workspace_bytes, stream);
+    return prefill_gemm(w, M, act_global_scale, Y_dev, ldy, workspace_dev, workspace_bytes, stream, false, plan_rows);
 }
+
+extern "C" {
 
 static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
                         void *stream, int variant, int csize = 0)

@@ -168,6 +168,9 @@ struct DeviceInfo { int device; int arch; int sms; StatusWord *status; };
 const DeviceInfo *device_info();
 
 bool handle_on_current_device(const dq_weights *w);      // defined beside the handle (dq_api.cu)
+// dq_prefill_linear on M rows of a call of plan_rows: the bits that call would give them
+int prefill_linear_rows(const dq_weights *w, const void *A_dev, int64_t M, int64_t lda, float act_global_scale, void *Y_dev, int64_t ldy,
+                        void *workspace_dev, size_t workspace_bytes, int64_t plan_rows, void *stream);
 
 // ---- launchers (each enqueues on `stream`, returns a cudaError_t) ----
 cudaError_t launch_pack_header(PackedHeader *hdr, const uint16_t *codebook_f16_host, cudaStream_t stream);
@@ -222,6 +225,7 @@ struct GemmArgs {
     float act_scale;
     void *Y; int64_t ldy;
     int64_t M, N, K;
+    int64_t plan_rows = 0;   // kernel and K split of a GEMM of that many rows, of which these M are a part; 0 = M
     StatusWord *status;
     bool w_const = false;    // w_codes / w_sf belong to the handle (not cast into the workspace for this call)
     int clocks = 0;          // 1: the launch leaves its cycles and nanoseconds in the status word, 2: adds them (the pair kernel always leaves its)

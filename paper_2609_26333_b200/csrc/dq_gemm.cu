@@ -585,12 +585,17 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
     GemmArgs a = args;
-    a.clocks = a.M > BM ? 1 : 0;
+    if (a.plan_rows == 0) a.plan_rows = a.M;
+    a.clocks = a.plan_rows > BM ? 1 : 0;
     Plan p = {a.N, 256, {1, 0.0}};
     // The measurement mode exists in the pair kernel only, and up to 128 tokens the gated epilogue too.  Above, a gated call adds its
     // products up as the plain call does: clusters where that takes clusters.  A lone CTA's sums are those of the pair kernel bit
     // for bit, k-step after k-step, so there the gated call keeps to the pair kernel, whose epilogue overlaps.
-    if (!a.mma_only && !(a.gated.codes && a.M <= BM)) p = choose_plan(a, di->device, di->sms);
+    if (!a.mma_only && !(a.gated.codes && a.plan_rows <= BM)) {
+        GemmArgs whole = a;
+        whole.M = a.plan_rows;
+        p = choose_plan(whole, di->device, di->sms);
+    }
     if (a.gated.codes && p.sp.csize == 1) p.head = a.N;
     if (p.head > 0) {
         GemmArgs front = a;

@@ -108,8 +108,9 @@ int dq_prefill_linear_host(const dq_weights *w, const void *A_host, int64_t M, i
     for (int c = 0; c < chunks; ++c) {
         const int64_t r0 = c * rows, mc = (M - r0 < rows) ? (M - r0) : rows;
         if (cudaStreamWaitEvent(s, p->a_ready[c], 0) != cudaSuccess) return DQ_ERR_CUDA;
-        st = dq_prefill_linear(w, A_dev + (size_t)r0 * K * 2, mc, K, act_global_scale, Y_dev + (size_t)r0 * N * 2, N, ws,
-                               ws_bytes, s);
+        // as rows of a call on all M: how the GEMM takes its sums over K depends on the number of rows
+        st = dq::prefill_linear_rows(w, A_dev + (size_t)r0 * K * 2, mc, K, act_global_scale, Y_dev + (size_t)r0 * N * 2, N, ws, ws_bytes,
+                                     M, s);
         if (st != DQ_OK) return st;
         if (cudaEventRecord(p->y_ready[c], s) != cudaSuccess) return DQ_ERR_CUDA;
         if (cudaStreamWaitEvent(p->s_out, p->y_ready[c], 0) != cudaSuccess) return DQ_ERR_CUDA;

@@ -665,6 +665,26 @@ def test_host_buffer_entry_points_match_device_calls(dq, oracle):
     _status_ok(dq)
 
 
+@pytest.mark.parametrize("M,N,K", [(2500, 5120, 17408), (1100, 5120, 17408), (1100, 528, 8192), (1025, 1024, 4096)])
+def test_host_chunks_add_up_as_the_whole_call_does(dq, M, N, K):
+    """Chunks of 1024 rows on their own would take another kernel and another split of K than all M rows: the same bits all the same, on
+    operands whose sums depend on the order they are taken in."""
+    g = torch.Generator(device=DEV).manual_seed(M + N)
+
+    def wide(rows, std):
+        e = torch.randint(-9, 1, (rows, K // 16), generator=g, device=DEV).float()
+        return (torch.randn(rows, K, generator=g, device=DEV) * std * torch.exp2(e).repeat_interleave(16, 1)).to(torch.bfloat16)
+
+    w = dq.pack_weights(wide(N, 0.02), formats=dq.FMT_NVFP4)
+    A = wide(M, 1.0)
+    sa = float(A.abs().max()) / 2688.0
+    A_host, Y_host = A.cpu().pin_memory(), torch.empty(M, N, dtype=torch.bfloat16).pin_memory()
+    dq.prefill_linear_host(w, A_host, sa, Y_host, dq.alloc_workspace(dq.prefill_host_staging_bytes(w, M), DEV))
+    want = dq.prefill_linear(w, A, sa)
+    _status_ok(dq)
+    assert torch.equal(Y_host, want.cpu())
+
+
 # ---- the tcgen05 decode kernel (test-hook variant 3; batch 1): same arithmetic, other machinery ----
 
 @pytest.mark.parametrize("N,K,seed", DECODE_SHAPES + [(400, 5120, 64), (3072, 12288, 65)])
