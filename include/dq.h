@@ -374,7 +374,8 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           a device-side wait budget of `wait_cycles` SM clocks (0 = the default of about two
  *           seconds).  variant 1 additionally leaves out one bulk copy (the first atom of warp 0 of
  *           CTA 0), so that the wait for it runs out after `wait_cycles`: the kernel returns normally,
- *           writes partial output and records DQ_ERR_TIMEOUT for dq_get_status.  variant 2 is the
+ *           writes partial output and records DQ_ERR_TIMEOUT for dq_get_status.  It runs the kernel of 8-row tiles
+ *           or, where dq_decode_linear takes it, the batch kernel; the other two keep every copy.  variant 2 is the
  *           same kernel as variant 0.  variant 3 (B = 1 only; DQ_ERR_INVALID_ARG where the row is
  *           too long for its shared-memory layout, about K > 12288) runs the tcgen05 kernel instead:
  *           levels stored to tensor memory, one tcgen05.mma per 16-weight block, the same exact

@@ -1387,14 +1387,15 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     const bool choose = a.kernel == 0 && a.force_P == 0;
     const int want_cols = B;                    // the split decides how many of them one pass takes
     Split sp = choose_split(a.bits, N, K, sms, want_cols);
+    const bool all = !a.drop_first_copy;        // the 16-row and the slice-by-slice kernel have no way to leave a copy out (test hook)
     if (choose && B >= 4 && B <= 8) {
-        if (B == 4 && few_rows(N, K, sms)) return launch_rows16(a, sms, stream);
+        if (B == 4 && all && few_rows(N, K, sms)) return launch_rows16(a, sms, stream);
         if (B > 4 && a.split_exact && one_half_slice(N, K)) return launch_decode_tc(a, stream);
-        if (B > 4 && rows16_is_faster(a.bits, N, K, B, sms, sp)) return launch_rows16(a, sms, stream);
+        if (B > 4 && all && rows16_is_faster(a.bits, N, K, B, sms, sp)) return launch_rows16(a, sms, stream);
         if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);
     }
-    if (choose && B > 8 && a.split_exact) return tc_is_faster(N, K, B, sms) ? launch_decode_tc(a, stream) : launch_wide(a, sms, stream);
-    if (a.kernel == 3 || (choose && B > 8 && wide_rows(N, K, B))) return launch_wide(a, sms, stream);
+    if (choose && B > 8 && a.split_exact && tc_is_faster(N, K, B, sms)) return launch_decode_tc(a, stream);
+    if (a.kernel == 3 || (choose && B > 8 && all && (a.split_exact || wide_rows(N, K, B)))) return launch_wide(a, sms, stream);
     LutPlan L;
     if (a.force_P > 0 && a.force_G > 0) {
         if (a.force_P * a.force_G > 32 || a.force_G > kMaxGroups) return cudaErrorInvalidValue;

@@ -272,6 +272,20 @@ def test_decode_batch_wait_runs_out(dq):
     _status_ok(dq)
 
 
+@pytest.mark.parametrize("N,K,B", [(1024, 1024, 4), (1024, 1024, 6), (1024, 1024, 12), (8192, 2048, 12), (2048, 2048, 24), (4096, 512, 40)])
+def test_decode_left_out_copy_is_missed_at_every_batch(dq, N, K, B):
+    """The hook that leaves a copy out does so whichever kernel the shape would take."""
+    w = dq.pack_weights(dq_inputs.gaussian_bf16(N, K, 0.02, 1).to(DEV), formats=dq.FMT_LUT3)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 2).to(DEV)
+    good = dq.decode_linear(w, X)
+    dq.test_decode_linear(w, dq.FMT_LUT3, X, variant=1, wait_cycles=2_000_000)
+    torch.cuda.synchronize()
+    st, _ = dq.get_status()
+    assert dq.status_string(st) == "device-side wait ran out"
+    assert torch.equal(dq.decode_linear(w, X), good)
+    _status_ok(dq)
+
+
 @pytest.mark.parametrize("fmt", ["lut3", "lut2"])
 @pytest.mark.parametrize("N,K", SHAPES + [(4112, 1536)])
 @pytest.mark.parametrize("B", [1, 5, 8])
