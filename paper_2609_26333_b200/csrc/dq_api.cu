@@ -642,6 +642,7 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
         if (ce == cudaSuccess) ce = dq::launch_pack_done(s);
         if (ce == cudaSuccess) ce = dq::launch_gemv_nvfp4(g, s);
     }
+    if (variant != 0 && ce == cudaErrorInvalidValue) return DQ_ERR_INVALID_ARG;      // the test hook's kernel does not take this call
     if (ce != cudaSuccess) return DQ_ERR_CUDA;
     return DQ_OK;
 }
@@ -706,8 +707,11 @@ int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int
                           int ring_stages, long long wait_cycles, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev,
                           int64_t ldy, void *stream)
 {
-    if (format == DQ_FMT_NVFP4 || format == DQ_FMT_NVFP4_FROM_LUT3)
+    if (format == DQ_FMT_NVFP4 || format == DQ_FMT_NVFP4_FROM_LUT3) {
+        if (variant != 0 && variant != 1 && variant != 5 && variant != 6) return DQ_ERR_INVALID_ARG;
+        if (warps_per_group < 0) return DQ_ERR_INVALID_ARG;
         return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 ? warps_per_group : 0);
+    }
     if (warps_per_group < 0 || groups_per_cta < 0 || ring_stages < 0 || ring_stages > 8 || wait_cycles < 0)
         return DQ_ERR_INVALID_ARG;
     if (variant < 0 || variant > 6) return DQ_ERR_INVALID_ARG;

@@ -345,3 +345,18 @@ def test_decode_columns_of_very_different_magnitude(dq, oracle, fmt, N, K, B):
         _status_ok(dq)
         for b in range(B):
             check_outputs(Y[b:b + 1], Yr[b:b + 1], S[b:b + 1], f"{fmt} {B}x{N}x{K} column {b}")
+
+
+def test_decode_nvfp4_hook_refuses_what_it_does_not_know(dq):
+    """Variants that do not exist for this encoding and cluster sizes that do not fit are argument errors, not another kernel's run."""
+    N, K = 272, 1024
+    w = dq.pack_weights(dq_inputs.gaussian_bf16(N, K, 0.02, 3).to(DEV), formats=dq.FMT_NVFP4)
+    X = dq_inputs.gaussian_bf16(2, K, 1.0, 4).to(DEV)
+    for kw in ({"variant": -1}, {"variant": 2}, {"variant": 3}, {"variant": 4}, {"variant": 7}, {"variant": 99},
+               {"variant": TC, "warps_per_group": 3}, {"variant": TC, "warps_per_group": 9}, {"variant": TC, "warps_per_group": -1}):
+        with pytest.raises(dq.DQError) as e:
+            dq.test_decode_linear(w, dq.FMT_NVFP4, X, **kw)
+        assert e.value.code == 1, kw
+    for variant in (0, 1, TC, 6):
+        dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=variant)
+    _status_ok(dq)
