@@ -1204,15 +1204,18 @@ cudaError_t launch_rows16_bits(const GemvArgs &a, const LutPlan &L, int grid, cu
                               (int)a.B, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.N, (int)a.K, L, a.status);
 }
 
+cudaError_t launch_rows16(const GemvArgs &a, LutPlan L, int grid, cudaStream_t stream)
+{
+    L.wait_cycles = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitBudgetCycles;
+    return a.bits == 3 ? launch_rows16_bits<3>(a, L, grid, stream) : launch_rows16_bits<2>(a, L, grid, stream);
+}
 // B <= 8 columns in one pass; cudaErrorInvalidValue where the row is too long for it
 cudaError_t launch_rows16(const GemvArgs &a, int sms, cudaStream_t stream)
 {
     LutPlan L = {};
     double cost;
     const int grid = a.B <= 8 ? choose_rows16(a.bits, a.N, a.K, sms, (int)a.B, L, cost) : 0;
-    if (grid == 0) return cudaErrorInvalidValue;
-    L.wait_cycles = a.wait_cycles > 0 ? a.wait_cycles : tc::kWaitBudgetCycles;
-    return a.bits == 3 ? launch_rows16_bits<3>(a, L, grid, stream) : launch_rows16_bits<2>(a, L, grid, stream);
+    return grid == 0 ? cudaErrorInvalidValue : launch_rows16(a, L, grid, stream);
 }
 
 }  // namespace
@@ -1323,14 +1326,15 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
 // than the model's stretch, and long rows' activations take their time to convert.  Over 520 points the pick is never the slower one by more
 // than 2 % and on average 0.3 % off the better (1024x4096 batch 5: 7.9 / 6.6; 4096x5120 batch 8: 11.6 / 11.4; 8192x12288 batch 5:
 // 38 / 25.8; stays with 8 rows: 5120x3072 batch 5 8.3 / 9.2, 1024x8192 batch 6 10.1 / 11.4).  Below 128 rows neither fills the chip.
-static bool rows16_is_faster(int bits, int64_t N, int64_t K, int B, int sms, const Split &narrow)
+// The grid of the 16-row launch and its plan in L, 0 for 8-row tiles.
+static int rows16_if_faster(int bits, int64_t N, int64_t K, int B, int sms, const Split &narrow, LutPlan &L)
 {
-    LutPlan L = {};
     double cost;
-    if (N < 128 || choose_rows16(bits, N, K, sms, B, L, cost) == 0) return false;
+    const int grid = N < 128 ? 0 : choose_rows16(bits, N, K, sms, B, L, cost);
+    if (grid == 0) return 0;
     const double warps = (double)(L.P * L.G);
     if (warps < 12.0) cost *= std::sqrt(std::sqrt(12.0 / warps));
-    return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost;
+    return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost ? grid : 0;
 }
 
 // Four columns: 16-row tiles only where every CTA gets one of them at most and the rows are short (512x1024: 5.7 / 5.0; 1024x2048: 6.1 / 5.4;
@@ -1366,7 +1370,7 @@ static bool tc_is_faster(int64_t N, int64_t K, int B, int sms)
     return tc < wide;
 }
 
-// up to eight columns per pass
+// Which kernel a call takes; the kernel of 8-row tiles takes up to eight columns per pass.
 cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
 {
     const int K = (int)a.K, N = (int)a.N, B = (int)a.B;
@@ -1376,7 +1380,7 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     if (!di) return cudaErrorInvalidDevice;
     const int sms = di->sms;
     // The tcgen05 kernel runs only where the caller asks for it (test hook): measured, it is the slower of the two
-    // (23.7 against 16.3 us on 17408x5120; its header says why).
+    // (20.9 against 15.3 us on 17408x5120; its header says why).
     if (a.kernel == 2) {
         const int wgs = gemv_lut_tc_warpgroups(a.bits, N, K, B, sms, true);
         if (wgs == 0) return cudaErrorInvalidValue;
@@ -1385,17 +1389,19 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
     if (a.kernel == 4) return a.split_exact ? launch_decode_tc(a, stream) : cudaErrorInvalidValue;
     if (a.kernel == 5) return launch_rows16(a, sms, stream);
     const bool choose = a.kernel == 0 && a.force_P == 0;
-    const int want_cols = B;                    // the split decides how many of them one pass takes
-    Split sp = choose_split(a.bits, N, K, sms, want_cols);
     const bool all = !a.drop_first_copy;        // the 16-row and the slice-by-slice kernel have no way to leave a copy out (test hook)
-    if (choose && B >= 4 && B <= 8) {
-        if (B == 4 && all && few_rows(N, K, sms)) return launch_rows16(a, sms, stream);
-        if (B > 4 && a.split_exact && one_half_slice(N, K)) return launch_decode_tc(a, stream);
-        if (B > 4 && all && rows16_is_faster(a.bits, N, K, B, sms, sp)) return launch_rows16(a, sms, stream);
-        if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);
-    }
+    if (choose && B == 4 && all && few_rows(N, K, sms)) return launch_rows16(a, sms, stream);
+    if (choose && B > 4 && B <= 8 && a.split_exact && one_half_slice(N, K)) return launch_decode_tc(a, stream);
     if (choose && B > 8 && a.split_exact && tc_is_faster(N, K, B, sms)) return launch_decode_tc(a, stream);
     if (a.kernel == 3 || (choose && B > 8 && all && (a.split_exact || wide_rows(N, K, B)))) return launch_wide(a, sms, stream);
+    const int want_cols = B;                    // the split decides how many of them one pass takes
+    Split sp = choose_split(a.bits, N, K, sms, want_cols);
+    if (choose && B >= 4 && B <= 8) {
+        LutPlan L16 = {};
+        const int grid16 = B > 4 && all ? rows16_if_faster(a.bits, N, K, B, sms, sp, L16) : 0;
+        if (grid16 > 0) return launch_rows16(a, L16, grid16, stream);
+        if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);
+    }
     LutPlan L;
     if (a.force_P > 0 && a.force_G > 0) {
         if (a.force_P * a.force_G > 32 || a.force_G > kMaxGroups) return cudaErrorInvalidValue;
