@@ -812,58 +812,84 @@ bool make_codes_tmap(CUtensorMap *tm, const void *ptr, int64_t N, int64_t K)
 constexpr int kMaxCluster = 8;
 
 template <int FMT, int NC>
-cudaError_t launch_one(const CUtensorMap &tmap, TcDecodeArgs P, int force_csize, cudaStream_t stream)
+cudaError_t set_attributes(int dev)
 {
-    using C = Cfg<FMT, NC>;
+    static std::atomic<bool> done[kMaxDevices];
+    if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
     auto kernel = decode_tc_kernel<FMT, NC>;
-    static std::atomic<bool> attr_set[kMaxDevices];
-    static std::atomic<int> max_clusters[kMaxDevices][kMaxCluster + 1];          // + 1; 0 = not asked yet
-    const DeviceInfo *di = device_info();
-    if (!di) return cudaErrorInvalidDevice;
-    const int dev = di->device, sms = di->sms;
-    if (!attr_set[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::kSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-        if (e != cudaSuccess) return e;
-        attr_set[dev].store(true, std::memory_order_release);
-    }
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<FMT, NC>::kSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+    if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
+    return e;
+}
+
+template <int FMT, int NC>
+cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int csize, cudaStream_t stream)
+{
     cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.dynamicSmemBytes = Cfg<FMT, NC>::kSmem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    attr[1].val.clusterDim.x = (unsigned)csize;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
+    cfg.numAttrs = csize > 1 ? 2 : 1;
+    return cfg;
+}
 
-    // CTAs per tile: the fewest slices on the busiest CTA, a cluster's exchange counted as half a slice.  Clusters take one
-    // tile each and must all be resident; how many fit is asked once per size and device.
-    const int tiles = (P.N + 255) / 256, ns = (P.K + kSlice - 1) / kSlice;
-    int best_c = 1;
-    double best = (double)((tiles + sms - 1) / sms) * ns;
-    for (int c = 2; c <= kMaxCluster && c <= ns && tiles * c <= sms; ++c) {
-        int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
-        if (fit == 0) {
-            cfg.gridDim = dim3((unsigned)(c * (sms / c)));
-            attr[1].val.clusterDim.x = (unsigned)c;
-            cfg.numAttrs = 2;
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-            fit = n + 1;
-            max_clusters[dev][c].store(fit, std::memory_order_relaxed);
+// How many clusters of c CTAs a device holds at once: they do not straddle its groups of SMs, so some SMs stay out, on a B200 28 of
+// them at eight CTAs.  Every instantiation has an SM to itself, so one answers for all; asked once per size and device, and
+// again where the runtime did not answer.
+int clusters_that_fit(int dev, int c, int sms)
+{
+    static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];                 // + 1; 0 = not known
+    int fit = known[dev][c].load(std::memory_order_relaxed);
+    if (fit == 0) {
+        cudaLaunchAttribute attr[2];
+        const cudaLaunchConfig_t cfg = launch_config<0, 16>(attr, c * (sms / c), c, nullptr);
+        int n = 0;
+        if (set_attributes<0, 16>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, decode_tc_kernel<0, 16>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
         }
-        if (tiles > fit - 1) continue;
-        const double cost = (double)((ns + c - 1) / c) + 0.5;
-        if (force_csize > 0 ? c == force_csize : cost < best) { best = cost; best_c = c; }
+        fit = n + 1;
+        known[dev][c].store(fit, std::memory_order_relaxed);
     }
-    if (force_csize > 0 && best_c != force_csize) return cudaErrorInvalidValue;
-    P.csize = best_c;
-    attr[1].val.clusterDim.x = (unsigned)best_c;
-    cfg.numAttrs = best_c > 1 ? 2 : 1;
-    cfg.gridDim = dim3((unsigned)(best_c > 1 ? tiles * best_c : (tiles < sms ? tiles : sms)));
-    return cudaLaunchKernelEx(&cfg, kernel, tmap, P);
+    return fit - 1;
+}
+
+// CTAs per tile: the fewest slices of 512 weights on the busiest CTA, a cluster's exchange counted as half a slice.  Clusters take one
+// tile each and must all be resident.
+struct TileSplit { int csize; double slices; };
+TileSplit split_tiles(int64_t N, int64_t K, int dev, int sms, int force_csize)
+{
+    const int64_t tiles = (N + 255) / 256, ns = (K + kSlice - 1) / kSlice;
+    TileSplit best = {1, (double)((tiles + sms - 1) / sms) * (double)ns};
+    for (int c = 2; c <= kMaxCluster && c <= ns && tiles * c <= sms; ++c) {
+        if (force_csize > 0 && c != force_csize) continue;
+        const double cost = (double)((ns + c - 1) / c) + 0.5;
+        if ((force_csize > 0 || cost < best.slices) && tiles <= clusters_that_fit(dev, c, sms)) best = {c, cost};
+    }
+    return best;
+}
+
+template <int FMT, int NC>
+cudaError_t launch_one(const CUtensorMap &tmap, TcDecodeArgs P, int force_csize, cudaStream_t stream)
+{
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    const cudaError_t e = set_attributes<FMT, NC>(di->device);
+    if (e != cudaSuccess) return e;
+    const int tiles = (P.N + 255) / 256;
+    P.csize = split_tiles(P.N, P.K, di->device, di->sms, force_csize).csize;
+    if (force_csize > 0 && P.csize != force_csize) return cudaErrorInvalidValue;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = launch_config<FMT, NC>(attr, P.csize > 1 ? tiles * P.csize : (tiles < di->sms ? tiles : di->sms), P.csize, stream);
+    return cudaLaunchKernelEx(&cfg, decode_tc_kernel<FMT, NC>, tmap, P);
 }
 
 template <int FMT>
@@ -877,17 +903,11 @@ cudaError_t launch_cols(const CUtensorMap &tmap, const TcDecodeArgs &P, int forc
 
 }  // namespace
 
-// 512-weight slices the busiest CTA of a launch works through, before the exchange of a cluster (the launcher's own choice,
-// by what fits a B200 at once: clusters do not straddle its groups of SMs, so the last few SMs stay out, more of them at eight CTAs)
-double decode_tc_slices(int64_t N, int64_t K, int sms)
+// 512-weight slices the busiest CTA of a launch works through, an exchange included
+double decode_tc_slices(int64_t N, int64_t K)
 {
-    const int tiles = (int)((N + 255) / 256), ns = (int)((K + kSlice - 1) / kSlice);
-    double best = (double)((tiles + sms - 1) / sms) * ns;
-    for (int c = 2; c <= kMaxCluster && c <= ns && tiles * c <= sms - (c == 8 ? 28 : 8); ++c) {
-        const double cost = (double)((ns + c - 1) / c) + 0.5;
-        if (cost < best) best = cost;
-    }
-    return best;
+    const DeviceInfo *di = device_info();
+    return di ? split_tiles(N, K, di->device, di->sms, 0).slices : 1e300;
 }
 
 cudaError_t launch_decode_tc(const GemvArgs &a, cudaStream_t stream)

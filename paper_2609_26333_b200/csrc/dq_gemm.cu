@@ -483,7 +483,7 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
             int n = 0;
             if (set_attributes<BN, 1, false, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false, false>, &cfg) != cudaSuccess) {
                 cudaGetLastError();
-                n = 0;
+                continue;                                                        // asked again the next time
             }
             fit = n + 1;
             max_clusters[dev][c].store(fit, std::memory_order_relaxed);

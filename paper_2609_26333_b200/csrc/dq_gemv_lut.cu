@@ -1364,7 +1364,7 @@ static bool tc_is_faster(int64_t N, int64_t K, int B, int sms)
     const int64_t per_round = 8 * (int64_t)sms;
     const double rounds = (double)((N / 16 + per_round - 1) / per_round) * (double)lut_slices(K);
     const double wide = rounds * (B <= 16 ? 3.95 : B <= 24 ? 5.2 : 6.25) + 1.15;
-    const double slices = decode_tc_slices(N, K, sms);
+    const double slices = decode_tc_slices(N, K);
     const double tc = K <= 512 ? slices * 1.05 * (double)((K + 127) / 128) + (B > 16 ? 4.2 : 2.7)
                                : B > 16 ? slices * 5.72 + 1.8 : slices * 5.05 + 1.1;
     return tc < wide;

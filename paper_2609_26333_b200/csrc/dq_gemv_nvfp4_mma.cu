@@ -326,7 +326,7 @@ bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms)
     const int64_t cols = cols_max < 8 ? cols_max : 8;
     const double rounds = (double)((ntiles + G * sms - 1) / (G * sms)), passes = (double)((B + cols - 1) / cols);
     const double here = passes * (2.4 + 4.6 * rounds * (K < 1280 ? (double)K / 1280.0 : 1.0)) + 0.58 * (double)B * (0.8 + 0.2 * rounds);
-    const double there = 2.2 + 2.7 * decode_tc_slices(N, K, sms) * (K < 512 ? (double)K / 512.0 : 1.0);
+    const double there = 2.2 + 2.7 * decode_tc_slices(N, K) * (K < 512 ? (double)K / 512.0 : 1.0);
     return there < here;
 }
 
