@@ -399,6 +399,16 @@ int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int
                           int groups_per_cta, int ring_stages, long long wait_cycles, const void *X_dev,
                           int64_t B, int64_t ldx, void *Y_dev, int64_t ldy, void *stream);
 
+/*
+ * dq_prefill_gemm with the kernel forced, so that tests reach every kernel and split at sizes that dq_prefill_gemm would not choose
+ * them for.  kernel 1: CTA pairs on 256 x 256 tiles; 2 / 3: tiles of 128 rows and 128 / 256 columns; 4: CTA pairs for all
+ * blocks of 256 columns but the last (N > 256), tiles of 128 columns for that one in a launch of their own.  ctas_per_tile (0..8; kernels 2 to
+ * 4) CTAs share the k-steps of a tile, 0 and 1 = one.  DQ_ERR_INVALID_ARG where so many have no k-step each or do not fit the GPU at
+ * once.  Other arguments, results and status codes as dq_prefill_gemm.
+ */
+int dq_test_prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, int kernel, int ctas_per_tile, void *Y_dev,
+                         int64_t ldy, const void *workspace_dev, size_t workspace_bytes, void *stream);
+
 /* ---- measurement hooks (the paper has no counterpart; they give bench.py its two measured ceilings) ---- */
 
 /*

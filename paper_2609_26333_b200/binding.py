@@ -21,7 +21,7 @@ DT_FP32 = 1
 SYMBOLS = ("dq_version", "dq_status_string", "dq_packed_bytes", "dq_pack_weights", "dq_free_weights",
            "dq_prefill_workspace_bytes", "dq_prefill_linear", "dq_prefill_quantize", "dq_prefill_gemm",
            "dq_prefill_linear_static",
-           "dq_decode_linear", "dq_decode_linear_nvfp4", "dq_decode_linear_lut2", "dq_test_decode_linear",
+           "dq_decode_linear", "dq_decode_linear_nvfp4", "dq_decode_linear_lut2", "dq_test_decode_linear", "dq_test_prefill_gemm",
            "dq_bench_gemm_mma_only", "dq_bench_stream_read", "dq_bench_gemm_clocks",
            "dq_prefill_rmsnorm_quantize", "dq_prefill_silu_mul_quantize", "dq_prefill_gemm_silu_mul_quantize",
            "dq_rmsnorm_quantize_activations",
@@ -82,6 +82,8 @@ def lib() -> C.CDLL:
         L.dq_decode_linear_nvfp4.argtypes = [vp, vp, i64, i64, vp, i64, vp]
         L.dq_decode_linear_lut2.restype = C.c_int
         L.dq_decode_linear_lut2.argtypes = [vp, vp, i64, i64, vp, i64, vp]
+        L.dq_test_prefill_gemm.restype = C.c_int
+        L.dq_test_prefill_gemm.argtypes = [vp, i64, C.c_float, C.c_int, C.c_int, vp, i64, vp, C.c_size_t, vp]
         L.dq_test_decode_linear.restype = C.c_int
         L.dq_test_decode_linear.argtypes = [vp, C.c_uint, C.c_int, C.c_int, C.c_int, C.c_int, C.c_longlong, vp, i64, i64,
                                             vp, i64, vp]
@@ -417,6 +419,15 @@ def test_decode_linear(w: DQWeights, fmt: int, X: torch.Tensor, out: torch.Tenso
     return out
 
 
+def test_prefill_gemm(w: DQWeights, M: int, act_global_scale: float, out: torch.Tensor, workspace: torch.Tensor, kernel: int,
+                      ctas_per_tile: int = 0, stream=None) -> torch.Tensor:
+    """dq_test_prefill_gemm: stage 2 of the prefill linear with the kernel forced (test hook)."""
+    _check(lib().dq_test_prefill_gemm(w.handle, M, float(act_global_scale), kernel, ctas_per_tile, out.data_ptr(), out.stride(0),
+                                      workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)), "dq_test_prefill_gemm")
+    return out
+
+
+test_prefill_gemm.__test__ = False
 test_decode_linear.__test__ = False      # not a pytest test
 test_silu.__test__ = False
 

@@ -483,7 +483,8 @@ int dq_prefill_silu_mul_quantize(const dq_weights *w, const void *GU_dev, int64_
 }
 
 static int prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, void *Y_dev, int64_t ldy,
-                        const void *workspace_dev, size_t workspace_bytes, void *stream, bool mma_only, int64_t plan_rows = 0)
+                        const void *workspace_dev, size_t workspace_bytes, void *stream, bool mma_only, int64_t plan_rows = 0,
+                        int force_kernel = 0, int force_csize = 0)
 {
     if (!Y_dev) return DQ_ERR_INVALID_ARG;
     int st = prefill_checks(w, M, act_global_scale, workspace_dev, workspace_bytes);
@@ -512,14 +513,24 @@ static int prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, 
     g.K = w->K;
     g.status = sw;
     g.mma_only = mma_only;
-    if (dq::launch_gemm_nvfp4(g, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return DQ_ERR_CUDA;
-    return DQ_OK;
+    g.force_kernel = force_kernel;
+    g.force_csize = force_csize;
+    const cudaError_t e = dq::launch_gemm_nvfp4(g, reinterpret_cast<cudaStream_t>(stream));
+    if (force_kernel != 0 && e == cudaErrorInvalidValue) return DQ_ERR_INVALID_ARG;
+    return e == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
 }
 
 int dq_prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, void *Y_dev, int64_t ldy,
                     const void *workspace_dev, size_t workspace_bytes, void *stream)
 {
     return prefill_gemm(w, M, act_global_scale, Y_dev, ldy, workspace_dev, workspace_bytes, stream, false);
+}
+
+int dq_test_prefill_gemm(const dq_weights *w, int64_t M, float act_global_scale, int kernel, int ctas_per_tile, void *Y_dev,
+                         int64_t ldy, const void *workspace_dev, size_t workspace_bytes, void *stream)
+{
+    if (kernel < 1 || kernel > 4 || ctas_per_tile < 0 || ctas_per_tile > 8) return DQ_ERR_INVALID_ARG;
+    return prefill_gemm(w, M, act_global_scale, Y_dev, ldy, workspace_dev, workspace_bytes, stream, false, 0, kernel, ctas_per_tile);
 }
 
 int dq_prefill_gemm_silu_mul_quantize(const dq_weights *w_gate_up, int64_t M, float act_global_scale,

@@ -229,6 +229,7 @@ struct GemmArgs {
     StatusWord *status;
     bool w_const = false;    // w_codes / w_sf belong to the handle (not cast into the workspace for this call)
     int clocks = 0;          // 1: the launch leaves its cycles and nanoseconds in the status word, 2: adds them (the pair kernel always leaves its)
+    int force_kernel = 0, force_csize = 0;                 // test hook: 1 pair, 2 / 3 tiles of 128 x 128 / 256, 4 the last columns on tiles; CTAs per tile
     bool mma_only = false;   // measurement: MMA issue sequence only (pair kernel; no loads, scale copies or stores)
     // gated epilogue where gated.codes is not null: W is a fused gate/up matrix with interleaved rows, and instead of Y the kernel
     // writes NVFP4(bf16(SiLU(gate) * up))

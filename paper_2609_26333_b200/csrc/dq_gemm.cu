@@ -459,16 +459,37 @@ cudaError_t set_attributes(int dev)
     return e;
 }
 
+// Whether clusters of c CTAs may share the tiles of 128 x BN: each takes one tile and at least one k-step, and all must be resident.  How
+// many of a size fit is asked once per device, and again where the runtime did not answer.
+template <int BN>
+bool clusters_fit(const GemmArgs &a, int c, int dev, int sms)
+{
+    static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];                 // + 1; 0 = not known
+    const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
+    if (c > kMaxCluster || c > (a.K / 64 + kKbPerStage - 1) / kKbPerStage || tiles * c > sms) return false;
+    int fit = known[dev][c].load(std::memory_order_relaxed);
+    if (fit == 0) {
+        cudaLaunchAttribute attr[2];
+        const cudaLaunchConfig_t cfg = launch_config<BN, 1, false>(attr, c * (sms / c), c, nullptr);
+        int n = 0;
+        if (set_attributes<BN, 1, false, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false, false>, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        fit = n + 1;
+        known[dev][c].store(fit, std::memory_order_relaxed);
+    }
+    return tiles <= fit - 1;
+}
+
 // CTAs per tile of 128 x BN: bytes of weights (rows x k-steps) that the busiest CTA streams, the activation tile of a step counted
-// as 48 rows (it comes from L2) and a cluster's exchange as 600.  A cluster takes one tile, and all must be resident;
-// how many of a size fit is asked once per device.
+// as 48 rows (it comes from L2) and a cluster's exchange as 600.
 // Against the pair kernel, above one tile of rows, the output counts as well: a round takes no less than its epilogue and half its k-steps
 // (34816 columns, 16384 rows: 2.3 us a round at K = 128, 2.9 at 1024), the exchange of full row tiles up to 1500 more where few
 // k-steps hide it (512x1536, 793 rows: 9.6 us against 8.2 in the pair kernel; 5120x17408, 300 rows: 25.2 with it, 27.0 without), and the ramp is 600 shorter than the pair kernel's.
 template <int BN>
 Split choose_split(const GemmArgs &a, int dev, int sms)
 {
-    static std::atomic<int> max_clusters[kMaxDevices][kMaxCluster + 1];          // + 1; 0 = not asked yet
     const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
     const int num_ks = (int)((a.K / 64 + kKbPerStage - 1) / kKbPerStage);
     const double step = BN + 48.0;
@@ -476,19 +497,7 @@ Split choose_split(const GemmArgs &a, int dev, int sms)
     const bool many = a.M > BM;
     Split best = {1, many ? rounds * (stream > output ? stream : output) - 600.0 : rounds * stream};
     for (int c = 2; c <= kMaxCluster && c <= num_ks && tiles * c <= sms; ++c) {
-        int fit = max_clusters[dev][c].load(std::memory_order_relaxed);
-        if (fit == 0) {
-            cudaLaunchAttribute attr[2];
-            const cudaLaunchConfig_t cfg = launch_config<BN, 1, false>(attr, c * (sms / c), c, nullptr);
-            int n = 0;
-            if (set_attributes<BN, 1, false, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, gemm_nvfp4_kernel<BN, 1, false, false>, &cfg) != cudaSuccess) {
-                cudaGetLastError();
-                continue;                                                        // asked again the next time
-            }
-            fit = n + 1;
-            max_clusters[dev][c].store(fit, std::memory_order_relaxed);
-        }
-        if (tiles > fit - 1) continue;
+        if (!clusters_fit<BN>(a, c, dev, sms)) continue;
         const double cost = (double)((num_ks + c - 1) / c) * step + 600.0 + (many && num_ks < 50 ? 1500.0 - 30.0 * num_ks : 0.0);
         if (cost < best.cost) best = {c, cost};
     }
@@ -579,6 +588,19 @@ static Plan choose_plan(const GemmArgs &a, int dev, int sms)
     return tiles_only;
 }
 
+// The plan a test asks for; false where it does not fit
+static bool forced_plan(const GemmArgs &a, int dev, int sms, Plan &p)
+{
+    const int c = a.force_csize > 1 ? a.force_csize : 1;
+    p = {0, a.force_kernel == 3 ? 256 : 128, {c, 0.0}};
+    if (a.force_kernel == 1) p.head = a.N;
+    if (a.force_kernel == 4) p.head = (a.N - 1) / 256 * 256;
+    GemmArgs rest = a;
+    rest.N -= p.head;
+    if (a.force_kernel == 1 || c == 1) return a.force_kernel != 4 || p.head > 0;
+    return (a.force_kernel != 4 || p.head > 0) && (p.bn == 128 ? clusters_fit<128>(rest, c, dev, sms) : clusters_fit<256>(rest, c, dev, sms));
+}
+
 cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
 {
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
@@ -591,7 +613,9 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
     // The measurement mode exists in the pair kernel only, and up to 128 tokens the gated epilogue too.  Above, a gated call adds its
     // products up as the plain call does: clusters where that takes clusters.  A lone CTA's sums are those of the pair kernel bit
     // for bit, k-step after k-step, so there the gated call keeps to the pair kernel, whose epilogue overlaps.
-    if (!a.mma_only && !(a.gated.codes && a.plan_rows <= BM)) {
+    if (a.force_kernel != 0) {
+        if (!forced_plan(a, di->device, di->sms, p)) return cudaErrorInvalidValue;
+    } else if (!a.mma_only && !(a.gated.codes && a.plan_rows <= BM)) {
         GemmArgs whole = a;
         whole.M = a.plan_rows;
         p = choose_plan(whole, di->device, di->sms);
