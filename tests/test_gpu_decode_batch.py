@@ -360,3 +360,99 @@ def test_decode_nvfp4_hook_refuses_what_it_does_not_know(dq):
     for variant in (0, 1, TC, 6):
         dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=variant)
     _status_ok(dq)
+
+
+@pytest.mark.parametrize("N,K", [(16, 128), (144, 384), (784, 1152), (272, 7168), (400, 9216), (144, 17408), (48, 21632), (80, 32768)])
+@pytest.mark.parametrize("B", [1, 3, 8, 17])
+def test_decode_nvfp4_every_kernel(dq, oracle, N, K, B):
+    """The NVFP4 kernels at every ring depth of the mma.sync kernel (one warp a row group up to 32), in one pass over the columns and in
+    several, whichever of them the public call would take."""
+    W, ref = _layer(oracle, N, K)
+    w = dq.pack_weights(W.to(DEV), formats=dq.FMT_NVFP4)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 950 + B)
+    Yr, S = _reference(oracle, ref, "nvfp4", X)
+    for variant in (0, 1, TC, 6):
+        out = torch.full((B + 1, N + 8), 7.0, dtype=torch.bfloat16, device=DEV)
+        dq.test_decode_linear(w, dq.FMT_NVFP4, X.to(DEV), out=out[:B, :N], variant=variant)
+        _status_ok(dq)
+        check_outputs(_f64(out[:B, :N]), Yr, S, f"variant {variant}, {B}x{N}x{K}")
+        assert torch.all(out[B] == 7.0) and torch.all(out[:, N:] == 7.0)
+
+
+def _decode_calls(dq, w, X):
+    """Calls that reach the batch kernel, the 16-row kernel and the slice-by-slice kernel, and what the public entry points take."""
+    calls = [(dq.FMT_LUT3, X[:9], TC), (dq.FMT_LUT3, X[:7], 6), (dq.FMT_LUT3, X[:20], 4), (dq.FMT_LUT2, X[:24], TC), (dq.FMT_LUT2, X[:5], 6),
+             (dq.FMT_LUT2, X[:33], 4), (dq.FMT_NVFP4, X[:6], TC), (dq.FMT_NVFP4, X[:2], 6)]
+    calls += [(f, X[:b], 0) for f in (dq.FMT_LUT3, dq.FMT_LUT2, dq.FMT_NVFP4) for b in (6, 12, 40)]
+    return [lambda out, f=f, x=x, v=v, **kw: dq.test_decode_linear(w, f, x, out=out, variant=v, **kw) for f, x, v in calls], \
+        [x.shape[0] for _, x, _ in calls]
+
+
+@pytest.mark.parametrize("N,K", [(1040, 2048), (144, 4224)])
+def test_decode_kernels_replay_from_a_cuda_graph(dq, N, K):
+    """Every decode kernel captured in one graph, launch after launch; replays on new activations give what eager calls give."""
+    w = dq.pack_weights(dq_inputs.gaussian_bf16(N, K, 0.02, 11).to(DEV), formats=dq.FMT_NVFP4 | dq.FMT_LUT3 | dq.FMT_LUT2)
+    X = dq_inputs.gaussian_bf16(40, K, 1.0, 12).to(DEV)
+    calls, rows = _decode_calls(dq, w, X)
+    outs = [torch.zeros(b, N, dtype=torch.bfloat16, device=DEV) for b in rows]
+    for call, y in zip(calls, outs):
+        call(y)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for call, y in zip(calls, outs):
+            call(y)
+    for seed in (13, 14):
+        X.copy_(dq_inputs.gaussian_bf16(40, K, 1.0, seed).to(DEV))
+        for y in outs:
+            y.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        for call, y in zip(calls, outs):
+            got = y.clone()
+            call(y)
+            torch.cuda.synchronize()
+            assert torch.equal(got, y) and float(got.float().abs().max()) > 0.0
+    _status_ok(dq)
+
+
+def test_decode_kernels_on_several_streams_at_once(dq):
+    """Every decode kernel on three streams at a time, on one handle: the bits of the calls one after the other."""
+    N, K = 1040, 2048
+    w = dq.pack_weights(dq_inputs.gaussian_bf16(N, K, 0.02, 15).to(DEV), formats=dq.FMT_NVFP4 | dq.FMT_LUT3 | dq.FMT_LUT2)
+    streams = [torch.cuda.Stream(device=DEV) for _ in range(3)]
+    work, want = [], []
+    for i in range(3):
+        calls, rows = _decode_calls(dq, w, dq_inputs.gaussian_bf16(40, K, 1.0, 16 + i).to(DEV))
+        work.append((calls, [torch.zeros(b, N, dtype=torch.bfloat16, device=DEV) for b in rows]))
+        want.append([call(torch.empty(b, N, dtype=torch.bfloat16, device=DEV)) for call, b in zip(calls, rows)])
+    torch.cuda.synchronize()
+    for _ in range(4):
+        for i, st in enumerate(streams):
+            with torch.cuda.stream(st):
+                for call, y in zip(*work[i]):
+                    call(y, stream=st)
+    torch.cuda.synchronize()
+    _status_ok(dq)
+    for i in range(3):
+        for y, z in zip(work[i][1], want[i]):
+            assert torch.equal(y, z)
+
+
+@pytest.mark.parametrize("fmt,limit", [("lut3", 6e-4), ("lut2", 6e-4), ("nvfp4", 3e-4)])
+@pytest.mark.parametrize("K", [512, 2048, 5120, 17408])
+def test_decode_batch_share_of_misrounded_outputs(dq, fmt, limit, K):
+    """Outputs that differ from the exact sum rounded to bf16 once.  A sum that is off by e ulp of fp32 moves a rounding with probability
+    e * 2^-15 (half a bf16 step is 2^15 fp32 ulp of a sum without cancellation, fewer with it): measured 1.6e-4 to 2.8e-4 for the LUT formats in groups
+    of 128 weights and 0.4e-4 to 1.2e-4 for NVFP4; the mma.sync kernels 0.9e-4 to 3.1e-4 and 0.6e-4 to 1.6e-4.  Groups of 512
+    gave the LUT formats 7e-4.  The limits are at least twice the largest; 655360 outputs scatter by about 0.2e-4."""
+    N, B = 10240, 64
+    g = torch.Generator(device=DEV).manual_seed(K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2, "nvfp4": dq.FMT_NVFP4}[fmt]
+    w = dq.pack_weights((torch.randn(N, K, generator=g, device=DEV) * 0.02).to(torch.bfloat16), formats=code)
+    X = torch.randn(B, K, generator=g, device=DEV).to(torch.bfloat16)
+    y = dq.test_decode_linear(w, code, X, variant=TC)
+    _status_ok(dq)
+    exact = (X.double() @ _dequantised(dq, w, fmt).T).to(torch.float32).to(torch.bfloat16)
+    share = float((y != exact).double().mean())
+    assert share < limit, f"{share:.2e}"

@@ -304,29 +304,32 @@ def test_decode_nvfp4_parity(dq, oracle, N, K, seed, B):
             dq.decode_linear_nvfp4(w3, X.to(DEV))
 
 
-@pytest.mark.parametrize("N,K,seed,B", [(19200, 1152, 35, 1), (9600, 5120, 36, 9), (3200, 17408, 37, 2)])
+@pytest.mark.parametrize("N,K,seed,B", [(24064, 1152, 35, 1), (9600, 5120, 36, 9), (3200, 17408, 37, 2), (4880, 8192, 38, 3),
+                                        (2432, 21632, 39, 1), (35600, 640, 40, 2)])
 def test_decode_nvfp4_several_row_tiles_per_cta(dq, oracle, N, K, seed, B):
-    """More row tiles than the grid takes in one round, at the row lengths whose warps keep three chunks in flight (the
-    eight chunks of a tile are not a multiple of three)."""
+    """The mma.sync kernel with more row tiles than its grid takes in one round, so that a warp's register ring of chunks goes on from one
+    tile to the next: three chunks deep (1152, 5120, 17408; the eight chunks of a tile are not a multiple of three), four (640,
+    8192) and two (21632); several passes over the columns; and what the public call takes."""
     W, ref = _layer(oracle, N, K, seed)
     w = dq.pack_weights(W.to(DEV), formats=dq.FMT_NVFP4)
     X = dq_inputs.gaussian_bf16(B, K, 1.0, seed + 200 + B)
-    Y = dq.decode_linear_nvfp4(w, X.to(DEV))
-    _status_ok(dq)
     Yr, S = oracle.decode_linear_nvfp4(dq_inputs.bf16_to_f32_numpy(X), ref["nvfp4_codes"], ref["nvfp4_scales"], ref["s"])
-    check_outputs(_f64(Y), Yr, S, f"nvfp4 decode {B}x{N}x{K}")
+    for variant in (0, 6):
+        Y = dq.test_decode_linear(w, dq.FMT_NVFP4, X.to(DEV), variant=variant)
+        _status_ok(dq)
+        check_outputs(_f64(Y), Yr, S, f"nvfp4 decode {B}x{N}x{K}, variant {variant}")
 
 
 def test_decode_nvfp4_kernels_agree_and_handle_wide_range_activations(dq, oracle):
-    """The tensor-core kernel (default) and the CUDA-core kernel both meet the oracle; activations spanning
-    many binades (the tensor-core kernel rescales them to fp16) and strided, guarded outputs."""
+    """The public call, the CUDA-core, batch and mma.sync kernels all meet the oracle; activations spanning
+    many binades (the tensor-core kernels rescale them to fp16) and strided, guarded outputs."""
     N, K, B = 400, 2048, 5
     W, ref = _layer(oracle, N, K, 90)
     w = dq.pack_weights(W.to(DEV), formats=dq.FMT_NVFP4)
     g = torch.Generator().manual_seed(91)
     X = (torch.randn(B, K, generator=g) * torch.exp2(torch.randint(-20, 12, (B, K), generator=g).float())).to(torch.bfloat16)
     Yr, S = oracle.decode_linear_nvfp4(dq_inputs.bf16_to_f32_numpy(X), ref["nvfp4_codes"], ref["nvfp4_scales"], ref["s"])
-    for variant in (0, 1):
+    for variant in (0, 1, 5, 6):
         out = torch.full((B, N + 8), -3.0, dtype=torch.bfloat16, device=DEV)
         dq.test_decode_linear(w, dq.FMT_NVFP4, X.to(DEV), out=out[:, :N], variant=variant)
         _status_ok(dq)
