@@ -1341,9 +1341,18 @@ static int rows16_if_faster(int bits, int64_t N, int64_t K, int B, int sms, cons
 // 2048x256: 5.2 / 4.6; longer, 1024x2560: 6.2 / 6.5; more rows, 3072x1024: 4.4 / 5.3)
 static bool few_rows(int64_t N, int64_t K, int sms) { return N >= 512 && N <= 16 * (int64_t)sms && K <= 2048; }
 
-// Where shared memory cuts four to eight columns into passes, the batch kernel of dq_decode_tc.cu, which has no such limit, is ahead once the
-// passes add up (3072x12288 batch 6: 22.7 / 19.5; 5120x17408 batch 8: 52 / 35; not yet for 1024x12288 batch 8: 17.3 / 18.5).
-static bool passes_add_up(int B, const Split &narrow) { return B >= 4 && narrow.cols < B && narrow.cost > 100.0 - 5.0 * B; }
+// Where shared memory cuts four to eight columns into passes, the batch kernel of dq_decode_tc.cu, which has no such limit, once it is well
+// ahead by models of both: here 0.13 for each unit of the split's cost, 2.7 a pass, 0.054 for each thousand activations and 1.7; there
+// 5.05 a slice of 512 and 1.1 (749 points of 6144 to 32768 weights, 16 to 20480 rows; the models are within 23 % of the times, and with 7 %
+// to spare the pick is slower than the passes at none: 3072x12288 batch 6 22.7 / 19.5, 5120x17408 batch 8 52 / 35; passes stay for
+// 1024x17408 batch 7 23.7 / 28.4, 8704x14336 batch 6 43.1 / 52.5, 1024x32768 batch 4 26.5 / 42.8).
+static bool passes_add_up(int64_t N, int64_t K, int B, const Split &narrow)
+{
+    if (B < 4 || narrow.cols >= B) return false;
+    const double passes = (double)((B + narrow.cols - 1) / narrow.cols);
+    const double here = 0.129 * narrow.cost + 2.67 * passes + 0.0536e-3 * (double)B * (double)K + 1.74;
+    return decode_tc_slices(N, K) * 5.05 + 1.1 < 0.93 * here;
+}
 
 // The batch kernel at up to eight columns on very short rows: one half slice, 4.5 to 4.8 whatever the batch (1024x256 batch 5 / 8: 4.8 / 5.9
 // with 16-row tiles).
@@ -1400,7 +1409,7 @@ cudaError_t launch_gemv_lut(const GemvArgs &a, cudaStream_t stream)
         LutPlan L16 = {};
         const int grid16 = B > 4 && all ? rows16_if_faster(a.bits, N, K, B, sms, sp, L16) : 0;
         if (grid16 > 0) return launch_rows16(a, L16, grid16, stream);
-        if (a.split_exact && passes_add_up(B, sp)) return launch_decode_tc(a, stream);
+        if (a.split_exact && passes_add_up(N, K, B, sp)) return launch_decode_tc(a, stream);
     }
     LutPlan L;
     if (a.force_P > 0 && a.force_G > 0) {
