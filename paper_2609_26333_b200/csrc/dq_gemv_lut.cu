@@ -1319,19 +1319,24 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
     return launch_one<BITS, 1024, 1, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
 }
 
-// The choices between the kernels, from launch after launch of one matrix at 130 shapes from 16 to 16384 rows of 128 to 12288 weights
-// (LUT3 and LUT2; us).
+// The choices between the kernels, from launch after launch of one matrix (LUT3 and LUT2; us).
 
 // Five to eight columns, 16-row tiles against 8-row tiles: the two cost models in one unit; a CTA with few warps loses a little more
-// than the model's stretch, and long rows' activations take their time to convert.  Over 520 points the pick is never the slower one by more
-// than 2 % and on average 0.3 % off the better (1024x4096 batch 5: 7.9 / 6.6; 4096x5120 batch 8: 11.6 / 11.4; 8192x12288 batch 5:
-// 38 / 25.8; stays with 8 rows: 5120x3072 batch 5 8.3 / 9.2, 1024x8192 batch 6 10.1 / 11.4).  Below 128 rows neither fills the chip.
+// than the model's stretch, and long rows' activations take their time to convert.  The models do not see that warps with one unit of 512
+// each have nothing to hide a wait behind: an odd number of them, which the four schedulers share unevenly, loses to 12 and more warps of
+// 8-row tiles (2016x5632 batch 8: 9.7 / 11.2; 128x4352 9.8 / 10.7) and 13 of them to any (352x6528 batch 5: 8.6 / 9.7).  Of 4960 points (128 to
+// 34816 rows of 384 to 14336 weights) the pick is more than 2 % slower than 8-row tiles at 67, at most 9 %, and on average 0.3 % off the better
+// (1024x4096 batch 5: 7.9 / 6.6; 4096x5120 batch 8: 11.6 / 11.4; 8192x12288 batch 5: 38 / 25.8; stays with 8 rows: 5120x3072 batch 5
+// 8.3 / 9.2, 1024x8192 batch 6 10.1 / 11.4).  Above 10240 rows it stays with 8 rows at some points where 16 would be
+// faster (17408x5120 batch 8: 22.1 / 20.8, 14336x8192 38.9 / 30.9).  Below 128 rows neither fills the chip.
 // The grid of the 16-row launch and its plan in L, 0 for 8-row tiles.
 static int rows16_if_faster(int bits, int64_t N, int64_t K, int B, int sms, const Split &narrow, LutPlan &L)
 {
     double cost;
     const int grid = N < 128 ? 0 : choose_rows16(bits, N, K, sms, B, L, cost);
     if (grid == 0) return 0;
+    const bool one_unit = L.P == (K + kLutAtomK - 1) / kLutAtomK && L.P % 2 == 1 && L.P >= 7;
+    if (one_unit && (narrow.P * narrow.G >= 12 || L.P == 13)) return 0;
     const double warps = (double)(L.P * L.G);
     if (warps < 12.0) cost *= std::sqrt(std::sqrt(12.0 / warps));
     return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost ? grid : 0;
