@@ -263,7 +263,7 @@ cudaError_t launch_gemv_lut_tc(const GemvArgs &args, int warpgroups, cudaStream_
 // dq_decode_tc.cu: up to 64 columns in one pass, dequantised weights through tcgen05.  LUT3 asks for a codebook whose levels
 // are multiples of 2^-15 up to 146.2 in magnitude (split_exact); force_P = CTAs per tile (test hook)
 cudaError_t launch_decode_tc(const GemvArgs &args, cudaStream_t stream);
-double decode_tc_slices(int64_t N, int64_t K);
+double decode_tc_slices(int64_t N, int64_t K, bool *crowded = nullptr);
 
 struct GemvNvArgs {
     const uint8_t *codes; const uint8_t *sf;              // NVFP4 view: [N][K/2] codes, MMA-layout scales

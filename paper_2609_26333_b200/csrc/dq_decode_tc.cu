@@ -903,11 +903,15 @@ cudaError_t launch_cols(const CUtensorMap &tmap, const TcDecodeArgs &P, int forc
 
 }  // namespace
 
-// 512-weight slices the busiest CTA of a launch works through, an exchange included
-double decode_tc_slices(int64_t N, int64_t K)
+// 512-weight slices the busiest CTA of a launch works through, an exchange included.  crowded: clusters of three or five, all or all but one
+// that fit: a slice then takes 2.8 to 4.1 us instead of 2.6 (NVFP4, 11296x2816, 45 clusters of three: 11.6; not seen at other sizes)
+double decode_tc_slices(int64_t N, int64_t K, bool *crowded)
 {
     const DeviceInfo *di = device_info();
-    return di ? split_tiles(N, K, di->device, di->sms, 0).slices : 1e300;
+    if (!di) return 1e300;
+    const TileSplit t = split_tiles(N, K, di->device, di->sms, 0);
+    if (crowded) *crowded = (t.csize == 3 || t.csize == 5) && (N + 255) / 256 >= clusters_that_fit(di->device, t.csize, di->sms) - 1;
+    return t.slices;
 }
 
 cudaError_t launch_decode_tc(const GemvArgs &a, cudaStream_t stream)

@@ -312,12 +312,13 @@ static int row_groups(int W)
     return G < 1 ? 1 : G > 15 ? 15 : G;
 }
 
-// Whether the batch kernel of dq_decode_tc.cu is ahead of this file's, from 396 points between 16x256 and 17408x8192, batch 1 to 8, launch
-// after launch of one matrix: here 2.4 us a pass, 4.6 for each round over the rows (less where a slice is short) and about half a
-// microsecond a column; there 2.2 and 2.7 for each slice of 512 weights that a CTA dequantises, whatever the batch.  The pick is never
-// the slower one by more than 2 % (us, here / there: 2048x4096 batch 1 / 4 7.6 / 6.6, 9.3 / 6.7; 8192x256 batch 4 5.6 / 3.8; 1024x8192
-// batch 1 / 8 7.1 / 8.8, 20.4 / 9.2; 8192x5120 batch 5 10.5 / 12.3; 17408x5120 batch 5 / 6 15.8 / 17.4, 16.4 / 17.4).  Above eight columns a second
-// pass is due here.
+// Whether the batch kernel of dq_decode_tc.cu is ahead of this file's, launch after launch of one matrix at batch 1 to 8: here 2.4 us a pass,
+// 4.6 for each round over the rows (less where a slice is short, or up to 12 warps share the CTA) and about half a microsecond a column; there
+// 2.2 and 2.7 for each slice of 512 weights that a CTA dequantises, whatever the batch, and a tenth more where its clusters
+// crowd the chip (us, here / there: 2048x4096 batch 1 / 4 7.6 / 6.6, 9.3 / 6.7; 8192x256 batch 4 5.6 / 3.8; 1024x8192 batch 1 / 8
+// 7.1 / 8.8, 20.4 / 9.2; 8192x5120 batch 5 10.5 / 12.3; 17408x5120 batch 5 / 6 15.8 / 17.4, 16.4 / 17.4; 2448x11008 batch 1 10.2 / 11.9;
+// 11312x11392 batch 1 22.4 / 32.6).  Of 1494 points (512 to 12288 rows of 1024 to 17408 weights) the pick is more than 2 % slower than this
+// kernel at 11, at most 7 %.  Above eight columns a second pass is due here.
 bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms)
 {
     const int64_t W = (K + 1023) / 1024, G = row_groups((int)W), ntiles = ((N + 127) / 128) * 8;
@@ -325,8 +326,11 @@ bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms)
     if (B > 8 || cols_max < 1) return true;
     const int64_t cols = cols_max < 8 ? cols_max : 8;
     const double rounds = (double)((ntiles + G * sms - 1) / (G * sms)), passes = (double)((B + cols - 1) / cols);
-    const double here = passes * (2.4 + 4.6 * rounds * (K < 1280 ? (double)K / 1280.0 : 1.0)) + 0.58 * (double)B * (0.8 + 0.2 * rounds);
-    const double there = 2.2 + 2.7 * decode_tc_slices(N, K) * (K < 512 ? (double)K / 512.0 : 1.0);
+    const double round = 4.6 * (K < 1280 ? (double)K / 1280.0 : 1.0) * (W * G <= 12 ? 0.84 : 1.0);
+    const double here = passes * (2.4 + rounds * round) + 0.58 * (double)B * (0.8 + 0.2 * rounds);
+    bool crowded = false;
+    const double slices = decode_tc_slices(N, K, &crowded);
+    const double there = 2.2 + 2.7 * slices * (K < 512 ? (double)K / 512.0 : 1.0) * (crowded ? 1.1 : 1.0);
     return there < here;
 }
 
