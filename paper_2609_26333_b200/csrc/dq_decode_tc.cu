@@ -41,7 +41,8 @@ using namespace tc;
 constexpr int kSlice = 512;                        // weights along K per accumulator
 constexpr int kThreads = 512;
 constexpr uint32_t kSmemMax = 227 * 1024;
-constexpr uint32_t kXinvOff = 512;                 // [4][4][64] floats: inverse activation scales of the last slices' 128-weight groups
+constexpr uint32_t kXinvOff = 512;                 // [4][4][64] floats: inverse activation scales of the last slices' 128-weight groups,
+constexpr uint32_t kXinvGroup = 68;                // a group's 64 padded: the four stores of a column go to different banks
 constexpr uint32_t kRingOff = 5120;
 
 // FMT: 0 = NVFP4, 2 = LUT2, 3 = LUT3; NC: batch columns of the pass, padded
@@ -81,7 +82,7 @@ enum : uint32_t {
     kXEmpty = kXFull + 16,
     kBarEnd = kXEmpty + 16,
 };
-static_assert(kBarEnd <= kXinvOff, "barriers");
+static_assert(kBarEnd <= kXinvOff && kXinvOff + 16u * 4u * kXinvGroup <= kRingOff, "barriers, scales");
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
 {
@@ -165,7 +166,7 @@ __device__ __noinline__ void stage_infinite(const __nv_bfloat16 *X, int64_t ldx,
         for (int i = 0; i < 2; ++i)
             asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
                          ::"r"(xb + (uint32_t)c * 16u + (uint32_t)(lane + 32 * i) * stride), "r"(x[i].x), "r"(x[i].y), "r"(x[i].z), "r"(x[i].w) : "memory");
-        if (lane < 4) xinv[lane * 64 + c] = (inf >> lane) & 1u ? __uint_as_float(0x7F800000u) : 1.0f;
+        if (lane < 4) xinv[lane * kXinvGroup + c] = (inf >> lane) & 1u ? __uint_as_float(0x7F800000u) : 1.0f;
     }
 }
 // four code bytes -> four fp16 pairs (low nibble first)
@@ -431,7 +432,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 ++grp;
                 open = true;
                 open_xi = next_xi;
-                if (kLut) next_xi += 256u;
+                if (kLut) next_xi += 4u * kXinvGroup;
             }
         };
         for (int tile = first_tile; tile < ntiles && ok; tile += tile_stride) {
@@ -440,7 +441,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
             for (int c = 0; c < NC; ++c) acc[c] = 0.0f;
             for (int sl = s0; sl < s1 && ok; ++sl, ++cnt) {
                 const int ng = groups(sl);
-                next_xi = win0 + kXinvOff + (cnt & 3u) * 1024u;
+                next_xi = win0 + kXinvOff + (cnt & 3u) * 16u * kXinvGroup;
                 if constexpr (kLut) {
                     // Index words and scales of this warp's 32 rows: four atoms.  Scales of the slice and words of one half of it at a time
                     // are held in registers, and the halves are a loop: unrolled over the slice the code outgrows the instruction
@@ -639,7 +640,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                         top = max(top, m);
                         const int ex = max(-100, (int)(m >> 7) - 127);              // floor(log2(max)); -127 for zero / subnormal
                         const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
-                        if (lane < 4) xinv_s[((cnt & 3u) * 4u + (uint32_t)lane) * 64u + c] = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
+                        if (lane < (kLut ? 4 : 1)) xinv_s[((cnt & 3u) * 4u + (uint32_t)lane) * kXinvGroup + c] = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
                             const uint32_t ww[4] = {v[u][i].x, v[u][i].y, v[u][i].z, v[u][i].w};
@@ -667,7 +668,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant
                 }
                 if (kLut && top >= 0x7F80u)
                     stage_infinite(P.X + (int64_t)P.b0 * P.ldx + sl * kSlice, P.ldx, sw, P.cols, live, xb, C::kXStride,
-                                   xinv_s + (cnt & 3u) * 256u);
+                                   xinv_s + (cnt & 3u) * 4u * kXinvGroup);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");        // the tensor cores read them
                 __syncwarp();
                 if (lane == 0) mbar_arrive(win0 + kXFull + (cnt & 1u) * 8u);
