@@ -235,7 +235,7 @@ struct GemmArgs {
     // writes NVFP4(bf16(SiLU(gate) * up))
     GatedOut gated = {nullptr, nullptr, 0.0f, 0};
 };
-cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream);
+cudaError_t launch_gemm_nvfp4(GemmArgs &args, cudaStream_t stream);      // args: scratch of the call
 cudaError_t launch_gemm_nvfp4_pair(const GemmArgs &args, void *encode_fn, cudaStream_t stream);
 int gemm_init_driver_api();   // resolves the tensor-map encoder; 0 on success
 void *gemm_encode_fn();       // the encoder, after gemm_init_driver_api

@@ -462,11 +462,11 @@ cudaError_t set_attributes(int dev)
 // Whether clusters of c CTAs may share the tiles of 128 x BN: each takes one tile and at least one k-step, and all must be resident.  How
 // many of a size fit is asked once per device, and again where the runtime did not answer.
 template <int BN>
-bool clusters_fit(const GemmArgs &a, int c, int dev, int sms)
+bool clusters_fit(int64_t M, int64_t N, int64_t K, int c, int dev, int sms)
 {
     static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];                 // + 1; 0 = not known
-    const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
-    if (c > kMaxCluster || c > (a.K / 64 + kKbPerStage - 1) / kKbPerStage || tiles * c > sms) return false;
+    const int64_t tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    if (c > kMaxCluster || c > (K / 64 + kKbPerStage - 1) / kKbPerStage || tiles * c > sms) return false;
     int fit = known[dev][c].load(std::memory_order_relaxed);
     if (fit == 0) {
         cudaLaunchAttribute attr[2];
@@ -488,16 +488,16 @@ bool clusters_fit(const GemmArgs &a, int c, int dev, int sms)
 // (34816 columns, 16384 rows: 2.3 us a round at K = 128, 2.9 at 1024), the exchange of full row tiles up to 1500 more where few
 // k-steps hide it (512x1536, 793 rows: 9.6 us against 8.2 in the pair kernel; 5120x17408, 300 rows: 25.2 with it, 27.0 without), and the ramp is 600 shorter than the pair kernel's.
 template <int BN>
-Split choose_split(const GemmArgs &a, int dev, int sms)
+Split choose_split(int64_t M, int64_t N, int64_t K, int dev, int sms)
 {
-    const int64_t tiles = ((a.M + BM - 1) / BM) * ((a.N + BN - 1) / BN);
-    const int num_ks = (int)((a.K / 64 + kKbPerStage - 1) / kKbPerStage);
+    const int64_t tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
+    const int num_ks = (int)((K / 64 + kKbPerStage - 1) / kKbPerStage);
     const double step = BN + 48.0;
     const double rounds = (double)((tiles + sms - 1) / sms), stream = num_ks * step, output = 0.54 * stream + 1290.0 * (BN / 128);
-    const bool many = a.M > BM;
+    const bool many = M > BM;
     Split best = {1, many ? rounds * (stream > output ? stream : output) - 600.0 : rounds * stream};
     for (int c = 2; c <= kMaxCluster && c <= num_ks && tiles * c <= sms; ++c) {
-        if (!clusters_fit<BN>(a, c, dev, sms)) continue;
+        if (!clusters_fit<BN>(M, N, K, c, dev, sms)) continue;
         const double cost = (double)((num_ks + c - 1) / c) * step + 600.0 + (many && num_ks < 50 ? 1500.0 - 30.0 * num_ks : 0.0);
         if (cost < best.cost) best = {c, cost};
     }
@@ -555,18 +555,18 @@ void *gemm_encode_fn() { return reinterpret_cast<void *>(g_encode); }
 // Kernel and tile of a GEMM: the pair kernel for the first `head` columns, tiles of 128 x bn with clusters of sp.csize for the rest
 struct Plan { int64_t head; int bn; Split sp; };
 
-static Plan choose_plan(const GemmArgs &a, int dev, int sms)
+static Plan choose_plan(int64_t M, int64_t N, int64_t K, int dev, int sms)
 {
-    const Split s128 = choose_split<128>(a, dev, sms), s256 = choose_split<256>(a, dev, sms);
+    const Split s128 = choose_split<128>(M, N, K, dev, sms), s256 = choose_split<256>(M, N, K, dev, sms);
     const Plan tiles_only = s128.cost < s256.cost ? Plan{0, 128, s128} : Plan{0, 256, s256};
-    if (a.M <= BM) return tiles_only;
+    if (M <= BM) return tiles_only;
     // CTA pairs on 256 x 256 tiles move half as many bytes per flop but have few tiles to share out: 0.36 us per k-step and round
     // and 1 us per tile against 1.75 ns per unit of the other cost, and no less than the output of a round on short rows
     // (34816x256, 16384 rows: 293 us here, 568 with the other kernel; 5120x1024, 2048 rows 13.3 / 16.7).  Measured (us, quantiser included, pair / here): 5120x17408
     // 200 tokens 29.7 / 21.7, 300 tokens 31.3 / 26.0, 512 tokens 32.7 / 37.3; 6144x4096 256 tokens 12.6 / 11.5, 512 tokens
     // 14.1 / 15.2; 10240x5120 256 tokens 15.2 / 17.7, 300 tokens 22.3 / 17.9; 34816x5120 129 tokens 28.3 / 32.9.
-    const int64_t tiles = ((a.M + 255) / 256) * ((a.N + 255) / 256);
-    const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (a.K + 255) / 256;
+    const int64_t tiles = ((M + 255) / 256) * ((N + 255) / 256);
+    const int64_t rounds = (tiles + sms / 2 - 1) / (sms / 2), num_ks = (K + 255) / 256;
     const auto pair_cost = [&](int64_t r) {
         const double stream = (double)num_ks * 206.0 + 571.0, output = (double)num_ks * 150.0 + 900.0;
         return (double)r * (stream > output ? stream : output);
@@ -574,17 +574,16 @@ static Plan choose_plan(const GemmArgs &a, int dev, int sms)
     // Where the last round would be nearly empty its columns go to the cluster kernel in a launch of their own, about 7 us of
     // ramp before its k-steps count (5120x17408, 1000 tokens, 80 tiles on 74 pairs: 59.6 -> 50.0 us; 10240x5120,
     // where a round is 9 us, would lose: 31.7 -> 37.3)
-    const int64_t tiles_m = (a.M + 255) / 256, head = (rounds - 1) * (sms / 2) / tiles_m;      // 256-column blocks of the full rounds
-    if (rounds > 1 && head > 0 && head * 256 < a.N) {
-        GemmArgs tail = a;
-        tail.N = a.N - head * 256;
-        const Split t128 = choose_split<128>(tail, dev, sms), t256 = choose_split<256>(tail, dev, sms);
+    const int64_t tiles_m = (M + 255) / 256, head = (rounds - 1) * (sms / 2) / tiles_m;      // 256-column blocks of the full rounds
+    if (rounds > 1 && head > 0 && head * 256 < N) {
+        const int64_t rest = N - head * 256;
+        const Split t128 = choose_split<128>(M, rest, K, dev, sms), t256 = choose_split<256>(M, rest, K, dev, sms);
         const double tail_cost = (t128.cost < t256.cost ? t128.cost : t256.cost) + 4000.0;
         const double split_cost = pair_cost(rounds - 1) + tail_cost;
         if (split_cost < pair_cost(rounds) && split_cost < s128.cost && split_cost < s256.cost)
             return t128.cost < t256.cost ? Plan{head * 256, 128, t128} : Plan{head * 256, 256, t256};
     }
-    if (pair_cost(rounds) <= s128.cost && pair_cost(rounds) <= s256.cost) return {a.N, 256, {1, 0.0}};
+    if (pair_cost(rounds) <= s128.cost && pair_cost(rounds) <= s256.cost) return {N, 256, {1, 0.0}};
     return tiles_only;
 }
 
@@ -595,18 +594,16 @@ static bool forced_plan(const GemmArgs &a, int dev, int sms, Plan &p)
     p = {0, a.force_kernel == 3 ? 256 : 128, {c, 0.0}};
     if (a.force_kernel == 1) p.head = a.N;
     if (a.force_kernel == 4) p.head = (a.N - 1) / 256 * 256;
-    GemmArgs rest = a;
-    rest.N -= p.head;
+    const int64_t rest = a.N - p.head;
     if (a.force_kernel == 1 || c == 1) return a.force_kernel != 4 || p.head > 0;
-    return (a.force_kernel != 4 || p.head > 0) && (p.bn == 128 ? clusters_fit<128>(rest, c, dev, sms) : clusters_fit<256>(rest, c, dev, sms));
+    return (a.force_kernel != 4 || p.head > 0) && (p.bn == 128 ? clusters_fit<128>(a.M, rest, a.K, c, dev, sms) : clusters_fit<256>(a.M, rest, a.K, c, dev, sms));
 }
 
-cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
+cudaError_t launch_gemm_nvfp4(GemmArgs &a, cudaStream_t stream)
 {
     if (gemm_init_driver_api() != 0) return cudaErrorNotSupported;
     const DeviceInfo *di = device_info();
     if (!di) return cudaErrorInvalidDevice;
-    GemmArgs a = args;
     if (a.plan_rows == 0) a.plan_rows = a.M;
     a.clocks = a.plan_rows > BM ? 1 : 0;
     Plan p = {a.N, 256, {1, 0.0}};
@@ -616,17 +613,15 @@ cudaError_t launch_gemm_nvfp4(const GemmArgs &args, cudaStream_t stream)
     if (a.force_kernel != 0) {
         if (!forced_plan(a, di->device, di->sms, p)) return cudaErrorInvalidValue;
     } else if (!a.mma_only && !(a.gated.codes && a.plan_rows <= BM)) {
-        GemmArgs whole = a;
-        whole.M = a.plan_rows;
-        p = choose_plan(whole, di->device, di->sms);
+        p = choose_plan(a.plan_rows, a.N, a.K, di->device, di->sms);
     }
     if (a.gated.codes && p.sp.csize == 1) p.head = a.N;
     if (p.head > 0) {
-        GemmArgs front = a;
-        front.N = p.head;
-        const cudaError_t e = launch_gemm_nvfp4_pair(front, reinterpret_cast<void *>(g_encode), stream);
-        if (e != cudaSuccess || p.head == a.N) return e;
-        a.N -= p.head;
+        const int64_t rest = a.N - p.head;
+        a.N = p.head;
+        const cudaError_t e = launch_gemm_nvfp4_pair(a, reinterpret_cast<void *>(g_encode), stream);
+        if (e != cudaSuccess || rest == 0) return e;
+        a.N = rest;
         a.w_codes += p.head * (a.K / 2);
         a.w_sf += p.head * (a.K / kBlock);
         a.clocks = 2;
