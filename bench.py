@@ -37,7 +37,7 @@ L2_BYTES = 126 * 1024 * 1024
 # DRAM bytes per launch measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum) on the kernel named in the
 # roofline object of the same line.  None = not captured for that workload.
 NCU_TRAFFIC_BYTES = {
-    ("gemm", "c3_gate_up27b"): 80.95e6 + 239.5e6,     # gemm_nvfp4_pair_kernel, full size (one-pass launch list)
+    ("gemm", "c3_gate_up27b"): 78.91e6 + 239.8e6,     # gemm_nvfp4_pair_kernel, full size (one-pass launch list)
     ("gemv", "c3_gate_up27b"): 39.04e6,               # gemv_lut_kernel<3, 640, 1, 1, true>, full size, batch 1 (reads; writes are 35 KB)
     ("gemv_nvfp4", "c3_gate_up27b"): 50.19e6,         # gemv_nvfp4_mma_kernel<640, 3>, full size (one-pass launch list)
 }
