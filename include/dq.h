@@ -215,15 +215,15 @@ int dq_prefill_linear_static(const dq_weights *w, const void *A_dev, int64_t M, 
  *   Y[b][n] = bf16( sum_k X[b][k] * W~[n][k] ),  W~ = s * d_b * codebook[idx],
  * a weight-only mat-vec / skinny GEMM on the handle's LUT3 weights with raw bf16
  * activations.  1 <= B <= 64.
- * Arithmetic: the products codebook[idx] * x are formed exactly (fp16 levels and the
- * activations, scaled by one power of two into fp16, on tensor cores) and summed in fp32 per
- * 16-weight block; the block sum is multiplied by d_b and accumulated in fp32; s is applied to
- * the total.  Nothing is rounded before the fp32 accumulation, so the error per output is a few
- * fp32 rounding errors of sum_k |x w| plus the bf16 rounding of the result, for any activation
- * pattern.  An activation more than 2^28 times smaller in magnitude than the largest activation
- * it shares a power-of-two scale with loses low bits or reads as zero: at most those of the rows of X that go
- * through one pass together (eight consecutive rows), in most calls with batches above 8 only those of its own row
- * in the same slice of K (512 or 1024 elements).
+ * Arithmetic: the products d_b * codebook[idx] * x are formed exactly (levels in fp16 against activations scaled by a power of
+ * two into fp16, on tensor cores) and summed in fp32: per 16-weight block, the block sum then multiplied by d_b, or, in
+ * calls that dequantise a weight once for a batch (two fp16 numbers whose sum is d_b * level), per group of 128 weights; sums of
+ * blocks and groups are added in fp32; s is applied to the total.  Nothing is rounded before the fp32 accumulation, so the error per
+ * output is a few fp32 rounding errors of sum_k |x w| plus the bf16 rounding of the result, for any activation
+ * pattern.  An activation more than 2^28 times smaller in magnitude than the largest activation it shares
+ * a power-of-two scale with loses low bits or reads as zero: at most those of the rows of X that go through
+ * one pass together (up to eight consecutive rows), in most calls with batches above 8 only those of its own
+ * row in the same slice of K (512 or 1024 elements).
  * X_dev: B x K bf16, row stride ldx; Y_dev: B x N bf16, row stride ldy.
  */
 int dq_decode_linear(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx,
@@ -243,7 +243,8 @@ int dq_decode_linear_lut2(const dq_weights *w, const void *X_dev, int64_t B, int
  * this mat-vec):
  *   Y[b][n] = bf16( sum_k X[b][k] * W^[n][k] ),  W^ = s * d_b * e2m1(code),
  * raw bf16 activations, fp32 accumulation.  Needs DQ_FMT_NVFP4 or DQ_FMT_NVFP4_FROM_LUT3 in the
- * handle (DQ_ERR_INVALID_ARG otherwise).  Arguments and limits as dq_decode_linear.
+ * handle (DQ_ERR_INVALID_ARG otherwise).  Arguments and limits as dq_decode_linear; products d_b * e2m1 * x are exact,
+ * summed in fp32 along K.
  */
 int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx,
                            void *Y_dev, int64_t ldy, void *stream);
@@ -254,9 +255,10 @@ int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, in
 /*
  * dq_prefill_linear on host memory: A_host (M x K bf16, row stride lda) is copied to the device, the
  * prefill linear runs, Y_host (M x N bf16, row stride ldy) receives the result, bit for bit that of
- * dq_prefill_linear on the same M rows.  M is cut into row chunks; the copy in of the next chunk and the copy out of the previous one overlap the kernels of the
- * current one on two internal streams per device (created at the first call on that device, which
- * therefore must not happen during a stream capture; these calls are not capturable at all).
+ * dq_prefill_linear on the same M rows.  M is cut into row chunks; the copy in of the next chunk and the
+ * copy out of the previous one overlap the kernels of the current one on two internal streams per device
+ * (created at the first call on that device, which therefore must not happen during a stream capture;
+ * these calls are not capturable at all).
  * A_host and Y_host should be pinned (cudaHostAlloc / cudaHostRegister), else the copies serialise.
  * staging_dev: caller-owned device buffer of at least dq_prefill_host_staging_bytes(w, M) bytes
  * (device copies of A and Y plus the prefill workspace of one chunk), 1024-byte aligned.
@@ -388,7 +390,7 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           batch kernel that dequantises every weight once into tensor memory (all columns in one pass,
  *           256-row tiles; DQ_ERR_INVALID_ARG for a codebook with levels that are not multiples of
  *           2^-15 or beyond +-146.2); warps_per_group (1..8) then sets the CTAs that share a tile.  variant 6 runs the kernel
- *           with 16-row tiles that dq_decode_linear takes for most batches of 5 to 8 (DQ_ERR_INVALID_ARG where
+ *           with 16-row tiles that dq_decode_linear takes for many batches of 4 to 8 (DQ_ERR_INVALID_ARG where
  *           the row is too long for it).
  *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what
  *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 5 = the batch

@@ -252,10 +252,10 @@ struct GemvArgs {
     int force_P = 0, force_G = 0, force_S = 0;
     long long wait_cycles = 0;
     int drop_first_copy = 0;                              // one warp's first copy is never requested (its wait must run out)
-    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = mma.sync kernel, 2 = tcgen05 kernel (batch 1), 3 = slice-by-slice kernel (batches above 8), 4 = dequantised through tcgen05 (any batch), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns), 5 = 16-row tiles (up to eight columns)
+    int kernel = 0;                                       // 0 = chosen by the launcher, 1 = 8-row tiles, 2 = tcgen05 kernel of one column, 3 = slice by slice, 4 = batch kernel (dq_decode_tc.cu), 5 = 16-row tiles (up to eight columns)
     bool split_exact = true;                              // codebook levels times block scales are exact as pairs of fp16 numbers (launch_decode_tc)
 };
-cudaError_t launch_gemv_lut(const GemvArgs &args, cudaStream_t stream);     // picks one of the two kernels below
+cudaError_t launch_gemv_lut(const GemvArgs &args, cudaStream_t stream);     // picks the kernel
 // tcgen05 kernel (batch 1): number of warpgroups it would run this shape with, 0 where it does not take it
 int gemv_lut_tc_warpgroups(int bits, int64_t N, int64_t K, int64_t B, int sms, bool any_size);
 cudaError_t launch_gemv_lut_tc(const GemvArgs &args, int warpgroups, cudaStream_t stream);

@@ -6,7 +6,8 @@
 // One CTA per SM and 128-row tile: the kernel of short prompts, where the weights stream from HBM and what counts is that every
 // SM streams its share of them.  Tiles are 128 x 256 or 128 x 128; where there are too few of them for the chip a cluster of up to
 // 8 CTAs shares one, each taking a range of k-steps, and they exchange partial sums through distributed shared memory at
-// the end (added in rank order; no workspace).  256-element k-steps.
+// the end (added in rank order; no workspace).  256-element k-steps.  Also the columns that a larger call leaves to it, and gate/up
+// matrices whose gating and quantising replaces the output (GATED; clusters only, the sums are then those of the plain call).
 //   warp 0      : TMA producer (packed FP4 tiles, 128B swizzle) + bulk copies of the scale atoms; weights that are part of the
 //                 handle are requested before the kernel ahead (the activation quantiser) has finished
 //   warp 1      : tcgen05.cp of the scales into TMEM and tcgen05.mma (kind::mxf4nvf4, block 16)

@@ -14,12 +14,12 @@ constexpr long long kWaitBudgetCycles = 4000000000ll;   // about two seconds
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// True in one lane of a converged warp, always the same one.  The warps that issue tcgen05 and TMA instructions walk their
-// loops and waits together and only wrap the instructions themselves in this: inside the branch the compiler knows that
-// one thread is left and keeps descriptors and addresses in uniform registers.  Under `lane == 0` it cannot, and a
-// tcgen05.mma takes 45 cycles to issue whatever its size; under elect.sync it takes what the tensor pipe needs
-// (128 x 16 x 16 with A in tensor memory: 9 cycles, 128 x 64 x 16: 32).  The branch holds straight-line code only: no lane
-// of the warp runs anything else meanwhile.
+// True in one lane of a converged warp, always the same one.  The warps that issue tcgen05 and TMA instructions wrap them in this: inside
+// the branch the compiler knows that one thread is left and keeps descriptors and addresses in uniform registers.  Under
+// `lane == 0` it cannot, and a tcgen05.mma takes 45 cycles to issue whatever its size; under elect.sync it takes what the tensor pipe
+// needs (128 x 16 x 16 with A in tensor memory: 9 cycles, 128 x 64 x 16: 32).  In one of two ways: the pair kernel's warps walk
+// loops and waits together and elect around the instructions alone; elsewhere the whole role, its loops and bounded waits included,
+// runs in the elected thread and the others wait for it at the __syncwarp behind.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
