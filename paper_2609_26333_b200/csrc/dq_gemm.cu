@@ -463,11 +463,10 @@ cudaError_t set_attributes(int dev)
 // Whether clusters of c CTAs may share the tiles of 128 x BN: each takes one tile and at least one k-step, and all must be resident.  How
 // many of a size fit is asked once per device, and again where the runtime did not answer.
 template <int BN>
-bool clusters_fit(int64_t M, int64_t N, int64_t K, int c, int dev, int sms)
+bool clusters_fit(int64_t tiles, int num_ks, int c, int dev, int sms)
 {
     static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];                 // + 1; 0 = not known
-    const int64_t tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-    if (c > kMaxCluster || c > (K / 64 + kKbPerStage - 1) / kKbPerStage || tiles * c > sms) return false;
+    if (c > kMaxCluster || c > num_ks || tiles * c > sms) return false;
     int fit = known[dev][c].load(std::memory_order_relaxed);
     if (fit == 0) {
         cudaLaunchAttribute attr[2];
@@ -497,9 +496,13 @@ Split choose_split(int64_t M, int64_t N, int64_t K, int dev, int sms)
     const double rounds = (double)((tiles + sms - 1) / sms), stream = num_ks * step, output = 0.54 * stream + 1290.0 * (BN / 128);
     const bool many = M > BM;
     Split best = {1, many ? rounds * (stream > output ? stream : output) - 600.0 : rounds * stream};
-    for (int c = 2; c <= kMaxCluster && c <= num_ks && tiles * c <= sms; ++c) {
-        if (!clusters_fit<BN>(M, N, K, c, dev, sms)) continue;
-        const double cost = (double)((num_ks + c - 1) / c) * step + 600.0 + (many && num_ks < 50 ? 1500.0 - 30.0 * num_ks : 0.0);
+    // the more CTAs the fewer k-steps each: the largest cluster that fits, less the CTAs that make no step fewer
+    int c = num_ks < kMaxCluster ? num_ks : kMaxCluster;
+    while (c > 1 && !clusters_fit<BN>(tiles, num_ks, c, dev, sms)) --c;
+    if (c > 1) {
+        const int steps = (num_ks + c - 1) / c;
+        c = (num_ks + steps - 1) / steps;
+        const double cost = steps * step + 600.0 + (many && num_ks < 50 ? 1500.0 - 30.0 * num_ks : 0.0);
         if (cost < best.cost) best = {c, cost};
     }
     return best;
@@ -595,9 +598,10 @@ static bool forced_plan(const GemmArgs &a, int dev, int sms, Plan &p)
     p = {0, a.force_kernel == 3 ? 256 : 128, {c, 0.0}};
     if (a.force_kernel == 1) p.head = a.N;
     if (a.force_kernel == 4) p.head = (a.N - 1) / 256 * 256;
-    const int64_t rest = a.N - p.head;
+    const int64_t tiles = (a.M + BM - 1) / BM * ((a.N - p.head + p.bn - 1) / p.bn);
+    const int num_ks = (int)((a.K / 64 + kKbPerStage - 1) / kKbPerStage);
     if (a.force_kernel == 1 || c == 1) return a.force_kernel != 4 || p.head > 0;
-    return (a.force_kernel != 4 || p.head > 0) && (p.bn == 128 ? clusters_fit<128>(a.M, rest, a.K, c, dev, sms) : clusters_fit<256>(a.M, rest, a.K, c, dev, sms));
+    return (a.force_kernel != 4 || p.head > 0) && (p.bn == 128 ? clusters_fit<128>(tiles, num_ks, c, dev, sms) : clusters_fit<256>(tiles, num_ks, c, dev, sms));
 }
 
 cudaError_t launch_gemm_nvfp4(GemmArgs &a, cudaStream_t stream)
