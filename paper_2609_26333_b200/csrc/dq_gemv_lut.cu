@@ -208,6 +208,106 @@ __device__ __forceinline__ uint32_t x_offset(int i)
     return atom * 1024u + (bb >> 3) * 256u + (bb & 1u) * 128u + h * 64u + ((bb >> 1) & 3u) * 8u;
 }
 
+// Kernels of 16-row tiles: an atom (32 blocks) takes 1024 bytes ordered [word group 4][block pair 4][quarter t 4][block parity 2]
+// [4 weights], so that the B fragments lane (., t) needs for a pair of blocks are 16 contiguous bytes.  Byte offset of weights
+// 4t .. 4t+3 of block blk (0..63) of a slice of 1024:
+__device__ __forceinline__ uint32_t x16_offset(uint32_t blk, uint32_t t)
+{
+    return (blk >> 5) * 1024u + ((blk & 31u) >> 3) * 256u + ((blk & 7u) >> 1) * 64u + t * 16u + (blk & 1u) * 8u;
+}
+
+// ---- Activations of a pass (columns b0 .. b0 + cols - 1 of X), global memory -> fp16 in shared memory, one power-of-two scale for all
+__device__ __forceinline__ float max_magnitude(uint4 v, float m)
+{
+    // |bf16| pairs compare like unsigned integers once the sign bits are cleared
+    const uint32_t a0 = v.x & 0x7FFF7FFFu, a1 = v.y & 0x7FFF7FFFu, a2 = v.z & 0x7FFF7FFFu, a3 = v.w & 0x7FFF7FFFu;
+    const uint32_t hi = max(max(a0 >> 16, a1 >> 16), max(a2 >> 16, a3 >> 16));
+    const uint32_t lo = max(max(a0 & 0xFFFFu, a1 & 0xFFFFu), max(a2 & 0xFFFFu, a3 & 0xFFFFu));
+    return fmaxf(m, __uint_as_float(max(hi, lo) << 16));
+}
+// exponent of the largest magnitude of the CTA: floor(log2(max)); -127 for zero / subnormal
+__device__ __forceinline__ int max_exponent(float m, float *xmax_s)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) xmax_s[threadIdx.x >> 5] = m;
+    __syncthreads();
+    m = (lane < (int)(blockDim.x >> 5)) ? xmax_s[lane] : 0.0f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const int ex = (int)((__float_as_uint(m) >> 23) & 0xFFu) - 127;
+    return max(-100, min(100, ex));
+}
+// eight bf16 times a power of two as fp16
+__device__ __forceinline__ void scale_to_f16(uint2 va, uint2 vb, float xscale, uint32_t (&r)[4])
+{
+    const uint32_t ww[4] = {va.x, va.y, vb.x, vb.y};
+#pragma unroll
+    for (int z = 0; z < 4; ++z) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(ww[z] << 16) * xscale, __uint_as_float(ww[z] & 0xFFFF0000u) * xscale);
+        r[z] = *reinterpret_cast<const uint32_t *>(&h);
+    }
+}
+// Three columns and more: a warp takes whole atoms of 512 weights, whatever column they are in, four at a time, so that eight 16-byte
+// loads of a lane are in flight together where column after column each would wait for the one before (0.35 us a column; 6144x4096:
+// batch 4 9.8 -> 9.2 us, batch 8 11.3 -> 9.8; 34816x5120 batch 8 32.6 -> 30.3).  They are parked raw while the largest magnitude is
+// found and converted in place: an atom takes the same 1024 bytes raw and converted, and one warp reads all of it before it writes.  Up
+// to two columns there are too few atoms for the warps (6144x4096 batch 1 7.4 / 7.7).  One bulk copy per column instead of the loads
+// takes 0.8 us longer to arrive.  Returns the inverse of the scale.  ROWS16: the layout of 16-row tiles.
+template <bool ROWS16>
+__device__ __forceinline__ float load_columns(const __nv_bfloat16 *__restrict__ X, int64_t ldx, int b0, int cols, int K, int kpad, uint32_t xs,
+                                              uint32_t col_stride, float *xmax_s)
+{
+    constexpr int kBatch = 4;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int per_col = kpad >> 9, atoms = cols * per_col;
+    auto atom_at = [&](int a) { return xs + (uint32_t)(a / per_col) * col_stride + (uint32_t)(a % per_col) * 1024u; };
+    float m = 0.0f;
+    for (int a0 = warp; a0 < atoms; a0 += kBatch * nwarps) {
+        uint4 v[kBatch][2];
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int a = a0 + u * nwarps, c = a / per_col, k8 = (a % per_col) * 64 + lane;       // pieces of eight weights
+            const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)(b0 + c) * ldx) + k8;
+#pragma unroll
+            for (int j = 0; j < 2; ++j)                          // the padding of a short last slice reads as zero
+                v[u][j] = (a < atoms && k8 + 32 * j < K / 8) ? __ldg(xp + 32 * j) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            const int a = a0 + u * nwarps;
+            if (a >= atoms) break;
+            const uint32_t at = atom_at(a) + (uint32_t)lane * 16u;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                m = max_magnitude(v[u][j], m);
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(at + 512u * j), "r"(v[u][j].x), "r"(v[u][j].y), "r"(v[u][j].z), "r"(v[u][j].w) : "memory");
+            }
+        }
+    }
+    const int ex = max_exponent(m, xmax_s);
+    const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
+    for (int a = warp; a < atoms; a += nwarps) {
+        const uint32_t at = atom_at(a);
+        const uint4 v0 = lds_v4_at<0>(at + (uint32_t)lane * 16u), v1 = lds_v4_at<512>(at + (uint32_t)lane * 16u);
+        __syncwarp();                                                   // the atom is in registers
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const uint32_t i = (uint32_t)(lane + 32 * j);               // eight weights 8 i ..: a quarter pair of one block
+            const uint4 v = j ? v1 : v0;
+            const uint32_t dst = at + (ROWS16 ? x16_offset(i >> 1, (i & 1u) * 2u) : x_offset((int)i));
+            uint32_t r[4];
+            scale_to_f16(make_uint2(v.x, v.y), make_uint2(v.z, v.w), xscale, r);
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst), "r"(r[0]), "r"(r[1]) : "memory");
+            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst + (ROWS16 ? 16u : 32u)), "r"(r[2]), "r"(r[3]) : "memory");
+        }
+    }
+    __syncthreads();
+    return __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
+}
+
 __device__ __forceinline__ uint32_t lds_u32_volatile(uint32_t addr)
 {
     uint32_t v;
@@ -216,12 +316,16 @@ __device__ __forceinline__ uint32_t lds_u32_volatile(uint32_t addr)
 }
 __device__ __forceinline__ void fence_cta() { asm volatile("fence.acq_rel.cta;" ::: "memory"); }
 
-template <int BITS, int MAXT, int MINB, int CG, bool ONE>
+// CLS, the columns of a pass: 1 = one, two of the four accumulator columns are not kept up; 2 = one or two; 3 = three and more.  2 and 3 differ in
+// how the activations are loaded: with both ways in one instantiation the registers left to the main loop make one or two columns
+// slower (6144x4096 batch 1 7.4 -> 8.0 us, 4096x4096 batch 2 6.3 -> 6.9).
+template <int BITS, int MAXT, int MINB, int CG, int CLS>
 __global__ void __launch_bounds__(MAXT, MINB)
 gemv_lut_kernel(const uint8_t *__restrict__ lut, const PackedHeader *__restrict__ hdr,
                 const __nv_bfloat16 *__restrict__ X, int64_t ldx, int b0, int cols,
                 __nv_bfloat16 *__restrict__ Y, int64_t ldy, int N, int K, LutPlan L, StatusWord *status)
 {
+    constexpr bool ONE = CLS == 1;
     constexpr uint32_t kAtom = (uint32_t)lut_atom_bytes(BITS);
     constexpr uint32_t kChunk = 2u * kAtom;                 // one ring stage: 8 rows x 1024 weights
     constexpr uint32_t kPlanes = (uint32_t)lut_plane_bytes(BITS);
@@ -299,53 +403,39 @@ gemv_lut_kernel(const uint8_t *__restrict__ lut, const PackedHeader *__restrict_
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // ---- activations of this pass: one read from global memory (raw bf16 parked in shared memory, largest
-    //      magnitude on the way), then power-of-two scale -> fp16 in place
-    uint8_t *xh = smem_raw + L.x_off;
-    float m = 0.0f;
-    for (int c = 0; c < cols; ++c) {
-        const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)(b0 + c) * ldx);
-        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);                 // the padding of a short last slice reads as zero
-            if (i < K / 8) v = __ldg(xp + i);
-            // |bf16| pairs compare like unsigned integers once the sign bits are cleared
-            const uint32_t a0 = v.x & 0x7FFF7FFFu, a1 = v.y & 0x7FFF7FFFu, a2 = v.z & 0x7FFF7FFFu, a3 = v.w & 0x7FFF7FFFu;
-            const uint32_t hi = max(max(a0 >> 16, a1 >> 16), max(a2 >> 16, a3 >> 16));
-            const uint32_t lo = max(max(a0 & 0xFFFFu, a1 & 0xFFFFu), max(a2 & 0xFFFFu, a3 & 0xFFFFu));
-            m = fmaxf(m, __uint_as_float(max(hi, lo) << 16));
-            uint8_t *dst = xh + (size_t)c * L.col_stride + x_offset(i);
-            *reinterpret_cast<uint2 *>(dst) = make_uint2(v.x, v.y);
-            *reinterpret_cast<uint2 *>(dst + 32) = make_uint2(v.z, v.w);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) xmax_s[warp] = m;
-    __syncthreads();
-    m = (lane < nwarps) ? xmax_s[lane] : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    int ex = (int)((__float_as_uint(m) >> 23) & 0xFFu) - 127;           // floor(log2(max)); -127 for zero / subnormal
-    ex = max(-100, min(100, ex));
-    const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
-    const float xinv = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
-    for (int c = 0; c < cols; ++c) {
-        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {        // every thread converts what it parked itself
-            uint8_t *px = xh + (size_t)c * L.col_stride + x_offset(i);
-            const uint2 va = *reinterpret_cast<const uint2 *>(px), vb = *reinterpret_cast<const uint2 *>(px + 32);
-            const uint32_t ww[4] = {va.x, va.y, vb.x, vb.y};
-            uint32_t r[4];
-#pragma unroll
-            for (int z = 0; z < 4; ++z) {
-                const __half2 h = __floats2half2_rn(__uint_as_float(ww[z] << 16) * xscale,
-                                                    __uint_as_float(ww[z] & 0xFFFF0000u) * xscale);
-                r[z] = *reinterpret_cast<const uint32_t *>(&h);
+    float xinv;
+    if constexpr (CLS == 3) {
+        xinv = load_columns<false>(X, ldx, b0, cols, K, kpad, win0 + L.x_off, L.col_stride, xmax_s);
+    } else {
+        // one or two columns: the threads share a column piece by piece, raw bf16 parked in its place while the largest magnitude is found
+        uint8_t *xh = smem_raw + L.x_off;
+        float m = 0.0f;
+        for (int c = 0; c < cols; ++c) {
+            const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)(b0 + c) * ldx);
+            for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);                 // the padding of a short last slice reads as zero
+                if (i < K / 8) v = __ldg(xp + i);
+                m = max_magnitude(v, m);
+                uint8_t *dst = xh + (size_t)c * L.col_stride + x_offset(i);
+                *reinterpret_cast<uint2 *>(dst) = make_uint2(v.x, v.y);
+                *reinterpret_cast<uint2 *>(dst + 32) = make_uint2(v.z, v.w);
             }
-            *reinterpret_cast<uint2 *>(px) = make_uint2(r[0], r[1]);
-            *reinterpret_cast<uint2 *>(px + 32) = make_uint2(r[2], r[3]);
         }
+        const int ex = max_exponent(m, xmax_s);
+        const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
+        xinv = __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
+        for (int c = 0; c < cols; ++c) {
+            for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {        // every thread converts what it parked itself
+                uint8_t *px = xh + (size_t)c * L.col_stride + x_offset(i);
+                const uint2 va = *reinterpret_cast<const uint2 *>(px), vb = *reinterpret_cast<const uint2 *>(px + 32);
+                uint32_t r[4];
+                scale_to_f16(va, vb, xscale, r);
+                *reinterpret_cast<uint2 *>(px) = make_uint2(r[0], r[1]);
+                *reinterpret_cast<uint2 *>(px + 32) = make_uint2(r[2], r[3]);
+            }
+        }
+        __syncthreads();
     }
-    __syncthreads();
     const float out_scale = s_w * xinv;
     // B operand of this lane in column group c: column 4c + g % 4 (column 0 where the pass has fewer), block parity g / 4,
     // weights 4t .. 4t+3
@@ -496,7 +586,7 @@ give_up:
     }
 }
 
-template <int BITS, int MAXT, int MINB, int CG, bool ONE>
+template <int BITS, int MAXT, int MINB, int CG, int CLS>
 cudaError_t launch_one(const GemvArgs &a, int b0, int cols, int grid, int threads, const LutPlan &L, uint32_t smem,
                        cudaStream_t stream)
 {
@@ -505,13 +595,13 @@ cudaError_t launch_one(const GemvArgs &a, int b0, int cols, int grid, int thread
     if (!di) return cudaErrorInvalidDevice;
     const int dev = di->device;
     if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(gemv_lut_kernel<BITS, MAXT, MINB, CG, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(gemv_lut_kernel<BITS, MAXT, MINB, CG, CLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kSmemLimit);
         if (e != cudaSuccess) return e;
         // every instantiation asks for the same split of the SM's memory between L1 and shared memory: a change of
         // the split between two launches has to wait until the SM is empty, which would undo the overlap of one
         // launch's set-up with the tail of the launch before it
-        e = cudaFuncSetAttribute(gemv_lut_kernel<BITS, MAXT, MINB, CG, ONE>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        e = cudaFuncSetAttribute(gemv_lut_kernel<BITS, MAXT, MINB, CG, CLS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared);
         if (e != cudaSuccess) return e;
         attr_set[dev] = true;
@@ -526,7 +616,7 @@ cudaError_t launch_one(const GemvArgs &a, int b0, int cols, int grid, int thread
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemv_lut_kernel<BITS, MAXT, MINB, CG, ONE>, a.lut, a.hdr, reinterpret_cast<const __nv_bfloat16 *>(a.X),
+    return cudaLaunchKernelEx(&cfg, gemv_lut_kernel<BITS, MAXT, MINB, CG, CLS>, a.lut, a.hdr, reinterpret_cast<const __nv_bfloat16 *>(a.X),
                               (int64_t)a.ldx, b0, cols, reinterpret_cast<__nv_bfloat16 *>(a.Y), (int64_t)a.ldy, (int)a.N,
                               (int)a.K, L, a.status);
 }
@@ -548,13 +638,6 @@ struct WidePlan {
     long long wait_cycles;
 };
 
-// Activations of one column and slice, fp16: an atom (32 blocks) takes 1024 bytes ordered [word group 4][block pair 4]
-// [quarter t 4][block parity 2][4 weights], so that the B fragments lane (., t) needs for a pair of blocks are 16
-// contiguous bytes.  Byte offset of weights 4t .. 4t+3 of block blk (0..63) of the slice:
-__device__ __forceinline__ uint32_t x16_offset(uint32_t blk, uint32_t t)
-{
-    return (blk >> 5) * 1024u + ((blk & 31u) >> 3) * 256u + ((blk & 7u) >> 1) * 64u + t * 16u + (blk & 1u) * 8u;
-}
 
 // One word group of two atoms (rows g and g + 8 of the tile): eight blocks, one mma each per group of eight columns.
 template <int BITS, int WI, int CG8>
@@ -981,54 +1064,8 @@ gemv_lut_rows16_kernel(const uint8_t *__restrict__ lut, const PackedHeader *__re
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-    // ---- activations: raw bf16 parked in shared memory, largest magnitude on the way, then power-of-two scale -> fp16 in place
-    uint8_t *xh = smem_raw + L.x_off;
-    auto x_at = [&](int c, int i) {                              // eight weights 8 i .. 8 i + 7 of column c; the other quarter 16 bytes on
-        return xh + (size_t)c * L.col_stride + (size_t)(i >> 7) * 2048u + x16_offset(((uint32_t)i >> 1) & 63u, ((uint32_t)i & 1u) * 2u);
-    };
-    float m = 0.0f;
-    for (int c = 0; c < cols; ++c) {
-        const uint4 *xp = reinterpret_cast<const uint4 *>(X + (int64_t)(b0 + c) * ldx);
-        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);                 // the padding of a short last slice reads as zero
-            if (i < K / 8) v = __ldg(xp + i);
-            const uint32_t a0 = v.x & 0x7FFF7FFFu, a1 = v.y & 0x7FFF7FFFu, a2 = v.z & 0x7FFF7FFFu, a3 = v.w & 0x7FFF7FFFu;
-            const uint32_t hi = max(max(a0 >> 16, a1 >> 16), max(a2 >> 16, a3 >> 16));
-            const uint32_t lo = max(max(a0 & 0xFFFFu, a1 & 0xFFFFu), max(a2 & 0xFFFFu, a3 & 0xFFFFu));
-            m = fmaxf(m, __uint_as_float(max(hi, lo) << 16));
-            uint8_t *dst = x_at(c, i);
-            *reinterpret_cast<uint2 *>(dst) = make_uint2(v.x, v.y);
-            *reinterpret_cast<uint2 *>(dst + 16) = make_uint2(v.z, v.w);
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) xmax_s[warp] = m;
-    __syncthreads();
-    m = (lane < nwarps) ? xmax_s[lane] : 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    int ex = (int)((__float_as_uint(m) >> 23) & 0xFFu) - 127;           // floor(log2(max)); -127 for zero / subnormal
-    ex = max(-100, min(100, ex));
-    const float xscale = __uint_as_float((uint32_t)(127 + 14 - ex) << 23);   // 2^(14 - ex)
-    const float out_scale = s_w * __uint_as_float((uint32_t)(127 - 14 + ex) << 23);
-    for (int c = 0; c < cols; ++c) {
-        for (int i = threadIdx.x; i < kpad / 8; i += blockDim.x) {        // every thread converts what it parked itself
-            uint8_t *px = x_at(c, i);
-            const uint2 va = *reinterpret_cast<const uint2 *>(px), vb = *reinterpret_cast<const uint2 *>(px + 16);
-            const uint32_t ww[4] = {va.x, va.y, vb.x, vb.y};
-            uint32_t r[4];
-#pragma unroll
-            for (int z = 0; z < 4; ++z) {
-                const __half2 h = __floats2half2_rn(__uint_as_float(ww[z] << 16) * xscale,
-                                                    __uint_as_float(ww[z] & 0xFFFF0000u) * xscale);
-                r[z] = *reinterpret_cast<const uint32_t *>(&h);
-            }
-            *reinterpret_cast<uint2 *>(px) = make_uint2(r[0], r[1]);
-            *reinterpret_cast<uint2 *>(px + 16) = make_uint2(r[2], r[3]);
-        }
-    }
-    __syncthreads();
+    const float xinv = load_columns<true>(X, ldx, b0, cols, K, kpad, win0 + L.x_off, L.col_stride, xmax_s);
+    const float out_scale = s_w * xinv;
     // B operand of this lane: column g (column 0 where the pass has fewer), weights 4t .. 4t+3 of a pair of blocks per 16-byte load
     const uint32_t xlane = win0 + L.x_off + (uint32_t)(g < cols ? g : 0) * L.col_stride + (uint32_t)t * 16u;
     const uint32_t lane_plane = (uint32_t)lane * 16u;
@@ -1303,20 +1340,24 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
                                uint32_t smem, cudaStream_t stream)
 {
     const int cg = col_groups(cols);
+    const bool few = cols <= 2;
     if (slots == 2 && threads <= 384 && grid > 148) {
         // a single column with at most 8 warps per CTA: the variant that keeps up two of the four accumulator columns
         // (it needs more than 80 registers to gain from that)
-        if (cols == 1 && threads <= 256) return launch_one<BITS, 256, 2, 1, true>(a, b0, cols, grid, threads, L, smem, stream);
-        if (cg == 1) return launch_one<BITS, 384, 2, 1, false>(a, b0, cols, grid, threads, L, smem, stream);
-        return launch_one<BITS, 384, 2, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
+        if (cols == 1 && threads <= 256) return launch_one<BITS, 256, 2, 1, 1>(a, b0, cols, grid, threads, L, smem, stream);
+        if (few) return launch_one<BITS, 384, 2, 1, 2>(a, b0, cols, grid, threads, L, smem, stream);
+        if (cg == 1) return launch_one<BITS, 384, 2, 1, 3>(a, b0, cols, grid, threads, L, smem, stream);
+        return launch_one<BITS, 384, 2, 2, 3>(a, b0, cols, grid, threads, L, smem, stream);
     }
-    if (cols == 1 && threads <= 640) return launch_one<BITS, 640, 1, 1, true>(a, b0, cols, grid, threads, L, smem, stream);
+    if (cols == 1 && threads <= 640) return launch_one<BITS, 640, 1, 1, 1>(a, b0, cols, grid, threads, L, smem, stream);
     if (threads <= 768) {
-        if (cg == 1) return launch_one<BITS, 768, 1, 1, false>(a, b0, cols, grid, threads, L, smem, stream);
-        return launch_one<BITS, 768, 1, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
+        if (few) return launch_one<BITS, 768, 1, 1, 2>(a, b0, cols, grid, threads, L, smem, stream);
+        if (cg == 1) return launch_one<BITS, 768, 1, 1, 3>(a, b0, cols, grid, threads, L, smem, stream);
+        return launch_one<BITS, 768, 1, 2, 3>(a, b0, cols, grid, threads, L, smem, stream);
     }
-    if (cg == 1) return launch_one<BITS, 1024, 1, 1, false>(a, b0, cols, grid, threads, L, smem, stream);
-    return launch_one<BITS, 1024, 1, 2, false>(a, b0, cols, grid, threads, L, smem, stream);
+    if (few) return launch_one<BITS, 1024, 1, 1, 2>(a, b0, cols, grid, threads, L, smem, stream);
+    if (cg == 1) return launch_one<BITS, 1024, 1, 1, 3>(a, b0, cols, grid, threads, L, smem, stream);
+    return launch_one<BITS, 1024, 1, 2, 3>(a, b0, cols, grid, threads, L, smem, stream);
 }
 
 // The choices between the kernels, from launch after launch of one matrix (LUT3 and LUT2; us).
