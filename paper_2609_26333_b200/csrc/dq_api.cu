@@ -230,14 +230,14 @@ int dq_pack_weights(const void *W_dev, int w_dtype, int64_t N, int64_t K, int64_
     uint8_t *codes = (formats & DQ_FMT_NVFP4) ? base + L.nv_codes_off : nullptr;
     uint8_t *sf = codes ? base + L.nv_sf_off : nullptr;
     if (formats & DQ_FMT_LUT3) {
-        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, base + L.lut_off, 3, s) != cudaSuccess) return DQ_ERR_CUDA;
+        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, cb, hdr, codes, sf, base + L.lut_off, 3, s) != cudaSuccess) return DQ_ERR_CUDA;
         codes = sf = nullptr;
     }
     if (formats & DQ_FMT_LUT2) {
-        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, base + L.lut2_off, 2, s) != cudaSuccess) return DQ_ERR_CUDA;
+        if (dq::launch_pack(W_dev, w_dtype, N, K, ldw, cb, hdr, codes, sf, base + L.lut2_off, 2, s) != cudaSuccess) return DQ_ERR_CUDA;
         codes = sf = nullptr;
     }
-    if (codes && dq::launch_pack(W_dev, w_dtype, N, K, ldw, hdr, codes, sf, nullptr, 0, s) != cudaSuccess) return DQ_ERR_CUDA;
+    if (codes && dq::launch_pack(W_dev, w_dtype, N, K, ldw, cb, hdr, codes, sf, nullptr, 0, s) != cudaSuccess) return DQ_ERR_CUDA;
     if (formats & DQ_FMT_NVFP4_FROM_LUT3) {
         if (dq::launch_autocast(hdr, base + L.lut_off, N, K, base + L.nv_codes_off, base + L.nv_sf_off, s) !=
             cudaSuccess)

@@ -177,8 +177,8 @@ cudaError_t launch_pack_header(PackedHeader *hdr, const uint16_t *codebook_f16_h
 cudaError_t launch_absmax(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
                           cudaStream_t stream);
 // one pass over W: NVFP4 where codes is not null, a LUT format where bits is 3 (LUT3) or 2 (LUT2); writes hdr->s, hdr->rc6
-cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes,
-                        uint8_t *sf_swizzled, uint8_t *lut_dev, int bits, cudaStream_t stream);
+cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, const uint16_t *codebook_f16_host, PackedHeader *hdr,
+                        uint8_t *codes, uint8_t *sf_swizzled, uint8_t *lut_dev, int bits, cudaStream_t stream);
 // bits = 3 (LUT3) or 2 (LUT2) in the two LUT launchers below
 cudaError_t launch_autocast(const PackedHeader *hdr, const uint8_t *lut_dev, int64_t N,
                             int64_t K, uint8_t *codes, uint8_t *sf_swizzled, cudaStream_t stream);

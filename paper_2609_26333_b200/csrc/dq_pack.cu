@@ -5,6 +5,8 @@
 // Quantiser arithmetic is fp32 with explicit round-to-nearest intrinsics so the
 // compiler cannot contract or reorder it:
 //   rc6 = 1/(6 s);  t = extreme * rc6;  d = E4M3(t);  r = 1/(s * dec(d));  y = x * r
+#include <atomic>
+
 #include "dq_common.cuh"
 #include "dq_quant.cuh"
 
@@ -71,6 +73,12 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b)
 {
     uint32_t r;
     asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ uint32_t min_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("min.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
     return r;
 }
 // Largest magnitude of W: one streaming read, four 16-byte loads in flight per thread.  grid.y walks rows, grid.x the
@@ -146,16 +154,16 @@ __device__ __forceinline__ float tensor_scale(const PackedHeader *hdr)
     return (amax == 0.0f) ? 1.0f : __fdiv_rn(amax, 2688.0f);
 }
 
-// four floats -> two bytes of E2M1 codes (element 0 in the low nibble of byte 0)
-__device__ __forceinline__ uint32_t f32x4_to_e2m1x4(float f0, float f1, float f2, float f3)
+// four floats -> two bytes of E2M1 codes (element 0 in the low nibble of byte 0), at the low end
+__device__ __forceinline__ uint32_t f32x4_to_e2m1x4(const float (&f)[4])
 {
     uint32_t r;
     asm("{\n\t.reg .b8 b0, b1;\n\t"
         "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
         "cvt.rn.satfinite.e2m1x2.f32 b1, %4, %3;\n\t"
         "mov.b32 %0, {b0, b1, b0, b1};\n\t}"
-        : "=r"(r) : "f"(f0), "f"(f1), "f"(f2), "f"(f3));
-    return r & 0xFFFFu;
+        : "=r"(r) : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]));
+    return r;
 }
 // Transpose of 16-bit pieces between the four threads of a quad.  Thread t comes with v[j] = its pieces of blocks 2j (low
 // half) and 2j + 1 (high half) and leaves with the sixteen bytes of blocks 2t and 2t + 1, pieces in thread order.
@@ -173,192 +181,351 @@ __device__ __forceinline__ uint4 quad_transpose(const uint32_t (&v)[4], int t)
                       __byte_perm(u2, u3, 0x7632));
 }
 
-// Number of thresholds below y (the index of the nearest level, a value on a threshold taking the lower level), as index
-// bits in the sign bits of the results: T - y is negative exactly where y > T, and with increasing thresholds the bits of the count
-// are parities of those signs.
-template <int BITS>
-__device__ __forceinline__ void level_bits(float y, const float (&T)[(1 << BITS) - 1], uint32_t (&bit)[BITS])
+// Number of thresholds below y (the index of the nearest level, a value on a threshold taking the lower level).  The line is cut into
+// kBins bins, the outermost open-ended, none of which holds more than one threshold (pack_bins_fit); a bin's entry, found through
+// y's place on the line, says how many thresholds lie below the bin and where its own is, and one multiply-add that saturates at 0 and
+// 1 compares with that: y * 2^60 - T * 2^60 is rounded once, so it is positive exactly where y > T, and then at least 1.  A NaN
+// counts none: the saturated place of a NaN is 0, and so is the comparison.  Entries are 8 bytes, one copy per lane: no bank conflicts.
+// Nearly all of it is multiply-adds, whose pipe has room beside the logic, shifts and converts of the rest.
+constexpr int kBins = 64;
+constexpr float kBinSpan = 32.0f;                          // places from -16 to 16
+constexpr float kCmpScale = 1152921504606846976.0f;        // 2^60; thresholds are multiples of 2^-25 and at most 65504
+constexpr float kBinSlack = 1e-3f;                         // the place is rounded: by how much a bin may reach beyond its edges (2^-18 at most)
+__host__ __device__ inline float bin_edge(int b) { return ((float)b / (float)(kBins - 1) - 0.5f) * kBinSpan; }
+// thresholds (ascending) below bin b, and the one inside it or +inf; false where it holds more
+__host__ __device__ inline bool bin_entry(const float *T, int n, int b, int &below, float &own)
 {
-    uint32_t d[(1 << BITS) - 1];
-#pragma unroll
-    for (int l = 0; l < (1 << BITS) - 1; ++l) d[l] = __float_as_uint(__fsub_rn(T[l], y));
-    if (BITS == 3) {
-        bit[BITS - 1] = d[3];
-        bit[1] = d[1] ^ d[3] ^ d[BITS == 3 ? 5 : 0];
-        bit[0] = (d[0] ^ d[1] ^ d[2]) ^ (d[3] ^ d[BITS == 3 ? 4 : 0] ^ d[BITS == 3 ? 5 : 0]) ^ d[BITS == 3 ? 6 : 0];
-    } else {
-        bit[1] = d[1];
-        bit[0] = d[0] ^ d[1] ^ d[2];
+    below = 0;
+    own = INFINITY;
+    int inside = 0;
+    for (int l = 0; l < n; ++l) {
+        if (b > 0 && T[l] < bin_edge(b) - kBinSlack) ++below;
+        else if (b == kBins - 1 || T[l] <= bin_edge(b + 1) + kBinSlack) { if (inside++ == 0) own = T[l]; }
     }
+    return inside <= 1;
 }
-// appends a nibble [index bits, BITS of them][garbage bit] at the low end of acc (LUT2: [0][bits][garbage])
-template <int BITS>
-__device__ __forceinline__ uint32_t push_level(uint32_t acc, const uint32_t (&bit)[BITS])
+__device__ __forceinline__ float ffma_sat(float a, float b, float c)
 {
-    if (BITS == 2) acc <<= 1;
+    float r;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+// appends the level of y to a number in base 16
+__device__ __forceinline__ float push_level(float acc, float y, const float2 *bins, uint32_t lane8)
+{
+    const float place = ffma_sat(y, 1.0f / kBinSpan, 0.5f);
+    const uint32_t at = (__float_as_uint(__fmaf_rn(place, (float)(256 * (kBins - 1)), 8388608.0f)) & (uint32_t)(256 * (kBins - 1))) | lane8;
+    const float2 e = *reinterpret_cast<const float2 *>(reinterpret_cast<const uint8_t *>(bins) + at);
+    return __fadd_rn(__fmaf_rn(acc, 16.0f, e.x), ffma_sat(y, kCmpScale, e.y));
+}
+// The same by comparing with every threshold, for codebooks with two of them in a bin: T - y is negative exactly where y > T.
+template <int N>
+__device__ __forceinline__ float push_level_all(float acc, float y, const float (&T)[N])
+{
+    uint32_t n = 0;
 #pragma unroll
-    for (int b = BITS - 1; b > 0; --b) acc = __funnelshift_l(bit[b], acc, 1);
-    return __funnelshift_l(bit[0], acc, 2);
+    for (int l = 0; l < N; ++l) n += __float_as_uint(__fsub_rn(T[l], y)) >> 31;
+    return __fmaf_rn(acc, 16.0f, (float)n);
+}
+
+// Transpose of 32-bit words between the four threads of a quad: thread t comes with v[q] and leaves with word t of threads 0..3
+__device__ __forceinline__ void quad_transpose_words(uint32_t (&v)[4], int t)
+{
+    const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
+    const uint32_t a0 = hi2 ? v[2] : v[0], a1 = hi2 ? v[3] : v[1];
+    const uint32_t b0 = __shfl_xor_sync(0xffffffffu, hi2 ? v[0] : v[2], 2), b1 = __shfl_xor_sync(0xffffffffu, hi2 ? v[1] : v[3], 2);
+    const uint32_t k0 = hi1 ? a1 : a0, k1 = hi1 ? b1 : b0;              // of threads t and t ^ 2
+    const uint32_t g0 = __shfl_xor_sync(0xffffffffu, hi1 ? a0 : a1, 1), g1 = __shfl_xor_sync(0xffffffffu, hi1 ? b0 : b1, 1);
+    const uint32_t p0 = hi1 ? g0 : k0, p1 = hi1 ? k0 : g0, q0 = hi1 ? g1 : k1, q1 = hi1 ? k1 : g1;
+    v[0] = hi2 ? q0 : p0;
+    v[1] = hi2 ? q1 : p1;
+    v[2] = hi2 ? p0 : q0;
+    v[3] = hi2 ? p1 : q1;
+}
+
+// CTAs per SM: what the registers of bf16, and the copy buffers of fp32, leave room for
+constexpr int pack_ctas(bool fp32) { return fp32 ? 2 : 4; }
+__host__ __device__ constexpr int pack_stage_bytes(bool fp32) { return 8 * 128 * (fp32 ? 4 : 2); }      // one word group of a warp: 8 rows x 128 weights
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
 // Round-to-nearest packing of the master weights (App. A.3): NVFP4 (NV) and / or one LUT format (BITS = 3 or 2) in one
-// read of W.  A warp takes an atom of 8 rows x 512 weights; lane (g, t) = (row, quarter of a 16-block) takes weights
-// 4t .. 4t+3 of every block of its row, which is what its index words of the LUT layout store, 128 weights at a time.
-// Both encodings share the block's largest magnitude, its E4M3 scale and the reciprocal (a table of the 127 scales per CTA);
-// index words and scales leave as whole 512- and 256-byte rows of the atom, E2M1 codes after a transpose inside
-// the quad as 16 bytes per lane.
-// Bound by instruction issue (the thresholds: 7 subtractions, 4 logic ops and 3 shifts per weight).  17408 x 5120 bf16 to
-// NVFP4 and LUT3: 116 us, 2.3 TB/s; a pass per format with compares and one bit placed at a time took about 250.
-template <bool FP32IN, bool NV, int BITS>
-__global__ void __launch_bounds__(128) pack_kernel(const void *__restrict__ W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
-                                                   uint8_t *__restrict__ codes, uint8_t *__restrict__ sf, uint8_t *__restrict__ lut)
+// read of W.  A warp takes atoms of 8 rows x 512 weights, 128 weights (eight blocks) of every row at a time; lane (g, t) takes blocks
+// 2t and 2t + 1 of row g whole: extremes, scale and reciprocal (a table of the 127 scales per CTA), which serve both encodings, are its
+// own, and its E2M1 codes are 16 bytes of the output as they are.  The index words of the LUT layout hold quarters of eight blocks:
+// one transpose inside the quad brings them about.  Index words and scales leave as whole 512- and 256-byte rows of the atom.
+// The next word group is on its way to shared memory meanwhile (loaded straight into registers, a lane's 64 or 128 contiguous bytes touch
+// 16 or 32 lines per instruction); its 16-byte pieces are placed so that the lanes' reads hit different banks.
+// Bound by instruction issue.  17408 x 5120 bf16 to NVFP4 and LUT3: 73 us, 3.4 TB/s; with a quarter of every block per lane, its extremes reduced
+// and its scale made in all four lanes of the quad, and seven subtractions and seven logic operations and shifts per weight, 116 us.
+template <bool FP32IN, bool NV, int BITS, bool BINNED>
+__global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void *__restrict__ W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr,
+                                                                      uint8_t *__restrict__ codes, uint8_t *__restrict__ sf, uint8_t *__restrict__ lut)
 {
     constexpr bool LUT = BITS > 0;
     constexpr int B = LUT ? BITS : 2;                      // dummy where there is no LUT format
+    constexpr int NT = (1 << B) - 1;
+    __shared__ float2 bins[LUT && BINNED ? kBins * 32 : 1];
     __shared__ float rtab[128];                            // 1 / (s * d) by the byte of d; 0 for a scale that rounded to zero
+    extern __shared__ __align__(128) uint8_t stages[];     // [warp][2]
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const float s = tensor_scale(hdr);
     const float rc6 = __frcp_rn(__fmul_rn(6.0f, s));
     if (blockIdx.x == 0 && threadIdx.x == 0) { hdr->s = s; hdr->rc6 = rc6; }
-    rtab[threadIdx.x] = (threadIdx.x == 0) ? 0.0f : __frcp_rn(__fmul_rn(s, e4m3_to_f32(threadIdx.x)));
+    if (threadIdx.x < 128) rtab[threadIdx.x] = (threadIdx.x == 0) ? 0.0f : __frcp_rn(__fmul_rn(s, e4m3_to_f32(threadIdx.x)));
+    float T[NT];
+    if (LUT) {
+#pragma unroll
+        for (int l = 0; l < NT; ++l) T[l] = (BITS == 3) ? hdr->lut_thresholds[l] : hdr->lut2_thresholds[l & 3];
+    }
+    if (LUT && BINNED) {
+        for (int b = threadIdx.x >> 5; b < kBins; b += 8) {
+            int below;
+            float own;
+            bin_entry(T, NT, b, below, own);
+            bins[b * 32 + lane] = make_float2((float)below, __fmul_rn(own, -kCmpScale));
+        }
+    }
     __syncthreads();
     const uint32_t atoms_k = (uint32_t)(2 * lut_slices(K));               // atoms along a row, a short last slice padded
     const uint32_t katoms = NV && !LUT ? (uint32_t)((K + 511) / 512) : atoms_k;
-    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int64_t rowgrp = task / katoms;
-    if (rowgrp >= N / 8) return;
-    const uint32_t atom = (uint32_t)(task - rowgrp * katoms);
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t r = rowgrp * 8 + g;
-    const int nwi = max(0, min(4, (int)(K / 128) - 4 * (int)atom));
-    float T[(1 << B) - 1];
-    if (LUT) {
+    // tasks of this warp: atoms first, first + step, .. in row-major order, as (rows of eight, atom of the row) without a division each
+    const uint32_t step = gridDim.x * 8u, step_row = step / katoms, step_atom = step - step_row * katoms;
+    const uint32_t first = blockIdx.x * 8u + (threadIdx.x >> 5), rowgrps = (uint32_t)(N / 8);
+    struct Task { uint32_t row, atom; int groups; };                      // groups: word groups inside K, 0 for padding
+    const int kgroups = (int)(K / 128);
+    auto count = [&](Task &q) { q.groups = max(0, min(4, kgroups - 4 * (int)q.atom)); };
+    auto next = [&](Task &q) {
+        q.row += step_row;
+        q.atom += step_atom;
+        if (q.atom >= katoms) { q.atom -= katoms; ++q.row; }
+        count(q);
+    };
+    Task task = {first / katoms, first % katoms, 0};
+    count(task);
+
+    // copies: the word groups of this warp's tasks in turn, one ahead of the one in work.  Piece c of a row (16 bytes) goes to place
+    // c ^ swizzle: the four lanes of a quad and the rows g, g + 1 that read together then find theirs in eight different places of 128 bytes.
+    constexpr int kElem = FP32IN ? 4 : 2, kRow = 128 * kElem / 16, kPieces = kElem;      // pieces of a row, of a block
+    constexpr uint32_t kStage = (uint32_t)pack_stage_bytes(FP32IN);
+    const uint32_t ring = (uint32_t)__cvta_generic_to_shared(stages) + (threadIdx.x >> 5) * 2u * kStage;
+    auto swizzle = [](int row, int c) { return FP32IN ? (c >> 3) | ((row & 1) << 2) : (c >> 3) | ((row & 1) << 1); };
+    // an instruction copies 32 pieces: two rows of bf16 or one of fp32
+    constexpr int kRowsPer = 32 / kRow;
+    const int prow = lane / kRow, pc = lane % kRow;
+    const int64_t row_bytes = ldw * kElem, lane_src = prow * row_bytes + pc * 16;
+    Task ptask = task;
+    while (ptask.row < rowgrps && ptask.groups == 0) next(ptask);
+    auto source = [&]() { return reinterpret_cast<const uint8_t *>(W) + (int64_t)ptask.row * (8 * row_bytes) + (int64_t)ptask.atom * (512 * kElem) + lane_src; };
+    const uint8_t *psrc = source();
+    uint32_t pstage = 0;
+    auto copy_next = [&]() {
+        if (ptask.row < rowgrps) {
+            const uint8_t *q = psrc;
 #pragma unroll
-        for (int l = 0; l < (1 << B) - 1; ++l) T[l] = (BITS == 3) ? hdr->lut_thresholds[l] : hdr->lut2_thresholds[l & 3];
-    }
-    uint4 *out_codes = nullptr;
-    uint32_t *out_sf = nullptr;
-    if (NV) {
-        out_codes = reinterpret_cast<uint4 *>(codes + r * (K / 2) + (int64_t)atom * 256 + t * 16);
-        out_sf = reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, (int64_t)atom * 32 + 4 * (t & 1), K));
-    }
-    const int64_t src = r * ldw + (int64_t)atom * 512 + t * 4;
-    uint32_t words[4][B];
-    uint2 my_scales = make_uint2(0u, 0u);                  // LUT scale bytes of word group t
-#pragma unroll
-    for (int wi = 0; wi < 4; ++wi) {
-#pragma unroll
-        for (int p = 0; p < B; ++p) words[wi][p] = 0u;
-        if (wi >= nwi) continue;                           // whole warps
-        uint4 raw[8];                                      // bf16: two words of it are used
-#pragma unroll
-        for (int bb = 0; bb < 8; ++bb) {
-            if (FP32IN) {
-                raw[bb] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const float *>(W) + src + wi * 128 + bb * 16));
-            } else {
-                const uint2 v = __ldg(reinterpret_cast<const uint2 *>(reinterpret_cast<const __nv_bfloat16 *>(W) + src + wi * 128 + bb * 16));
-                raw[bb] = make_uint4(v.x, v.y, 0u, 0u);
+            for (int i = 0; i < kRow / 4; ++i, q += kRowsPer * row_bytes) {
+                const int row = i * kRowsPer + (kRowsPer > 1 ? prow : 0);
+                copy16(ring + pstage + (uint32_t)(row * kRow + (pc ^ swizzle(row, pc))) * 16u, q);
+            }
+            psrc += 128 * kElem;
+            if (--ptask.groups == 0) {
+                do next(ptask); while (ptask.row < rowgrps && ptask.groups == 0);
+                psrc = source();
             }
         }
-        uint32_t nv_pieces[4] = {0u, 0u, 0u, 0u};
-        uint32_t nv_sc[2] = {0u, 0u}, lut_sc[2] = {0u, 0u};
-        uint32_t sel[4];
+        pstage ^= kStage;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    copy_next();
+    uint32_t cstage = 0;
+    for (; task.row < rowgrps; next(task)) {
+        const int64_t rowgrp = task.row;
+        const uint32_t atom = task.atom;
+        const int64_t r = rowgrp * 8 + g;
+        const int nwi = task.groups;
+        uint4 *out_codes = nullptr;
+        uint32_t *out_sf = nullptr;
+        if (NV) {
+            out_codes = reinterpret_cast<uint4 *>(codes + r * (K / 2) + (int64_t)atom * 256 + t * 16);
+            out_sf = reinterpret_cast<uint32_t *>(sf + sf_swizzled_offset(r, (int64_t)atom * 32 + 4 * (t >> 1), K));
+        }
+        uint32_t words[4][B];
+        uint2 my_scales = make_uint2(0u, 0u);              // LUT scale bytes of word group t
 #pragma unroll
-        for (int a = 3; a >= 0; --a) {
-            uint32_t acc = 0u;
+        for (int wi = 0; wi < 4; ++wi) {
 #pragma unroll
-            for (int h = 1; h >= 0; --h) {                 // selector nibbles from the top: second block first
-                const int bb = 2 * a + h;
-                // largest and most negative value of the block across the quad
-                float mx, mn;
-                float x[4];
+            for (int p = 0; p < B; ++p) words[wi][p] = 0u;
+            if (wi >= nwi) continue;                       // whole warps
+            __syncwarp();                                  // everybody has read the stage that is filled next
+            copy_next();
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            __syncwarp();
+            uint4 raw[2][kPieces];
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int i = 0; i < kPieces; ++i) {
+                    const int c = (2 * t + j) * kPieces + i;
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(raw[j][i].x), "=r"(raw[j][i].y), "=r"(raw[j][i].z), "=r"(raw[j][i].w)
+                                 : "r"(ring + cstage + (uint32_t)(g * kRow + (c ^ swizzle(g, c))) * 16u) : "memory");
+                }
+            cstage ^= kStage;
+            float rs[2];
+            uint32_t sc = 0;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                float mx, mn;                              // largest value and largest of the negated values
                 if (FP32IN) {
-                    x[0] = __uint_as_float(raw[bb].x); x[1] = __uint_as_float(raw[bb].y);
-                    x[2] = __uint_as_float(raw[bb].z); x[3] = __uint_as_float(raw[bb].w);
-                    mx = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
-                    mn = fmaxf(fmaxf(-x[0], -x[1]), fmaxf(-x[2], -x[3]));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-                    mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 1));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-                    mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, 2));
+                    mx = mn = -INFINITY;
+#pragma unroll
+                    for (int i = 0; i < kPieces; ++i) {
+                        const float x0 = __uint_as_float(raw[j][i].x), x1 = __uint_as_float(raw[j][i].y), x2 = __uint_as_float(raw[j][i].z), x3 = __uint_as_float(raw[j][i].w);
+                        mx = fmaxf(mx, fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)));
+                        mn = fmaxf(mn, fmaxf(fmaxf(-x0, -x1), fmaxf(-x2, -x3)));
+                    }
                 } else {
-                    x[0] = __uint_as_float(raw[bb].x << 16); x[1] = __uint_as_float(raw[bb].x & 0xFFFF0000u);
-                    x[2] = __uint_as_float(raw[bb].y << 16); x[3] = __uint_as_float(raw[bb].y & 0xFFFF0000u);
-                    const uint32_t pm = max_bf16x2(raw[bb].x, raw[bb].y);
-                    const uint32_t nm = max_bf16x2(raw[bb].x ^ 0x80008000u, raw[bb].y ^ 0x80008000u);
-                    uint32_t e = max_bf16x2(__byte_perm(pm, nm, 0x5410), __byte_perm(pm, nm, 0x7632));    // (max, -min)
-                    e = max_bf16x2(e, __shfl_xor_sync(0xffffffffu, e, 1));
-                    e = max_bf16x2(e, __shfl_xor_sync(0xffffffffu, e, 2));
-                    mx = __uint_as_float(e << 16);
-                    mn = __uint_as_float(e & 0xFFFF0000u);
+                    const uint4 u = raw[j][0], v = raw[j][1];
+                    const uint32_t hi = max_bf16x2(max_bf16x2(max_bf16x2(u.x, u.y), max_bf16x2(u.z, u.w)), max_bf16x2(max_bf16x2(v.x, v.y), max_bf16x2(v.z, v.w)));
+                    const uint32_t lo = min_bf16x2(min_bf16x2(min_bf16x2(u.x, u.y), min_bf16x2(u.z, u.w)), min_bf16x2(min_bf16x2(v.x, v.y), min_bf16x2(v.z, v.w)));
+                    mx = fmaxf(__uint_as_float(hi << 16), __uint_as_float(hi & 0xFFFF0000u));
+                    mn = -fminf(__uint_as_float(lo << 16), __uint_as_float(lo & 0xFFFF0000u));
                 }
+                // the LUT scale takes the sign of the block's extreme, and the reciprocal with it: where both signs reach the
+                // magnitude, plus
                 const uint32_t d8 = f32_to_e4m3(__fmul_rn(fmaxf(mx, mn), rc6)) & 0x7Fu;
+                const bool neg = LUT && mn > mx;
                 const float rr = rtab[d8];
-                if (NV) {
-                    const uint32_t c = f32x4_to_e2m1x4(__fmul_rn(x[0], rr), __fmul_rn(x[1], rr), __fmul_rn(x[2], rr), __fmul_rn(x[3], rr));
-                    nv_pieces[a] |= (d8 ? c : 0u) << (16 * h);
-                    nv_sc[bb >> 2] |= d8 << (8 * (bb & 3));
-                }
-                if (LUT) {
-                    // the scale takes the sign of the block's extreme; where both signs reach the magnitude, plus
-                    const bool neg = mn > mx;
-                    lut_sc[bb >> 2] |= (d8 ? (d8 | (neg ? 0x80u : 0u)) : 0u) << (8 * (bb & 3));
-                    const float rs = neg ? -rr : rr;
+                rs[j] = neg ? -rr : rr;
+                sc |= (neg && d8 ? d8 | 0x80u : d8) << (8 * j);
+            }
+            const bool zeros = NV && __any_sync(0xffffffffu, !((sc & 0x7Fu) && (sc & 0x7F00u)));
+            const uint32_t s4 = __shfl_xor_sync(0xffffffffu, sc, 1);
+            const uint32_t sc4 = (t & 1) ? (sc << 16) | s4 : (s4 << 16) | sc;     // blocks 4 (t / 2) .. + 3
+            if (LUT) {
+                const uint32_t so = __shfl_xor_sync(0xffffffffu, sc4, 2);
+                if (t == wi) my_scales = (t & 2) ? make_uint2(so, sc4) : make_uint2(sc4, so);
+            }
+            uint32_t cw[4], sel[4];                        // E2M1 codes; levels, quarter q of both blocks
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                float acc[2];
+                uint32_t c2[2];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    float y[4];
+                    if (FP32IN) {
+                        const uint4 v = raw[j][FP32IN ? q : 0];
+                        y[0] = __uint_as_float(v.x); y[1] = __uint_as_float(v.y); y[2] = __uint_as_float(v.z); y[3] = __uint_as_float(v.w);
+                    } else {
+                        const uint4 v = raw[j][q >> 1];
+                        const uint32_t w0 = (q & 1) ? v.z : v.x, w1 = (q & 1) ? v.w : v.y;
+                        y[0] = __uint_as_float(w0 << 16); y[1] = __uint_as_float(w0 & 0xFFFF0000u);
+                        y[2] = __uint_as_float(w1 << 16); y[3] = __uint_as_float(w1 & 0xFFFF0000u);
+                    }
+                    acc[j] = 0.0f;
 #pragma unroll
                     for (int n4 = 3; n4 >= 0; --n4) {
-                        uint32_t bit[B];
-                        level_bits<B>(__fmul_rn(x[n4], rs), T, bit);
-                        acc = push_level<B>(acc, bit);
+                        y[n4] = __fmul_rn(y[n4], rs[j]);
+                        if (LUT) acc[j] = BINNED ? push_level(acc[j], y[n4], bins, (uint32_t)lane * 8u) : push_level_all(acc[j], y[n4], T);
                     }
+                    if (NV) c2[j] = f32x4_to_e2m1x4(y);
+                }
+                if (NV) {
+                    if (q & 1) { cw[q >> 1] = __byte_perm(cw[q >> 1], c2[0], 0x5410); cw[2 + (q >> 1)] = __byte_perm(cw[2 + (q >> 1)], c2[1], 0x5410); }
+                    else { cw[q >> 1] = c2[0]; cw[2 + (q >> 1)] = c2[1]; }
+                }
+                // the sixteen bits of each half sit at the low end of the significand
+                if (LUT) sel[q] = __byte_perm(__float_as_uint(__fadd_rn(acc[0], 8388608.0f)), __float_as_uint(__fadd_rn(acc[1], 8388608.0f)), 0x5410);
+            }
+            if (LUT) {
+                quad_transpose_words(sel, t);
+                if (BITS == 3) {
+#pragma unroll
+                    for (int p = 0; p < B; ++p) words[wi][p] = sel[p] | (((sel[3] >> p) & 0x11111111u) << 3);
+                } else {
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) words[wi][p] = sel[2 * p] | (sel[2 * p + 1] << 2);
                 }
             }
-            sel[a] = acc >> 1;
+            if (NV) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    // the NVFP4 scale has no sign: the codes take it back; under a zero scale they are zeros without a sign
+                    const uint32_t flip = LUT && rs[j] < 0.0f ? 0x88888888u : 0u, keep = zeros && rs[j] == 0.0f ? 0u : 0xFFFFFFFFu;
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) cw[2 * j + i] = (cw[2 * j + i] ^ flip) & keep;
+                }
+                out_codes[wi * 4] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
+                if ((t & 1) == 0) out_sf[wi * 256] = sc4 & 0x7F7F7F7Fu;           // two k atoms of 512 bytes per word group
+            }
         }
         if (LUT) {
-            if (BITS == 3) {
+            uint8_t *out = lut + lut_atom_offset(rowgrp * 8, atom, K, B);
 #pragma unroll
-                for (int p = 0; p < B; ++p)
-                    words[wi][p] = (sel[p] & 0x77777777u) | (((sel[3] >> p) & 0x11111111u) << 3);
-            } else {
-#pragma unroll
-                for (int p = 0; p < 2; ++p)
-                    words[wi][p] = (sel[2 * p] & 0x33333333u) | ((sel[2 * p + 1] & 0x33333333u) << 2);
-            }
-            if (t == wi) my_scales = make_uint2(lut_sc[0], lut_sc[1]);
+            for (int p = 0; p < B; ++p)
+                *reinterpret_cast<uint4 *>(out + p * 512 + lane * 16) = make_uint4(words[0][p], words[1][p], words[2][p], words[3][p]);
+            *reinterpret_cast<uint2 *>(out + lut_plane_bytes(B) + lane * 8) = my_scales;
         }
-        if (NV) {
-            out_codes[wi * 4] = quad_transpose(nv_pieces, t);
-            if (t < 2) out_sf[wi * 256] = t ? nv_sc[1] : nv_sc[0];              // two k atoms of 512 bytes per word group
-        }
-    }
-    if (LUT) {
-        uint8_t *out = lut + lut_atom_offset(rowgrp * 8, atom, K, B);
-#pragma unroll
-        for (int p = 0; p < B; ++p)
-            *reinterpret_cast<uint4 *>(out + p * 512 + lane * 16) = make_uint4(words[0][p], words[1][p], words[2][p], words[3][p]);
-        *reinterpret_cast<uint2 *>(out + lut_plane_bytes(B) + lane * 8) = my_scales;
     }
 }
 
-template <bool FP32IN>
-static void launch_pack_typed(const void *W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes, uint8_t *sf,
-                              uint8_t *lut, int bits, cudaStream_t stream)
+// Has no bin of the LUT3 codebook more than one threshold?  (Thresholds 0.51 apart never share one; the default codebook's are 1.2 apart.)
+static bool pack_bins_fit(const uint16_t *codebook_f16)
 {
-    const int64_t atoms_k = bits ? 2 * lut_slices(K) : (K + 511) / 512;
-    const unsigned blocks = (unsigned)((N / 8 * atoms_k + 3) / 4);
-    if (codes && bits == 3) pack_kernel<FP32IN, true, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
-    else if (codes && bits == 2) pack_kernel<FP32IN, true, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
-    else if (codes) pack_kernel<FP32IN, true, 0><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
-    else if (bits == 3) pack_kernel<FP32IN, false, 3><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
-    else pack_kernel<FP32IN, false, 2><<<blocks, 128, 0, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    float T[7];
+    for (int l = 0; l < 7; ++l) {
+        const float a = __half2float(__ushort_as_half(codebook_f16[l])), b = __half2float(__ushort_as_half(codebook_f16[l + 1]));
+        T[l] = (a + b) * 0.5f;
+    }
+    int below;
+    float own;
+    for (int b = 0; b < kBins; ++b)
+        if (!bin_entry(T, 7, b, below, own)) return false;
+    return true;
+}
+
+template <bool FP32IN, bool NV, int BITS, bool BINNED>
+static cudaError_t launch_pack_one(const void *W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes, uint8_t *sf, uint8_t *lut,
+                                   cudaStream_t stream)
+{
+    static std::atomic<bool> attr_set[kMaxDevices];
+    const DeviceInfo *di = device_info();
+    if (!di) return cudaErrorInvalidDevice;
+    auto kernel = pack_kernel<FP32IN, NV, BITS, BINNED>;
+    const int smem = 8 * 2 * pack_stage_bytes(FP32IN);
+    if (!attr_set[di->device].load(std::memory_order_acquire)) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+        if (e != cudaSuccess) return e;
+        attr_set[di->device].store(true, std::memory_order_release);
+    }
+    const int64_t atoms_k = BITS ? 2 * lut_slices(K) : (K + 511) / 512, need = (N / 8 * atoms_k + 7) / 8;
+    const int64_t slots = (int64_t)di->sms * pack_ctas(FP32IN);                  // all resident: a CTA makes its tables once
+    kernel<<<(unsigned)(need < slots ? need : slots), 256, smem, stream>>>(W, N, K, ldw, hdr, codes, sf, lut);
+    return cudaGetLastError();
+}
+template <bool FP32IN>
+static cudaError_t launch_pack_typed(const void *W, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes, uint8_t *sf,
+                                     uint8_t *lut, int bits, bool binned, cudaStream_t stream)
+{
+    if (codes && bits == 3 && binned) return launch_pack_one<FP32IN, true, 3, true>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    if (codes && bits == 3) return launch_pack_one<FP32IN, true, 3, false>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    if (codes && bits == 2) return launch_pack_one<FP32IN, true, 2, true>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    if (codes) return launch_pack_one<FP32IN, true, 0, false>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    if (bits == 3 && binned) return launch_pack_one<FP32IN, false, 3, true>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    if (bits == 3) return launch_pack_one<FP32IN, false, 3, false>(W, N, K, ldw, hdr, codes, sf, lut, stream);
+    return launch_pack_one<FP32IN, false, 2, true>(W, N, K, ldw, hdr, codes, sf, lut, stream);
 }
 
 // codes / sf: NVFP4 output or nullptr; lut with bits = 3 or 2: LUT output, bits = 0: none
-cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, PackedHeader *hdr, uint8_t *codes,
-                        uint8_t *sf_swizzled, uint8_t *lut_dev, int bits, cudaStream_t stream)
+cudaError_t launch_pack(const void *W, int w_dtype, int64_t N, int64_t K, int64_t ldw, const uint16_t *codebook_f16_host, PackedHeader *hdr,
+                        uint8_t *codes, uint8_t *sf_swizzled, uint8_t *lut_dev, int bits, cudaStream_t stream)
 {
-    if (w_dtype == DQ_DT_FP32) launch_pack_typed<true>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, stream);
-    else launch_pack_typed<false>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, stream);
-    return cudaGetLastError();
+    const bool binned = bits == 3 && pack_bins_fit(codebook_f16_host);
+    if (w_dtype == DQ_DT_FP32) return launch_pack_typed<true>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, binned, stream);
+    return launch_pack_typed<false>(W, N, K, ldw, hdr, codes, sf_swizzled, lut_dev, bits, binned, stream);
 }
 
 // ---------------------------------------------------------------- autocast
@@ -521,51 +688,58 @@ cudaError_t launch_export_nvfp4(const PackedHeader *hdr, const uint8_t *codes, c
 }
 
 // LSB-first bit-planes (App. C.2) from the device layout.  A warp takes an atom; lane (g, t) holds weights 4t .. 4t+3 of every
-// block of row g, i.e. bits 4t .. 4t+3 of each half of a canonical word.  It gathers its bits of the sixteen words of the atom
-// per plane; two exchanges inside the quad OR them together so that lane t ends up with the four words of word group t.
+// block of row g, i.e. bits 4t .. 4t+3 of each half of a canonical word.  Per plane and word group it has eight such nibbles, a pair for each
+// of four words: a multiplication brings the four bits of a half together (bit 4i times 2^(12 - 3j) lands on 12 + i where j = i,
+// and no two products meet anywhere else), and the pairs go into one word, so that one transpose inside the quad hands lane t
+// all nibbles of its word group; spread by two byte transposes they are the four words.  Bound by instruction issue
+// beside HBM: 17408 x 5120 LUT3 21 us a call (one word per nibble pair exchanged, 24.9).
 template <int BITS>
 __global__ void __launch_bounds__(128) export_lut_kernel(const PackedHeader *__restrict__ hdr, const uint8_t *__restrict__ lut, int64_t N,
                                                          int64_t K, uint32_t *__restrict__ planes_out, uint8_t *__restrict__ scales_out, float *s_out)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0 && s_out) *s_out = hdr->s;
     const uint32_t natoms = (uint32_t)((K + 511) / 512);
-    const int64_t task = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-    const int64_t rowgrp = task / natoms;
+    const uint32_t task = blockIdx.x * 4u + (threadIdx.x >> 5), rowgrp = task / natoms;
     if (rowgrp >= N / 8) return;
-    const uint32_t atom = (uint32_t)(task - rowgrp * natoms);
+    const uint32_t atom = task - rowgrp * natoms;
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int64_t r = rowgrp * 8 + g;
-    const uint8_t *src = lut + lut_atom_offset(rowgrp * 8, atom, K, BITS);
+    const int64_t r = (int64_t)rowgrp * 8 + g;
+    const uint8_t *src = lut + lut_atom_offset((int64_t)rowgrp * 8, atom, K, BITS);
     uint4 w[BITS];
 #pragma unroll
     for (int p = 0; p < BITS; ++p) w[p] = __ldg(reinterpret_cast<const uint4 *>(src + p * 512 + lane * 16));
     const uint2 s8 = __ldg(reinterpret_cast<const uint2 *>(src + lut_plane_bytes(BITS) + lane * 8));
     const bool mine = (int)(K / 128) - 4 * (int)atom > t;   // word group t of the atom lies inside the row
-    uint32_t sel[4][4];                                     // [word group][selector]
+    uint32_t v[BITS][4];                                    // [plane][word group]
 #pragma unroll
     for (int wi = 0; wi < 4; ++wi) {
-        uint32_t wd[BITS];
+        uint32_t wd[BITS], sel[4];
 #pragma unroll
         for (int p = 0; p < BITS; ++p) wd[p] = wi == 0 ? w[p].x : wi == 1 ? w[p].y : wi == 2 ? w[p].z : w[p].w;
-        lut_selectors<BITS>(wd, sel[wi]);
+        lut_selectors<BITS>(wd, sel);
+#pragma unroll
+        for (int p = 0; p < BITS; ++p) {
+            uint32_t m[4];                                  // nibbles of word a: top of bytes 1 (low half) and 3 (high half)
+#pragma unroll
+            for (int a = 0; a < 4; ++a) m[a] = ((sel[a] >> p) & 0x11111111u) * 0x1248u;
+            const uint32_t lo = __byte_perm(m[0], m[1], 0x7531), hi = __byte_perm(m[2], m[3], 0x7531);
+            v[p][wi] = ((lo >> 4) & 0x0F0F0F0Fu) | (hi & 0xF0F0F0F0u);     // bytes: words 0|2 low, 0|2 high, 1|3 low, 1|3 high
+        }
     }
-    const bool hi2 = (t & 2) != 0, hi1 = (t & 1) != 0;
 #pragma unroll
     for (int p = 0; p < BITS; ++p) {
+        quad_transpose_words(v[p], t);                      // word group t: the four lanes' nibbles
+        const uint32_t e0 = __byte_perm(v[p][0], v[p][1], 0x5140), e1 = __byte_perm(v[p][2], v[p][3], 0x5140);     // lanes 0, 1 (2, 3): low, low, high, high of words 0|2
+        const uint32_t f0 = __byte_perm(v[p][0], v[p][1], 0x7362), f1 = __byte_perm(v[p][2], v[p][3], 0x7362);     // of words 1|3
         uint32_t o[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            uint32_t z[4];
-#pragma unroll
-            for (int wi = 0; wi < 4; ++wi) {                // bit p of the eight nibbles -> bits 0-3 of both halves, then to 4t
-                uint32_t x = (sel[wi][a] >> p) & 0x11111111u;
-                x = (x | (x >> 3)) & 0x03030303u;
-                x = (x | (x >> 6)) & 0x000F000Fu;
-                z[wi] = x << (4 * t);
-            }
-            const uint32_t a0 = (hi2 ? z[2] : z[0]) | __shfl_xor_sync(0xffffffffu, hi2 ? z[0] : z[2], 2);
-            const uint32_t a1 = (hi2 ? z[3] : z[1]) | __shfl_xor_sync(0xffffffffu, hi2 ? z[1] : z[3], 2);
-            o[a] = (hi1 ? a1 : a0) | __shfl_xor_sync(0xffffffffu, hi1 ? a0 : a1, 1);
+        for (int a = 0; a < 2; ++a) {
+            const uint32_t x = a ? f0 : e0, y = a ? f1 : e1;
+            // bytes (lane 0, lane 1) of a half: low nibbles are word a's, high nibbles word a + 2's
+            const uint32_t l01 = (x & 0x000F000Fu) | ((x >> 4) & 0x00F000F0u), h01 = ((x >> 4) & 0x000F000Fu) | ((x >> 8) & 0x00F000F0u);
+            const uint32_t l23 = (y & 0x000F000Fu) | ((y >> 4) & 0x00F000F0u), h23 = ((y >> 4) & 0x000F000Fu) | ((y >> 8) & 0x00F000F0u);
+            o[a] = l01 | (l23 << 8);
+            o[a + 2] = h01 | (h23 << 8);
         }
         if (mine) {
             uint32_t *dst = planes_out + (r * BITS + p) * (K / 32) + (int64_t)atom * 16 + t * 4;
