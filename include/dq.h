@@ -249,6 +249,21 @@ int dq_decode_linear_lut2(const dq_weights *w, const void *X_dev, int64_t B, int
 int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx,
                            void *Y_dev, int64_t ldy, void *stream);
 
+/*
+ * The same decode, 5 to 16 columns, with a workspace of the caller's: the activations are written to it as FP4 digits and meet the
+ * stored matrix on the block-scaled tensor cores as it is, without dequantising.  (Up to four columns dq_decode_linear_nvfp4 does so
+ * without a workspace.)  Same products: an activation is held exactly within 2^27 of the largest of its 16-element block and rounded to
+ * 2^-35 of that below; summed in fp32 along K.
+ *   dq_decode_nvfp4_workspace_bytes  bytes that B columns need; 0 where dq_decode_linear_nvfp4 is the faster call or all there is
+ *                                    (any != 0: also where it is the faster one)
+ *   workspace_dev  256-byte aligned device memory, scratch of this call alone until the stream has passed it;
+ *                  DQ_ERR_WORKSPACE where it is too small
+ * Other arguments, limits and status codes as dq_decode_linear_nvfp4; DQ_ERR_INVALID_ARG for other batches.
+ */
+int dq_decode_nvfp4_workspace_bytes(const dq_weights *w, int64_t B, int any, size_t *bytes_host);
+int dq_decode_linear_nvfp4_ws(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
+                              void *workspace_dev, size_t workspace_bytes, void *stream);
+
 /* ---- host-buffer entry points (the paper has no counterpart; they exist to use and to measure the path
  *      end to end through this interface, copies included) ---- */
 
@@ -393,7 +408,8 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           with 16-row tiles that dq_decode_linear takes for many batches of 4 to 8 (DQ_ERR_INVALID_ARG where
  *           the row is too long for it).
  *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what
- *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 5 = the batch
+ *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 8 = the kernel on
+ *           the FP4 tensor cores (up to four columns, with warps_per_group CTAs per tile), 5 = the batch
  *           kernel as above, 6 = the mma.sync kernel.
  * Other arguments as dq_decode_linear.
  */

@@ -21,7 +21,8 @@ DT_FP32 = 1
 SYMBOLS = ("dq_version", "dq_status_string", "dq_packed_bytes", "dq_pack_weights", "dq_free_weights",
            "dq_prefill_workspace_bytes", "dq_prefill_linear", "dq_prefill_quantize", "dq_prefill_gemm",
            "dq_prefill_linear_static",
-           "dq_decode_linear", "dq_decode_linear_nvfp4", "dq_decode_linear_lut2", "dq_test_decode_linear", "dq_test_prefill_gemm",
+           "dq_decode_linear", "dq_decode_linear_nvfp4", "dq_decode_nvfp4_workspace_bytes", "dq_decode_linear_nvfp4_ws",
+           "dq_decode_linear_lut2", "dq_test_decode_linear", "dq_test_prefill_gemm",
            "dq_bench_gemm_mma_only", "dq_bench_stream_read", "dq_bench_gemm_clocks",
            "dq_prefill_rmsnorm_quantize", "dq_prefill_silu_mul_quantize", "dq_prefill_gemm_silu_mul_quantize",
            "dq_rmsnorm_quantize_activations",
@@ -80,6 +81,10 @@ def lib() -> C.CDLL:
         L.dq_decode_linear_host.argtypes = [vp, vp, i64, i64, vp, i64, vp, C.c_size_t, vp]
         L.dq_decode_linear_nvfp4.restype = C.c_int
         L.dq_decode_linear_nvfp4.argtypes = [vp, vp, i64, i64, vp, i64, vp]
+        L.dq_decode_nvfp4_workspace_bytes.restype = C.c_int
+        L.dq_decode_nvfp4_workspace_bytes.argtypes = [vp, i64, C.c_int, C.POINTER(sz)]
+        L.dq_decode_linear_nvfp4_ws.restype = C.c_int
+        L.dq_decode_linear_nvfp4_ws.argtypes = [vp, vp, i64, i64, vp, i64, vp, sz, vp]
         L.dq_decode_linear_lut2.restype = C.c_int
         L.dq_decode_linear_lut2.argtypes = [vp, vp, i64, i64, vp, i64, vp]
         L.dq_test_prefill_gemm.restype = C.c_int
@@ -167,6 +172,7 @@ class DQWeights:
         self.handle = handle
         self.packed = packed
         self.N, self.K, self.formats = N, K, formats
+        self.nvfp4_ws = {}               # workspace bytes of decode_linear_nvfp4 by batch
 
     def free(self):
         if self.handle:
@@ -383,12 +389,49 @@ def decode_linear(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None, strea
     return out
 
 
-def decode_linear_nvfp4(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
-    """dq_decode_linear_nvfp4: Y = X @ NVFP4(W)^T (weight-only NVFP4A16), bf16 out, batch 1..64."""
+def decode_nvfp4_workspace_bytes(w: DQWeights, B: int, any: bool = False) -> int:
+    """dq_decode_nvfp4_workspace_bytes: 0 where decode_linear_nvfp4 does without a workspace (any: what it would need)."""
+    out = C.c_size_t(0)
+    _check(lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, int(any), C.byref(out)), "dq_decode_nvfp4_workspace_bytes")
+    return int(out.value)
+
+
+def decode_linear_nvfp4_ws(w: DQWeights, X: torch.Tensor, workspace: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
+    """dq_decode_linear_nvfp4_ws: decode_linear_nvfp4, 5 to 16 columns, on the caller's workspace."""
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     B = X.shape[0]
     if out is None:
         out = torch.empty(B, w.N, dtype=torch.bfloat16, device=X.device)
+    _check(lib().dq_decode_linear_nvfp4_ws(w.handle, X.data_ptr(), B, X.stride(0), out.data_ptr(), out.stride(0), workspace.data_ptr(),
+                                           workspace.numel(), _stream_ptr(stream)), "dq_decode_linear_nvfp4_ws")
+    return out
+
+
+def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
+    """The workspace that makes decode_linear_nvfp4 faster, from torch's allocator on the call's stream; None where there is none."""
+    need = w.nvfp4_ws.get(B)
+    if need is None:
+        nbytes = C.c_size_t(0)               # stays 0 for arguments that the call itself refuses
+        lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, 0, C.byref(nbytes))
+        need = w.nvfp4_ws[B] = int(nbytes.value)
+    if not need or (stream is not None and int(stream.cuda_stream) != _current_stream_ptr()):
+        return None
+    try:
+        return torch.empty(need, dtype=torch.uint8, device=X.device)
+    except torch.OutOfMemoryError:           # the call does without
+        return None
+
+
+def decode_linear_nvfp4(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
+    """dq_decode_linear_nvfp4: Y = X @ NVFP4(W)^T (weight-only NVFP4A16), bf16 out, batch 1..64.  From 5 to 16 columns torch's allocator
+    lends a workspace for the call where that makes it faster (dq_decode_linear_nvfp4_ws)."""
+    assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
+    B = X.shape[0]
+    if out is None:
+        out = torch.empty(B, w.N, dtype=torch.bfloat16, device=X.device)
+    ws = _lent_workspace(w, X, B, stream) if 4 < B <= 16 else None
+    if ws is not None:
+        return decode_linear_nvfp4_ws(w, X, ws, out, stream)
     _check(lib().dq_decode_linear_nvfp4(w.handle, X.data_ptr(), B, X.stride(0), out.data_ptr(), out.stride(0),
                                         _stream_ptr(stream)), "dq_decode_linear_nvfp4")
     return out

@@ -615,7 +615,7 @@ int dq::prefill_linear_rows(const dq_weights *w, const void *A_dev, int64_t M, i
 extern "C" {
 
 static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
-                        void *stream, int variant, int csize = 0)
+                        void *stream, int variant, int csize = 0, void *ws = nullptr, size_t ws_bytes = 0)
 {
     if (!valid_handle(w) || !X_dev || !Y_dev) return DQ_ERR_INVALID_ARG;
     if (!has_nvfp4_view(w) || !on_handle_device(w)) return DQ_ERR_INVALID_ARG;
@@ -642,8 +642,11 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
     const dq::DeviceInfo *di = dq::device_info();
     if (!di) return DQ_ERR_CUDA;
     // Rows above 32768 are refused by the mma.sync kernel, as for every batch.
+    const bool fp4 = variant == 8 || (variant == 0 && w->K <= 32768 && B <= 4 && dq::decode_fp4_is_faster(w->N, w->K, B, di->sms));
     const bool tc = variant == 5 || (variant == 0 && w->K <= 32768 && dq::nvfp4_batch_kernel_is_faster(w->N, w->K, B, di->sms));
-    if (tc) {
+    if (fp4) {
+        ce = dq::launch_decode_fp4(g, csize, ws, ws_bytes, s);
+    } else if (tc) {
         ce = dq::launch_decode_tc_nvfp4(g, csize, s);
     } else if (variant == 0 || variant == 6) {
         ce = dq::launch_gemv_nvfp4_mma(g, s);
@@ -662,6 +665,30 @@ int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, in
                            void *stream)
 {
     return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, 0);
+}
+
+int dq_decode_nvfp4_workspace_bytes(const dq_weights *w, int64_t B, int any, size_t *bytes_host)
+{
+    if (!valid_handle(w) || !bytes_host) return DQ_ERR_INVALID_ARG;
+    if (!has_nvfp4_view(w) || !on_handle_device(w)) return DQ_ERR_INVALID_ARG;
+    if (B < 1 || B > 64) return DQ_ERR_INVALID_ARG;
+    const int st = check_arch();
+    if (st != DQ_OK) return st;
+    const dq::DeviceInfo *di = dq::device_info();
+    if (!di) return DQ_ERR_CUDA;
+    // rows above 32768 weights are refused by dq_decode_linear_nvfp4, and here
+    const bool use = w->K <= 32768 && B > 4 && B <= 16 && (any || dq::decode_fp4_is_faster(w->N, w->K, B, di->sms));
+    *bytes_host = use ? dq::decode_fp4_workspace(w->K) : 0;
+    return DQ_OK;
+}
+
+int dq_decode_linear_nvfp4_ws(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy, void *workspace_dev,
+                              size_t workspace_bytes, void *stream)
+{
+    if (!valid_handle(w) || !workspace_dev || B < 5 || B > 16 || w->K > 32768) return DQ_ERR_INVALID_ARG;
+    if (!aligned(workspace_dev, 256)) return DQ_ERR_ALIGN;
+    if (workspace_bytes < dq::decode_fp4_workspace(w->K)) return DQ_ERR_WORKSPACE;
+    return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, 8, 0, workspace_dev, workspace_bytes);
 }
 
 static int decode_lut(const dq_weights *w, unsigned format, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev,
@@ -719,9 +746,9 @@ int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int
                           int64_t ldy, void *stream)
 {
     if (format == DQ_FMT_NVFP4 || format == DQ_FMT_NVFP4_FROM_LUT3) {
-        if (variant != 0 && variant != 1 && variant != 5 && variant != 6) return DQ_ERR_INVALID_ARG;
+        if (variant != 0 && variant != 1 && variant != 5 && variant != 6 && variant != 8) return DQ_ERR_INVALID_ARG;
         if (warps_per_group < 0) return DQ_ERR_INVALID_ARG;
-        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 ? warps_per_group : 0);
+        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 || variant == 8 ? warps_per_group : 0);
     }
     if (warps_per_group < 0 || groups_per_cta < 0 || ring_stages < 0 || ring_stages > 8 || wait_cycles < 0)
         return DQ_ERR_INVALID_ARG;
