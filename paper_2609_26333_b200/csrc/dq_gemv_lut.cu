@@ -26,9 +26,10 @@
 // fp16 pairs.  The 256 block scales of an atom are converted to fp32 once per warp (eight per lane) and parked in a
 // small per-warp buffer; a lane reads its row's scales and its B fragments with 16-byte loads, two mmas per load.
 //
-// What bounds it.  On this GPU a warp instruction of the integer / logic / permute class occupies the issue port of
-// its SM sub-partition for two cycles (measured: 8 PRMT + 8 FFMA take 24 cycles, not 16), so the kernel is bound by
-// instruction issue: about 8 permutes, 2 logic ops, 2 shifts, 1 mma, 4 FFMA and 2 shared loads per 8 weights of a lane.
+// What bounds it.  A warp instruction of the integer / logic / permute class occupies its pipe in an SM sub-partition for
+// two cycles (FFMA runs beside it: 8 PRMT + 8 FFMA take 16.2 cycles), so the kernel is bound by that pipe: about 8 permutes, 2 logic
+// ops and 2 shifts per 8 weights of a lane, 24.4 cycles; with the mma, 4 FFMA and 2 shared loads the loop takes 28.4 from shared
+// memory alone, and about 38 in the kernel.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -1365,11 +1366,12 @@ static cudaError_t launch_bits(const GemvArgs &a, int b0, int cols, int grid, in
 // Five to eight columns, 16-row tiles against 8-row tiles: the two cost models in one unit; a CTA with few warps loses a little more
 // than the model's stretch, and long rows' activations take their time to convert.  The models do not see that warps with one unit of 512
 // each have nothing to hide a wait behind: an odd number of them, which the four schedulers share unevenly, loses to 12 and more warps of
-// 8-row tiles (2016x5632 batch 8: 9.7 / 11.2; 128x4352 9.8 / 10.7) and 13 of them to any (352x6528 batch 5: 8.6 / 9.7).  Of 4960 points (128 to
-// 34816 rows of 384 to 14336 weights) the pick is more than 2 % slower than 8-row tiles at 67, at most 9 %, and on average 0.3 % off the better
-// (1024x4096 batch 5: 7.9 / 6.6; 4096x5120 batch 8: 11.6 / 11.4; 8192x12288 batch 5: 38 / 25.8; stays with 8 rows: 5120x3072 batch 5
-// 8.3 / 9.2, 1024x8192 batch 6 10.1 / 11.4).  Above 10240 rows it stays with 8 rows at some points where 16 would be
-// faster (17408x5120 batch 8: 22.1 / 20.8, 14336x8192 38.9 / 30.9).  Below 128 rows neither fills the chip.
+// 8-row tiles (2016x5632 batch 8: 9.7 / 11.2; 128x4352 9.8 / 10.7) and 13 of them to any (352x6528 batch 5: 8.6 / 9.7).  Rows of up to 6144
+// weights, whose activations are loaded in a batch or two, take 16-row tiles up to 1.18 of the other model's cost: of 166 points (256 to 34816 rows
+// of 384 to 6144 weights) where that changes the pick 9 are more than 2 % slower for it, at most 4 %, and on average they are 11 % faster
+// (10240x5120 batch 8: 17.3 / 16.0; 17408x5120 batch 8 21.0 / 18.9; 19168x896 batch 6 7.5 / 6.5; 20752x3200 batch 7 21.5 / 17.4; slower: 6432x2816
+// batch 8 8.6 / 8.9).  Longer rows leave room for fewer warps, and the model favours 16 rows too often (12784x12288 batch 5 34.6 / 39.2, 496x7552 7.4 / 8.4):
+// there they have to be well ahead by it (8192x12288 batch 5: 38 / 25.8).  Below 128 rows neither fills the chip.
 // The grid of the 16-row launch and its plan in L, 0 for 8-row tiles.
 static int rows16_if_faster(int bits, int64_t N, int64_t K, int B, int sms, const Split &narrow, LutPlan &L)
 {
@@ -1380,7 +1382,8 @@ static int rows16_if_faster(int bits, int64_t N, int64_t K, int B, int sms, cons
     if (one_unit && (narrow.P * narrow.G >= 12 || L.P == 13)) return 0;
     const double warps = (double)(L.P * L.G);
     if (warps < 12.0) cost *= std::sqrt(std::sqrt(12.0 / warps));
-    return cost + (double)lut_slices(K) - 6.0 <= 0.94 * narrow.cost ? grid : 0;
+    const double slices = (double)lut_slices(K);
+    return cost + slices - 6.0 <= (slices <= 6.0 ? 1.18 : 0.94) * narrow.cost ? grid : 0;
 }
 
 // Four columns: 16-row tiles only where every CTA gets one of them at most and the rows are short (512x1024: 5.7 / 5.0; 1024x2048: 6.1 / 5.4;
