@@ -407,13 +407,24 @@ def decode_linear_nvfp4_ws(w: DQWeights, X: torch.Tensor, workspace: torch.Tenso
     return out
 
 
+_nvfp4_ws_known = {}                     # by device, matrix and batch: the answer depends on nothing else, and a new handle need not ask again
+
+
 def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
     """The workspace that makes decode_linear_nvfp4 faster, from torch's allocator on the call's stream; None where there is none."""
     need = w.nvfp4_ws.get(B)
     if need is None:
-        nbytes = C.c_size_t(0)               # stays 0 for arguments that the call itself refuses
-        lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, 0, C.byref(nbytes))
-        need = w.nvfp4_ws[B] = int(nbytes.value)
+        key = (X.device, w.packed.device, w.N, w.K, w.formats, B)
+        need = _nvfp4_ws_known.get(key)
+        if need is None:
+            nbytes = C.c_size_t(0)
+            st = lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, 0, C.byref(nbytes))
+            need = int(nbytes.value)         # 0 for arguments that the call itself refuses
+            if st == 0:
+                if len(_nvfp4_ws_known) >= 1024:
+                    _nvfp4_ws_known.clear()
+                _nvfp4_ws_known[key] = need
+        w.nvfp4_ws[B] = need
     if not need or (stream is not None and int(stream.cuda_stream) != _current_stream_ptr()):
         return None
     try:
@@ -429,7 +440,7 @@ def decode_linear_nvfp4(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None,
     B = X.shape[0]
     if out is None:
         out = torch.empty(B, w.N, dtype=torch.bfloat16, device=X.device)
-    ws = _lent_workspace(w, X, B, stream) if 4 < B <= 16 else None
+    ws = _lent_workspace(w, X, B, stream) if 4 < B <= 16 and w.nvfp4_ws.get(B) != 0 else None
     if ws is not None:
         return decode_linear_nvfp4_ws(w, X, ws, out, stream)
     _check(lib().dq_decode_linear_nvfp4(w.handle, X.data_ptr(), B, X.stride(0), out.data_ptr(), out.stride(0),
