@@ -21,8 +21,10 @@
 //   warp 13        : weights of the next slices, bulk / TMA copies into a ring per half
 // Two accumulators per half alternate, so reading one back overlaps the MMAs of the next.
 //
-// What bounds it: instruction issue of the dequantising warps.  The MMAs cost N / 2 cycles each whatever K-slice they are in
-// (issued under elect.sync), well below that; a weight is dequantised once for all columns.
+// What bounds it: look-ups and stores of the dequantising warps, which add up on a scheduler (32 PRMT, 16 HFMA2 and a store of 16
+// registers: 89 to 97 cycles a warp in every store shape) on top of the loop's hand-overs.  34816x5120 LUT3 batch 40 takes 70.0 us;
+// without staging 63.8, without read-back 67.9, without MMAs (N / 2 cycles each) 65.1, without all three 57.0, of these without
+// look-ups 39.2, without stores too 31.7.  It is not latency: sixteen dequantising warps take 73.6, waits that spin 72.4.
 #include <atomic>
 
 #include <cuda.h>
