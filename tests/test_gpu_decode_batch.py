@@ -308,6 +308,25 @@ def test_decode_rows16_parity(dq, oracle, fmt, N, K, B):
         check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K} public")
 
 
+@pytest.mark.parametrize("fmt,N,K,B,rows16", [("lut3", 19216, 640, 7, True), ("lut2", 10304, 1664, 8, True), ("lut3", 4464, 4608, 5, True),
+                                              ("lut2", 464, 6144, 6, None), ("lut2", 496, 7552, 5, False)])
+def test_decode_line_between_row_tiles(dq, oracle, fmt, N, K, B, rows16):
+    """Both sides of the line between 8-row and 16-row tiles: the public call against the oracle, and bit for bit the 16-row kernel where
+    that is the one taken."""
+    W, ref = _layer(oracle, N, K)
+    code = {"lut3": dq.FMT_LUT3, "lut2": dq.FMT_LUT2}[fmt]
+    w = dq.pack_weights(W.to(DEV), formats=code)
+    X = dq_inputs.gaussian_bf16(B, K, 1.0, 700 + B)
+    Yr, S = _reference(oracle, ref, fmt, X)
+    y = {"lut3": dq.decode_linear, "lut2": dq.decode_linear_lut2}[fmt](w, X.to(DEV))
+    forced = dq.test_decode_linear(w, code, X.to(DEV), variant=6)
+    _status_ok(dq)
+    check_outputs(_f64(y), Yr, S, f"{fmt} {B}x{N}x{K} public")
+    check_outputs(_f64(forced), Yr, S, f"{fmt} {B}x{N}x{K} 16 rows")
+    if rows16:
+        assert torch.equal(y, forced)
+
+
 @pytest.mark.parametrize("fmt", ["lut3", "lut2", "nvfp4"])
 @pytest.mark.parametrize("N,K", [(512, 256), (528, 1024), (1024, 2176), (2384, 640)])
 @pytest.mark.parametrize("B", [4, 6, 9, 16, 24])
