@@ -62,6 +62,7 @@ struct Cfg {
     static constexpr int kWorkers = 8, kThreads = 64 + 32 * kWorkers;          // warps
     static constexpr int kPerCol = 2;                                          // warps that share a column where they make the digits, step by step
     static_assert(PRE || kPerCol * 4 * NG == kWorkers, "a column per two warps");
+    static_assert(S < kGroupSteps, "the scales' slots rely on a full group being longer than the ring");
     static_assert(S >= 3 && STAGE_BYTES % 1024 == 0 && kSfBase + 2 * kSfCols <= kTmemCols, "shared memory, tensor memory");
     static_assert((NG + kMaxCluster) * 4096u <= S * STAGE_BYTES, "partial sums of a cluster must fit the ring");
 };
@@ -75,9 +76,15 @@ enum : uint32_t {
     kDEmpty = 184,               // [2]
     kTmemPtr = 208,
     kAbort = 212,
-    kScales = 256,               // [2 groups][16 columns] float
-    kSpecial = 512,              // [2][16] int: the column's group holds an infinity or a NaN
+    kScales = 256,               // [kSlots groups][16 columns] float
+    kSpecial = 512,              // [kSlots][16] int: the column's group holds an infinity or a NaN
 };
+// Groups whose scales and flags are held where the CTAs make the digits: group n's lie in slot n % 3.  They are written with the group's first
+// step, when the writer has read the sums of group n - 2, and of n - 1 too where n begins a tile.  Every warp has then read slot n - 3:
+//   n begins a tile: the sums of n - 1 exist, so every warp has handed over the first step of n - 1, and reads the sums of n - 3 before that;
+//   n does not: n - 1 has eight steps, more than the ring, so the stage that the writer got last held one of its steps but the first.
+// Two slots are not enough: group n - 2 is read after the first step of n - 1, which may be the only one (rows of 17, 25, .. steps).
+constexpr uint32_t kSlots = 3;
 
 struct Fp4Args {
     const uint8_t *codes, *w_sf;
@@ -309,7 +316,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
             const uint32_t st = i / (C::X_BYTES / 16u), at = i % (C::X_BYTES / 16u);
             asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(ring0 + st * C::STAGE_BYTES + C::A_BYTES + C::SFA_BYTES + at * 16u), "r"(0u) : "memory");
         }
-        if (threadIdx.x < 32) { scales[threadIdx.x] = 0.0f; specials[threadIdx.x] = 0; }
+        if (threadIdx.x < 16 * kSlots) { scales[threadIdx.x] = 0.0f; specials[threadIdx.x] = 0; }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
@@ -451,7 +458,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                 if (!ok) return;
                 tc_fence_after();
                 // the columns' powers of two: lane c has column c's
-                const int gi = ks / kGroupSteps * 16 + (lane & 15), si = (int)(n & 1u) * 16 + (lane & 15);
+                const int gi = ks / kGroupSteps * 16 + (lane & 15), si = (int)(n % kSlots) * 16 + (lane & 15);
                 const float gs = PRE ? __uint_as_float(__ldcg(P.group_scale + gi)) : scales[si];
                 const int sp_lane = PRE ? (int)__ldcg(P.group_scale + P.ngroups * 16 + gi) : specials[si];
 #pragma unroll
@@ -506,8 +513,8 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                     if (!ok) break;
                     const uint32_t b = ring0 + stage * C::STAGE_BYTES;
                     if (s == 0 && turn == 0 && lane == 0 && col < P.cols) {
-                        scales[(grp & 1u) * 16u + col] = __uint_as_float(scale_of_group(top, eg));
-                        specials[(grp & 1u) * 16u + col] = special;
+                        scales[grp % kSlots * 16u + col] = __uint_as_float(scale_of_group(top, eg));
+                        specials[grp % kSlots * 16u + col] = special;
                     }
                     if (col < P.cols && s % C::kPerCol == turn) {
                         const uint4 x = special ? make_uint4(0u, 0u, 0u, 0u) : next;

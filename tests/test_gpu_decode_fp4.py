@@ -58,6 +58,26 @@ def test_fp4_decode_every_cluster_size(dq, N, K, csize):  # noqa: F811
     _check(Y, X, Wd, f"{csize} CTAs per tile")
 
 
+@pytest.mark.parametrize("N,K", [(38160, 2304), (38160, 4352), (38160, 6400)])
+def test_fp4_decode_several_tiles_and_groups_per_cta(dq, N, K):  # noqa: F811
+    """More tiles than SMs and rows of two to four groups of 2048 weights, the last of them one step long: ring, accumulators and the
+    groups' powers of two go on across the tiles.  A column has one large group, the others 2^30 below: the scale of another group, or of
+    the next tile's, would show."""
+    g, w, Wd = _pack(dq, N, K, K)
+    groups = (K + 2047) // 2048
+    X = torch.randn(16, K, generator=g, device=DEV)
+    at = torch.arange(K, device=DEV) // 2048
+    for b in range(16):
+        X[b, at != b % groups] *= 2.0 ** -30
+    X = X.to(torch.bfloat16)
+    Yr, S = (X.double() @ Wd.T).cpu().numpy(), (X.double().abs() @ Wd.abs().T).cpu().numpy()
+    for first, B in [(b, 1) for b in range(groups)] + [(0, 4), (1, 4), (0, 5), (0, 8), (3, 9), (0, 16)]:
+        for _ in range(3):
+            Y = _call(dq, w, X[first:first + B])
+            _status_ok(dq)
+            check_outputs(_f64(Y), Yr[first:first + B], S[first:first + B], f"{N}x{K}, columns {first} to {first + B - 1}")
+
+
 @pytest.mark.parametrize("B", [2, 7, 12])
 def test_fp4_decode_magnitudes(dq, B):  # noqa: F811
     """Rows of 40 binades; elements 2^27 below the largest of their block under a weight of zero there; subnormals; very large
