@@ -8,7 +8,8 @@
 // the column's 2048 weights (a group), down to 2^-17 of it; blocks below share that exponent (2^-52 of the group's largest).  A batch
 // column thus becomes twelve columns of the MMA's other operand.  Products and block scales are exact; the tensor cores sum a group
 // (32 instructions, as many as one of decode_tc_kernel's), its twelve sums are put together and added to the running sum by FMA in
-// fp32 with the group's power of two.  An infinity or a NaN: the group's products with it, one by one (special_sum).
+// fp32 with the powers of two of the group and, as far as fp32's range allows (scale_exponent), of the tensor scale: without that,
+// finite outputs of activations of 2^104 and more were lost.  An infinity or a NaN: the group's products with it, one by one (special_sum).
 //
 // Work split.  A tile is 256 rows in two halves, the tensor-memory lanes; a step 256 weights.  Where there are too few tiles for the chip
 // a cluster of up to 8 CTAs shares one, each taking a range of steps; at the end they exchange partial sums through distributed
@@ -156,6 +157,14 @@ __device__ __forceinline__ uint32_t max_abs_of(uint4 v) { return max_abs_bf16x2(
 // fp32 bits of a group's power of two, 2^(eg - 135) with eg the largest exponent; a subnormal for the smallest.  0 beside infinities and NaN:
 // no sums of the tensor cores
 __device__ __forceinline__ uint32_t scale_of_group(uint32_t top, int eg) { return top >= 0x7F80u ? 0u : eg >= 9 ? (uint32_t)(eg - 8) << 23 : 1u << (eg + 14); }
+// The part of a tensor scale's power of two, 2^e, that goes with the groups' scales: their product is a number of fp32 whatever the group.  The
+// scale is looked at here and not before: it comes from memory, and the first digits are not to wait for it.
+__device__ __forceinline__ int scale_exponent(float s)
+{
+    asm volatile("" : "+f"(s));
+    return max(-15, min(8, (int)((__float_as_uint(s) >> 23) & 255u) - 127));
+}
+__device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(e + 127) << 23); }
 // Digits and block scales of a lane's eight activations x; lanes 2i and 2i + 1 share a block, eight lanes the word of four scales
 __device__ __forceinline__ void digits_and_scales(const uint4 x, int eg, uint32_t (&w)[kDigits], uint32_t &sf)
 {
@@ -441,25 +450,25 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
             sf_place[u] = C::A_BYTES + C::SFA_BYTES + C::B_BYTES + (n >> 7) * 2048u + ((uint32_t)lane >> 3) * 512u + (rr & 31u) * 16u + (rr >> 5) * 4u;
         }
         asm volatile("griddepcontrol.wait;" ::: "memory");     // X may come from the kernel ahead
-        const float s_w = P.hdr->s;
+        const float s_all = P.hdr->s;
         float acc[4 * NG];
         bool ok = true;
         int stage = 0;
-        uint32_t phase = 0, grp = 0;                           // groups whose digits are begun
+        uint32_t phase = 0, grp = 0, slot = 0;                 // groups whose digits are begun; grp % kSlots
         for (int tile = first_tile; tile < tiles && ok; tile += tile_stride) {
             const int row = tile * 256 + r;
 #pragma unroll
             for (int c = 0; c < 4 * NG; ++c) acc[c] = 0.0f;
             // where the group that step ks is in ends: groups of the workspace are counted from the row's start, others from the CTA's first step
             auto group_end = [&](int ks) { return PRE ? (ks / kGroupSteps + 1) * kGroupSteps : ks + kGroupSteps; };
-            // group n of the kernel, of steps from ks: from its accumulator into the running sums
-            auto flush = [&](uint32_t n, int ks) {
+            // group n of the kernel, of steps from ks, its scales in slot sl: from its accumulator into the running sums
+            auto flush = [&](uint32_t n, uint32_t sl, int ks) {
                 if (ok) ok = wait_warp(dfull_bar(n), (n / C::kAccs) & 1u, abort_flag);
                 if (!ok) return;
                 tc_fence_after();
                 // the columns' powers of two: lane c has column c's
-                const int gi = ks / kGroupSteps * 16 + (lane & 15), si = (int)(n % kSlots) * 16 + (lane & 15);
-                const float gs = PRE ? __uint_as_float(__ldcg(P.group_scale + gi)) : scales[si];
+                const int gi = ks / kGroupSteps * 16 + (lane & 15), si = (int)sl * 16 + (lane & 15);
+                const float gs = (PRE ? __uint_as_float(__ldcg(P.group_scale + gi)) : scales[si]) * pow2(scale_exponent(s_all));
                 const int sp_lane = PRE ? (int)__ldcg(P.group_scale + P.ngroups * 16 + gi) : specials[si];
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
@@ -499,8 +508,8 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                 for (int s = 0; s < kGroupSteps; ++s) gm = max_abs_bf16x2(gm, max_abs_of(piece(k0 + s)));
                 next = piece(k0 + turn);
             }
-            for (int kg = k0; PRE && kg < k1 && ok; kg = group_end(kg)) flush(grp++, kg);
-            for (int kg = k0; !PRE && kg < k1 && ok; kg += kGroupSteps, ++grp) {
+            for (int kg = k0; PRE && kg < k1 && ok; kg = group_end(kg)) flush(grp++, 0u, kg);
+            for (int kg = k0; !PRE && kg < k1 && ok; kg += kGroupSteps, ++grp, slot = slot + 1u == kSlots ? 0u : slot + 1u) {
                 const int nk = min(kGroupSteps, k1 - kg);
                 const uint32_t top = __reduce_max_sync(0xffffffffu, max_magnitude(gm));
                 const bool special = top >= 0x7F80u;
@@ -513,8 +522,8 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                     if (!ok) break;
                     const uint32_t b = ring0 + stage * C::STAGE_BYTES;
                     if (s == 0 && turn == 0 && lane == 0 && col < P.cols) {
-                        scales[grp % kSlots * 16u + col] = __uint_as_float(scale_of_group(top, eg));
-                        specials[grp % kSlots * 16u + col] = special;
+                        scales[slot * 16u + col] = __uint_as_float(scale_of_group(top, eg));
+                        specials[slot * 16u + col] = special;
                     }
                     if (col < P.cols && s % C::kPerCol == turn) {
                         const uint4 x = special ? make_uint4(0u, 0u, 0u, 0u) : next;
@@ -541,11 +550,12 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                     if (lane == 0) mbar_arrive(xfull_bar(stage));
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                     gm = max_abs_bf16x2(gm, max_abs_of(ahead));
-                    if (s == 0 && kg > k0) flush(grp - 1u, kg - kGroupSteps);
+                    if (s == 0 && kg > k0) flush(grp - 1u, (slot == 0 ? kSlots : slot) - 1u, kg - kGroupSteps);
                 }
             }
-            if (!PRE && ok && k1 > k0) flush(grp - 1u, k0 + (k1 - k0 - 1) / kGroupSteps * kGroupSteps);
+            if (!PRE && ok && k1 > k0) flush(grp - 1u, (slot == 0 ? kSlots : slot) - 1u, k0 + (k1 - k0 - 1) / kGroupSteps * kGroupSteps);
             if (ok && csize == 1 && row < P.N) {
+                const float s_w = s_all * pow2(-scale_exponent(s_all));        // what the groups' scales have left of it
                 __nv_bfloat16 *y = P.Y + row;
 #pragma unroll
                 for (int c = 0; c < 4 * NG; ++c)
@@ -563,6 +573,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                 st_cluster_v4(mine + (uint32_t)((int)rank * per + i / csize) * 4096u, (uint32_t)(i % csize), acc[4 * i], acc[4 * i + 1], acc[4 * i + 2], acc[4 * i + 3]);
             cluster_sync();
             const int row = first_tile * 256 + r;
+            const float s_w = s_all * pow2(-scale_exponent(s_all));
             if (ok && row < P.N) {
                 for (int i = (int)rank, l = 0; i < NG && 4 * i < P.cols; i += csize, ++l) {
                     float tot[4] = {0.0f, 0.0f, 0.0f, 0.0f};

@@ -104,6 +104,20 @@ def test_fp4_decode_magnitudes(dq, B):  # noqa: F811
         assert (Y[4] == 0).all()
 
 
+@pytest.mark.parametrize("B", [1, 4, 8, 16])
+@pytest.mark.parametrize("w_exp,x_exp", [(0, 116), (-60, 124), (60, 60), (100, -110), (-90, -20), (0, -100)])
+def test_fp4_decode_sums_beyond_fp32_before_the_tensor_scale(dq, B, w_exp, x_exp):  # noqa: F811
+    """Outputs are finite and right wherever bf16 holds them, also where sums without the tensor scale, or a group's power of two with it, are beyond
+    fp32's range."""
+    N, K = 272, 4352
+    g = torch.Generator(device=DEV).manual_seed(B)
+    w = dq.pack_weights((torch.randn(N, K, generator=g, device=DEV) * 2.0 ** (w_exp - 6)).to(torch.bfloat16), formats=dq.FMT_NVFP4)
+    X = (torch.randn(B, K, generator=g, device=DEV).double() * 2.0 ** x_exp).to(torch.bfloat16)
+    Y = _call(dq, w, X)
+    _status_ok(dq)
+    _check(Y, X, _dequantised(dq, w, "nvfp4"), f"weights 2^{w_exp - 6}, activations 2^{x_exp}")
+
+
 @pytest.mark.parametrize("B", [4, 16])
 def test_fp4_decode_infinities_and_nan(dq, B):  # noqa: F811
     N, K = 272, 2304
