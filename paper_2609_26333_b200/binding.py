@@ -410,21 +410,28 @@ def decode_linear_nvfp4_ws(w: DQWeights, X: torch.Tensor, workspace: torch.Tenso
 _nvfp4_ws_known = {}                     # by device, matrix and batch: the answer depends on nothing else, and a new handle need not ask again
 
 
-def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
-    """The workspace that makes decode_linear_nvfp4 faster, from torch's allocator on the call's stream; None where there is none."""
+def _nvfp4_ws_need(w: DQWeights, device, B: int) -> int:
+    """Bytes of the workspace that makes decode_linear_nvfp4 faster, 0 where there is none.  An answer is kept; where there was none (another
+    device is current, a CUDA error) the call does without, and the next one asks again."""
     need = w.nvfp4_ws.get(B)
     if need is None:
-        key = (X.device, w.packed.device, w.N, w.K, w.formats, B)
+        key = (device, w.packed.device, w.N, w.K, w.formats, B)
         need = _nvfp4_ws_known.get(key)
         if need is None:
             nbytes = C.c_size_t(0)
-            st = lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, 0, C.byref(nbytes))
-            need = int(nbytes.value)         # 0 for arguments that the call itself refuses
-            if st == 0:
-                if len(_nvfp4_ws_known) >= 1024:
-                    _nvfp4_ws_known.clear()
-                _nvfp4_ws_known[key] = need
+            if lib().dq_decode_nvfp4_workspace_bytes(w.handle, B, 0, C.byref(nbytes)) != 0:
+                return 0
+            need = int(nbytes.value)
+            if len(_nvfp4_ws_known) >= 1024:
+                _nvfp4_ws_known.clear()
+            _nvfp4_ws_known[key] = need
         w.nvfp4_ws[B] = need
+    return need
+
+
+def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
+    """That workspace, from torch's allocator on the call's stream; None where there is none."""
+    need = _nvfp4_ws_need(w, X.device, B)
     if not need or (stream is not None and int(stream.cuda_stream) != _current_stream_ptr()):
         return None
     try:

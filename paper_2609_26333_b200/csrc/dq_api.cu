@@ -677,7 +677,9 @@ int dq_decode_nvfp4_workspace_bytes(const dq_weights *w, int64_t B, int any, siz
     const dq::DeviceInfo *di = dq::device_info();
     if (!di) return DQ_ERR_CUDA;
     // rows above 32768 weights are refused by dq_decode_linear_nvfp4, and here
-    const bool use = w->K <= 32768 && B > 4 && B <= 16 && (any || dq::decode_fp4_is_faster(w->N, w->K, B, di->sms));
+    bool sure = true;
+    const bool use = w->K <= 32768 && B > 4 && B <= 16 && (any || dq::decode_fp4_is_faster(w->N, w->K, B, di->sms, &sure));
+    if (!sure) return DQ_ERR_CUDA;                       // the caller may keep the answer, so there is none
     *bytes_host = use ? dq::decode_fp4_workspace(w->K) : 0;
     return DQ_OK;
 }

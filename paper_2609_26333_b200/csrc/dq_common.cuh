@@ -281,7 +281,7 @@ cudaError_t launch_decode_tc_nvfp4(const GemvNvArgs &args, int force_csize, cuda
 // bytes, 256-byte aligned).  force_csize: CTAs per tile (test hook)
 size_t decode_fp4_workspace(int64_t K);
 cudaError_t launch_decode_fp4(const GemvNvArgs &args, int force_csize, void *ws, size_t ws_bytes, cudaStream_t stream);
-bool decode_fp4_is_faster(int64_t N, int64_t K, int64_t B, int sms);
+bool decode_fp4_is_faster(int64_t N, int64_t K, int64_t B, int sms, bool *sure = nullptr);
 cudaError_t launch_fill_e2m1_table(cudaStream_t stream);
 // read-only streaming sum with 128-bit loads (measurement): 8 bytes of result at out_dev
 cudaError_t launch_stream_read(const void *src_dev, size_t bytes, void *out_dev, cudaStream_t stream);   // value-pair table of the NVFP4 decode kernel

@@ -648,8 +648,8 @@ cudaLaunchConfig_t launch_config(cudaLaunchAttribute (&attr)[2], int grid, int c
 }
 
 // How many clusters of c CTAs the device holds at once (one CTA per SM in every instantiation); asked once per size and device, and again
-// where the runtime did not answer
-int clusters_that_fit(int dev, int c, int sms)
+// where the runtime did not answer: 0 and sure = false then
+int clusters_that_fit(int dev, int c, int sms, bool &sure)
 {
     static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];                 // + 1; 0 = not known
     int fit = known[dev][c].load(std::memory_order_relaxed);
@@ -659,6 +659,7 @@ int clusters_that_fit(int dev, int c, int sms)
         int n = 0;
         if (set_attributes<1, false>(dev) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, decode_fp4_kernel<1, false>, &cfg) != cudaSuccess) {
             cudaGetLastError();
+            sure = false;
             return 0;
         }
         fit = n + 1;
@@ -667,17 +668,17 @@ int clusters_that_fit(int dev, int c, int sms)
     return fit - 1;
 }
 
-// CTAs per tile, and the steps of the busiest CTA.  Clusters take one tile each and must all be resident.
-struct Split { int csize; int steps; };
+// CTAs per tile, and the steps of the busiest CTA.  Clusters take one tile each and must all be resident.  sure: the runtime has said how many are
+struct Split { int csize; int steps; bool sure; };
 Split split_tiles(int64_t N, int64_t K, int dev, int sms, int force_csize)
 {
     const int64_t tiles = (N + 255) / 256, ksteps = (K + 255) / 256;
-    Split best = {1, (int)((tiles + sms - 1) / sms * ksteps)};
+    Split best = {1, (int)((tiles + sms - 1) / sms * ksteps), true};
     double cost = (double)best.steps;
     for (int c = 2; c <= kMaxCluster && c <= ksteps && tiles * c <= sms; ++c) {
         if (force_csize > 0 && c != force_csize) continue;
         const int steps = (int)((ksteps + c - 1) / c);
-        if ((force_csize > 0 || steps + 0.5 < cost) && tiles <= clusters_that_fit(dev, c, sms)) { best = {c, steps}; cost = steps + 0.5; }
+        if ((force_csize > 0 || steps + 0.5 < cost) && tiles <= clusters_that_fit(dev, c, sms, best.sure)) { best = {c, steps, best.sure}; cost = steps + 0.5; }
     }
     return best;
 }
@@ -721,14 +722,18 @@ cudaError_t launch_ng(const CUtensorMap &tmap, Fp4Args P, int force_csize, const
 // columns on, with the workspace: 4.3 (5.6 above eight) for both launches, 0.51 (0.74) a step of the busiest CTA, 0.078 (0.070) a megabyte, 1.4 for a
 // cluster's exchange, against 1.9, 2.75 a slice of 512 and 0.033 a megabyte; its second launch costs the host 3, so that short calls stay
 // (1536x8192 batch 8 9.4 / 8.7); clusters of three or five that crowd the chip wait for a free group of SMs (11408x11776 batch 9 27.4 / 33.9).
-bool decode_fp4_is_faster(int64_t N, int64_t K, int64_t B, int sms)
+// sure = false: the answer rests on one that the runtime did not give
+bool decode_fp4_is_faster(int64_t N, int64_t K, int64_t B, int sms, bool *sure)
 {
+    if (sure) *sure = true;
     if (B > 16) return false;
     if (B <= 4) return !(K > 256 && K <= 512 && N >= 9216) && !(B == 1 && K > 10240 && N <= 2304);
     const DeviceInfo *di = device_info();
     if (!di || K <= 1024) return false;
-    const Split t = split_tiles(N, K, di->device, sms, 0);
-    if ((t.csize == 3 || t.csize == 5) && (N + 255) / 256 >= clusters_that_fit(di->device, t.csize, sms) - 1) return false;
+    Split t = split_tiles(N, K, di->device, sms, 0);
+    const bool crowded = (t.csize == 3 || t.csize == 5) && (N + 255) / 256 >= clusters_that_fit(di->device, t.csize, sms, t.sure) - 1;
+    if (sure) *sure = t.sure;
+    if (crowded) return false;
     const double mb = (double)N * (double)K * 0.5625e-6;
     const double here = (B <= 8 ? 4.29 + 0.507 * t.steps + 0.0778 * mb : 5.62 + 0.736 * t.steps + 0.0704 * mb) + (t.csize > 1 ? 1.42 : 0.0);
     const double there = 1.87 + 2.75 * decode_tc_slices(N, K) + 0.033 * mb;
