@@ -429,20 +429,32 @@ def _nvfp4_ws_need(w: DQWeights, device, B: int) -> int:
     return need
 
 
+def _borrow(nbytes: int, device):
+    """A workspace from torch's allocator on the current stream, None where it has none: the call does without."""
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        return None
+
+
 def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
     """That workspace, from torch's allocator on the call's stream; None where there is none."""
     need = _nvfp4_ws_need(w, X.device, B)
-    if not need or (stream is not None and int(stream.cuda_stream) != _current_stream_ptr()):
+    if not need:
         return None
-    try:
-        return torch.empty(need, dtype=torch.uint8, device=X.device)
-    except torch.OutOfMemoryError:           # the call does without
-        return None
+    if stream is None or int(stream.cuda_stream) == _current_stream_ptr():
+        return _borrow(need, X.device)
+    if not isinstance(stream, torch.cuda.Stream):        # another library's: torch knows it by its address
+        p = int(stream.cuda_stream)
+        stream = torch.cuda.ExternalStream(p, device=X.device) if p else torch.cuda.default_stream(X.device)
+    with torch.cuda.stream(stream):
+        return _borrow(need, X.device)
 
 
 def decode_linear_nvfp4(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
     """dq_decode_linear_nvfp4: Y = X @ NVFP4(W)^T (weight-only NVFP4A16), bf16 out, batch 1..64.  From 5 to 16 columns torch's allocator
-    lends a workspace for the call where that makes it faster (dq_decode_linear_nvfp4_ws)."""
+    lends a workspace on the call's stream where that makes it faster (dq_decode_linear_nvfp4_ws), also with `out` given.  Where torch has no memory
+    left the call does without: another kernel, the same products, sums that may round differently."""
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     B = X.shape[0]
     if out is None:

@@ -181,7 +181,7 @@ def test_fp4_decode_workspace_arguments_and_graphs(dq):  # noqa: F811
         with torch.cuda.stream(streams[i % 3]):
             outs.append(dq.decode_linear_nvfp4(w, X[:5 + i % 3 * 4]))
     torch.cuda.synchronize()
-    other = dq.decode_linear_nvfp4(w, X, stream=streams[0])  # another stream than the current one: no borrowed workspace
+    other = dq.decode_linear_nvfp4(w, X, stream=streams[0])  # another stream than the current one: it is borrowed there
     torch.cuda.synchronize()
     _status_ok(dq)
     _check(other, X, Wd, "explicit stream")
@@ -189,3 +189,31 @@ def test_fp4_decode_workspace_arguments_and_graphs(dq):  # noqa: F811
         n = 5 + i % 3 * 4
         assert torch.equal(Y, outs[i % 3]) and Y.shape[0] == n
         _check(Y, X[:n], Wd, f"stream {i % 3}")
+
+
+class _ForeignStream:
+    def __init__(self, cuda_stream):
+        self.cuda_stream = cuda_stream
+
+
+def test_fp4_decode_same_bits_on_every_stream(dq):  # noqa: F811
+    """A call gives the same bits on the current stream, on another of torch's, on one that torch knows by its address alone and on the
+    default one; what it borrows belongs to the stream that it runs on."""
+    g, w, Wd = _pack(dq, 28672, 4096, 8)
+    assert dq.decode_nvfp4_workspace_bytes(w, 8) > 0
+    X = torch.randn(8, 4096, generator=g, device=DEV).to(torch.bfloat16)
+    Y0 = dq.decode_linear_nvfp4(w, X)
+    assert not torch.equal(Y0, dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=5)) and not torch.equal(Y0, dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=6))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    outs = []
+    for _ in range(4):
+        for s in (side, _ForeignStream(side.cuda_stream), _ForeignStream(0), torch.cuda.default_stream()):
+            outs.append(dq.decode_linear_nvfp4(w, X, stream=s))
+        with torch.cuda.stream(side):
+            outs.append(dq.decode_linear_nvfp4(w, X, stream=_ForeignStream(0)))
+            outs.append(dq.decode_linear_nvfp4(w, X))
+    torch.cuda.synchronize()
+    _status_ok(dq)
+    for Y in outs:
+        assert torch.equal(Y, Y0)
