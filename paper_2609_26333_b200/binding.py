@@ -154,6 +154,8 @@ try:                                     # the same without building a Stream ob
 except ImportError:                      # a build of torch without CUDA
     pass
 
+_capturing = getattr(torch._C, "_cuda_isCurrentStreamCapturing", torch.cuda.is_current_stream_capturing)
+
 
 def _stream_ptr(stream=None) -> int:
     return _current_stream_ptr() if stream is None else int(stream.cuda_stream)
@@ -429,12 +431,20 @@ def _nvfp4_ws_need(w: DQWeights, device, B: int) -> int:
     return need
 
 
+def _of_a_private_pool(t: torch.Tensor) -> bool:
+    p = t.data_ptr()
+    return any(s["address"] <= p < s["address"] + s["total_size"] and tuple(s["segment_pool_id"]) != (0, 0) for s in torch.cuda.memory_snapshot())
+
+
 def _borrow(nbytes: int, device):
-    """A workspace from torch's allocator on the current stream, None where it has none: the call does without."""
+    """A workspace from torch's allocator on the current stream, None where it has none: the call does without.  In a stream capture it has
+    to come from the graph's own pool, as in torch.cuda.graph: in a capture that torch does not know of it would go to somebody else
+    when the call returns, and every replay would write to it."""
     try:
-        return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
     except torch.OutOfMemoryError:
         return None
+    return ws if not _capturing() or _of_a_private_pool(ws) else None
 
 
 def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
@@ -454,7 +464,7 @@ def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
 def decode_linear_nvfp4(w: DQWeights, X: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
     """dq_decode_linear_nvfp4: Y = X @ NVFP4(W)^T (weight-only NVFP4A16), bf16 out, batch 1..64.  From 5 to 16 columns torch's allocator
     lends a workspace on the call's stream where that makes it faster (dq_decode_linear_nvfp4_ws), also with `out` given.  Where torch has no memory
-    left the call does without: another kernel, the same products, sums that may round differently."""
+    left, or does not know that the stream is being captured, the call does without: another kernel, the same products, sums that may round differently."""
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     B = X.shape[0]
     if out is None:

@@ -217,3 +217,48 @@ def test_fp4_decode_same_bits_on_every_stream(dq):  # noqa: F811
     _status_ok(dq)
     for Y in outs:
         assert torch.equal(Y, Y0)
+
+
+def test_fp4_decode_captures_that_torch_does_not_know_of(dq):  # noqa: F811
+    """A graph captured without torch keeps no hold on torch's memory: a call with `out` given may leave nothing of torch's in it.  Whatever
+    torch hands out afterwards stays as it is while the graph is replayed.  (In torch's own captures the workspace is the graph's.)"""
+    runtime = pytest.importorskip("cuda.bindings.runtime")
+    g, w, Wd = _pack(dq, 28672, 4096, 8)
+    X = torch.randn(8, 4096, generator=g, device=DEV).to(torch.bfloat16)
+    need = dq.decode_nvfp4_workspace_bytes(w, 8)
+    assert need > 0
+    out = torch.empty(8, 28672, dtype=torch.bfloat16, device=DEV)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for warm in (True, False):                               # with a free block of that size in torch's hands, and with nothing
+        torch.cuda.empty_cache()
+        with torch.cuda.stream(side):
+            if warm:
+                torch.empty(need, dtype=torch.uint8, device=DEV)
+            ok, = runtime.cudaStreamBeginCapture(side.cuda_stream, runtime.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal)
+            assert int(ok) == 0
+            dq.decode_linear_nvfp4(w, X, out=out)
+            ok, graph = runtime.cudaStreamEndCapture(side.cuda_stream)
+            assert int(ok) == 0
+            ok, exe = runtime.cudaGraphInstantiate(graph, 0)
+            assert int(ok) == 0
+            others = [torch.full((need,), 171, dtype=torch.uint8, device=DEV) for _ in range(4)]
+            out.zero_()
+            for _ in range(2):
+                ok, = runtime.cudaGraphLaunch(exe, side.cuda_stream)
+                assert int(ok) == 0
+        side.synchronize()
+        _status_ok(dq)
+        assert all(bool((t == 171).all()) for t in others)
+        _check(out, X, Wd, "replayed")
+        assert int(runtime.cudaGraphExecDestroy(exe)[0]) == 0 and int(runtime.cudaGraphDestroy(graph)[0]) == 0
+    # torch's own capture: the kernel with a workspace, which stays the graph's
+    Y0 = dq.decode_linear_nvfp4(w, X)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dq.decode_linear_nvfp4(w, X, out=out)
+    others = [torch.full((need,), 171, dtype=torch.uint8, device=DEV) for _ in range(4)]
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, Y0) and all(bool((t == 171).all()) for t in others)

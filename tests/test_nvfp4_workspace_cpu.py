@@ -30,6 +30,7 @@ def test_a_question_without_an_answer_is_asked_again(monkeypatch):
     L = _Library(1, 6, 0)
     monkeypatch.setattr(binding, "lib", lambda: L)
     monkeypatch.setattr(binding, "_nvfp4_ws_known", {})
+    monkeypatch.setattr(binding, "_capturing", lambda: False)
     w, other, X = _handle(), _handle(), torch.empty(8, 2048)
     lent = [binding._lent_workspace(w, X, 8, None) for _ in range(4)]
     assert [None if t is None else t.numel() for t in lent] == [None, None, 4096, 4096]
