@@ -401,11 +401,12 @@ def decode_nvfp4_workspace_bytes(w: DQWeights, B: int, any: bool = False) -> int
 def decode_linear_nvfp4_ws(w: DQWeights, X: torch.Tensor, workspace: torch.Tensor, out: torch.Tensor = None, stream=None) -> torch.Tensor:
     """dq_decode_linear_nvfp4_ws: decode_linear_nvfp4, 5 to 16 columns, on the caller's workspace."""
     assert X.is_cuda and X.dtype == torch.bfloat16 and X.dim() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
+    assert workspace.is_cuda and workspace.is_contiguous()
     B = X.shape[0]
     if out is None:
         out = torch.empty(B, w.N, dtype=torch.bfloat16, device=X.device)
     _check(lib().dq_decode_linear_nvfp4_ws(w.handle, X.data_ptr(), B, X.stride(0), out.data_ptr(), out.stride(0), workspace.data_ptr(),
-                                           workspace.numel(), _stream_ptr(stream)), "dq_decode_linear_nvfp4_ws")
+                                           workspace.numel() * workspace.element_size(), _stream_ptr(stream)), "dq_decode_linear_nvfp4_ws")
     return out
 
 

@@ -262,3 +262,15 @@ def test_fp4_decode_captures_that_torch_does_not_know_of(dq):  # noqa: F811
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, Y0) and all(bool((t == 171).all()) for t in others)
+
+
+def test_fp4_decode_workspace_is_memory_of_its_size(dq):  # noqa: F811
+    """A workspace whose elements do not lie one after the other, or that is not on the GPU, is refused; its size counts in bytes."""
+    g, w, Wd = _pack(dq, 512, 512, 3)
+    X = torch.randn(9, 512, generator=g, device=DEV).to(torch.bfloat16)
+    need = dq.decode_nvfp4_workspace_bytes(w, 9, True)
+    for ws in (torch.empty(1, dtype=torch.uint8, device=DEV).expand(need), torch.empty(2 * need, dtype=torch.uint8, device=DEV)[::2],
+               torch.empty(need, dtype=torch.uint8)):
+        with pytest.raises(AssertionError):
+            dq.decode_linear_nvfp4_ws(w, X, ws)
+    _check(dq.decode_linear_nvfp4_ws(w, X, torch.empty((need + 3) // 4, dtype=torch.float32, device=DEV)), X, Wd, "fp32 workspace")
