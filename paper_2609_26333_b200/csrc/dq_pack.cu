@@ -210,21 +210,21 @@ __device__ __forceinline__ float ffma_sat(float a, float b, float c)
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// appends the level of y to a number in base 16
-__device__ __forceinline__ float push_level(float acc, float y, const float2 *bins, uint32_t lane8)
+// appends the level of y, or of -y for sign = -1, to a number in base 16
+__device__ __forceinline__ float push_level(float acc, float y, float sign, const float2 *bins, uint32_t lane8)
 {
-    const float place = ffma_sat(y, 1.0f / kBinSpan, 0.5f);
+    const float place = ffma_sat(y, sign / kBinSpan, 0.5f);
     const uint32_t at = (__float_as_uint(__fmaf_rn(place, (float)(256 * (kBins - 1)), 8388608.0f)) & (uint32_t)(256 * (kBins - 1))) | lane8;
     const float2 e = *reinterpret_cast<const float2 *>(reinterpret_cast<const uint8_t *>(bins) + at);
-    return __fadd_rn(__fmaf_rn(acc, 16.0f, e.x), ffma_sat(y, kCmpScale, e.y));
+    return __fadd_rn(__fmaf_rn(acc, 16.0f, e.x), ffma_sat(y, sign * kCmpScale, e.y));
 }
 // The same by comparing with every threshold, for codebooks with two of them in a bin: T - y is negative exactly where y > T.
 template <int N>
-__device__ __forceinline__ float push_level_all(float acc, float y, const float (&T)[N])
+__device__ __forceinline__ float push_level_all(float acc, float y, float sign, const float (&T)[N])
 {
     uint32_t n = 0;
 #pragma unroll
-    for (int l = 0; l < N; ++l) n += __float_as_uint(__fsub_rn(T[l], y)) >> 31;
+    for (int l = 0; l < N; ++l) n += __float_as_uint(__fmaf_rn(y, -sign, T[l])) >> 31;
     return __fmaf_rn(acc, 16.0f, (float)n);
 }
 
@@ -372,18 +372,18 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
                                  : "r"(ring + cstage + (uint32_t)(g * kRow + (c ^ swizzle(g, c))) * 16u) : "memory");
                 }
             cstage ^= kStage;
-            float rs[2];
+            float rs[2], sign[2];
             uint32_t sc = 0;
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 float mx, mn;                              // largest value and largest of the negated values
                 if (FP32IN) {
-                    mx = mn = -INFINITY;
 #pragma unroll
                     for (int i = 0; i < kPieces; ++i) {
                         const float x0 = __uint_as_float(raw[j][i].x), x1 = __uint_as_float(raw[j][i].y), x2 = __uint_as_float(raw[j][i].z), x3 = __uint_as_float(raw[j][i].w);
-                        mx = fmaxf(mx, fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)));
-                        mn = fmaxf(mn, fmaxf(fmaxf(-x0, -x1), fmaxf(-x2, -x3)));
+                        const float px = fmaxf(fmaxf(x0, x1), fmaxf(x2, x3)), pn = fmaxf(fmaxf(-x0, -x1), fmaxf(-x2, -x3));
+                        mx = i ? fmaxf(mx, px) : px;       // NaN only where all of the block is
+                        mn = i ? fmaxf(mn, pn) : pn;
                     }
                 } else {
                     const uint4 u = raw[j][0], v = raw[j][1];
@@ -392,12 +392,14 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
                     mx = fmaxf(__uint_as_float(hi << 16), __uint_as_float(hi & 0xFFFF0000u));
                     mn = -fminf(__uint_as_float(lo << 16), __uint_as_float(lo & 0xFFFF0000u));
                 }
-                // the LUT scale takes the sign of the block's extreme, and the reciprocal with it: where both signs reach the
-                // magnitude, plus
+                // the LUT scale takes the sign of the block's extreme; where both signs reach the magnitude, plus.  It goes with the reciprocal, but
+                // where there are E2M1 codes too, with the levels' constants: codes have the plain reciprocal (taken back from the codes, it would
+                // leave one on those of a NaN, which come without)
                 const uint32_t d8 = f32_to_e4m3(__fmul_rn(fmaxf(mx, mn), rc6)) & 0x7Fu;
                 const bool neg = LUT && mn > mx;
                 const float rr = rtab[d8];
-                rs[j] = neg ? -rr : rr;
+                rs[j] = neg && !NV ? -rr : rr;
+                sign[j] = neg && NV ? -1.0f : 1.0f;
                 sc |= (neg && d8 ? d8 | 0x80u : d8) << (8 * j);
             }
             const bool zeros = NV && __any_sync(0xffffffffu, !((sc & 0x7Fu) && (sc & 0x7F00u)));
@@ -428,7 +430,7 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
 #pragma unroll
                     for (int n4 = 3; n4 >= 0; --n4) {
                         y[n4] = __fmul_rn(y[n4], rs[j]);
-                        if (LUT) acc[j] = BINNED ? push_level(acc[j], y[n4], bins, (uint32_t)lane * 8u) : push_level_all(acc[j], y[n4], T);
+                        if (LUT) acc[j] = BINNED ? push_level(acc[j], y[n4], sign[j], bins, (uint32_t)lane * 8u) : push_level_all(acc[j], y[n4], sign[j], T);
                     }
                     if (NV) c2[j] = f32x4_to_e2m1x4(y);
                 }
@@ -452,10 +454,10 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
             if (NV) {
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    // the NVFP4 scale has no sign: the codes take it back; under a zero scale they are zeros without a sign
-                    const uint32_t flip = LUT && rs[j] < 0.0f ? 0x88888888u : 0u, keep = zeros && rs[j] == 0.0f ? 0u : 0xFFFFFFFFu;
+                    // under a zero scale: zeros without a sign
+                    const uint32_t keep = zeros && rs[j] == 0.0f ? 0u : 0xFFFFFFFFu;
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) cw[2 * j + i] = (cw[2 * j + i] ^ flip) & keep;
+                    for (int i = 0; i < 2; ++i) cw[2 * j + i] &= keep;
                 }
                 out_codes[wi * 4] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
                 if ((t & 1) == 0) out_sf[wi * 256] = sc4 & 0x7F7F7F7Fu;           // two k atoms of 512 bytes per word group

@@ -65,3 +65,37 @@ def test_pack_lut2_at_thresholds(dq, oracle, fmts):  # noqa: F811
     _status_ok(dq)
     p, s = oracle.quant_lut2(W, 1.0)
     assert np.array_equal(_np(sc), s) and np.array_equal(_np(planes).view(np.uint32), p)
+
+
+@pytest.mark.parametrize("kind", ["nan", "nan blocks", "one nan at the end", "infinity", "subnormal", "zero times a reciprocal beyond fp32"])
+@pytest.mark.parametrize("N,K", [(48, 640), (272, 1152)])
+def test_pack_encodings_do_not_depend_on_their_company(dq, kind, N, K):  # noqa: F811
+    """An encoding has the same bytes whatever else is packed with it, and from fp32 as from bf16, also beside NaN, infinities and zeros that a
+    reciprocal beyond fp32 turns into NaN: their E2M1 code has no sign that a negative block scale could turn round."""
+    g = torch.Generator(device=DEV).manual_seed(N)
+    W = torch.randn(N, K, generator=g, device=DEV) * 0.02
+    blocks = W.view(-1, 16)
+    if kind == "nan":
+        W.view(-1)[torch.randperm(N * K, generator=g, device=DEV)[:N * K // 50]] = float("nan")
+    elif kind == "nan blocks":
+        blocks[::7], blocks[3::11, 5] = float("nan"), float("nan")
+    elif kind == "one nan at the end":
+        blocks[-1, 15], blocks[-1, 3] = float("nan"), -1.0
+    elif kind == "infinity":
+        W.view(-1)[torch.randperm(N * K, generator=g, device=DEV)[:20]] = float("-inf")
+    else:
+        W *= 1e-36 if kind == "subnormal" else 1e-37
+        W.view(-1, 16)[::3, ::2] = 0.0
+    Wb = W.to(torch.bfloat16)
+    assert kind not in ("nan", "nan blocks", "one nan at the end") or torch.isnan(Wb).any()
+    alone = {}
+    for f in (dq.FMT_NVFP4, dq.FMT_LUT3, dq.FMT_LUT2):
+        alone[f] = [t.clone() for t in dq.export_canonical(dq.pack_weights(Wb, formats=f), f)[:2]]
+    for formats in (dq.FMT_NVFP4, dq.FMT_LUT3, dq.FMT_LUT2, dq.FMT_NVFP4 | dq.FMT_LUT3, dq.FMT_NVFP4 | dq.FMT_LUT2, dq.FMT_NVFP4 | dq.FMT_LUT3 | dq.FMT_LUT2):
+        for M in (Wb, Wb.float()):
+            w = dq.pack_weights(M, formats=formats)
+            for f in alone:
+                if formats & f:
+                    codes, scales, _ = dq.export_canonical(w, f)
+                    assert torch.equal(codes, alone[f][0]) and torch.equal(scales, alone[f][1]), (formats, M.dtype, f)
+    _status_ok(dq)
