@@ -190,7 +190,10 @@ __device__ __forceinline__ uint4 quad_transpose(const uint32_t (&v)[4], int t)
 constexpr int kBins = 64;
 constexpr float kBinSpan = 32.0f;                          // places from -16 to 16
 constexpr float kCmpScale = 1152921504606846976.0f;        // 2^60; thresholds are multiples of 2^-25 and at most 65504
-constexpr float kBinSlack = 1e-3f;                         // the place is rounded: by how much a bin may reach beyond its edges (2^-18 at most)
+// By how much a bin may reach beyond its edges: the place is rounded to 1/256 of a bin, so it begins up to 1/512 of one early (9.92e-4), and
+// places and edges are rounded in fp32 (about 2^-24 of the span); a quarter more
+constexpr float kBinReach = kBinSpan / (512.0f * (kBins - 1)), kBinSlack = 1.25f * kBinReach;
+static_assert(kBinSlack > kBinReach + kBinSpan / 4194304.0f && kBinSlack < kBinSpan / (4.0f * (kBins - 1)), "room for the rounding, well inside a bin");
 __host__ __device__ inline float bin_edge(int b) { return ((float)b / (float)(kBins - 1) - 0.5f) * kBinSpan; }
 // thresholds (ascending) below bin b, and the one inside it or +inf; false where it holds more
 __host__ __device__ inline bool bin_entry(const float *T, int n, int b, int &below, float &own)
@@ -473,7 +476,7 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
     }
 }
 
-// Has no bin of the LUT3 codebook more than one threshold?  (Thresholds 0.51 apart never share one; the default codebook's are 1.2 apart.)
+// Has no bin of the LUT3 codebook more than one threshold?  (Thresholds 0.52 apart never share one; the default codebook's are 1.2 apart.)
 static bool pack_bins_fit(const uint16_t *codebook_f16)
 {
     float T[7];

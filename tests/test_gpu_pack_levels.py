@@ -14,6 +14,8 @@ CODEBOOKS = {
     "two in a bin": (-0.3, -0.2, -0.1, 0, 0.1, 0.2, 0.3, 6),
     "one far below the bins": (-300, -3, -1.5, 0, 1, 2.25, 4, 6),
     "two below the bins": (-300, -80, -20, 0, 1, 2.25, 4, 6),
+    "threshold 0.95e-3 below a bin edge": (-4.703125, -2.869140625, -1.369140625, 0, 0.07489013671875, 2.462890625, 4.046875, 6),
+    "threshold 0.97e-3 below a bin edge": (-4.703125, -3.5, -2.470703125, -0.0709228515625, 0, 2.5, 4, 6),
     "subnormal levels": (-3, -2, -2.0 ** -24, 0, 2.0 ** -24, 2, 4, 6),
 }
 
