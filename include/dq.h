@@ -409,8 +409,9 @@ int dq_weights_shape(const dq_weights *w, int64_t *N_host, int64_t *K_host, unsi
  *           the row is too long for it).
  *   format  DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3: the NVFP4A16 decode; variant 0 = what
  *           dq_decode_linear_nvfp4 runs, 1 = the CUDA-core kernel kept for comparison, 8 = the kernel on
- *           the FP4 tensor cores (up to four columns, with warps_per_group CTAs per tile), 5 = the batch
- *           kernel as above, 6 = the mma.sync kernel.
+ *           the FP4 tensor cores (up to four columns, with warps_per_group CTAs per tile and a wait budget of
+ *           wait_cycles), 9 = the same with one bulk copy left out, so that its waits run out as above, 5 = the
+ *           batch kernel as above, 6 = the mma.sync kernel.
  * Other arguments as dq_decode_linear.
  */
 int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int warps_per_group,

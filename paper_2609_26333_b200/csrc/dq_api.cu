@@ -615,7 +615,7 @@ int dq::prefill_linear_rows(const dq_weights *w, const void *A_dev, int64_t M, i
 extern "C" {
 
 static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx, void *Y_dev, int64_t ldy,
-                        void *stream, int variant, int csize = 0, void *ws = nullptr, size_t ws_bytes = 0)
+                        void *stream, int variant, int csize = 0, void *ws = nullptr, size_t ws_bytes = 0, long long wait_cycles = 0)
 {
     if (!valid_handle(w) || !X_dev || !Y_dev) return DQ_ERR_INVALID_ARG;
     if (!has_nvfp4_view(w) || !on_handle_device(w)) return DQ_ERR_INVALID_ARG;
@@ -642,7 +642,9 @@ static int decode_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64
     const dq::DeviceInfo *di = dq::device_info();
     if (!di) return DQ_ERR_CUDA;
     // Rows above 32768 are refused by the mma.sync kernel, as for every batch.
-    const bool fp4 = variant == 8 || (variant == 0 && w->K <= 32768 && B <= 4 && dq::decode_fp4_is_faster(w->N, w->K, B, di->sms));
+    g.wait_cycles = wait_cycles;
+    g.drop_first_copy = variant == 9;
+    const bool fp4 = variant >= 8 || (variant == 0 && w->K <= 32768 && B <= 4 && dq::decode_fp4_is_faster(w->N, w->K, B, di->sms));
     const bool tc = variant == 5 || (variant == 0 && w->K <= 32768 && dq::nvfp4_batch_kernel_is_faster(w->N, w->K, B, di->sms));
     if (fp4) {
         ce = dq::launch_decode_fp4(g, csize, ws, ws_bytes, s);
@@ -748,9 +750,9 @@ int dq_test_decode_linear(const dq_weights *w, unsigned format, int variant, int
                           int64_t ldy, void *stream)
 {
     if (format == DQ_FMT_NVFP4 || format == DQ_FMT_NVFP4_FROM_LUT3) {
-        if (variant != 0 && variant != 1 && variant != 5 && variant != 6 && variant != 8) return DQ_ERR_INVALID_ARG;
-        if (warps_per_group < 0) return DQ_ERR_INVALID_ARG;
-        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 || variant == 8 ? warps_per_group : 0);
+        if (variant != 0 && variant != 1 && variant != 5 && variant != 6 && variant != 8 && variant != 9) return DQ_ERR_INVALID_ARG;
+        if (warps_per_group < 0 || wait_cycles < 0) return DQ_ERR_INVALID_ARG;
+        return decode_nvfp4(w, X_dev, B, ldx, Y_dev, ldy, stream, variant, variant == 5 || variant >= 8 ? warps_per_group : 0, nullptr, 0, wait_cycles);
     }
     if (warps_per_group < 0 || groups_per_cta < 0 || ring_stages < 0 || ring_stages > 8 || wait_cycles < 0)
         return DQ_ERR_INVALID_ARG;

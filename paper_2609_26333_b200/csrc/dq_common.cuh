@@ -272,12 +272,14 @@ struct GemvNvArgs {
     const void *X; int64_t ldx; int64_t B;
     void *Y; int64_t ldy;
     int64_t N, K;
+    long long wait_cycles = 0;                            // decode_fp4_kernel: device-side wait budget, 0 = the default
+    int drop_first_copy = 0;                              // decode_fp4_kernel: the weights of CTA 0's first step are never requested
 };
 cudaError_t launch_gemv_nvfp4(const GemvNvArgs &args, cudaStream_t stream);          // CUDA cores, pair-table lookups
 cudaError_t launch_gemv_nvfp4_mma(const GemvNvArgs &args, cudaStream_t stream);      // tensor cores (mma.sync), no lookups
 bool nvfp4_batch_kernel_is_faster(int64_t N, int64_t K, int64_t B, int sms);
 cudaError_t launch_decode_tc_nvfp4(const GemvNvArgs &args, int force_csize, cudaStream_t stream);     // dq_decode_tc.cu
-// dq_decode_fp4.cu: activations as digits against the stored FP4 matrix, up to 16 columns; above 8 with a workspace for the digits (decode_fp4_workspace
+// dq_decode_fp4.cu: activations as digits against the stored FP4 matrix, up to 16 columns; above 4 with a workspace for the digits (decode_fp4_workspace
 // bytes, 256-byte aligned).  force_csize: CTAs per tile (test hook)
 size_t decode_fp4_workspace(int64_t K);
 cudaError_t launch_decode_fp4(const GemvNvArgs &args, int force_csize, void *ws, size_t ws_bytes, cudaStream_t stream);

@@ -99,6 +99,8 @@ struct Fp4Args {
     uint8_t *digits;             // [steps][X_BYTES]
     uint32_t *group_scale;       // [groups][16 columns] fp32 bits, then the same number of flags: an infinity or a NaN
     int ngroups;
+    long long wait_cycles;
+    int drop_first_copy;         // test hook: the weights of CTA 0's first step are never requested
     StatusWord *status;
 };
 
@@ -250,23 +252,23 @@ __device__ __forceinline__ bool try_park(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity), "r"(20000u) : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ bool wait_one(uint32_t bar, uint32_t parity, volatile int *abort_flag)
+__device__ __forceinline__ bool wait_one(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long budget)
 {
     if (try_park(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
         if (try_park(bar, parity)) return true;
         if (*abort_flag) return false;
-        if (clock64() - t0 > kWaitBudgetCycles) { *abort_flag = 1; return false; }
+        if (clock64() - t0 > budget) { *abort_flag = 1; return false; }
     }
 }
-__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag)
+__device__ __forceinline__ bool wait_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag, long long budget)
 {
     if (__all_sync(0xffffffffu, try_park(bar, parity))) return true;
     const long long t0 = clock64();
     while (true) {
         if (__all_sync(0xffffffffu, try_park(bar, parity))) return true;
-        const bool over = clock64() - t0 > kWaitBudgetCycles;
+        const bool over = clock64() - t0 > budget;
         if (__any_sync(0xffffffffu, over || *abort_flag != 0)) { *abort_flag = 1; return false; }
     }
 }
@@ -343,10 +345,12 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
     if (warp == 0) {
         // -------------------------- weights: constant data, nothing to wait for; digits that the kernel ahead has made
         if (elect_one()) {
+            bool drop = P.drop_first_copy && blockIdx.x == 0;
             auto load_w = [&](int stage, int tile, int ks) {
                 const uint32_t a = ring0 + stage * C::STAGE_BYTES, sf = (uint32_t)min(4, katoms - 4 * ks) * 512u;
                 mbar_expect_tx(full_bar(stage), C::A_BYTES + 2u * sf + (PRE ? C::X_BYTES : 0u));
-                tma_load_2d(a, &tmap_w, ks * 128, tile * 256, full_bar(stage));
+                if (!drop) tma_load_2d(a, &tmap_w, ks * 128, tile * 256, full_bar(stage));
+                drop = false;
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
                     bulk_load(a + C::A_BYTES + h * 2048u, P.w_sf + ((size_t)(tile * 2 + h) * katoms + (size_t)ks * 4) * 512, sf, full_bar(stage));
@@ -367,7 +371,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
                     if (PRE && early > 0) {
                         --early;
                     } else {
-                        ok = wait_one(empty_bar(stage), phase ^ 1u, abort_flag);
+                        ok = wait_one(empty_bar(stage), phase ^ 1u, abort_flag, P.wait_cycles);
                         if (!ok) break;
                         load_w(stage, tile, ks);
                     }
@@ -387,10 +391,10 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
             for (int tile = first_tile; tile < tiles && ok; tile += tile_stride) {
                 int in_group = 0;
                 for (int ks = k0; ks < k1; ++ks, ++it) {
-                    if (in_group == 0) ok = wait_one(dempty_bar(grp), ((grp / C::kAccs) & 1u) ^ 1u, abort_flag);
-                    if (ok && it >= 2) ok = wait_one(empty_bar(before[it & 1u]), before_phase[it & 1u], abort_flag);
-                    if (ok) ok = wait_one(full_bar(stage), phase, abort_flag);
-                    if (!PRE && ok) ok = wait_one(xfull_bar(stage), phase, abort_flag);
+                    if (in_group == 0) ok = wait_one(dempty_bar(grp), ((grp / C::kAccs) & 1u) ^ 1u, abort_flag, P.wait_cycles);
+                    if (ok && it >= 2) ok = wait_one(empty_bar(before[it & 1u]), before_phase[it & 1u], abort_flag, P.wait_cycles);
+                    if (ok) ok = wait_one(full_bar(stage), phase, abort_flag, P.wait_cycles);
+                    if (!PRE && ok) ok = wait_one(xfull_bar(stage), phase, abort_flag, P.wait_cycles);
                     if (!ok) break;
                     tc_fence_after();
                     const int nkb = min(4, katoms - 4 * ks);
@@ -463,7 +467,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
             auto group_end = [&](int ks) { return PRE ? (ks / kGroupSteps + 1) * kGroupSteps : ks + kGroupSteps; };
             // group n of the kernel, of steps from ks, its scales in slot sl: from its accumulator into the running sums
             auto flush = [&](uint32_t n, uint32_t sl, int ks) {
-                if (ok) ok = wait_warp(dfull_bar(n), (n / C::kAccs) & 1u, abort_flag);
+                if (ok) ok = wait_warp(dfull_bar(n), (n / C::kAccs) & 1u, abort_flag, P.wait_cycles);
                 if (!ok) return;
                 tc_fence_after();
                 // the columns' powers of two: lane c has column c's
@@ -518,7 +522,7 @@ decode_fp4_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_const
 #pragma unroll 1
                 for (int s = 0; s < nk; ++s) {
                     const uint4 ahead = piece(kg + kGroupSteps + s);
-                    ok = wait_warp(empty_bar(stage), phase ^ 1u, abort_flag);
+                    ok = wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, P.wait_cycles);
                     if (!ok) break;
                     const uint32_t b = ring0 + stage * C::STAGE_BYTES;
                     if (s == 0 && turn == 0 && lane == 0 && col < P.cols) {
@@ -771,6 +775,8 @@ cudaError_t launch_decode_fp4(const GemvNvArgs &a, int force_csize, void *ws, si
     P.N = (int)a.N;
     P.K = (int)a.K;
     P.csize = 1;
+    P.wait_cycles = a.wait_cycles > 0 ? a.wait_cycles : kWaitBudgetCycles;
+    P.drop_first_copy = a.drop_first_copy;
     P.status = a.status;
     if (a.B <= 4) return launch_ng<1, false>(tmap, P, force_csize, di, stream);
     const WsLayout L = ws_layout(a.K);

@@ -274,3 +274,59 @@ def test_fp4_decode_workspace_is_memory_of_its_size(dq):  # noqa: F811
         with pytest.raises(AssertionError):
             dq.decode_linear_nvfp4_ws(w, X, ws)
     _check(dq.decode_linear_nvfp4_ws(w, X, torch.empty((need + 3) // 4, dtype=torch.float32, device=DEV)), X, Wd, "fp32 workspace")
+
+
+@pytest.mark.parametrize("B", [5, 8, 9, 13, 16])
+@pytest.mark.parametrize("tiles", [74, 68, 49, 45, 36, 29, 24, 21, 18, 9])
+def test_fp4_decode_clusters_with_a_workspace(dq, tiles, B):  # noqa: F811
+    """Clusters of every size that tiles of these numbers can share, with one and with two times four columns to add up for each CTA of a
+    cluster, and groups that a CTA's share of the row cuts."""
+    for K in (2304, 4352):
+        N = tiles * 256 - 112
+        g, w, Wd = _pack(dq, N, K, tiles)
+        X = torch.randn(B, K, generator=g, device=DEV).to(torch.bfloat16)
+        Y = _call(dq, w, X)
+        _status_ok(dq)
+        _check(Y, X, Wd, f"{N}x{K} batch {B}")
+        assert torch.equal(Y, _call(dq, w, X))
+
+
+@pytest.mark.parametrize("B", [4, 16])
+@pytest.mark.parametrize("K", [2048, 16384])
+def test_fp4_decode_digits_larger_than_their_sum(dq, K, B):  # noqa: F811
+    """Activations just above half a digit beside larger ones, so that a value's digits add up to three times its magnitude, with sums that
+    cancel: inside the allowance of the other kernels, and no worse than the mma.sync and the batch kernel (2.9e-8 to 7.4e-8 of the sum of
+    magnitudes beyond the rounding to bf16, for 0 to 1.2e-7 of theirs)."""
+    N = 1024
+    g = torch.Generator(device=DEV).manual_seed(K)
+    half = (torch.randn(N, K // 2, generator=g, device=DEV) * 0.02).abs()
+    w = dq.pack_weights(torch.cat((half, -half), dim=1).to(torch.bfloat16), formats=dq.FMT_NVFP4)
+    Wd = _dequantised(dq, w, "nvfp4")
+    x = 0.5 + 2.0 ** -8 * torch.randint(1, 4, (B, K // 2), generator=g, device=DEV).float()
+    x[:, ::16] = 3.0
+    X = torch.cat((x, x), dim=1)
+    X[:, K // 2 + 5::16] += 2.0 ** -8                       # leaves a small sum
+    X = X.to(torch.bfloat16)
+    Y = _call(dq, w, X)
+    _status_ok(dq)
+    Yr, S = X.double() @ Wd.T, X.double().abs() @ Wd.abs().T
+    assert float((Yr.abs() / S).max()) < 1e-2               # they do cancel
+    ulp = torch.exp2(torch.floor(torch.log2(Yr.abs().clamp_min(2.0 ** -126))) - 7)
+    over = ((Y.double() - Yr).abs() - 0.5 * ulp) / S
+    assert float(over.max()) < 3e-7                         # four times the most that was seen
+
+
+@pytest.mark.parametrize("N,K,csize", [(1024, 4096, 1), (1024, 4096, 4), (40000, 512, 0)])
+@pytest.mark.parametrize("B", [1, 4])
+def test_fp4_decode_wait_runs_out(dq, N, K, csize, B):  # noqa: F811
+    """Weights that are never requested: the waits run out in every role, the clusters' barriers are met, the launch returns and reports, and
+    the next call is right."""
+    g, w, Wd = _pack(dq, N, K, 9)
+    X = torch.randn(B, K, generator=g, device=DEV).to(torch.bfloat16)
+    good = dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=FP4, warps_per_group=csize)
+    dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=9, warps_per_group=csize, wait_cycles=2_000_000)
+    torch.cuda.synchronize()
+    st, _ = dq.get_status()
+    assert dq.status_string(st) == "device-side wait ran out"
+    assert torch.equal(dq.test_decode_linear(w, dq.FMT_NVFP4, X, variant=FP4, warps_per_group=csize, wait_cycles=2_000_000), good)
+    _status_ok(dq)
