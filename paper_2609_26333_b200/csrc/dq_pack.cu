@@ -213,13 +213,13 @@ __device__ __forceinline__ float ffma_sat(float a, float b, float c)
     asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
-// appends the level of y, or of -y for sign = -1, to a number in base 16
-__device__ __forceinline__ float push_level(float acc, float y, float sign, const float2 *bins, uint32_t lane8)
+// appends the level of y, or of -y for per_bin = -1 / kBinSpan, to a number in base 16
+__device__ __forceinline__ float push_level(float acc, float y, float per_bin, const float2 *bins, uint32_t lane8)
 {
-    const float place = ffma_sat(y, sign / kBinSpan, 0.5f);
+    const float place = ffma_sat(y, per_bin, 0.5f);
     const uint32_t at = (__float_as_uint(__fmaf_rn(place, (float)(256 * (kBins - 1)), 8388608.0f)) & (uint32_t)(256 * (kBins - 1))) | lane8;
     const float2 e = *reinterpret_cast<const float2 *>(reinterpret_cast<const uint8_t *>(bins) + at);
-    return __fadd_rn(__fmaf_rn(acc, 16.0f, e.x), ffma_sat(y, sign * kCmpScale, e.y));
+    return __fadd_rn(__fmaf_rn(acc, 16.0f, e.x), ffma_sat(y, per_bin * (kBinSpan * kCmpScale), e.y));
 }
 // The same by comparing with every threshold, for codebooks with two of them in a bin: T - y is negative exactly where y > T.
 template <int N>
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
                 const bool neg = LUT && mn > mx;
                 const float rr = rtab[d8];
                 rs[j] = neg && !NV ? -rr : rr;
-                sign[j] = neg && NV ? -1.0f : 1.0f;
+                sign[j] = (BINNED ? 1.0f / kBinSpan : 1.0f) * (neg && NV ? -1.0f : 1.0f);
                 sc |= (neg && d8 ? d8 | 0x80u : d8) << (8 * j);
             }
             const bool zeros = NV && __any_sync(0xffffffffu, !((sc & 0x7Fu) && (sc & 0x7F00u)));
@@ -458,9 +458,7 @@ __global__ void __launch_bounds__(256, pack_ctas(FP32IN)) pack_kernel(const void
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
                     // under a zero scale: zeros without a sign
-                    const uint32_t keep = zeros && rs[j] == 0.0f ? 0u : 0xFFFFFFFFu;
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) cw[2 * j + i] &= keep;
+                    if (zeros && rs[j] == 0.0f) cw[2 * j] = cw[2 * j + 1] = 0u;
                 }
                 out_codes[wi * 4] = make_uint4(cw[0], cw[1], cw[2], cw[3]);
                 if ((t & 1) == 0) out_sf[wi * 256] = sc4 & 0x7F7F7F7Fu;           // two k atoms of 512 bytes per word group
