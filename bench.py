@@ -39,7 +39,7 @@ L2_BYTES = 126 * 1024 * 1024
 NCU_TRAFFIC_BYTES = {
     ("gemm", "c3_gate_up27b"): 78.91e6 + 239.8e6,     # gemm_nvfp4_pair_kernel, full size (one-pass launch list)
     ("gemv", "c3_gate_up27b"): 39.04e6,               # gemv_lut_kernel<3, 640, 1, 1, true>, full size, batch 1 (reads; writes are 35 KB)
-    ("gemv_nvfp4", "c3_gate_up27b"): 50.19e6,         # gemv_nvfp4_mma_kernel<640, 3>, full size (one-pass launch list)
+    ("gemv_nvfp4", "c3_gate_up27b"): 50.20e6,         # decode_fp4_kernel<1, false>, full size, batch 1
 }
 NOMINAL_FP4_TFLOPS = 9000.0                            # dense FP4, 4 x the 2250 TFLOP/s bf16 figure
 NOMINAL_HBM_GBS = 8000.0
@@ -731,10 +731,10 @@ def main():
                             "decode_ms_x_sm_mhz": d_ms * sm_mhz if sm_mhz else None},
     }
     nv_bytes = 0.5625 * N * K + 2.0 * B * (K + N)
-    line["roofline_decode_nvfp4a16"] = {"kernel": "gemv_nvfp4_mma_kernel", "bound": "hbm",
+    line["roofline_decode_nvfp4a16"] = {"kernel": "decode_fp4_kernel" if B <= 4 else "by models: decode_fp4_kernel, decode_tc_kernel, gemv_nvfp4_mma_kernel", "bound": "hbm",
                                         "achieved": nv_bytes / (d_nv_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                                         "frac": nv_bytes / (d_nv_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
-                                        "traffic": NCU_TRAFFIC_BYTES.get(("gemv_nvfp4", cfg.name)),
+                                        "traffic": NCU_TRAFFIC_BYTES.get(("gemv_nvfp4", cfg.name)) if B == 1 else None,
                                         "timing": "back-to-back launches replayed from one CUDA graph", "peak_source": f"{peaks['source']} copy bandwidth"}
     line["roofline_decode"]["back_to_back"] = {"achieved": dec_bytes / (d_b2b_ms * 1e-3) / 1e9,
                                                "frac": dec_bytes / (d_b2b_ms * 1e-3) / 1e9 / peaks["hbm_gbs"],

@@ -299,7 +299,7 @@ int dq_decode_linear_host(const dq_weights *w, const void *X_host, int64_t B, in
  *   DQ_FMT_NVFP4 / DQ_FMT_NVFP4_FROM_LUT3:
  *     codes  uint8[N][K/2]  element 2j in the low nibble, 2j+1 in the high nibble,
  *            code = sign<<3 | index into {0,.5,1,1.5,2,3,4,6} (App. A.3 "NVFP4")
- *     scales uint8[N][K/16] E4M3
+ *     scales uint8[N][K/16] E4M3, magnitudes: the top bit is 0
  *   DQ_FMT_LUT3 (b = 3) / DQ_FMT_LUT2 (b = 2):
  *     codes  uint32[N][b][K/32] bit-planes (App. C.2): bit i (LSB = 0) of word j of
  *            plane p is bit p of the index of weight 32*j + i

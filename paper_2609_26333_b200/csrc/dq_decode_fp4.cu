@@ -726,6 +726,8 @@ cudaError_t launch_ng(const CUtensorMap &tmap, Fp4Args P, int force_csize, const
 // columns on, with the workspace: 4.3 (5.6 above eight) for both launches, 0.51 (0.74) a step of the busiest CTA, 0.078 (0.070) a megabyte, 1.4 for a
 // cluster's exchange, against 1.9, 2.75 a slice of 512 and 0.033 a megabyte; its second launch costs the host 3, so that short calls stay
 // (1536x8192 batch 8 9.4 / 8.7); clusters of three or five that crowd the chip wait for a free group of SMs (11408x11776 batch 9 27.4 / 33.9).
+// The mma.sync kernel is not in it: where this one is taken for five to eight columns it is never the faster (144 points; 23600x10240 batch 5: mma.sync 39.4,
+// batch kernel 56.4, this one 28.6).
 // sure = false: the answer rests on one that the runtime did not give
 bool decode_fp4_is_faster(int64_t N, int64_t K, int64_t B, int sms, bool *sure)
 {
