@@ -430,9 +430,14 @@ def _nvfp4_ws_need(w: DQWeights, device, B: int) -> int:
     return need
 
 
-def _of_a_private_pool(t: torch.Tensor) -> bool:
+def _of_the_graph(t: torch.Tensor) -> bool:
+    """Whether memory from torch, taken in a capture, is the graph's: of a private pool, or, with the driver's allocator, a node of the graph."""
     p = t.data_ptr()
-    return any(s["address"] <= p < s["address"] + s["total_size"] and tuple(s["segment_pool_id"]) != (0, 0) for s in torch.cuda.memory_snapshot())
+    try:
+        segments = torch.cuda.memory_snapshot()
+    except RuntimeError:                 # an allocator that has none
+        return torch.cuda.get_allocator_backend() == "cudaMallocAsync"
+    return any(s["address"] <= p < s["address"] + s["total_size"] and tuple(s.get("segment_pool_id", (0, 0))) != (0, 0) for s in segments)
 
 
 def _borrow(nbytes: int, device):
@@ -443,7 +448,7 @@ def _borrow(nbytes: int, device):
         ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
     except torch.OutOfMemoryError:
         return None
-    return ws if not _capturing() or _of_a_private_pool(ws) else None
+    return ws if not _capturing() or _of_the_graph(ws) else None
 
 
 def _lent_workspace(w: DQWeights, X: torch.Tensor, B: int, stream):
