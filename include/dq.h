@@ -243,7 +243,8 @@ int dq_decode_linear_lut2(const dq_weights *w, const void *X_dev, int64_t B, int
  * this mat-vec):
  *   Y[b][n] = bf16( sum_k X[b][k] * W^[n][k] ),  W^ = s * d_b * e2m1(code),
  * raw bf16 activations, fp32 accumulation.  Needs DQ_FMT_NVFP4 or DQ_FMT_NVFP4_FROM_LUT3 in the
- * handle (DQ_ERR_INVALID_ARG otherwise).  Arguments and limits as dq_decode_linear; products d_b * e2m1 * x are exact,
+ * handle (DQ_ERR_INVALID_ARG otherwise).  Arguments and limits as dq_decode_linear; products d_b * e2m1 * x are exact
+ * (up to four columns for activations within 2^27 of the largest of their 16-element block, smaller ones being rounded to 2^-35 of it),
  * summed in fp32 along K.
  */
 int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, int64_t ldx,
@@ -253,7 +254,7 @@ int dq_decode_linear_nvfp4(const dq_weights *w, const void *X_dev, int64_t B, in
  * The same decode, 5 to 16 columns, with a workspace of the caller's: the activations are written to it as FP4 digits and meet the
  * stored matrix on the block-scaled tensor cores as it is, without dequantising.  (Up to four columns dq_decode_linear_nvfp4 does so
  * without a workspace.)  Same products: an activation is held exactly within 2^27 of the largest of its 16-element block and rounded to
- * 2^-35 of that below; summed in fp32 along K.
+ * 2^-35 of that below; summed in fp32 along K.  The sums may round differently from those of dq_decode_linear_nvfp4 at the same batch.
  *   dq_decode_nvfp4_workspace_bytes  bytes that B columns need; 0 where dq_decode_linear_nvfp4 is the faster call or all there is
  *                                    (any != 0: also where it is the faster one)
  *   workspace_dev  256-byte aligned device memory, scratch of this call alone until the stream has passed it;
